@@ -605,6 +605,11 @@ int plan_geom(const Request &q, const double lo[3], const double hi[3], long lon
         g.ncy = std::max(1, g.ncy / 2);
     }
     cap_columns(ntot, g.ncx, g.ncy);
+    // padded entries are indexed with 32-bit integers
+    while ((long long)g.ncx * g.ncy > 1 && ntot + 31ll * g.ncx * g.ncy > (1ll << 31) - 64) {
+        g.ncx = std::max(1, g.ncx / 2);
+        g.ncy = std::max(1, g.ncy / 2);
+    }
     g.ncols = g.ncx * g.ncy;
     g.reach_x = rx;
     g.reach_y = ry;
@@ -741,6 +746,8 @@ int run(Request &q)
     unsigned *d_err = nullptr, *d_ctr = nullptr, *d_wcount = nullptr;
     cf::WorkItem *work = nullptr;
     cf::Win *wins = nullptr;
+    cf::Nbr *nbr = nullptr;
+    unsigned *nbr_count = nullptr;
     long long win_cap = 0;
     long long *wscratch = nullptr;
     unsigned long long *d_hist = nullptr, *d_diag = nullptr;
@@ -861,10 +868,12 @@ int run(Request &q)
             bump.base = pass ? (char *)ws2 : nullptr;
             bump.off = 0;
             for (int t = 0; t < ncat; ++t) {
-                const long long n = cats[t]->n + 3ll * g.ncols;  // columns padded to 4
+                const long long n = cf::padded_max(cats[t]->n, g.ncols);
                 G[t].xs = bump.take<float>(n);
                 G[t].ys = bump.take<float>(n);
                 G[t].zs = bump.take<float>(n);
+                G[t].xyz = bump.take<float>(3 * n);
+                G[t].chunk_col = bump.take<int>(n / cf::COL_PAD);
                 G[t].ws = c->weighted ? bump.take<float>(n + 64) : nullptr;  // + slack for tile reads
                 if (resid) {  // float32 mean separation from inputs float32 cannot hold exactly
                     G[t].xl = bump.take<float>(n + 64);
@@ -879,15 +888,17 @@ int run(Request &q)
             }
             tmp.cell_of = bump.take<uint32_t>(nmax);
             tmp.slot = bump.take<uint32_t>(nmax);
-            tmp.tmp_idx = bump.take<int>(nmax + 3ll * g.ncols);
-            tmp.tmp_key = bump.take<unsigned long long>(nmax + 3ll * g.ncols);
+            tmp.tmp_idx = bump.take<int>(cf::padded_max(nmax, g.ncols));
+            tmp.tmp_key = bump.take<unsigned long long>(cf::padded_max(nmax, g.ncols));
             tmp.counts = bump.take<uint32_t>(g.ncells + 1);
             tmp.pad = bump.take<uint32_t>(g.ncols);
             tmp.bsum = bump.take<uint32_t>(g.ncells / 4096 + 2);
+            const int sx = 2 * g.reach_x + 1, sy = 2 * g.reach_y + 1;
+            const int nst = q.autocorr ? (sx * sy + 1) / 2 : sx * sy;
+            nbr = bump.take<cf::Nbr>((size_t)g.ncols * nst);
+            nbr_count = bump.take<unsigned>(g.ncols);
             work = bump.take<cf::WorkItem>((size_t)g.ncols * cf::MAX_STENCIL);
-            if (q.kind == 0 && !f64) {  // window records of the float32 DD(r) kernels
-                const int sx = 2 * g.reach_x + 1, sy = 2 * g.reach_y + 1;
-                const int nst = q.autocorr ? (sx * sy + 1) / 2 : sx * sy;
+            if (q.kind == 0 && !f64 && wacc) {  // window records of the weighted float32 DD(r) kernels
                 const int ch = cf::xi32_chunk(c->pair_chunk ? c->pair_chunk : 16,
                                               c->pair_pp ? c->pair_pp : 2, wacc,
                                               (c->flags & CF_FLAG_VERIFY_BAND) != 0);
@@ -921,6 +932,8 @@ int run(Request &q)
         double M = 0.0, Ls = 0.0;
         base_params(q, g, G[0], G[1], P, M, Ls);
         P.work = work;
+        P.nbr = nbr;
+        P.nbr_count = nbr_count;
         P.win = wins;
         P.win_cap = win_cap;
         P.win_count = d_err + 3;  // zeroed with the result block
@@ -967,7 +980,6 @@ int run(Request &q)
         PL.evals = (c->flags & (CF_FLAG_COUNT_EVALS | CF_FLAG_VERIFY_BAND)) ? 1 : 0;
         PL.verify = (!f64 && (c->flags & CF_FLAG_VERIFY_BAND)) ? 1 : 0;
         PL.max_blocks = wscratch ? sms * 2 : 0;
-        PL.pipe = 1;
         cf::plan_pairs(P, PL);
         if (!f64 && PL.smem > cf::SMEM_MAX) {
             // float32 weighted rows for this many bins exceed shared memory: count
@@ -1728,9 +1740,8 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     cf::Gridded G[2] = {};
     cf::GridTemps tmp = {};
     cf::WorkItem *work = nullptr;
-    cf::Win *wins = nullptr;
-    long long win_cap = 0;
-    const int win_ch = cf::xi32_chunk(16, 2, false, false);  // the kernel shape of this entry point
+    cf::Nbr *nbr = nullptr;
+    unsigned *nbr_count = nullptr;
     // Carve the grids, temporaries and the work list for the current geometry
     // out of the array; if they do not fit, plan coarser (columns at least
     // Rmax / refine wide stay correct at any width, and fewer z-cells only make
@@ -1740,11 +1751,13 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
         g.ncells = (long long)g.ncols * g.nz;
         Bump b = bump;
         for (int t = 0; t < ncat; ++t) {
-            const long long n = cats[t]->n + 3ll * g.ncols;  // columns padded to 4
+            const long long n = cf::padded_max(cats[t]->n, g.ncols);
             G[t] = cf::Gridded{};
             G[t].xs = b.take<float>(n);
             G[t].ys = b.take<float>(n);
             G[t].zs = b.take<float>(n);
+            G[t].xyz = b.take<float>(3 * n);
+            G[t].chunk_col = b.take<int>(n / cf::COL_PAD);
             G[t].pos64 = b.take<double4_32a>(n);
             G[t].perm = b.take<int>(n);
             G[t].cell_start = b.take<uint32_t>(g.ncells + 1);
@@ -1752,14 +1765,14 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
         }
         tmp.cell_of = b.take<uint32_t>(nmax);
         tmp.slot = b.take<uint32_t>(nmax);
-        tmp.tmp_idx = b.take<int>(nmax + 3ll * g.ncols);
-        tmp.tmp_key = b.take<unsigned long long>(nmax + 3ll * g.ncols);
+        tmp.tmp_idx = b.take<int>(cf::padded_max(nmax, g.ncols));
+        tmp.tmp_key = b.take<unsigned long long>(cf::padded_max(nmax, g.ncols));
         tmp.counts = b.take<uint32_t>(g.ncells + 1);
         tmp.pad = b.take<uint32_t>(g.ncols);
         tmp.bsum = b.take<uint32_t>(g.ncells / 4096 + 2);
         work = b.take<cf::WorkItem>((size_t)g.ncols * nstencil_max);
-        win_cap = f64 ? 0 : cf::win_bound(cats[0]->n, g.ncols, nstencil_max, win_ch);
-        wins = f64 ? nullptr : b.take<cf::Win>((size_t)win_cap);
+        nbr = b.take<cf::Nbr>((size_t)g.ncols * nstencil_max);
+        nbr_count = b.take<unsigned>(g.ncols);
         if (b.off <= NOALLOC_BYTES) {
             bump = b;
             break;
@@ -1809,9 +1822,8 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     P.n_items = g.ncols * P.nstencil;
     P.work = work;
     P.work_count = d_ctr + 1;
-    P.win = wins;
-    P.win_cap = win_cap;
-    P.win_count = d_ctr + 2;
+    P.nbr = nbr;
+    P.nbr_count = nbr_count;
     P.tile_max = 1024;
     P.flags = c->flags & (CF_FLAG_NO_PRUNE | CF_FLAG_COUNT_EVALS);
     P.wait_ns = wait_limit_ns(P.flags);
@@ -1855,7 +1867,6 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     PL.chunk = 16;
     PL.pp = 2;
     PL.evals = (P.flags & CF_FLAG_COUNT_EVALS) ? 1 : 0;
-    PL.pipe = 1;
     cf::plan_pairs(P, PL);
     if (P.n_items > 0 && (e = cf::launch_pairs(P, PL, sms, st)))
         return cuda_fail(e, "pair kernel launch");
@@ -2188,12 +2199,14 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
         for (int k = 0; k < nj; ++k) {
             BatchJob &j = b->jobs[k];
             for (int t = 0; t < j.ncat; ++t, ++q) {
-                const long long n = j.cat[t].n + 3ll * j.g.ncols;
+                const long long n = cf::padded_max(j.cat[t].n, j.g.ncols);
                 cf::Gridded &G = j.G[t];
                 G.n = j.cat[t].n;
                 G.xs = bump.take<float>(n);
                 G.ys = bump.take<float>(n);
                 G.zs = bump.take<float>(n);
+                G.xyz = bump.take<float>(3 * n);
+                G.chunk_col = bump.take<int>(n / cf::COL_PAD);
                 G.ws = nullptr;
                 G.pos64 = bump.take<double4_32a>(n);
                 G.perm = bump.take<int>(n);

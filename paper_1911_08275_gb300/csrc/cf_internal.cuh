@@ -47,13 +47,6 @@ constexpr int XI32_THR_OFF = XI32_TX_OFF + 3 * XI32_TSTRIDE;
 constexpr int XI32_E2_OFF = XI32_THR_OFF + 2 * (NB_MAX + 1) * 4;
 constexpr int XI32_HIST_OFF = XI32_E2_OFF + (NB_MAX + 1) * 8;
 
-// The pipelined float32 DD(r) kernel keeps one histogram copy shared by all
-// warps and places its second tile buffer after it.
-__host__ __device__ constexpr int pipe_slot1_off(int nbins)
-{
-    return (XI32_HIST_OFF + (nbins + 2) * 128 + 127) & ~127;
-}
-
 // The weighted float32 DD(rp, pi) kernel stages a weight tile after the squared
 // edges.
 constexpr int XIW_W_OFF = XI32_HIST_OFF;
@@ -83,17 +76,36 @@ struct Geom {
     int box_bits32[3];      // bits of the smallest float >= box (float32 inputs)
 };
 
-// A gridded catalogue, in (column, z, original index) order; every column is
-// padded with NaN entries to a multiple of 4 (see grid.cu).
+// Every column of a gridded catalogue is padded with NaN entries to a multiple
+// of this (see grid.cu).
+constexpr unsigned COL_PAD = 32;
+
+// Entries of a gridded catalogue of n points on ncols columns, at most.
+__host__ __device__ inline long long padded_max(long long n, int ncols)
+{
+    return (n + (COL_PAD - 1ll) * ncols + COL_PAD - 1) / COL_PAD * COL_PAD;
+}
+
+// Offset of entry d in the quad layout (x0..x3, y0..y3, z0..z3 per four
+// entries): its x; y and z are 4 and 8 floats further.
+__host__ __device__ __forceinline__ size_t quad_off(uint32_t d)
+{
+    return (size_t)(d >> 2) * 12u + (d & 3u);
+}
+
+// A gridded catalogue, in (column, z, original index) order, columns padded to
+// COL_PAD entries.
 struct Gridded {
     long long n;
     float *xs, *ys, *zs;  // float32 coordinates in the grid frame (padded columns)
+    float *xyz;           // the same in quads (quad_off): one address serves three 16-byte loads
     float *ws;            // float32 weights (padded columns, 64 floats of slack; NULL without weights)
     unsigned *wmax;       // bit pattern of max |w| as float (written by gridding; NULL without weights)
     float *xl, *yl, *zl;  // rounding residuals fl32((X - O) - xs) of the float32 coordinates
                           // (float32 mean separations from float64 inputs; else NULL)
     double4_32a *pos64;       // (x, y, z, w) binary64, exact inputs
     int *perm;            // original index of each sorted point
+    int *chunk_col;       // column of each run of COL_PAD entries
     uint32_t *cell_start; // ncells + 1
     double4_32a *colbox;      // per column (xmin, xmax, ymin, ymax)
 };
@@ -113,6 +125,13 @@ struct __align__(16) WorkItem {
 // empty range (lo == hi) when the image does not apply.
 struct __align__(8) Win {
     int lo[3], hi[3];
+};
+
+// A kept neighbour of a primary column: the column pair's z reach (float32,
+// rounded up, with the window slack) and its code (as WorkItem::code).
+struct __align__(8) Nbr {
+    float dz;
+    int code;
 };
 
 // Cell index along one axis from a float32 frame coordinate (monotone in it):
@@ -139,6 +158,9 @@ struct PairParams {
     unsigned *win_count;   // window records handed out by the work-list kernel
     long long win_cap;  // capacity of win (records)
     int win_chunk;      // primaries per chunk the windows are computed for (0 = no pre-pass)
+    Nbr *nbr;           // chunk tasks: nstencil entries per primary column, kept ones first
+    unsigned *nbr_count;   // kept entries per primary column
+    int parts;          // chunk tasks: shares a chunk's neighbour list is split into
     int tile_max;       // points per staged tile
     uint32_t flags;
     uint64_t wait_ns;   // limit of every tile-barrier wait (then the error word gets ERR_TIMEOUT)

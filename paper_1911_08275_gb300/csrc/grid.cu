@@ -7,14 +7,17 @@
 //   cell_start[ncells + 1]  counting-sort offsets; cell = column * nz + zcell,
 //                           column = cx * ncy + cy.  A column is the contiguous
 //                           range [cell_start[col*nz], cell_start[(col+1)*nz]),
-//                           padded at its end to a multiple of 4 entries (16 bytes
-//                           of float) so 1-D bulk copies of column slices are
-//                           aligned; padding entries are NaN and never counted.
+//                           padded at its end to a multiple of COL_PAD = 32
+//                           entries, so chunks of 8, 16 or 32 primaries and
+//                           aligned groups of secondaries never straddle two
+//                           columns; padding entries are NaN and never counted.
 //   xs, ys, zs[n']  float32 x - ox, y - oy, z - oz (grid frame), structure of arrays
+//   xyz[3 n']       the same in quads (x0..x3, y0..y3, z0..z3 per four points)
+//   chunk_col[n'/32] column of each run of 32 entries
 //   pos64[n']       double4 (x, y, z, w) exact binary64 copies (re-checks, FP64 path)
 //   perm[n']        original index of each sorted point (-1 for padding)
 //   colbox[ncols]   (xmin, xmax, ymin, ymax) of the column's points, binary64
-// with n' <= n + 3 * ncols.
+// with n' <= n + 31 * ncols.
 //
 // Within a cell the order is (z, original index), computed by ranking, so the
 // output is deterministic whatever the order of the atomic slot assignment.
@@ -207,7 +210,7 @@ __global__ void k_scan_add(uint32_t *__restrict__ out, long long n, const uint32
         out[i] += bsum[i / SCAN_ITEMS];
 }
 
-// One warp per column: padding that rounds the column up to a multiple of 4,
+// One warp per column: padding that rounds the column up to a multiple of COL_PAD,
 // written into the padded count of the column's last cell.
 __global__ void k_colpad(const uint32_t *__restrict__ count, int ncols, int nz,
                          uint32_t *__restrict__ pad, uint32_t *__restrict__ padded)
@@ -226,7 +229,7 @@ __global__ void k_colpad(const uint32_t *__restrict__ count, int ncols, int nz,
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
         tot += __shfl_xor_sync(FULL, tot, o);
-    const uint32_t pd = (4u - (tot & 3u)) & 3u;
+    const uint32_t pd = (COL_PAD - (tot & (COL_PAD - 1u))) & (COL_PAD - 1u);
     __syncwarp();
     if (lane == 0) {
         pad[col] = pd;
@@ -254,8 +257,9 @@ __device__ __forceinline__ void put_entry(const T *__restrict__ x, const T *__re
                                           const double *__restrict__ w, const Geom &g, uint32_t d,
                                           int iq, unsigned long long kq, float *__restrict__ xs,
                                           float *__restrict__ ys, float *__restrict__ zs,
-                                          float *__restrict__ ws, double4_32a *__restrict__ pos64,
-                                          int *__restrict__ perm, unsigned &wm)
+                                          float *__restrict__ xyz, float *__restrict__ ws,
+                                          double4_32a *__restrict__ pos64, int *__restrict__ perm,
+                                          unsigned &wm)
 {
     const double X = (double)x[iq], Y = (double)y[iq], Z = key_value(kq);
     const double W = w ? w[iq] : 0.0;
@@ -267,6 +271,10 @@ __device__ __forceinline__ void put_entry(const T *__restrict__ x, const T *__re
     xs[d] = fx;
     ys[d] = fy;
     zs[d] = fz;
+    float *qd = xyz + quad_off(d);
+    qd[0] = fx;
+    qd[4] = fy;
+    qd[8] = fz;
     if (ws) {
         ws[d] = (float)W;
         wm = max(wm, __float_as_uint(fabsf((float)W)));
@@ -303,8 +311,8 @@ __global__ void __launch_bounds__(SORT_THREADS)
                  long long ncells, Geom g, const uint32_t *__restrict__ count,
                  const uint32_t *__restrict__ start, const int *__restrict__ tmp_idx,
                  const unsigned long long *__restrict__ tmp_key, float *__restrict__ xs,
-                 float *__restrict__ ys, float *__restrict__ zs, float *__restrict__ ws,
-                 unsigned *__restrict__ wmax, double4_32a *__restrict__ pos64,
+                 float *__restrict__ ys, float *__restrict__ zs, float *__restrict__ xyz,
+                 float *__restrict__ ws, unsigned *__restrict__ wmax, double4_32a *__restrict__ pos64,
                  int *__restrict__ perm, unsigned *__restrict__ claim)
 {
     __shared__ ulonglong2 s_ent[SORT_THREADS / 32][SORT_BUF];
@@ -331,7 +339,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
             __syncwarp();
             const uint32_t rank = rank_in(be + half * 16, max(cnt0, cnt1), kq, iq);
             if (mine)
-                put_entry(x, y, w, g, s + rank, iq, kq, xs, ys, zs, ws, pos64, perm, wm);
+                put_entry(x, y, w, g, s + rank, iq, kq, xs, ys, zs, xyz, ws, pos64, perm, wm);
             continue;
         }
         for (int h = 0; h < 2; ++h) {  // whole warp, one cell after the other
@@ -371,7 +379,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
                     }
                 }
                 if (mine)
-                    put_entry(x, y, w, g, sc + rank, iq, kq, xs, ys, zs, ws, pos64, perm, wm);
+                    put_entry(x, y, w, g, sc + rank, iq, kq, xs, ys, zs, xyz, ws, pos64, perm, wm);
             }
         }
     }
@@ -390,25 +398,34 @@ __global__ void __launch_bounds__(SORT_THREADS)
     }
 }
 
-// Padding entries at the end of each column: NaN (never counted), perm -1.
-__global__ void k_padfill(const uint32_t *__restrict__ start, const uint32_t *__restrict__ pad,
-                          int ncols, int nz, float *__restrict__ xs, float *__restrict__ ys,
-                          float *__restrict__ zs, float *__restrict__ ws,
-                          double4_32a *__restrict__ pos64, int *__restrict__ perm)
+// One warp per column: its padding entries (NaN, never counted; perm -1) and
+// the column of each of its runs of COL_PAD entries.
+__device__ __forceinline__ void pad_column(const Gridded &G, int col, uint32_t s, uint32_t e,
+                                           uint32_t pad, int lane)
 {
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= ncols)
-        return;
-    const uint32_t e = start[(long long)(col + 1) * nz];
     const float fn = __int_as_float(0x7fc00000);
     const double dn = __longlong_as_double(0x7ff8000000000000ll);
-    for (uint32_t q = e - pad[col]; q < e; ++q) {
-        xs[q] = ys[q] = zs[q] = fn;
-        if (ws)
-            ws[q] = 0.0f;
-        pos64[q] = make_double4_32a(dn, dn, dn, dn);
-        perm[q] = -1;
+    if ((uint32_t)lane < pad) {
+        const uint32_t q = e - 1u - lane;
+        G.xs[q] = G.ys[q] = G.zs[q] = fn;
+        float *qd = G.xyz + quad_off(q);
+        qd[0] = qd[4] = qd[8] = fn;
+        if (G.ws)
+            G.ws[q] = 0.0f;
+        G.pos64[q] = make_double4_32a(dn, dn, dn, dn);
+        G.perm[q] = -1;
     }
+    for (uint32_t k = s / COL_PAD + lane; k < e / COL_PAD; k += 32)
+        G.chunk_col[k] = col;
+}
+
+__global__ void __launch_bounds__(256) k_padfill(const uint32_t *__restrict__ pad, int ncols, int nz,
+                                                 const __grid_constant__ Gridded G)
+{
+    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (col < ncols)
+        pad_column(G, col, G.cell_start[(long long)col * nz], G.cell_start[(long long)(col + 1) * nz],
+                   pad[col], threadIdx.x & 31);
 }
 
 // One block per column: (xmin, xmax, ymin, ymax) of its points, with min / max
@@ -655,7 +672,7 @@ __global__ void __launch_bounds__(256) kb_colpad(const GridBatch B)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
         tot += __shfl_xor_sync(FULL, tot, o);
-    const uint32_t pd = (4u - (tot & 3u)) & 3u;
+    const uint32_t pd = (COL_PAD - (tot & (COL_PAD - 1u))) & (COL_PAD - 1u);
     __syncwarp();
     if (lane == 0) {
         S.pad[col] = pd;
@@ -694,10 +711,10 @@ __device__ __forceinline__ void put_seg(const GridBatch &B, const GridSeg &S, ui
     const Geom &g = B.geom[S.job];
     if (S.f32)
         put_entry(static_cast<const float *>(S.x), static_cast<const float *>(S.y), nullptr, g, d, iq,
-                  kq, S.out.xs, S.out.ys, S.out.zs, nullptr, S.out.pos64, S.out.perm, wm);
+                  kq, S.out.xs, S.out.ys, S.out.zs, S.out.xyz, nullptr, S.out.pos64, S.out.perm, wm);
     else
         put_entry(static_cast<const double *>(S.x), static_cast<const double *>(S.y), nullptr, g, d,
-                  iq, kq, S.out.xs, S.out.ys, S.out.zs, nullptr, S.out.pos64, S.out.perm, wm);
+                  iq, kq, S.out.xs, S.out.ys, S.out.zs, S.out.xyz, nullptr, S.out.pos64, S.out.perm, wm);
 }
 
 // k_sort_cells over the concatenated cells of every segment (the two cells of
@@ -786,20 +803,13 @@ __global__ void __launch_bounds__(SORT_THREADS) kb_sort_cells(const GridBatch B)
 
 __global__ void __launch_bounds__(256) kb_padfill(const GridBatch B)
 {
-    const int s = block_seg(B.pre[GB_COLS], B.nseg);
+    const int s = block_seg(B.pre[GB_COLWARPS], B.nseg);
     const GridSeg &S = B.seg[s];
     const Geom &g = B.geom[S.job];
-    const int col = (int)(blockIdx.x - B.pre[GB_COLS][s]) * 256 + (int)threadIdx.x;
-    if (col >= g.ncols)
-        return;
-    const uint32_t e = S.out.cell_start[(long long)(col + 1) * g.nz];
-    const float fn = __int_as_float(0x7fc00000);
-    const double dn = __longlong_as_double(0x7ff8000000000000ll);
-    for (uint32_t q = e - S.pad[col]; q < e; ++q) {
-        S.out.xs[q] = S.out.ys[q] = S.out.zs[q] = fn;
-        S.out.pos64[q] = make_double4_32a(dn, dn, dn, dn);
-        S.out.perm[q] = -1;
-    }
+    const int col = (int)(blockIdx.x - B.pre[GB_COLWARPS][s]) * 8 + (int)(threadIdx.x >> 5);
+    if (col < g.ncols)
+        pad_column(S.out, col, S.out.cell_start[(long long)col * g.nz],
+                   S.out.cell_start[(long long)(col + 1) * g.nz], S.pad[col], threadIdx.x & 31);
 }
 
 // One block per column (as k_colbox).
@@ -878,15 +888,14 @@ cudaError_t build_grid_t(const void *x, const void *y, const void *z, const doub
         const long long cwarps = std::min<long long>((nc + 1) / 2, (long long)sms * 64);
         k_sort_cells<T><<<(int)((cwarps * 32 + SORT_THREADS - 1) / SORT_THREADS), SORT_THREADS, 0, st>>>(
             (const T *)x, (const T *)y, w, nc, g, t.counts, out.cell_start, t.tmp_idx, t.tmp_key,
-            out.xs, out.ys, out.zs, out.ws, out.ws ? out.wmax : nullptr, out.pos64, out.perm,
+            out.xs, out.ys, out.zs, out.xyz, out.ws, out.ws ? out.wmax : nullptr, out.pos64, out.perm,
             t.counts + nc);
     }
-    k_padfill<<<(g.ncols + 255) / 256, 256, 0, st>>>(out.cell_start, t.pad, g.ncols, g.nz, out.xs,
-                                                      out.ys, out.zs, out.ws, out.pos64, out.perm);
+    k_padfill<<<cb, 256, 0, st>>>(t.pad, g.ncols, g.nz, out);
     k_colbox<<<std::min(g.ncols, sms * 8), 256, 0, st>>>(out.pos64, out.cell_start, g.ncols, g.nz,
                                                           out.colbox);
     if (out.xl) {
-        const long long np = n + 3ll * g.ncols;  // padded length (an upper bound)
+        const long long np = padded_max(n, g.ncols);
         k_residual<<<grid_blocks(np, TB, sms), TB, 0, st>>>(out.pos64, out.xs, out.ys, out.zs,
                                                             out.cell_start, g, out.xl, out.yl,
                                                             out.zl);
@@ -935,8 +944,6 @@ unsigned grid_batch_blocks(int k, long long n, const Geom &g)
         return (unsigned)((n + 255) / 256);
     case GB_COLWARPS:
         return (unsigned)((g.ncols + 7) / 8);
-    case GB_COLS:
-        return (unsigned)((g.ncols + 255) / 256);
     case GB_COLBLK:
         return (unsigned)g.ncols;
     default:
@@ -964,7 +971,7 @@ cudaError_t build_grid_batch(const GridBatch &B, int sms, cudaStream_t st)
         const long long cwarps = std::min<long long>((B.ctot + 1) / 2, (long long)sms * 64);
         kb_sort_cells<<<(unsigned)((cwarps * 32 + SORT_THREADS - 1) / SORT_THREADS), SORT_THREADS, 0, st>>>(B);
     }
-    kb_padfill<<<B.blocks[GB_COLS], 256, 0, st>>>(B);
+    kb_padfill<<<B.blocks[GB_COLWARPS], 256, 0, st>>>(B);
     kb_colbox<<<B.blocks[GB_COLBLK], 256, 0, st>>>(B);
     return cudaGetLastError();
 }

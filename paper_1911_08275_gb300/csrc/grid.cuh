@@ -11,8 +11,8 @@ namespace cf {
 struct GridTemps {
     uint32_t *cell_of;   // n
     uint32_t *slot;      // n
-    int *tmp_idx;        // n + 3 * ncols (padded index space)
-    unsigned long long *tmp_key;  // n + 3 * ncols: order-preserving keys of z
+    int *tmp_idx;        // padded_max(n, ncols)
+    unsigned long long *tmp_key;  // padded_max(n, ncols): order-preserving keys of z
     uint32_t *counts;    // ncells + 1 (the last: the in-cell sort's claim counter)
     uint32_t *pad;       // ncols
     uint32_t *bsum;      // ceil(ncells / 4096)
@@ -41,8 +41,8 @@ struct GridSeg {
                             // (ncells + 1 entries per segment)
     Gridded out;            // output arrays (preallocated; no weights, no residuals)
     uint32_t *cell_of, *slot;      // n each
-    int *tmp_idx;                  // n + 3 ncols
-    unsigned long long *tmp_key;   // n + 3 ncols
+    int *tmp_idx;                  // padded_max(n, ncols)
+    unsigned long long *tmp_key;   // padded_max(n, ncols)
     uint32_t *pad;                 // ncols
     unsigned *err;                 // the job's error word
 };
@@ -52,7 +52,6 @@ struct GridSeg {
 enum GridBatchShape {
     GB_POINTS,    // 256 points per block
     GB_COLWARPS,  // 8 columns per block (one warp each)
-    GB_COLS,      // 256 columns per block (one thread each)
     GB_COLBLK,    // one column per block
     GB_CELLS,     // 256 entries of cell_start per block
     GB_SHAPES

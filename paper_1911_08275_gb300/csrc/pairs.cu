@@ -40,7 +40,9 @@
 #include <mutex>
 
 #include "cf_internal.cuh"
+#include "launch.cuh"
 #include "pairs.cuh"
+#include "pairs_dev.cuh"
 
 namespace cf {
 
@@ -69,11 +71,6 @@ void plan_pairs(PairParams &P, PairLaunch &L)
             P.hist_off = XI32_HIST_OFF;
             L.hist_words = planes * WARPS * (nb + 2) * 32;
             L.smem = align_up(XI32_HIST_OFF + L.hist_words * 4 + (nb + 2) * 4, 128);
-        } else if (L.pipe) {
-            // one histogram copy shared by all warps, then the second tile buffer
-            L.hist_words = (nb + 2) * 32;
-            P.hist_off = XI32_HIST_OFF;
-            L.smem = pipe_slot1_off(nb) + 3 * XI32_TSTRIDE;
         } else {
             L.hist_words = WARPS * (nb + 2) * 32;  // + a row for flagged table cells
             P.hist_off = XI32_HIST_OFF;
@@ -101,219 +98,6 @@ void plan_pairs(PairParams &P, PairLaunch &L)
 }
 
 namespace {
-
-typedef unsigned long long u64;
-
-__device__ __forceinline__ int floor_div(int a, int n)
-{
-    return a >= 0 ? a / n : -((-a + n - 1) / n);
-}
-
-// ---------------------------------------------------------------- packed f32x2
-__device__ __forceinline__ u64 pack2(float lo, float hi)
-{
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(u64 v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ u64 fsub2(u64 a, u64 b)
-{
-    u64 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ u64 fmul2(u64 a, u64 b)
-{
-    u64 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c)
-{
-    u64 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
-// ---------------------------------------------------------------- searches
-// First index p in [0, n) with key(p) >= v (upper = false) or key(p) > v
-// (upper = true); n if none.  Keys must be sorted.  All lanes call it with the
-// same arguments; each round probes 32 positions.
-template <class Key, class V>
-__device__ __forceinline__ int warp_bound(Key key, int n, V v, bool upper, int lane)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int s = (hi - lo + 31) >> 5;
-        const int p = lo + lane * s;
-        bool q = false;
-        if (p < hi) {
-            const V z = key(p);
-            q = upper ? (z <= v) : (z < v);
-        }
-        const int c = __popc(__ballot_sync(FULL, q));
-        if (c == 0)
-            break;
-        const int nlo = lo + (c - 1) * s + 1;
-        hi = min(hi, lo + c * s);
-        lo = nlo;
-    }
-    return lo;
-}
-
-// Bin of a binary64 squared separation: k with E2[k] <= r2 < E2[k+1], else -1.
-// Non-negative doubles order like their bit patterns, so integer compares suffice.
-__device__ __forceinline__ int bin_f64(double r2, const double *E2, int nb)
-{
-    const long long u = __double_as_longlong(r2);
-    const long long *e = reinterpret_cast<const long long *>(E2);
-    if (!(u >= e[0] && u < e[nb]))
-        return -1;
-    int lo = 0, hi = nb;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (e[mid] <= u)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ double canon_r2(const double4_32a &p, const double4_32a &q, double Sx,
-                                           double Sy, double Sz)
-{
-    const double dx = canon_comp(p.x, q.x, Sx);
-    const double dy = canon_comp(p.y, q.y, Sy);
-    const double dz = canon_comp(p.z, q.z, Sz);
-    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-}
-
-// The same for an image whose shifts are all zero (canon_comp's adds are then
-// skipped, so the value is bit-identical).  The binary64 sweeps choose between
-// the two once per window: a shift test inside the pair loop is compiled into
-// adds issued under a predicate, which still occupy the narrow binary64 pipe.
-__device__ __forceinline__ double plain_r2(const double4_32a &p, const double4_32a &q)
-{
-    const double dx = __dsub_rn(q.x, p.x), dy = __dsub_rn(q.y, p.y), dz = __dsub_rn(q.z, p.z);
-    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-}
-
-// Binary64 re-evaluation of one pair inside an error band: bin row or -1.
-__device__ __noinline__ int recheck64(const double *E2, int nb, const double4_32a *pa,
-                                      const double4_32a *pb, int i, int j, double Sx, double Sy,
-                                      double Sz)
-{
-    return bin_f64(canon_r2(pa[i], pb[j], Sx, Sy, Sz), E2, nb);
-}
-
-// Debug: does the float32 decision for d2 agree with binary64?  (1 = violation)
-__device__ __noinline__ int verify_pair(float d2, const float *thr, int nthr, int nb,
-                                        const double *E2, const double4_32a *pa,
-                                        const double4_32a *pb, int i, int j, double Sx, double Sy,
-                                        double Sz)
-{
-    int c = 0;
-    while (c < nthr && thr[c] <= d2)
-        ++c;
-    if (c & 1)
-        return 0;  // inside a band: re-checked, no float32 claim
-    const int k32 = (c >= 2 && c <= 2 * nb) ? (c - 2) >> 1 : -1;
-    const int k64 = bin_f64(canon_r2(pa[i], pb[j], Sx, Sy, Sz), E2, nb);
-    return k32 != k64;
-}
-
-__device__ __forceinline__ u64 warp_sum_u64(u64 v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        v += __shfl_xor_sync(FULL, v, o);
-    return v;
-}
-
-// Move one warp's per-lane counts to the global histogram (overflow guard).
-__device__ void warp_flush(uint32_t *hw, int nb, unsigned long long *ghist, int lane)
-{
-    for (int b = 0; b < nb; ++b) {
-        const u64 v = warp_sum_u64(hw[b * 32 + lane]);
-        hw[b * 32 + lane] = 0u;
-        if (lane == 0 && v)
-            atomicAdd(&ghist[b], v);
-    }
-}
-
-// The same for a copy that other warps add to concurrently: each count is read
-// and cleared in one atomic exchange, so no concurrent increment is lost.
-__device__ void warp_flush_shared(uint32_t *hw, int nb, unsigned long long *ghist, int lane)
-{
-    for (int b = 0; b < nb; ++b) {
-        const u64 v = warp_sum_u64(atomicExch(&hw[b * 32 + lane], 0u));
-        if (lane == 0 && v)
-            atomicAdd(&ghist[b], v);
-    }
-}
-
-// Candidate (column a, stencil offset) -> column pair, image, pruning
-// (Sec. 2.2) and z reach, in binary64.  Returns false if the pair has no work.
-__device__ __forceinline__ bool plan_item(const PairParams &P, int item, WorkItem &w)
-{
-    const int a = item / P.nstencil, s = item - a * P.nstencil;
-    const int2 o = P.stencil[s];
-    const int ax = a / P.g.ncy, ay = a - ax * P.g.ncy;
-    int bx = ax + o.x, by = ay + o.y;
-    int qx = 0, qy = 0;
-    if (P.g.periodic) {
-        qx = floor_div(bx, P.g.ncx);
-        qy = floor_div(by, P.g.ncy);
-        // an image two or more boxes away holds no pair within Rmax < L/2 (every
-        // coordinate difference is below L), even when pruning is switched off
-        if (qx < -1 || qx > 1 || qy < -1 || qy > 1)
-            return false;
-        bx -= qx * P.g.ncx;
-        by -= qy * P.g.ncy;
-    } else if (bx < 0 || bx >= P.g.ncx || by < 0 || by >= P.g.ncy) {
-        return false;
-    }
-    const double Sx = qx * P.g.box[0], Sy = qy * P.g.box[1];
-    const int b = bx * P.g.ncy + by;
-    const long long nz = P.g.nz;
-    if (P.shard_n > 1) {  // deterministic split of the primary columns over shards
-        const unsigned long long total = P.A.cell_start[(long long)P.g.ncols * nz];
-        const unsigned long long first = P.A.cell_start[a * nz];
-        const unsigned long long lo = total * (unsigned long long)P.shard_k / P.shard_n;
-        const unsigned long long hi = total * (unsigned long long)(P.shard_k + 1) / P.shard_n;
-        if (first < lo || first >= hi)
-            return false;
-    }
-    w.a0 = (int)P.A.cell_start[a * nz];
-    w.a1 = (int)P.A.cell_start[(a + 1) * nz];
-    w.b0 = (int)P.B.cell_start[b * nz];
-    w.b1 = (int)P.B.cell_start[(b + 1) * nz];
-    if (w.a0 >= w.a1 || w.b0 >= w.b1)
-        return false;
-    // minimum possible (x, y) separation of the two columns' bounding boxes
-    const double4_32a ba = P.A.colbox[a], bb = P.B.colbox[b];
-    const double gx = fmax(0.0, fmax(__dsub_rn(__dadd_rn(bb.x, Sx), ba.y),
-                                     __dsub_rn(ba.x, __dadd_rn(bb.y, Sx))));
-    const double gy = fmax(0.0, fmax(__dsub_rn(__dadd_rn(bb.z, Sy), ba.w),
-                                     __dsub_rn(ba.z, __dadd_rn(bb.w, Sy))));
-    const double g2 = __dadd_rn(__dmul_rn(gx, gx), __dmul_rn(gy, gy));
-    if (!(P.flags & CF_FLAG_NO_PRUNE) && g2 >= P.prune_r2)
-        return false;
-    // z reach: dz_max,all of Sec. 2.2 (xi); pimax (rp-pi)
-    double dzmax = P.rz;
-    if (P.kind == 0)
-        dzmax = sqrt(fmax(0.0, __dsub_rn(P.rxy2, __dmul_rn(g2, 1.0 - 1e-12))));
-    w.dzmax = __dmul_rn(dzmax, 1.0 + 1e-9);
-    const bool self = P.autocorr && o.x == 0 && o.y == 0;
-    w.code = (qx + 1) | ((qy + 1) << 2) | (self ? 16 : 0) | (b << 5);
-    w.wbase = 0;
-    return true;
-}
 
 // Work-list kernel (a3): one thread per candidate, kept pairs appended to
 // P.work with one warp-aggregated atomic per warp.  With the window pre-pass
@@ -614,12 +398,6 @@ __device__ __forceinline__ uint32_t lut_byte(const unsigned char *smem, uint32_t
     return smem[LUT_OFF + min(q, last)];
 }
 
-// Cells linear in d2: adding 2^23 in the fma rounds d2 * scale to an integer q
-// held in the sum's low bits (exact below 2^22; larger values, and NaN, give
-// larger bit patterns and clamp to the out-of-range entry).
-constexpr float LIN_MAGIC = 8388608.0f;  // 2^23: spacing 1 in [2^23, 2^24)
-constexpr uint32_t LIN_MAGIC_BITS = 0x4b000000u;
-
 __device__ __forceinline__ uint32_t lut_byte_lin(const unsigned char *smem, float scale,
                                                  uint32_t last, float d2)
 {
@@ -632,52 +410,6 @@ __device__ __forceinline__ uint32_t lut_entry(const unsigned char *smem, uint32_
                                               uint32_t last, float scale, float d2)
 {
     return LIN ? lut_byte_lin(smem, scale, last, d2) : lut_byte(smem, u0s, shift, last, d2);
-}
-
-// Number of thresholds T[c] <= d2 (T non-decreasing, d2 not NaN), scanning
-// down from the top: flagged cells are dominated by the largest edges (the
-// pair density grows with the separation), where this ends in a step or two.
-__device__ __forceinline__ int thr_count_top(const float *T, int nthr, float d2)
-{
-    int c = nthr;
-    while (c > 0 && T[c - 1] > d2)
-        --c;
-    return c;
-}
-
-// Number of thresholds T[c] <= d2 (T is non-decreasing; NaN counts none).
-__device__ __forceinline__ int thr_count(const float *T, int nthr, float d2)
-{
-    int lo = 0, hi = nthr;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (T[mid] <= d2)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ void red_shared1(uint32_t addr)
-{
-    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr));
-}
-
-// Table byte at a shared address, sign-extended: the flagged entry gives -1.
-__device__ __forceinline__ uint32_t lds_entry(uint32_t addr)
-{
-    uint32_t e;
-    asm volatile("ld.shared.s8 %0, [%1];" : "=r"(e) : "r"(addr));
-    return e;
-}
-
-// (m << 1) | (v >> 31): one funnel shift appends v's sign bit to the mask m.
-__device__ __forceinline__ uint32_t push_sign(uint32_t m, uint32_t v)
-{
-    uint32_t r;
-    asm("shf.l.wrap.b32 %0, %1, %2, 1;" : "=r"(r) : "r"(v), "r"(m));
-    return r;
 }
 
 // Flagged table cell: count the thresholds <= d2; inside a band re-evaluate in
@@ -2592,157 +2324,6 @@ __global__ void __launch_bounds__(THREADS, MINB) k_path(const __grid_constant__ 
     Path::fini(P, smem, st);
 }
 
-// ============================================ pipelined float32 DD(r) kernel
-// Two tile buffers: while the warps sweep the tile in one, the next tile is
-// already staged in the other, so no CTA-wide barrier separates work items.
-// A unit is one tile of one work item.  The warp that finishes a unit last
-// (counted in done[s]) refills its buffer with the unit after next: it claims
-// the next item when the cursor's item has no tile left, pads, and issues the
-// bulk copies; the other warps move straight on to the other buffer.  Within
-// a unit the warps claim chunks from claim[s].  Every wait is bounded.
-struct PipeHdr {
-    uint64_t full[2];    // tile-ready barrier of each buffer
-    WorkItem w[2];       // work item of each buffer's unit
-    int item[2];         // its index (-1: no more work)
-    int t0[2], nt[2];    // its tile of column b
-    int claim[2];        // next chunk of the unit
-    int done[2];         // warps finished with the unit
-    int cur, next_t0;    // cursor: item of the last issued unit, start of its next tile
-};
-static_assert(sizeof(PipeHdr) <= XI32_LUT_OFF, "pipeline header fits before the table");
-
-// Fill buffer s with the next unit (called by one whole warp; lane 0 claims,
-// every lane pads, lane 0 issues the copies and arrives on the barrier).
-__device__ __forceinline__ void pipe_issue(const PairParams &P, PipeHdr *H, int s, int n_work,
-                                           unsigned char *buf, int lane, bool stall = false)
-{
-    int item = -1, t0 = 0, nt = 0;
-    if (lane == 0) {
-        const int cur = H->cur;
-        if (cur >= 0 && H->next_t0 < H->w[s ^ 1].b1 && H->item[s ^ 1] == cur) {
-            item = cur;  // the cursor's item has tiles left (its record is in the other buffer)
-            t0 = H->next_t0;
-            H->w[s] = H->w[s ^ 1];
-        } else {
-            for (;;) {  // next item with points on both sides (bounded by the work count)
-                const int c = (int)atomicAdd(P.item_counter, 1u);
-                if (c >= n_work)
-                    break;
-                const WorkItem w = P.work[c];
-                if (w.a1 > w.a0 && w.b1 > w.b0) {
-                    item = c;
-                    t0 = w.b0;
-                    H->w[s] = w;
-                    break;
-                }
-            }
-            H->cur = item;
-        }
-        if (item >= 0) {
-            nt = min(TILE32, H->w[s].b1 - t0);
-            H->next_t0 = t0 + nt;
-        }
-    }
-    item = __shfl_sync(FULL, item, 0);
-    nt = __shfl_sync(FULL, nt, 0);
-    t0 = __shfl_sync(FULL, t0, 0);
-    if (item >= 0) {
-        float *t = reinterpret_cast<float *>(buf);
-        for (int q = lane; q < 3 * 64; q += 32)  // sentinels after the copied range: never counted
-            t[(q >> 6) * (XI32_TSTRIDE / 4) + nt + (q & 63)] = __int_as_float(0x7fc00000);
-    }
-    __syncwarp();
-    if (lane == 0) {
-        H->item[s] = item;
-        H->t0[s] = t0;
-        H->nt[s] = nt;
-        if (item >= 0) {
-            const unsigned bytes = (unsigned)nt * 4u;
-            fence_proxy_async_smem();
-            mbar_arrive_expect_tx(&H->full[s], 3u * bytes);
-            if (!stall) {  // diagnostic stall: the armed copy is never issued
-                bulk_g2s(buf, P.B.xs + t0, bytes, &H->full[s]);
-                bulk_g2s(buf + XI32_TSTRIDE, P.B.ys + t0, bytes, &H->full[s]);
-                bulk_g2s(buf + 2 * XI32_TSTRIDE, P.B.zs + t0, bytes, &H->full[s]);
-            }
-        } else {
-            mbar_arrive(&H->full[s]);
-        }
-    }
-}
-
-template <class Path, int MINB>
-__global__ void __launch_bounds__(THREADS, MINB) k_pipe(const __grid_constant__ PairParams P)
-{
-    extern __shared__ __align__(128) unsigned char smem[];
-    PipeHdr *H = reinterpret_cast<PipeHdr *>(smem);
-    unsigned char *buf0 = smem + XI32_TX_OFF, *buf1 = smem + pipe_slot1_off(P.nbins);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    Path::init(P, smem);
-    if (threadIdx.x == 0) {
-        mbar_init(&H->full[0], 1);
-        mbar_init(&H->full[1], 1);
-        fence_mbar_init();
-        H->item[0] = H->item[1] = -1;
-        H->claim[0] = H->claim[1] = 0;
-        H->done[0] = H->done[1] = 0;
-        H->cur = -1;
-        H->next_t0 = 0;
-    }
-    __syncthreads();
-    const int n_work = (int)*P.work_count;
-    if (warp == 0) {
-        pipe_issue(P, H, 0, n_work, buf0, lane, (P.flags & CF_FLAG_DEBUG_STALL) != 0);
-        pipe_issue(P, H, 1, n_work, buf1, lane);
-    }
-    PathState st = {0ull, 0ull, 0ull, 0u, 0u, 0u};
-    unsigned par = 0u;  // bit s: parity of buffer s's next phase
-    bool timed_out = false;
-    for (int u = 0;; ++u) {
-        const int s = u & 1;
-        unsigned char *buf = s ? buf1 : buf0;
-        if (!mbar_wait(&H->full[s], (par >> s) & 1u, P.wait_ns)) {
-            if (lane == 0)
-                atomicOr(P.err, ERR_TIMEOUT);
-            timed_out = true;
-            break;
-        }
-        par ^= 1u << s;
-        const int item = reinterpret_cast<volatile int *>(H->item)[s];
-        if (item < 0)
-            break;
-        Item it;
-        decode_record(P, H->w[s], it);
-        Path::tile(P, it, H->t0[s], H->nt[s], buf, &H->claim[s], smem, st);
-        __syncwarp();
-        int last = 0;
-        if (lane == 0) {
-            __threadfence_block();  // this warp's reads of the buffer come first
-            last = atomicAdd(&H->done[s], 1) == WARPS - 1;
-        }
-        if (__shfl_sync(FULL, last, 0)) {
-            if (lane == 0) {
-                __threadfence_block();
-                H->done[s] = 0;
-                H->claim[s] = 0;
-            }
-            __syncwarp();
-            pipe_issue(P, H, s, n_work, buf, lane);
-        }
-    }
-    if (__syncthreads_or(timed_out)) {
-        // every warp gave up at the same unit: let the copies still in flight (the
-        // other buffer's, and a late one of the stuck buffer) land before the CTA
-        // exits, each wait bounded again
-        if (threadIdx.x == 0) {
-            mbar_wait(&H->full[0], par & 1u, P.wait_ns);
-            mbar_wait(&H->full[1], (par >> 1) & 1u, P.wait_ns);
-        }
-        __syncthreads();
-    }
-    Path::fini(P, smem, st);
-}
-
 // ============================================================ batched kernel
 // Many independent jobs (catalogues, bins, modes) in one persistent launch: the
 // CTAs pull items from one global counter over the concatenation of the jobs'
@@ -2899,55 +2480,6 @@ __global__ void __launch_bounds__(THREADS, 2) k_batch(const __grid_constant__ Ba
         batch_fini(B.path[cur], B.jobs[cur], smem, st);
 }
 
-// Per (kernel, device): the dynamic shared-memory limit set so far (only ever
-// raised) and the occupancy per shared-memory size, queried once.
-struct OccCache {
-    const void *kern;
-    int dev, smem, occ;
-};
-struct AttrCache {
-    const void *kern;
-    int dev, limit;
-};
-OccCache g_occ[128];
-AttrCache g_attr[32];
-int g_nocc = 0, g_nattr = 0;
-std::mutex g_occ_mu;
-
-template <class K>
-cudaError_t occupancy(K kern, int smem, int &occ)
-{
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e)
-        return e;
-    std::lock_guard<std::mutex> lock(g_occ_mu);
-    AttrCache *a = nullptr;
-    for (int q = 0; q < g_nattr; ++q)
-        if (g_attr[q].kern == (const void *)kern && g_attr[q].dev == dev)
-            a = &g_attr[q];
-    if (!a || a->limit < smem) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e)
-            return e;
-        if (!a && g_nattr < 32)
-            a = &g_attr[g_nattr++];
-        if (a)
-            *a = AttrCache{(const void *)kern, dev, smem};
-    }
-    for (int q = 0; q < g_nocc; ++q)
-        if (g_occ[q].kern == (const void *)kern && g_occ[q].dev == dev && g_occ[q].smem == smem) {
-            occ = g_occ[q].occ;
-            return cudaSuccess;
-        }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, THREADS, smem);
-    if (e)
-        return e;
-    if (g_nocc < 128)
-        g_occ[g_nocc++] = OccCache{(const void *)kern, dev, smem, occ};
-    return cudaSuccess;
-}
-
 template <class K>
 cudaError_t launch_persistent(K kern, const PairParams &P, PairLaunch &L, int sms, cudaStream_t st)
 {
@@ -2968,6 +2500,57 @@ cudaError_t launch_persistent(K kern, const PairParams &P, PairLaunch &L, int sm
 }
 
 }  // namespace
+
+
+// Per (kernel, device): the dynamic shared-memory limit set so far (only ever
+// raised) and the occupancy per shared-memory size, queried once.
+namespace {
+struct OccCache {
+    const void *kern;
+    int dev, smem, occ;
+};
+struct AttrCache {
+    const void *kern;
+    int dev, limit;
+};
+OccCache g_occ[128];
+AttrCache g_attr[64];
+int g_nocc = 0, g_nattr = 0;
+std::mutex g_occ_mu;
+}  // namespace
+
+cudaError_t occupancy_of(const void *kern, int smem, int &occ)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e)
+        return e;
+    std::lock_guard<std::mutex> lock(g_occ_mu);
+    AttrCache *a = nullptr;
+    for (int q = 0; q < g_nattr; ++q)
+        if (g_attr[q].kern == kern && g_attr[q].dev == dev)
+            a = &g_attr[q];
+    if (!a || a->limit < smem) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e)
+            return e;
+        if (!a && g_nattr < 64)
+            a = &g_attr[g_nattr++];
+        if (a)
+            *a = AttrCache{kern, dev, smem};
+    }
+    for (int q = 0; q < g_nocc; ++q)
+        if (g_occ[q].kern == kern && g_occ[q].dev == dev && g_occ[q].smem == smem) {
+            occ = g_occ[q].occ;
+            return cudaSuccess;
+        }
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, THREADS, smem);
+    if (e)
+        return e;
+    if (g_nocc < 128)
+        g_occ[g_nocc++] = OccCache{kern, dev, smem, occ};
+    return cudaSuccess;
+}
 
 int batch_path(const PairParams &P, int f64, int chunk, int pp)
 {
@@ -3026,7 +2609,14 @@ cudaError_t launch_pairs(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
     if (P0.n_items <= 0)
         return cudaSuccess;
     PairParams P = P0;
-    // the float32 DD(r) kernels take their chunk windows from the window pre-pass
+    if (P.kind == 0 && !L.f64 && !P.wacc) {  // float32 DD(r) counts: chunk tasks
+        cudaError_t e0 = launch_neighbours(P, st);
+        if (!e0)
+            e0 = launch_count32(P, L, sms, st);
+        L.kernels = 2;
+        return e0;
+    }
+    // the weighted float32 DD(r) kernels take their chunk windows from the window pre-pass
     const bool xi32 = P.kind == 0 && !L.f64;
     if (xi32 && !P.win)
         return cudaErrorInvalidValue;  // the caller provides the window records
@@ -3099,37 +2689,7 @@ cudaError_t launch_pairs(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
         return L.evals ? launch_persistent(k_path<Xi32Path<16, 1, true, false, false, true, HW, PW>, 2>, P, L, sms, st)
                        : launch_persistent(k_path<Xi32Path<16, 1, false, false, false, true, HW, PW>, 2>, P, L, sms, st);
     }
-    if (!L.pipe) {  // single tile buffer, one histogram copy per warp
-        if (L.verify)
-            return launch_persistent(k_path<Xi32Path<8, 1, true, true, false, false, HW, PW>, 3>, P, L, sms, st);
-        return L.evals ? launch_persistent(k_path<Xi32Path<16, 2, true, false, false, false, HW, PW>, 3>, P, L, sms, st)
-                       : launch_persistent(k_path<Xi32Path<16, 2, false, false, false, false, HW, PW>, 3>, P, L, sms, st);
-    }
-    // two tile buffers, one shared histogram copy
-    constexpr int H1 = 1;
-    if (L.verify)
-        return launch_persistent(k_pipe<Xi32Path<8, 1, true, true, false, false, H1, PW>, 3>, P, L, sms, st);
-    if (L.pp == 4)
-        return L.evals ? launch_persistent(k_pipe<Xi32Path<8, 4, true, false, false, false, H1, PW>, 2>, P, L, sms, st)
-                       : launch_persistent(k_pipe<Xi32Path<8, 4, false, false, false, false, H1, PW>, 2>, P, L, sms, st);
-    if (L.pp == 2) {
-        if (L.chunk == 8)
-            return L.evals ? launch_persistent(k_pipe<Xi32Path<8, 2, true, false, false, false, H1, PW>, 3>, P, L, sms, st)
-                           : launch_persistent(k_pipe<Xi32Path<8, 2, false, false, false, false, H1, PW>, 3>, P, L, sms, st);
-        return L.evals ? launch_persistent(k_pipe<Xi32Path<16, 2, true, false, false, false, H1, PW>, 3>, P, L, sms, st)
-                       : launch_persistent(k_pipe<Xi32Path<16, 2, false, false, false, false, H1, PW>, 3>, P, L, sms, st);
-    }
-    switch (L.chunk) {
-    case 16:
-        return L.evals ? launch_persistent(k_pipe<Xi32Path<16, 1, true, false, false, false, H1, PW>, 3>, P, L, sms, st)
-                       : launch_persistent(k_pipe<Xi32Path<16, 1, false, false, false, false, H1, PW>, 3>, P, L, sms, st);
-    case 32:
-        return L.evals ? launch_persistent(k_pipe<Xi32Path<32, 1, true, false, false, false, H1, PW>, 3>, P, L, sms, st)
-                       : launch_persistent(k_pipe<Xi32Path<32, 1, false, false, false, false, H1, PW>, 3>, P, L, sms, st);
-    default:
-        return L.evals ? launch_persistent(k_pipe<Xi32Path<8, 1, true, false, false, false, H1, PW>, 3>, P, L, sms, st)
-                       : launch_persistent(k_pipe<Xi32Path<8, 1, false, false, false, false, H1, PW>, 3>, P, L, sms, st);
-    }
+    return cudaErrorNotSupported;
 }
 
 }  // namespace cf

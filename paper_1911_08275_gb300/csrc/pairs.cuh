@@ -42,7 +42,6 @@ struct PairLaunch {
     int smem;        // dynamic shared memory bytes
     int hist_words;  // shared histogram words
     int max_blocks;  // upper bound on the persistent grid (0 = none)
-    int pipe;        // float32 DD(r) without sums: two tile buffers (no CTA barrier per item)
     int kernels;     // kernels the launch issued (work list, window pre-pass, pair kernel)
 };
 
@@ -64,16 +63,22 @@ inline int xi32_chunk(int chunk, int pp, bool weighted, bool verify)
 
 // Upper bound on the window records of one launch: every kept column pair
 // (at most nstencil per column of d1) has one record per chunk of its column a,
-// and the columns of d1 hold n1 points plus at most 3 padding points each.
+// and the columns of d1 hold padded_max(n1, ncols) entries.
 inline long long win_bound(long long n1, int ncols, int nstencil, int chunk)
 {
-    return (long long)nstencil * ((n1 + 3ll * ncols) / chunk + ncols + 1);
+    return (long long)nstencil * (padded_max(n1, ncols) / chunk + ncols + 1);
 }
 
 // Fill the shared-memory plan of a launch: L.smem, L.hist_words and, for
 // rp-pi, P.hcopies and P.hist_off.  Needs P.kind, P.nbins, P.npibins,
 // P.tile_max and L.f64.
 void plan_pairs(PairParams &P, PairLaunch &L);
+
+// Chunk tasks (tasks.cuh): the neighbour lists of d1's columns (P.nbr,
+// P.nbr_count; kept pairs added to *P.work_count), and the float32 DD(r) counts.
+cudaError_t launch_neighbours(const PairParams &P, cudaStream_t st);
+cudaError_t launch_count32(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
+int count32_smem(int nbins);
 
 // Configure (max dynamic smem), pick the occupancy-based grid and launch
 // (the work-list kernel, then the pair kernel).
