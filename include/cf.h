@@ -20,7 +20,9 @@
  *   dx = x_j - x_i; periodic: if dx > L/2: dx -= L; elif dx < -L/2: dx += L;
  *   rp2 = dx*dx + dy*dy;  r2 = rp2 + dz*dz;  bin k iff e_k^2 <= r2 < e_{k+1}^2;
  *   pi bins [P_m, P_{m+1}) with P_m = (pimax*m)/npibins, P_npibins = pimax.
- * CF_MODE_FP64 evaluates exactly that.  CF_MODE_FP32_RECHECK evaluates the
+ * CF_MODE_FP64 evaluates exactly that for every pair that can count (pairs that a
+ * proven float32 bound places beyond Rmax or pimax are dropped, as the bounding
+ * boxes drop them).  CF_MODE_FP32_RECHECK evaluates the
  * distances in float32 and re-evaluates in binary64 every pair whose float32
  * value lies within a proven error bound of a bin edge, Rmin, Rmax or a pi
  * edge; its integer counts are therefore identical to CF_MODE_FP64.
@@ -61,7 +63,7 @@ extern "C" {
 typedef enum { CF_FLOAT32 = 0, CF_FLOAT64 = 1 } cf_dtype;
 
 typedef enum {
-    CF_MODE_FP64 = 0,          /* all distance arithmetic in binary64          */
+    CF_MODE_FP64 = 0,          /* every counted distance in binary64           */
     CF_MODE_FP32_RECHECK = 1   /* float32 bulk + binary64 re-check near edges   */
 } cf_mode;
 

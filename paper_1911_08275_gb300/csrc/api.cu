@@ -636,6 +636,21 @@ uint64_t wait_limit_ns(uint32_t flags)
     return (flags & CF_FLAG_DEBUG_STALL) ? 1000000ull : 2000000000ull;
 }
 
+// Float32 bounds beyond which the binary64 counts discard a pair: cull for the
+// squared distance (ncomp components), zcull for dz^2.  d2~ >= hi proves d2 >= E2
+// for hi = E2 + B (band_sq), d2~ the float32 value as the float32 counts compute
+// it; the kernel's fused sum d2 - cull differs from d2~ - cull by at most a few
+// 2^-24 cull, which the factor 1 + 1e-6 covers.  |dz~| >= pimax + zslack proves
+// |dz| >= pimax (zslack widens every float32 z decision); the sign of the
+// kernel's one fma dz~^2 - zcull is exact.
+void set_cull(cf::PairParams &P, double rmax, int ncomp, double M, double Ls, double R)
+{
+    const double e2 = rmax * rmax;
+    P.cull = f32_up((double)std::nextafter(f32_up(e2 + band_sq(e2, ncomp, M, Ls, R)), INFINITY) * (1.0 + 1e-6));
+    const double z = P.rz + (double)P.zslack;
+    P.zcull = f32_up(z * z * (1.0 + 1e-6));
+}
+
 // Pair-kernel parameters that depend only on the request and the geometry:
 // stencil (Sec. 2.1: half stencil for auto), pruning radius and z reach
 // (Sec. 2.2), float32 slacks, bins and the pi-bin error band.  M and Ls return
@@ -674,6 +689,7 @@ void base_params(const Request &q, const cf::Geom &g, const cf::Gridded &A, cons
     P.zslack = (float)(8.0 * U32 * (M + Ls + Rz) + 1e-6 * Rz);
     for (int a = 0; a < 3; ++a)
         P.boxf[a] = (float)g.box[a];
+    set_cull(P, q.edges.back(), q.kind == 0 ? 3 : 2, M, Ls, R);
     P.nbins = (int)q.edges.size() - 1;
     if (q.kind == 1) {
         P.npibins = q.npibins;
@@ -1836,6 +1852,7 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     P.zslack = (float)(8.0 * U32 * (M + Ls + R) + 1e-6 * R);
     for (int a = 0; a < 3; ++a)
         P.boxf[a] = (float)g.box[a];
+    set_cull(P, R, 3, M, Ls, R);
     P.nbins = nb;
     float T[2 * (cf::NB_MAX + 1)];
     uint8_t tab[cf::LUT_MAX];

@@ -181,7 +181,9 @@ struct PairParams {
     float pscale;       // rp-pi: fl32(npibins / pimax), pi edges at integer t = |dz| * pscale
     float pband;        // rp-pi: |t - 1/2 - round(t - 1/2)| > pband means t is near an edge
     int hcopies;        // rp-pi: shared histogram copies per CTA (warp w uses w % hcopies)
-    int hist_off;       // byte offset of the shared histograms (rp-pi kernels)
+    int hist_off;       // byte offset of the shared histograms
+    int guess_off, e2_off, ring_off, queue_off;  // binary64 counts: start table, edges, rings, queues
+    float cull, zcull;  // binary64 counts: float32 squared distance / dz^2 proven out of reach
     // weighted sums (Code 1's weight per bin) and mean separation
     int weighted;       // pair weight w_i * w_j (else 1)
     int want_r;         // accumulate r (xi) or rp (rp-pi) times the pair weight

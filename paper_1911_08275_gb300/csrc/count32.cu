@@ -1,355 +1,12 @@
-// Float32 DD(r) without sums: the hot loop of the paper (Sec. 2.2, Codes 2-4)
-// over chunk tasks (tasks.cuh).
-//
-// Each lane holds PP primaries, each broadcast into both halves of a 64-bit
-// register, and evaluates them against four consecutive secondaries (one
-// 16-byte load per axis, two packed pairs) with the packed f32x2 instructions.
-// The squared distance indexes (clamped, branch-free) a byte table built on the
-// host from float32 thresholds lo_k < e_k^2 < hi_k that bracket every squared
-// edge by a proven error bound; a safe cell gives the bin row, out-of-range
-// distances a dummy row, and every lane adds one to its own column of the CTA's
-// shared histogram with a shared-memory atomic (no bank conflicts, no branch).
-// A pair in a flagged cell (touching a band) sets a bit of the lane's mask;
-// once per 8 steps a warp-uniform test moves the recorded pairs to the warp's
-// queue, and whenever 32 wait there they are settled together, one per lane: compared
-// with the thresholds, a distance inside a band re-evaluated with the canonical
-// binary64 formula, so counts are bit-identical to the binary64 definition.
-//
-// Bounds, and what was measured (1.2M clustered points, box 420, 20 log bins,
-// Rmax 25, 2.3e9 evaluations, GB300): a step of 8 pairs per lane takes 96
-// instructions (28 packed float32, 8 each of table byte, atomic, address, clamp
-// and flag bit, 3 tile loads) and 28 wavefronts of the L1's data path, which is
-// 81 % busy, issue 68 %: the data path binds first.  Kernel 1.127 ms, against
-// 1.193 ms for CTAs that staged one column pair at a time in two tile buffers and
-// settled flagged pairs where they were found (0.5M pairs in a third of all
-// blocks of 8 steps, a whole warp waiting for one lane); without the queue the
-// chunk tasks took 1.218 ms, and reading the secondaries through the L1 instead
-// of the ring 1.245 ms (four wavefronts per 16-byte load).  Rmax 5 / 10 / 50: 0.282 /
-// 0.280 / 5.285 ms before, 0.219 / 0.270 / 5.12 ms now.
+// Launches of the float32 DD(r) counts (count32.cuh) and the neighbour lists of the
+// chunk tasks.
 #include <cuda_runtime.h>
 
-#include <algorithm>
-
-#include "cf_internal.cuh"
-#include "launch.cuh"
-#include "pairs.cuh"
-#include "tasks.cuh"
+#include "count32.cuh"
 
 namespace cf {
 
 namespace {
-
-// Shared layout: [0, 128) the table's barrier; table; thresholds; squared edges;
-// per warp a ring of secondaries and a queue of flagged pairs; histogram of
-// (nbins + 2) rows of 32 words (row -1 of flagged pairs, the bins, the not-counted
-// row), shared by the CTA's warps.
-constexpr int C32_LUT = 128;
-constexpr int C32_THR = C32_LUT + LUT_MAX;
-constexpr int C32_E2 = C32_THR + 2 * (NB_MAX + 1) * 4;
-constexpr int C32_RING = (C32_E2 + (NB_MAX + 1) * 8 + 127) / 128 * 128;
-constexpr int C32_QUEUE = C32_RING + WARPS * RING_BYTES;
-constexpr int C32_HIST = C32_QUEUE + WARPS * (int)sizeof(FlagQueue);
-
-// What a sweep needs beside the primaries.
-struct Sweep {
-    uint32_t lutb, hl;  // shared addresses: table, this lane's histogram column (row 0)
-    uint32_t u0, lut_last;
-    int shift, nthr, nb;
-    float lscale;
-    FlagQueue *fq;
-    int qn;  // flagged pairs waiting in the warp's queue
-};
-
-// Settle the last min(32, qn) flagged pairs of the warp's queue, one per lane: the
-// float32 d2 with the sweep's operations, counted against the thresholds; inside
-// a band re-evaluated in binary64.  Each pair goes to its true bin (the sweep has
-// put it in row -1, which is never read).  Returns 1 in lanes that re-evaluated.
-__device__ __noinline__ int settle(const PairParams &P, const unsigned char *smem, uint32_t hl,
-                                   const FlagQueue *fq, int qn)
-{
-    const int lane = threadIdx.x & 31, first = max(0, qn - 32);
-    int row = -1, re = 0;
-    __syncwarp();
-    if (first + lane < qn) {
-        const int i = fq->i[first + lane], j = fq->j[first + lane], m = fq->image[first + lane];
-        const int qx = (m & 3) - 1, qy = ((m >> 2) & 3) - 1, qz = ((m >> 4) & 3) - 1;
-        const float *a = P.A.xyz + quad_off((uint32_t)i), *b = P.B.xyz + quad_off((uint32_t)j);
-        const float dx = __fsub_rn(b[0], __fsub_rn(a[0], (float)qx * P.boxf[0]));
-        const float dy = __fsub_rn(b[4], __fsub_rn(a[4], (float)qy * P.boxf[1]));
-        const float dz = __fsub_rn(b[8], __fsub_rn(a[8], (float)qz * P.boxf[2]));
-        const float d2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
-        const int c = thr_count(reinterpret_cast<const float *>(smem + C32_THR), P.nthr, d2);
-        if (!(c & 1)) {
-            row = (c >= 2 && c <= 2 * P.nbins) ? (c - 2) >> 1 : -1;
-        } else {
-            row = bin_f64(canon_r2(P.A.pos64[i], P.B.pos64[j], (double)qx * P.g.box[0],
-                                   (double)qy * P.g.box[1], (double)qz * P.g.box[2]),
-                          reinterpret_cast<const double *>(smem + C32_E2), P.nbins);
-            re = 1;
-        }
-    }
-    if (row >= 0)
-        red_shared1(hl + (uint32_t)row * 128u);
-    __syncwarp();
-    return re;
-}
-
-// Sweep the piece [j0, j1) of a window [jlo, jhi), its secondaries at shared
-// address addr.  Lane (ii, jj) holds PP primaries and evaluates them against the
-// quad 4 jj .. 4 jj + 3 of each step; a step covers I PP primaries x JS = 128 / I
-// secondaries and starts at a multiple of JS, so it never leaves the column
-// (columns are padded to 32).  Secondaries outside the window are farther than
-// Rmax in z and never counted.  TRI: pairs with j <= i do not count.
-template <int I, int PP, bool TRI, bool EVALS, bool VERIFY, bool LIN>
-__device__ __forceinline__ void sweep(const PairParams &P, const unsigned char *smem, Sweep &S,
-                                      uint32_t addr, int j0, int j1, int jlo, int jhi, int jj,
-                                      const u64 (&XH)[PP], const u64 (&YH)[PP], const u64 (&ZH)[PP], int ib,
-                                      int image, unsigned vmask, u64 &n_eval, u64 &n_rck, u64 &n_viol)
-{
-    constexpr int JS = 128 / I;
-    const float qnan = __int_as_float(0x7fc00000);
-    const u64 LS = pack2(S.lscale, S.lscale), LM = pack2(LIN_MAGIC, LIN_MAGIC);
-    const uint32_t lut_lo = S.lutb - LIN_MAGIC_BITS, lut_hi = S.lutb + S.lut_last;
-    const int ii = (threadIdx.x & 31) % I;
-    const uint32_t p0 = addr + 48u * jj;  // this lane's first quad
-    const int jf = j0 + 4 * jj;           // its first secondary
-    uint32_t p = p0;
-    for (int nit = (j1 - j0 + JS - 1) / JS; nit > 0; nit -= 8) {
-        const int tend = min(8, nit);
-        const uint32_t pb = p, pend = p + (uint32_t)tend * (12u * JS);
-        uint32_t fm[PP];
-#pragma unroll
-        for (int q = 0; q < PP; ++q)
-            fm[q] = 0u;
-#pragma unroll 1
-        for (; p != pend; p += 12 * JS) {
-            const int jt = jf + (int)((p - p0) / 12u);  // (TRI and diagnostics only)
-            ulonglong2 vx, vy, vz;
-            lds128<0>(p, vx);
-            lds128<16>(p, vy);
-            lds128<32>(p, vz);
-            float d[PP][4];
-            uint32_t cq[PP][4];
-#pragma unroll
-            for (int q = 0; q < PP; ++q) {
-                u64 dx = fsub2(vx.x, XH[q]), dy = fsub2(vy.x, YH[q]), dz = fsub2(vz.x, ZH[q]);
-                const u64 dA = ffma2(dz, dz, ffma2(dy, dy, fmul2(dx, dx)));
-                dx = fsub2(vx.y, XH[q]);
-                dy = fsub2(vy.y, YH[q]);
-                dz = fsub2(vz.y, ZH[q]);
-                const u64 dB = ffma2(dz, dz, ffma2(dy, dy, fmul2(dx, dx)));
-                unpack2(dA, d[q][0], d[q][1]);
-                unpack2(dB, d[q][2], d[q][3]);
-                if (LIN) {  // one packed fma gives two cells; the sum is >= 2^23 (NaN larger)
-                    float c[4];
-                    unpack2(ffma2(dA, LS, LM), c[0], c[1]);
-                    unpack2(ffma2(dB, LS, LM), c[2], c[3]);
-#pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        cq[q][r] = min(__float_as_uint(c[r]) + lut_lo, lut_hi);
-                } else {
-#pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        cq[q][r] = S.lutb + min((__float_as_uint(d[q][r]) >> S.shift) - S.u0, S.lut_last);
-                }
-            }
-            if (TRI) {
-#pragma unroll
-                for (int q = 0; q < PP; ++q)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const bool live = jt + r > ib + q * I + ii;
-                        cq[q][r] = live ? cq[q][r] : lut_hi;
-                        d[q][r] = live ? d[q][r] : qnan;
-                    }
-            }
-            if (EVALS) {
-#pragma unroll
-                for (int q = 0; q < PP; ++q)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        n_eval += (((vmask >> q) & 1u) && jt + r >= jlo && jt + r < jhi &&
-                                   (!TRI || jt + r > ib + q * I + ii)) ? 1ull : 0ull;
-            }
-#pragma unroll
-            for (int q = 0; q < PP; ++q)
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const uint32_t e = lds_entry(cq[q][r]);  // the row: bin, dummy or flagged (-1)
-                    red_shared1(S.hl + e * 128u);
-                    fm[q] = push_sign(fm[q], e);  // pair (t, r) ends at bit 4 tend - 1 - (4 t + r)
-                }
-            if (VERIFY) {
-                const float *T = reinterpret_cast<const float *>(smem + C32_THR);
-                const double *E2 = reinterpret_cast<const double *>(smem + C32_E2);
-#pragma unroll
-                for (int q = 0; q < PP; ++q)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r)  // sentinels and padding give NaN
-                        if (((vmask >> q) & 1u) && !isnan(d[q][r]))
-                            n_viol += verify_pair(d[q][r], T, S.nthr, S.nb, E2, P.A.pos64, P.B.pos64,
-                                                  ib + q * I + ii, jt + r,
-                                                  (double)((image & 3) - 1) * P.g.box[0],
-                                                  (double)(((image >> 2) & 3) - 1) * P.g.box[1],
-                                                  (double)(((image >> 4) & 3) - 1) * P.g.box[2]);
-            }
-        }
-        uint32_t anyf = 0u;
-#pragma unroll
-        for (int q = 0; q < PP; ++q)
-            anyf |= fm[q];
-        if (__any_sync(FULL, anyf != 0u)) {  // queue the flagged pairs; settle them 32 at a time
-#pragma unroll
-            for (int q = 0; q < PP; ++q) {
-                uint32_t m = fm[q];
-                for (unsigned bm; (bm = __ballot_sync(FULL, m != 0u)) != 0u;) {
-                    if (m) {
-                        const int b = 4 * tend - __ffs(m);  // = 4 t + r
-                        const int at = S.qn + __popc(bm & ((1u << (threadIdx.x & 31)) - 1u));
-                        S.fq->i[at] = ib + q * I + ii;
-                        S.fq->j[at] = jf + (int)((pb - p0) / 12u) + (b >> 2) * JS + (b & 3);
-                        S.fq->image[at] = image;
-                        m &= m - 1u;
-                    }
-                    S.qn += __popc(bm);
-                    if (S.qn >= 32) {
-                        n_rck += settle(P, smem, S.hl, S.fq, S.qn);
-                        S.qn -= 32;
-                    }
-                }
-            }
-        }
-    }
-}
-
-template <int I, int PP, bool EVALS, bool VERIFY, bool LIN, int MINB>
-__global__ void __launch_bounds__(THREADS, MINB) k_count32(const __grid_constant__ PairParams P)
-{
-    constexpr int CH = I * PP;
-    extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
-    const int tid = threadIdx.x, lane = tid & 31, ii = lane % I, jj = lane / I, nb = P.nbins;
-    uint32_t *hist = reinterpret_cast<uint32_t *>(smem + C32_HIST);
-
-    // the table by one bulk copy (bounded wait), the rest by the threads
-    if (tid == 0) {
-        mbar_init(bar, 1);
-        fence_mbar_init();
-        const unsigned bytes = ((unsigned)P.lut_n + 15u) & ~15u;
-        mbar_arrive_expect_tx(bar, bytes);
-        if (!(P.flags & CF_FLAG_DEBUG_STALL))  // diagnostic stall: the armed copy is never issued
-            bulk_g2s(smem + C32_LUT, P.lut, bytes, bar);
-    }
-    for (int q = tid; q < P.nthr; q += THREADS)
-        reinterpret_cast<float *>(smem + C32_THR)[q] = P.thr[q];
-    for (int q = tid; q <= nb; q += THREADS)
-        reinterpret_cast<double *>(smem + C32_E2)[q] = P.E2[q];
-    for (int q = tid; q < (nb + 2) * 32; q += THREADS)
-        hist[q] = 0u;
-    __syncthreads();
-    if (__syncthreads_or(!mbar_wait(bar, 0u, P.wait_ns))) {
-        if (tid == 0) {
-            atomicOr(P.err, ERR_TIMEOUT);
-            mbar_wait(bar, 0u, P.wait_ns);  // a late copy lands before the CTA exits
-        }
-        return;
-    }
-
-    Sweep S;
-    S.lutb = smem_u32(smem + C32_LUT);
-    S.hl = smem_u32(hist + 32 + lane);  // row 0 (row -1 before it)
-    S.u0 = P.u0;
-    S.lut_last = (uint32_t)(P.lut_n - 1);
-    S.shift = P.lut_shift;
-    S.nthr = P.nthr;
-    S.nb = nb;
-    S.lscale = P.lut_scale;
-    S.fq = reinterpret_cast<FlagQueue *>(smem + C32_QUEUE) + (tid >> 5);
-    S.qn = 0;
-    const uint32_t ring = smem_u32(smem + C32_RING) + (uint32_t)(tid >> 5) * RING_BYTES;
-    const TaskSplit split(__ldg(P.A.cell_start + P.g.ncells) / CH, (unsigned)P.parts);
-    u64 n_eval = 0, n_rck = 0, n_viol = 0;
-    unsigned pending = 0;
-
-    unsigned nxt = 0;
-    if (lane == 0)
-        nxt = atomicAdd(P.item_counter, 1u);
-    for (unsigned t = __shfl_sync(FULL, nxt, 0); t < split.ntask; t = __shfl_sync(FULL, nxt, 0)) {
-        if (lane == 0)
-            nxt = atomicAdd(P.item_counter, 1u);  // read at the end of this task
-        unsigned c, part, parts;
-        split.task(t, c, part, parts);
-        const int ib = (int)(c * CH);
-        const int col = __ldg(P.A.chunk_col + ib / (int)COL_PAD);
-        float xq[PP], yq[PP], zq[PP];
-        int zb = 0;
-        unsigned vmask = 0;
-#pragma unroll
-        for (int q = 0; q < PP; ++q) {
-            const float *p = P.A.xyz + quad_off((uint32_t)(ib + q * I + ii));
-            xq[q] = __ldg(p);
-            yq[q] = __ldg(p + 4);
-            zq[q] = __ldg(p + 8);
-            const bool v = !isnan(xq[q]);  // column padding is NaN
-            vmask |= (unsigned)v << q;
-            if (v)  // frame coordinates are >= 0: they order like their bits (-0 below)
-                zb = max(zb, __float_as_int(zq[q]));
-        }
-        const float zlo = __shfl_sync(FULL, zq[0], 0);
-        if (isnan(zlo))
-            continue;  // a chunk of padding
-        const float zhi = __int_as_float(__reduce_max_sync(FULL, zb));
-        u64 XH[PP], YH[PP], ZH[PP];
-        int image = 0;  // of the current window: qx + 1, qy + 1, qz + 1 in two bits each
-        for_windows<128 / I>(
-            P, col, ib, zlo, zhi, (int)part, (int)parts, lane, ring,
-            [&](int k, int code) {
-                image = (code & 15) | ((k + 1) << 4);
-                const float Sx = (float)((code & 3) - 1) * P.boxf[0];
-                const float Sy = (float)(((code >> 2) & 3) - 1) * P.boxf[1], Sz = (float)k * P.boxf[2];
-#pragma unroll
-                for (int q = 0; q < PP; ++q) {
-                    const float xh = __fsub_rn(xq[q], Sx), yh = __fsub_rn(yq[q], Sy), zh = __fsub_rn(zq[q], Sz);
-                    XH[q] = pack2(xh, xh);
-                    YH[q] = pack2(yh, yh);
-                    ZH[q] = pack2(zh, zh);
-                }
-            },
-            [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {
-                pending += (unsigned)((j1 - j0) / (128 / I) + 1) * 4u * PP;
-                if (tri)
-                    sweep<I, PP, true, EVALS, VERIFY, LIN>(P, smem, S, addr, j0, j1, jlo, jhi, jj, XH, YH, ZH,
-                                                           ib, image, vmask, n_eval, n_rck, n_viol);
-                else
-                    sweep<I, PP, false, EVALS, VERIFY, LIN>(P, smem, S, addr, j0, j1, jlo, jhi, jj, XH, YH, ZH,
-                                                            ib, image, vmask, n_eval, n_rck, n_viol);
-                if (pending > (1u << 30) / WARPS) {  // keep every shared u32 count far from overflow
-                    __syncwarp();
-                    warp_flush_shared(hist + 32, nb, P.hist, lane);
-                    pending = 0;
-                }
-            });
-    }
-    if (S.qn)
-        n_rck += settle(P, smem, S.hl, S.fq, S.qn);
-    __syncthreads();
-    for (int b = tid >> 5; b < nb; b += WARPS) {
-        const u64 v = warp_sum_u64(hist[(b + 1) * 32 + lane]);
-        if (lane == 0 && v)
-            atomicAdd(&P.hist[b], v);
-    }
-    n_eval = warp_sum_u64(n_eval);
-    n_rck = warp_sum_u64(n_rck);
-    n_viol = warp_sum_u64(n_viol);
-    if (lane == 0) {
-        if (n_eval)
-            atomicAdd(&P.diag[1], n_eval);
-        if (n_rck)
-            atomicAdd(&P.diag[2], n_rck);
-        if (n_viol)
-            atomicAdd(&P.diag[3], n_viol);
-    }
-}
 
 // Neighbour lists (Sec. 2.1, 2.2): one warp per primary column, one stencil
 // offset per lane; the kept column pairs are listed in stencil order with
@@ -385,24 +42,10 @@ __global__ void __launch_bounds__(128) k_neighbours(const __grid_constant__ Pair
 }
 
 template <int I, int PP, bool EVALS, bool VERIFY, int MINB>
-cudaError_t launch_shape(PairParams &P, PairLaunch &L, int sms, cudaStream_t st)
+cudaError_t launch_shape(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st)
 {
-    const long long chunks = (P.A.n + (long long)P.g.ncols * (COL_PAD / 2)) / (I * PP) + 1;
-    auto go = [&](auto kern) {
-        int occ = 0;
-        cudaError_t e = occupancy(kern, L.smem, occ);
-        if (e)
-            return e;
-        if (occ < 1)
-            return cudaErrorInvalidConfiguration;
-        P.parts = std::min(P.nstencil, TASK_PARTS);
-        const long long tasks = chunks * P.parts;
-        L.blocks = (int)std::max(1ll, std::min<long long>((long long)sms * occ, (tasks + WARPS - 1) / WARPS));
-        kern<<<L.blocks, THREADS, L.smem, st>>>(P);
-        return cudaGetLastError();
-    };
-    return P.lut_lin ? go(k_count32<I, PP, EVALS, VERIFY, true, MINB>)
-                     : go(k_count32<I, PP, EVALS, VERIFY, false, MINB>);
+    return P.lut_lin ? launch_tasks<Count32<I, PP, EVALS, VERIFY, 1>, MINB>(P, L, sms, st)
+                     : launch_tasks<Count32<I, PP, EVALS, VERIFY, 0>, MINB>(P, L, sms, st);
 }
 
 }  // namespace
@@ -415,9 +58,8 @@ cudaError_t launch_neighbours(const PairParams &P, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_count32(const PairParams &P0, PairLaunch &L, int sms, cudaStream_t st)
+cudaError_t launch_count32(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st)
 {
-    PairParams P = P0;
     L.smem = count32_smem(P.nbins);
     if (L.verify)
         return launch_shape<8, 1, true, true, 3>(P, L, sms, st);

@@ -1,0 +1,55 @@
+// Launches of the binary64 counts (cull64.cuh).
+#include <cuda_runtime.h>
+
+#include "cull64.cuh"
+
+namespace cf {
+
+// Shared memory of a binary64 count: [0, 128) free, start table of the
+// binning, squared edges and pi edges,
+// per warp a ring of secondaries and a queue of pairs, histograms, binary64 sums.
+// DD(rp, pi): one histogram copy per warp while three CTAs fit an SM, else fewer
+// copies shared by several warps.
+int plan_count64(PairParams &P)
+{
+    const int slots = P.kind == 0 ? P.nbins : P.nbins * P.npibins;
+    P.guess_off = 128;
+    P.e2_off = P.guess_off + GUESS;
+    P.ring_off = align_up(P.e2_off + (P.nbins + 1 + (P.kind == 1 ? P.npibins + 1 : 0)) * 8, 128);
+    P.queue_off = P.ring_off + WARPS * RING_BYTES;
+    P.hist_off = align_up(P.queue_off + WARPS * (int)sizeof(FlagQueue), 128);
+    const int sums = P.wacc ? slots * 16 : 0;
+    if (P.kind == 0) {
+        P.hcopies = P.wacc ? WARPS : 1;  // of the sums; the counts have a word per lane
+        P.acc_off = P.hist_off + P.nbins * 128;
+        return align_up(P.acc_off + P.hcopies * sums, 128);
+    }
+    P.hcopies = 1;
+    for (int c = WARPS; c > 1; c >>= 1)
+        if (P.hist_off + c * (slots * 4 + sums) <= 75 * 1024) {
+            P.hcopies = c;
+            break;
+        }
+    P.acc_off = align_up(P.hist_off + P.hcopies * slots * 4, 16);
+    return align_up(P.acc_off + P.hcopies * sums, 128);
+}
+
+cudaError_t launch_count64(const PairParams &P0, PairLaunch &L, int sms, cudaStream_t st)
+{
+    PairParams P = P0;
+    L.smem = plan_count64(P);
+    if (P.kind == 0) {
+        if (P.wacc)
+            return L.evals ? launch_tasks<Cull64<0, true, true>, 3>(P, L, sms, st)
+                           : launch_tasks<Cull64<0, false, true>, 3>(P, L, sms, st);
+        return L.evals ? launch_tasks<Cull64<0, true, false>, 3>(P, L, sms, st)
+                       : launch_tasks<Cull64<0, false, false>, 3>(P, L, sms, st);
+    }
+    if (P.wacc)
+        return L.evals ? launch_tasks<Cull64<1, true, true>, 3>(P, L, sms, st)
+                       : launch_tasks<Cull64<1, false, true>, 3>(P, L, sms, st);
+    return L.evals ? launch_tasks<Cull64<1, true, false>, 3>(P, L, sms, st)
+                   : launch_tasks<Cull64<1, false, false>, 3>(P, L, sms, st);
+}
+
+}  // namespace cf

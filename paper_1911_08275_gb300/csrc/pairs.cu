@@ -2609,10 +2609,10 @@ cudaError_t launch_pairs(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
     if (P0.n_items <= 0)
         return cudaSuccess;
     PairParams P = P0;
-    if (P.kind == 0 && !L.f64 && !P.wacc) {  // float32 DD(r) counts: chunk tasks
+    if (L.f64 || (P.kind == 0 && !P.wacc)) {  // chunk tasks
         cudaError_t e0 = launch_neighbours(P, st);
         if (!e0)
-            e0 = launch_count32(P, L, sms, st);
+            e0 = L.f64 ? launch_count64(P, L, sms, st) : launch_count32(P, L, sms, st);
         L.kernels = 2;
         return e0;
     }
@@ -2634,13 +2634,6 @@ cudaError_t launch_pairs(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
         L.kernels = 3;
     }
     if (P.kind == 1) {
-        if (L.f64) {
-            if (P.wacc)
-                return L.evals ? launch_persistent(k_path<Rppi64Path<8, true, true>, 1>, P, L, sms, st)
-                               : launch_persistent(k_path<Rppi64Path<8, false, true>, 1>, P, L, sms, st);
-            return L.evals ? launch_persistent(k_path<Rppi64Path<8, true, false>, 1>, P, L, sms, st)
-                           : launch_persistent(k_path<Rppi64Path<8, false, false>, 1>, P, L, sms, st);
-        }
         if (P.wacc)
             return L.evals ? launch_persistent(k_path<Rppi32Path<16, true, false, true>, 3>, P, L, sms, st)
                            : launch_persistent(k_path<Rppi32Path<16, false, false, true>, 3>, P, L, sms, st);
@@ -2663,13 +2656,6 @@ cudaError_t launch_pairs(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
     }
     if (P.kind != 0)
         return cudaErrorNotSupported;
-    if (L.f64) {
-        if (P.wacc)
-            return L.evals ? launch_persistent(k_path<Xi64Path<8, true, true>, 1>, P, L, sms, st)
-                           : launch_persistent(k_path<Xi64Path<8, false, true>, 1>, P, L, sms, st);
-        return L.evals ? launch_persistent(k_path<Xi64Path<8, true, false>, 1>, P, L, sms, st)
-                       : launch_persistent(k_path<Xi64Path<8, false, false>, 1>, P, L, sms, st);
-    }
     constexpr int HW = WARPS;
     constexpr bool PW = true;
     if (P.wacc) {  // pair weights and / or mean separation: integer sums in the same sweep

@@ -12,6 +12,10 @@
 // column may be as narrow as a chunk.
 #pragma once
 
+#include <algorithm>
+
+#include "launch.cuh"
+#include "pairs.cuh"
 #include "pairs_dev.cuh"
 
 namespace cf {
@@ -110,6 +114,54 @@ __device__ __forceinline__ void cp_wait()
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// A chunk's primaries: lane ii of I holds the entries ib + q I + ii.
+template <int I, int PP>
+struct Chunk {
+    float x[PP], y[PP], z[PP];
+    float zlo, zhi;  // z range of the real entries
+    unsigned vmask;  // bit q: entry q is real (column padding is NaN)
+    int col;
+
+    // False if the chunk holds only padding.
+    __device__ __forceinline__ bool load(const PairParams &P, int ib, int ii)
+    {
+        col = __ldg(P.A.chunk_col + ib / (int)COL_PAD);
+        int zb = 0;
+        vmask = 0;
+#pragma unroll
+        for (int q = 0; q < PP; ++q) {
+            const float *p = P.A.xyz + quad_off((uint32_t)(ib + q * I + ii));
+            x[q] = __ldg(p);
+            y[q] = __ldg(p + 4);
+            z[q] = __ldg(p + 8);
+            const bool v = !isnan(x[q]);
+            vmask |= (unsigned)v << q;
+            if (v)  // frame coordinates are >= 0: they order like their bits (-0 below)
+                zb = max(zb, __float_as_int(z[q]));
+        }
+        zlo = __shfl_sync(FULL, z[0], 0);
+        zhi = __int_as_float(__reduce_max_sync(FULL, zb));
+        return !isnan(zlo);
+    }
+
+    // The primaries shifted for image code / k, broadcast into packed pairs;
+    // returns the image (qx + 1, qy + 1, qz + 1 in two bits each).
+    __device__ __forceinline__ int shift(const PairParams &P, int k, int code, u64 (&XH)[PP], u64 (&YH)[PP],
+                                         u64 (&ZH)[PP]) const
+    {
+        const float Sx = (float)((code & 3) - 1) * P.boxf[0];
+        const float Sy = (float)(((code >> 2) & 3) - 1) * P.boxf[1], Sz = (float)k * P.boxf[2];
+#pragma unroll
+        for (int q = 0; q < PP; ++q) {
+            const float xh = __fsub_rn(x[q], Sx), yh = __fsub_rn(y[q], Sy), zh = __fsub_rn(z[q], Sz);
+            XH[q] = pack2(xh, xh);
+            YH[q] = pack2(yh, yh);
+            ZH[q] = pack2(zh, zh);
+        }
+        return (code & 15) | ((k + 1) << 4);
+    }
+};
+
 // The windows of the chunk [ib, ib + CH) of column col against its neighbours
 // part, part + parts, ...; all lanes call it together.  For every window,
 // open(k, code) sets the primaries up for the image, then for every piece
@@ -184,6 +236,49 @@ __device__ __forceinline__ void for_windows(const PairParams &P, int col, int ib
             }
         }
     }
+}
+
+// Persistent kernel over the chunk tasks of one count.  Path: CH (primaries per
+// chunk), State, init (false in every thread if the CTA has to give up), task,
+// fini.
+template <class Path, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB) k_tasks(const __grid_constant__ PairParams P)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    typename Path::State st;
+    if (!Path::init(P, smem, st))
+        return;
+    const int lane = threadIdx.x & 31;
+    const TaskSplit split(__ldg(P.A.cell_start + P.g.ncells) / Path::CH, (unsigned)P.parts);
+    unsigned nxt = 0;
+    if (lane == 0)
+        nxt = atomicAdd(P.item_counter, 1u);
+    for (unsigned t = __shfl_sync(FULL, nxt, 0); t < split.ntask; t = __shfl_sync(FULL, nxt, 0)) {
+        if (lane == 0)
+            nxt = atomicAdd(P.item_counter, 1u);  // read at the end of this task
+        unsigned c, part, parts;
+        split.task(t, c, part, parts);
+        Path::task(P, smem, st, c, part, parts);
+    }
+    Path::fini(P, smem, st);
+}
+
+// Launch k_tasks with L.smem bytes of shared memory per CTA.
+template <class Path, int MINB>
+cudaError_t launch_tasks(const PairParams &P0, PairLaunch &L, int sms, cudaStream_t st)
+{
+    PairParams P = P0;
+    int occ = 0;
+    const cudaError_t e = occupancy(k_tasks<Path, MINB>, L.smem, occ);
+    if (e)
+        return e;
+    if (occ < 1)
+        return cudaErrorInvalidConfiguration;
+    const long long chunks = (P.A.n + (long long)P.g.ncols * (COL_PAD / 2)) / Path::CH + 1;
+    P.parts = std::min(P.nstencil, TASK_PARTS);
+    L.blocks = (int)std::max(1ll, std::min<long long>((long long)sms * occ, (chunks * P.parts + WARPS - 1) / WARPS));
+    k_tasks<Path, MINB><<<L.blocks, THREADS, L.smem, st>>>(P);
+    return cudaGetLastError();
 }
 
 }  // namespace
