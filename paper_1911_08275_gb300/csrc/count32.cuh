@@ -228,22 +228,15 @@ struct Count32 {
         Sweep S;
         u64 n_eval, n_rck, n_viol;
         unsigned pending;  // pairs added to this lane's column since the last flush
-        unsigned phase;    // parity of the table's barrier
     };
 
-    // First use of the barrier by this CTA.
-    static __device__ __forceinline__ void arm(unsigned char *smem)
+    static __device__ __forceinline__ bool init(const PairParams &P, unsigned char *smem, State &st)
     {
         if (threadIdx.x == 0) {
             mbar_init(reinterpret_cast<uint64_t *>(smem), 1);
             fence_mbar_init();
         }
         __syncthreads();
-    }
-
-    static __device__ __forceinline__ bool init(const PairParams &P, unsigned char *smem, State &st)
-    {
-        arm(smem);
         return load(P, smem, st, 0u);
     }
 
@@ -251,30 +244,16 @@ struct Count32 {
     static __device__ __forceinline__ bool load(const PairParams &P, unsigned char *smem, State &st,
                                                 unsigned phase)
     {
-        uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
         uint32_t *hist = reinterpret_cast<uint32_t *>(smem + C32_HIST);
         const int tid = threadIdx.x, nb = P.nbins;
-        // the table by one bulk copy (bounded wait), the rest by the threads
-        if (tid == 0) {
-            const unsigned bytes = ((unsigned)P.lut_n + 15u) & ~15u;
-            fence_proxy_async_smem();
-            mbar_arrive_expect_tx(bar, bytes);
-            if (!(P.flags & CF_FLAG_DEBUG_STALL))  // diagnostic stall: the armed copy is never issued
-                bulk_g2s(smem + C32_LUT, P.lut, bytes, bar);
-        }
-        for (int q = tid; q < P.nthr; q += THREADS)
-            reinterpret_cast<float *>(smem + C32_THR)[q] = P.thr[q];
-        for (int q = tid; q <= nb; q += THREADS)
-            reinterpret_cast<double *>(smem + C32_E2)[q] = P.E2[q];
-        for (int q = tid; q < (nb + 2) * 32; q += THREADS)
-            hist[q] = 0u;
-        if (__syncthreads_or(!mbar_wait(bar, phase, P.wait_ns))) {
-            if (tid == 0) {
-                atomicOr(P.err, ERR_TIMEOUT);
-                mbar_wait(bar, phase, P.wait_ns);  // a late copy lands before the CTA exits
-            }
-            return false;
-        }
+        const bool ok = load_table(P, smem, C32_LUT, phase, [&]() {
+            for (int q = tid; q < P.nthr; q += THREADS)
+                reinterpret_cast<float *>(smem + C32_THR)[q] = P.thr[q];
+            for (int q = tid; q <= nb; q += THREADS)
+                reinterpret_cast<double *>(smem + C32_E2)[q] = P.E2[q];
+            for (int q = tid; q < (nb + 2) * 32; q += THREADS)
+                hist[q] = 0u;
+        });
         st.n_eval = st.n_rck = st.n_viol = 0ull;
         st.pending = 0u;
         Sweep &S = st.S;
@@ -288,7 +267,7 @@ struct Count32 {
         S.lscale = P.lut_scale;
         S.fq = reinterpret_cast<FlagQueue *>(smem + C32_QUEUE) + (tid >> 5);
         S.qn = 0;
-        return true;
+        return ok;
     }
 
     static __device__ __forceinline__ void task(const PairParams &P, unsigned char *smem, State &st,

@@ -1309,13 +1309,6 @@ struct Xi64Path {
 constexpr float PI_MAGIC = 12582912.0f;        // 1.5 * 2^23: spacing 1 in [2^23, 2^24)
 constexpr uint32_t PI_MAGIC_BITS = 0x4b400000u;  // its bit pattern
 
-__device__ __forceinline__ u64 fadd2(u64 a, u64 b)
-{
-    u64 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 __device__ __forceinline__ u64 fabs2(u64 a) { return a & 0x7fffffff7fffffffull; }
 
 __device__ __forceinline__ void red_shared(uint32_t addr, uint32_t v)
@@ -2609,10 +2602,11 @@ cudaError_t launch_pairs(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
     if (P0.n_items <= 0)
         return cudaSuccess;
     PairParams P = P0;
-    if (L.f64 || (P.kind == 0 && !P.wacc)) {  // chunk tasks
+    if (L.f64 || !P.wacc) {  // chunk tasks
         cudaError_t e0 = launch_neighbours(P, st);
         if (!e0)
-            e0 = L.f64 ? launch_count64(P, L, sms, st) : launch_count32(P, L, sms, st);
+            e0 = L.f64 ? launch_count64(P, L, sms, st)
+                       : P.kind == 0 ? launch_count32(P, L, sms, st) : launch_countrp32(P, L, sms, st);
         L.kernels = 2;
         return e0;
     }
@@ -2637,22 +2631,7 @@ cudaError_t launch_pairs(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
         if (P.wacc)
             return L.evals ? launch_persistent(k_path<Rppi32Path<16, true, false, true>, 3>, P, L, sms, st)
                            : launch_persistent(k_path<Rppi32Path<16, false, false, true>, 3>, P, L, sms, st);
-        if (L.verify)
-            return launch_persistent(k_path<Rppi32Path<8, true, true, false>, 3>, P, L, sms, st);
-        if (L.pp == 2)  // two primaries per lane, deferred flags
-            return L.evals ? launch_persistent(k_path<Rppi32PathPP<16, 2, true>, 3>, P, L, sms, st)
-                           : launch_persistent(k_path<Rppi32PathPP<16, 2, false>, 3>, P, L, sms, st);
-        switch (L.chunk) {
-        case 16:
-            return L.evals ? launch_persistent(k_path<Rppi32Path<16, true, false, false>, 3>, P, L, sms, st)
-                           : launch_persistent(k_path<Rppi32Path<16, false, false, false>, 3>, P, L, sms, st);
-        case 32:
-            return L.evals ? launch_persistent(k_path<Rppi32Path<32, true, false, false>, 3>, P, L, sms, st)
-                           : launch_persistent(k_path<Rppi32Path<32, false, false, false>, 3>, P, L, sms, st);
-        default:
-            return L.evals ? launch_persistent(k_path<Rppi32Path<8, true, false, false>, 3>, P, L, sms, st)
-                           : launch_persistent(k_path<Rppi32Path<8, false, false, false>, 3>, P, L, sms, st);
-        }
+        return cudaErrorNotSupported;
     }
     if (P.kind != 0)
         return cudaErrorNotSupported;

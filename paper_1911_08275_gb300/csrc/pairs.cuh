@@ -79,6 +79,9 @@ void plan_pairs(PairParams &P, PairLaunch &L);
 cudaError_t launch_neighbours(const PairParams &P, cudaStream_t st);
 cudaError_t launch_count32(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
 int count32_smem(int nbins);
+// Float32 DD(rp, pi) counts.
+cudaError_t launch_countrp32(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
+int countrp32_smem(int nbins, int npibins);
 // Binary64 counts: offsets and histogram copies into P, bytes of shared memory back.
 int plan_count64(PairParams &P);
 cudaError_t launch_count64(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);

@@ -114,6 +114,32 @@ __device__ __forceinline__ void cp_wait()
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// The job's byte table by one bulk copy into smem + lut_off, while fill() writes
+// what else the CTA needs (the barrier at smem is initialised; its phase parity is
+// phase).  False in every thread if the wait gave up.
+template <class Fill>
+__device__ __forceinline__ bool load_table(const PairParams &P, unsigned char *smem, int lut_off,
+                                           unsigned phase, Fill fill)
+{
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
+    if (threadIdx.x == 0) {
+        const unsigned bytes = ((unsigned)P.lut_n + 15u) & ~15u;
+        fence_proxy_async_smem();
+        mbar_arrive_expect_tx(bar, bytes);
+        if (!(P.flags & CF_FLAG_DEBUG_STALL) || P.kind != 0)  // diagnostic stall: never issued
+            bulk_g2s(smem + lut_off, P.lut, bytes, bar);
+    }
+    fill();
+    if (__syncthreads_or(!mbar_wait(bar, phase, P.wait_ns))) {
+        if (threadIdx.x == 0) {
+            atomicOr(P.err, ERR_TIMEOUT);
+            mbar_wait(bar, phase, P.wait_ns);  // a late copy lands before the CTA exits
+        }
+        return false;
+    }
+    return true;
+}
+
 // A chunk's primaries: lane ii of I holds the entries ib + q I + ii.
 template <int I, int PP>
 struct Chunk {
