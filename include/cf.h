@@ -220,10 +220,11 @@ int cf_countpairs_xi_noalloc(int autocorr, const cf_catalog *d1, const cf_catalo
  * of uneven sizes, DD(r) or DD(rp, pi), float32+re-check or binary64, auto or
  * cross, periodic or open -- are added to a batch and then run together: every
  * gridding stage runs once for all catalogues of all jobs (each catalogue a
- * segment of the launch), the work lists of all jobs in one more launch, and
- * one persistent kernel pulls column pairs from a single queue over all jobs'
- * work lists (the GPU analogue of the paper's OpenMP loop over cell pairs,
- * Sec. 2.1): a run is 16 launches whatever the number of jobs.  With
+ * segment of the launch), the neighbour lists of all jobs in one more launch, and
+ * one persistent kernel per kind of count (DD(r) or DD(rp, pi), float32 or
+ * binary64, kernel shape) whose CTAs attach to one job after another (the GPU
+ * analogue of the paper's OpenMP loop over cell pairs, Sec. 2.1): a run is 13
+ * launches plus one per kind, whatever the number of jobs.  With
  * use_graph the whole sequence is captured once into a CUDA graph and replayed
  * by later runs.  A job's res->n_kernels is 0 (the launches are shared; the
  * batch's count is in cf_batch_stats).
@@ -255,12 +256,12 @@ typedef struct cf_batch cf_batch;
 
 typedef struct {
     uint64_t n_jobs;
-    uint64_t n_kernels;   /* kernels of one run (gridding, work lists, offsets, batched kernel) */
+    uint64_t n_kernels;   /* kernels of one run (gridding, neighbour lists, a pair kernel per kind) */
     uint64_t pairs;       /* sum over jobs of the counted pairs                   */
     int used_graph;       /* 1 if the run launched the captured graph             */
     int planned;          /* 1 if the run (re)planned the jobs                    */
-    int blocks;           /* CTAs of the batched kernel                           */
-    double kernel_ms;     /* device time of the batched pair kernel (-1 when the
+    int blocks;           /* CTAs of the largest pair kernel                      */
+    double kernel_ms;     /* device time of the batched pair kernels (-1 when the
                              run replayed a graph: only the whole run is timed)  */
     double total_ms;      /* device time of the run (memsets to the final copy)   */
 } cf_batch_stats;

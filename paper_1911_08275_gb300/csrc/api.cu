@@ -1949,17 +1949,17 @@ struct BatchJob {
 struct cf_batch {
     std::vector<BatchJob> jobs;
     bool planned = false;
-    int dev = -1, sms = 0, smem_max = 0, blocks = 0;
+    int dev = -1, sms = 0, blocks = 0;
+    cf::BatchPlan plan;
     void *ws = nullptr;                  // one device workspace for every job
     unsigned long long *d_out = nullptr; // output block (all jobs)
     size_t out_words = 0;
     unsigned long long *h_out = nullptr; // page-locked copy of the output block
     cf::PairParams *d_jobs = nullptr;
-    int *d_path = nullptr;
-    unsigned *d_offsets = nullptr, *d_counter = nullptr;
+    int *d_list = nullptr, *d_start = nullptr;  // device copies of the plan's
     unsigned long long *d_bbox = nullptr;
     cf::GridBatch grid = {};             // every catalogue of every job, gridded in one pass
-    unsigned *d_wpre = nullptr;          // work-list blocks: prefix over the jobs
+    unsigned *d_wpre = nullptr;          // neighbour-list blocks: prefix over the jobs
     unsigned wblocks = 0;
     cudaStream_t own = nullptr;
     cudaEvent_t ev[4] = {};
@@ -1969,6 +1969,24 @@ struct cf_batch {
 };
 
 namespace {
+
+// First jobs a plan holds, per SM: at most 12 kinds of count (2 of them binary64)
+// with at most 8 CTAs per SM each.
+constexpr int BATCH_STARTS = 12 * 8;
+
+// Estimated work of a job: pairs in the windows (points times the secondaries
+// within reach of a column), and a fixed part per point.
+double batch_work(const BatchJob &j)
+{
+    const double R = j.edges.back(), rz = j.q.kind == 0 ? R : j.q.pimax;
+    double frac = 1.0;
+    const double len[3] = {3.0 * R, 3.0 * R, 2.5 * rz};
+    for (int a = 0; a < 3; ++a)
+        if (j.g.extent[a] > len[a])
+            frac *= len[a] / j.g.extent[a];
+    const double na = (double)j.cat[0].n, nb = (double)j.cat[j.ncat - 1].n;
+    return na * nb * frac * (j.q.autocorr ? 0.5 : 1.0) + 200.0 * (na + 1.0);
+}
 
 void batch_free_plan(cf_batch *b)
 {
@@ -2196,9 +2214,8 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
         bump.off = 0;
         b->d_out = bump.take<unsigned long long>(out_words);
         b->d_jobs = bump.take<cf::PairParams>(nj);
-        b->d_path = bump.take<int>(nj);
-        b->d_offsets = bump.take<unsigned>(nj + 1);
-        b->d_counter = bump.take<unsigned>(1);
+        b->d_list = bump.take<int>(nj);
+        b->d_start = bump.take<int>((size_t)BATCH_STARTS * b->sms);
         cf::GridBatch &gb = b->grid;
         gb.seg = bump.take<cf::GridSeg>(nseg);
         gb.geom = bump.take<cf::Geom>(nj);
@@ -2240,7 +2257,9 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
             if (j.ncat == 1)
                 j.G[1] = j.G[0];
             const int nb = (int)j.edges.size() - 1;
-            j.P.work = bump.take<cf::WorkItem>((size_t)j.g.ncols * cf::MAX_STENCIL);
+            const int sx = 2 * j.g.reach_x + 1, sy = 2 * j.g.reach_y + 1;
+            j.P.nbr = bump.take<cf::Nbr>((size_t)j.g.ncols * (j.q.autocorr ? (sx * sy + 1) / 2 : sx * sy));
+            j.P.nbr_count = bump.take<unsigned>(j.g.ncols);
             j.P.thr = bump.take<float>(2 * (nb + 1));
             j.P.lut = bump.take<uint8_t>(cf::LUT_MAX);
             j.P.E2 = bump.take<double>(nb + 1);
@@ -2256,20 +2275,22 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
     b->out_words = out_words;
     // parameters and tables of every job
     std::vector<cf::PairParams> hp(nj);
-    std::vector<int> hpath(nj);
-    b->smem_max = 0;
+    std::vector<int> hpath(nj), hsmem(nj);
+    std::vector<double> hwork(nj);
     for (int k = 0; k < nj; ++k) {
         BatchJob &j = b->jobs[k];
         const int nb = (int)j.edges.size() - 1;
         const bool f64 = j.cfg.mode == CF_MODE_FP64;
-        cf::WorkItem *work = j.P.work;
+        cf::Nbr *nbr = j.P.nbr;
+        unsigned *nbr_count = j.P.nbr_count;
         const float *dthr = j.P.thr;
         const uint8_t *dlut = j.P.lut;
         const double *dE2 = j.P.E2, *dP = j.P.P;
         double M = 0.0, Ls = 0.0;
         base_params(j.q, j.g, j.G[0], j.G[1], j.P, M, Ls);
         j.P.flags = j.cfg.flags & CF_FLAG_NO_PRUNE;
-        j.P.work = work;
+        j.P.nbr = nbr;
+        j.P.nbr_count = nbr_count;
         j.P.thr = dthr;
         j.P.lut = dlut;
         j.P.E2 = dE2;
@@ -2304,19 +2325,12 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
         j.P.err = reinterpret_cast<unsigned *>(o + j.nslots + 4);
         j.P.item_counter = j.P.err + 1;
         j.P.work_count = j.P.err + 2;
-        cf::PairLaunch PL;
-        std::memset(&PL, 0, sizeof(PL));
-        PL.f64 = f64;
-        PL.chunk = j.chunk;
-        PL.pp = j.pp;
-        cf::plan_pairs(j.P, PL);
-        j.smem = PL.smem;
-        j.path = cf::batch_path(j.P, f64, j.chunk, j.pp);
-        b->smem_max = std::max(b->smem_max, PL.smem);
+        j.path = hpath[k] = cf::batch_path(j.P, f64, j.chunk, j.pp);
+        j.smem = hsmem[k] = cf::batch_smem(j.P, j.path);
+        hwork[k] = batch_work(j);
         hp[k] = j.P;
-        hpath[k] = j.path;
         j.n_kernels = 0;  // the batch's launches are shared by all jobs (batch statistics)
-        wpre[k + 1] = wpre[k] + (unsigned)((std::max(j.P.n_items, 0) + 255) / 256);
+        wpre[k + 1] = wpre[k] + (unsigned)((j.g.ncols + 7) / 8);
     }
     for (auto &sg : seg)
         sg.err = b->jobs[sg.job].P.err;
@@ -2324,8 +2338,17 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
     for (int k = 0; k < nj; ++k)
         geom[k] = b->jobs[k].g;
     b->wblocks = wpre[nj];
+    if ((e = cf::plan_batch(hpath, hsmem, hwork, b->sms, hp, b->plan)))
+        return cuda_fail(e, "batch plan");
+    if (b->plan.start.size() > (size_t)BATCH_STARTS * b->sms)
+        return fail(CF_EDEVICE, "batch plan: more CTAs than expected");
+    b->blocks = 0;
+    for (const auto &gr : b->plan.groups)
+        b->blocks = std::max(b->blocks, gr.blocks);
     if ((e = cudaMemcpy(b->d_jobs, hp.data(), sizeof(cf::PairParams) * nj, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(b->d_path, hpath.data(), sizeof(int) * nj, cudaMemcpyHostToDevice)) ||
+        (e = cudaMemcpy(b->d_list, b->plan.list.data(), sizeof(int) * nj, cudaMemcpyHostToDevice)) ||
+        (e = cudaMemcpy(b->d_start, b->plan.start.data(), sizeof(int) * b->plan.start.size(),
+                        cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy((void *)b->grid.seg, seg.data(), sizeof(cf::GridSeg) * nseg, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy((void *)b->grid.geom, geom.data(), sizeof(cf::Geom) * nj, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(b->d_wpre, wpre.data(), sizeof(unsigned) * (nj + 1), cudaMemcpyHostToDevice)))
@@ -2334,8 +2357,8 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
         if ((e = cudaMemcpy((void *)b->grid.pre[k], pre[k].data(), sizeof(unsigned) * (nseg + 1),
                             cudaMemcpyHostToDevice)))
             return cuda_fail(e, "H2D batch gridding plan");
-    // two memsets, the batched gridding, the work lists, offsets + batched pair kernel
-    b->n_kernels = 2 + cf::grid_batch_kernels() + 1 + 2;
+    // a memset, the batched gridding, the neighbour lists, a pair kernel per kind of count
+    b->n_kernels = 1 + cf::grid_batch_kernels() + 1 + b->plan.groups.size();
     b->planned = true;
     (void)st;
     return CF_OK;
@@ -2348,22 +2371,15 @@ int batch_issue(cf_batch *b, cudaStream_t st, bool capturing)
     cudaError_t e;
     const int nj = (int)b->jobs.size();
     if ((!capturing && (e = cudaEventRecord(b->ev[0], st))) ||
-        (e = cudaMemsetAsync(b->d_out, 0, b->out_words * 8, st)) ||
-        (e = cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned), st)))
+        (e = cudaMemsetAsync(b->d_out, 0, b->out_words * 8, st)))
         return cuda_fail(e, "batch start");
-    // every catalogue of every job gridded stage by stage, then every work list
+    // every catalogue of every job gridded stage by stage, then every neighbour list
     if ((e = cf::build_grid_batch(b->grid, b->sms, st)))
         return cuda_fail(e, "batched gridding");
-    if ((e = cf::launch_worklist_batch(b->d_jobs, b->d_wpre, nj, b->wblocks, st)))
-        return cuda_fail(e, "batched work lists");
-    cf::BatchParams B;
-    B.jobs = b->d_jobs;
-    B.path = b->d_path;
-    B.njobs = nj;
-    B.offsets = b->d_offsets;
-    B.item_counter = b->d_counter;
+    if ((e = cf::launch_neighbours_batch(b->d_jobs, b->d_wpre, nj, b->wblocks, st)))
+        return cuda_fail(e, "batched neighbour lists");
     if ((!capturing && (e = cudaEventRecord(b->ev[1], st))) ||
-        (e = cf::launch_batch(B, b->smem_max, b->sms, b->blocks, st)) ||
+        (e = cf::launch_batch(b->plan, b->d_jobs, b->d_list, b->d_start, st)) ||
         (!capturing && (e = cudaEventRecord(b->ev[2], st))) ||
         (e = cudaMemcpyAsync(b->h_out, b->d_out, b->out_words * 8, cudaMemcpyDeviceToHost, st)) ||
         (!capturing && (e = cudaEventRecord(b->ev[3], st))))

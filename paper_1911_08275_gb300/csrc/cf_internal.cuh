@@ -161,6 +161,7 @@ struct PairParams {
     Nbr *nbr;           // chunk tasks: nstencil entries per primary column, kept ones first
     unsigned *nbr_count;   // kept entries per primary column
     int parts;          // chunk tasks: shares a chunk's neighbour list is split into
+    int split_all;      // batches: every chunk is split (else the last eighth)
     int tile_max;       // points per staged tile
     uint32_t flags;
     uint64_t wait_ns;   // limit of every tile-barrier wait (then the error word gets ERR_TIMEOUT)

@@ -8,34 +8,6 @@ namespace cf {
 
 namespace {
 
-// Neighbour lists (Sec. 2.1, 2.2): one warp per primary column, one stencil
-// offset per lane; the kept column pairs are listed in stencil order with
-// their z reach (float32, rounded up, with the window slack).
-__device__ __forceinline__ void neighbours_body(const PairParams &P, int col, int lane)
-{
-    if (col >= P.g.ncols)
-        return;
-    int n = 0;
-    for (int s0 = 0; s0 < P.nstencil; s0 += 32) {
-        const int s = s0 + lane;
-        WorkItem w;
-        const bool keep = s < P.nstencil && plan_item(P, col * P.nstencil + s, w);
-        const unsigned m = __ballot_sync(FULL, keep);
-        if (keep) {
-            Nbr r;
-            r.dz = __fadd_ru(__double2float_ru(w.dzmax), P.zslack);
-            r.code = w.code;
-            P.nbr[(long long)col * P.nstencil + n + __popc(m & ((1u << lane) - 1u))] = r;
-        }
-        n += __popc(m);
-    }
-    if (lane == 0) {
-        P.nbr_count[col] = (unsigned)n;
-        if (n)
-            atomicAdd(P.work_count, (unsigned)n);
-    }
-}
-
 __global__ void __launch_bounds__(128) k_neighbours(const __grid_constant__ PairParams P)
 {
     neighbours_body(P, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), threadIdx.x & 31);

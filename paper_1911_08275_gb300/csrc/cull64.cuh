@@ -130,6 +130,11 @@ struct Cull64 {
         return KIND == 0 ? P.nbins : P.nbins * P.npibins;
     }
 
+    static __device__ __forceinline__ bool load(const PairParams &P, unsigned char *smem, State &st, unsigned)
+    {
+        return init(P, smem, st);
+    }
+
     static __device__ __forceinline__ bool init(const PairParams &P, unsigned char *smem, State &st)
     {
         double *E2 = reinterpret_cast<double *>(smem + P.e2_off), *Pe = E2 + P.nbins + 1;

@@ -15,8 +15,16 @@ cudaError_t occupancy(K kern, int smem, int &occ)
     return occupancy_of((const void *)kern, smem, occ);
 }
 
-// Parts a split chunk task has, at most (TaskSplit); a part takes every
-// TASK_PARTS-th neighbour.
+// Parts a split chunk task has (TaskSplit; a part takes every parts-th
+// neighbour) for a count of about `chunks` chunks on `warps` warps: 8, more where
+// there are fewer than two chunks per warp, so that there are some 16 tasks per
+// warp (a chunk of a dense catalogue against all neighbours is a long task).
 constexpr int TASK_PARTS = 8;
+inline int task_parts(double chunks, double warps, int nstencil)
+{
+    const double want = 16.0 * warps / (chunks > 1.0 ? chunks : 1.0);
+    const int parts = want > TASK_PARTS ? (want < 1024.0 ? (int)want : 1024) : TASK_PARTS;
+    return parts < nstencil ? parts : nstencil;
+}
 
 }  // namespace cf

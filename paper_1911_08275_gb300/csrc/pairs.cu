@@ -148,28 +148,6 @@ __global__ void __launch_bounds__(256) k_worklist(const __grid_constant__ PairPa
     worklist_body(P, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// The work lists of every job of a batch in one launch: job j owns blocks
-// [pre[j], pre[j + 1]) (one thread per candidate, as k_worklist).
-__global__ void __launch_bounds__(256) k_worklist_batch(const PairParams *__restrict__ jobs,
-                                                        const unsigned *__restrict__ pre, int njobs)
-{
-    __shared__ int s_job;
-    if (threadIdx.x == 0) {
-        int lo = 0, hi = njobs - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (pre[mid] <= blockIdx.x)
-                lo = mid;
-            else
-                hi = mid - 1;
-        }
-        s_job = lo;
-    }
-    __syncthreads();
-    const int j = s_job;
-    worklist_body(jobs[j], (int)(blockIdx.x - pre[j]) * blockDim.x + threadIdx.x);
-}
-
 // One kept column pair, as the pair kernels use it (identical in every thread
 // of the CTA: all read the same record).
 struct Item {
@@ -1136,168 +1114,6 @@ __device__ __forceinline__ float sqrt_approx(float v)
     return r;
 }
 
-// ============================================================ binary64 kernel
-template <int I, bool EVALS, bool WACC>
-struct Xi64Path {
-    static __device__ __forceinline__ void init(const PairParams &P, unsigned char *smem)
-    {
-        const int nb = P.nbins;
-        const Smem64 L = smem64_layout(P.tile_max, nb, 0, WARPS * (nb + 1) * 32);
-        double *E2 = reinterpret_cast<double *>(smem + L.e2);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + L.hist);
-        double *acc = WACC ? reinterpret_cast<double *>(smem + P.acc_off) : nullptr;  // [warp][bin][2]
-
-        const int tid = threadIdx.x;
-        for (int q = tid; q <= nb; q += THREADS)
-            E2[q] = P.E2[q];
-        for (int q = tid; q < WARPS * (nb + 1) * 32; q += THREADS)
-            hist[q] = 0u;
-        if (WACC)
-            for (int q = tid; q < WARPS * nb * 2; q += THREADS)
-                acc[q] = 0.0;
-    }
-
-    static __device__ __forceinline__ bool item(const PairParams &P, const Item &it,
-                                                unsigned char *smem, PathState &st)
-    {
-        constexpr int J = 32 / I;
-        const int nb = P.nbins;
-        const Smem64 L = smem64_layout(P.tile_max, nb, 0, WARPS * (nb + 1) * 32);
-        uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
-        double4_32a *tile = reinterpret_cast<double4_32a *>(smem + L.tile);
-        double *E2 = reinterpret_cast<double *>(smem + L.e2);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + L.hist);
-        double *acc = WACC ? reinterpret_cast<double *>(smem + P.acc_off) : nullptr;  // [warp][bin][2]
-
-        const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-        unsigned &phase = st.phase;
-        u64 &n_eval = st.n_eval;
-        unsigned &pending = st.pending;
-
-        uint32_t *hw = hist + warp * (nb + 1) * 32;
-        uint32_t *hl = hw + lane;
-        const int ii = lane % I, jj = lane / I;
-        const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-
-        const double dzw = __dadd_rn(it.dzmax, 1e-9 * (P.rz + P.g.box[2] + 1.0));
-        const int nchunks = (it.a1 - it.a0 + I - 1) / I;
-
-        for (int t0 = it.b0; t0 < it.b1; t0 += P.tile_max) {
-            const int nt = min(P.tile_max, it.b1 - t0);
-            if (!stage_tile(tile, P.B.pos64 + t0, nt, 32, bar, phase, P.err, P.wait_ns)) {
-                return false;
-            }
-            const double zt_lo = tile[0].z, zt_hi = tile[nt - 1].z;
-            auto zkey = [&](int p) { return tile[p].z; };
-            auto next_chunk = [&]() {  // chunks in increasing order, claimed by the warps
-                int v = 0;
-                if (lane == 0)
-                    v = atomicAdd(reinterpret_cast<int *>(smem + CLAIM_OFF), 1);
-                return __shfl_sync(FULL, v, 0);
-            };
-            for (int c = next_chunk(); c < nchunks; c = next_chunk()) {
-                const int ib = it.a0 + c * I;
-                const int nvi = min(I, it.a1 - ib);
-                const int i = ib + ii;
-                const bool vi = ii < nvi;
-                double4_32a pi = make_double4_32a(qnan, qnan, qnan, qnan);
-                if (vi)
-                    pi = P.A.pos64[i];  // column padding entries are NaN
-                const double zlo = __shfl_sync(FULL, pi.z, 0);
-                double zhi = pi.z;
-    #pragma unroll
-                for (int o = 1; o < I; o <<= 1) {  // largest real z of the chunk
-                    const double t = __shfl_xor_sync(FULL, zhi, o);
-                    zhi = (isnan(zhi) || t > zhi) ? t : zhi;
-                }
-                if (isnan(zlo))
-                    continue;
-                for (int k = it.kmin; k <= it.kmax; ++k) {
-                    const double kz = k * P.g.box[2];
-                    const double wlo = zlo - kz - dzw, whi = zhi - kz + dzw;
-                    if (whi < zt_lo || wlo > zt_hi)
-                        continue;
-                    int jlo = warp_bound(zkey, nt, wlo, false, lane);
-                    const int jhi = warp_bound(zkey, nt, whi, true, lane);
-                    const bool tri = it.self && k == 0;
-                    if (tri)
-                        jlo = max(jlo, ib + 1 - t0);
-                    if (jlo >= jhi)
-                        continue;
-                    pending += (unsigned)((jhi - jlo + J - 1) / J);
-                    const bool noshift = it.Sx == 0.0 && it.Sy == 0.0 && kz == 0.0;
-                    for (int jb = jlo; jb < jhi; jb += J) {
-                        const int j = jb + jj;
-                        const double4_32a pj = tile[j];
-                        const bool live = !tri || (t0 + j > i);
-                        if (EVALS)
-                            n_eval += (vi && j < jhi && live) ? 1ull : 0ull;
-                        double r2;
-                        if (noshift)
-                            r2 = plain_r2(pi, pj);
-                        else
-                            r2 = canon_r2(pi, pj, it.Sx, it.Sy, kz);
-                        if (!live)
-                            r2 = qnan;
-                        const int kb = bin_f64(r2, E2, nb);
-                        if (kb >= 0) {
-                            hl[kb * 32] += 1u;
-                            if (WACC) {  // Code 1's weight; the oracle's product and sqrt
-                                double *aw = acc + (warp * nb + kb) * 2;
-                                const double pw = P.weighted ? __dmul_rn(pi.w, pj.w) : 1.0;
-                                atomicAdd(aw, pw);
-                                if (P.want_r)
-                                    atomicAdd(aw + 1, __dmul_rn(__dsqrt_rn(r2), pw));
-                            }
-                        }
-                    }
-                }
-                if (pending > (1u << 30)) {
-                    warp_flush(hw, nb, P.hist, lane);
-                    pending = 0;
-                }
-            }
-        }
-        return true;
-    }
-
-    static __device__ __forceinline__ void fini(const PairParams &P, unsigned char *smem, PathState &st)
-    {
-        const int nb = P.nbins;
-        const Smem64 L = smem64_layout(P.tile_max, nb, 0, WARPS * (nb + 1) * 32);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + L.hist);
-        double *acc = WACC ? reinterpret_cast<double *>(smem + P.acc_off) : nullptr;  // [warp][bin][2]
-
-        const int tid = threadIdx.x, lane = tid & 31;
-        u64 &n_eval = st.n_eval;
-
-        __syncthreads();
-        for (int bn = tid; bn < nb; bn += THREADS) {
-            u64 sum = 0;
-            double ws = 0.0, rs = 0.0;
-            for (int w = 0; w < WARPS; ++w) {
-                for (int l = 0; l < 32; ++l)
-                    sum += hist[(w * (nb + 1) + bn) * 32 + l];
-                if (WACC) {
-                    ws += acc[(w * nb + bn) * 2];
-                    rs += acc[(w * nb + bn) * 2 + 1];
-                }
-            }
-            if (sum) {
-                atomicAdd(&P.hist[bn], sum);
-                if (WACC) {
-                    atomicAdd(&P.wsum[bn], ws);
-                    if (P.want_r)
-                        atomicAdd(&P.rsum[bn], rs);
-                }
-            }
-        }
-        n_eval = warp_sum_u64(n_eval);
-        if (lane == 0 && n_eval)
-            atomicAdd(&P.diag[1], n_eval);
-    }
-};
-
 // ============================================================ DD(rp, pi) kernels
 // rp^2 = dx^2 + dy^2 is binned like r^2 (bits-indexed table of float32
 // thresholds with 2-component error bands).  pi = |dz| is binned by
@@ -1816,474 +1632,6 @@ struct Rppi32Path {
     }
 };
 
-// A pair recorded by sweep_rppi32_pp: recompute rp^2 and t' from the staged
-// tile with the same IEEE operations as the packed main path, then settle it
-// as resolve_rppi does (the main path added it at addr_main).
-template <bool LIN>
-__device__ __forceinline__ int resolve_local_rppi(const unsigned char *smem, const SweepRP &S,
-                                                  float xh, float yh, float zh, float s,
-                                                  int i, int jl)
-{
-    const float *tx = reinterpret_cast<const float *>(smem + TX_OFF);
-    const float dx = __fsub_rn(tx[jl], xh);
-    const float dy = __fsub_rn(tx[jl + TSTRIDE / 4], yh);
-    const float dz = __fsub_rn(tx[jl + TSTRIDE / 2], zh);
-    const float rp2 = __fmaf_rn(dy, dy, __fmul_rn(dx, dx));
-    const float t = __fmaf_rn(fabsf(dz), s, -0.5f);
-    const float q = __fadd_rn(t, PI_MAGIC);
-    const float f = __fsub_rn(t, __fsub_rn(q, PI_MAGIC));
-    // the entry as the main path loaded it (sign-extended: flagged = -1)
-    const uint32_t e = (uint32_t)(int)(signed char)lut_entry<LIN>(smem, S.u0, S.shift, S.lut_last,
-                                                                  S.lscale, rp2);
-    const uint32_t m = min(__float_as_uint(q) - PI_MAGIC_BITS, (uint32_t)S.npi);
-    const uint32_t addr = S.hbase + e * S.rowb + m * 4u;  // as the main path added it
-    return resolve_rppi<false>(smem, S, e, rp2, m, fabsf(f) > S.pband, addr, i, S.t0 + jl, 1.0f);
-}
-
-// Sweep one window with PP primaries per lane (lane layout as in sweep32): per
-// pair rp^2 and t' = |dz| s - 1/2 in packed float32, the rp table byte, the pi
-// index from the rounding, one shared atomic into the warp's 2-D histogram copy.
-// A pair whose rp cell is flagged, or whose t' lies within the error bound of
-// a pi edge (|t' - round(t')| >= pband), sets a bit of the lane's mask; once
-// per block of 8 steps a warp-uniform test settles the recorded pairs.
-template <int I, int PP, bool TRI, bool EVALS, bool LIN>
-__device__ __forceinline__ void sweep_rppi32_pp(unsigned char *smem, const SweepRP &S, int jlo,
-                                                int jhi, int jj, const u64 *XH, const u64 *YH,
-                                                const u64 *ZH, u64 SC, float sc, const int *iv,
-                                                const bool *vv, u64 &n_eval, u64 &n_rck)
-{
-    const float qnan = __int_as_float(0x7fc00000);
-    const u64 MH = pack2(-0.5f, -0.5f), MG = pack2(PI_MAGIC, PI_MAGIC);
-    const u64 PB = pack2(S.pband, S.pband);
-    const u64 LS = pack2(S.lscale, S.lscale), LM = pack2(LIN_MAGIC, LIN_MAGIC);
-    const uint32_t npiu = (uint32_t)S.npi;
-    // shared addresses of the rp table, the base folded into the clamp (as in sweep32)
-    const uint32_t lutb = smem_u32(smem + LUT_OFF), lut_lo = lutb - LIN_MAGIC_BITS,
-                   lut_hi = lutb + S.lut_last;
-    const int jstart = jlo & ~1;
-    constexpr int JS = 64 / I;
-    const int nit = (jhi - jstart + 2 * JS - 1) / (2 * JS);
-    for (int b0 = 0; b0 < nit; b0 += 8) {
-        const int jAb = jstart + 2 * jj + b0 * 2 * JS;
-        const uint32_t pb = smem_u32(smem + TX_OFF) + jAb * 4;
-        const int tend = min(8, nit - b0);
-        uint32_t fm[PP];
-#pragma unroll
-        for (int q = 0; q < PP; ++q)
-            fm[q] = 0u;
-        for (int t = 0; t < tend; ++t) {
-            const uint32_t p = pb + t * 8 * JS;
-            const u64 xA = lds64<0>(p);
-            const u64 yA = lds64<TSTRIDE>(p);
-            const u64 zA = lds64<2 * TSTRIDE>(p);
-            const u64 xB = lds64<4 * JS>(p);
-            const u64 yB = lds64<4 * JS + TSTRIDE>(p);
-            const u64 zB = lds64<4 * JS + 2 * TSTRIDE>(p);
-            const int jA = jAb + t * 2 * JS;
-            const int gA = S.t0 + jA, gB = gA + JS;  // global indices of (a0, b0); a1, b1 are +1
-            const int gv[4] = {gA, gA + 1, gB, gB + 1};
-#pragma unroll
-            for (int q = 0; q < PP; ++q) {
-                u64 dx = fsub2(xA, XH[q]), dy = fsub2(yA, YH[q]);
-                const u64 rA = ffma2(dy, dy, fmul2(dx, dx));
-                const u64 tA = ffma2(fabs2(fsub2(zA, ZH[q])), SC, MH);
-                dx = fsub2(xB, XH[q]);
-                dy = fsub2(yB, YH[q]);
-                const u64 rB = ffma2(dy, dy, fmul2(dx, dx));
-                const u64 tB = ffma2(fabs2(fsub2(zB, ZH[q])), SC, MH);
-                const u64 qA = fadd2(tA, MG), qB = fadd2(tB, MG);
-                // pband - |t' - round(t')|: sign bit set = near a pi edge (a NaN
-                // sentinel gives a positive NaN: never flagged)
-                const u64 gA2 = fsub2(PB, fabs2(fsub2(tA, fsub2(qA, MG))));
-                const u64 gB2 = fsub2(PB, fabs2(fsub2(tB, fsub2(qB, MG))));
-                float r[4], qv[4], g[4];
-                unpack2(rA, r[0], r[1]);
-                unpack2(rB, r[2], r[3]);
-                unpack2(qA, qv[0], qv[1]);
-                unpack2(qB, qv[2], qv[3]);
-                unpack2(gA2, g[0], g[1]);
-                unpack2(gB2, g[2], g[3]);
-                uint32_t cq[4];
-                if (LIN) {
-                    float c[4];
-                    unpack2(ffma2(rA, LS, LM), c[0], c[1]);
-                    unpack2(ffma2(rB, LS, LM), c[2], c[3]);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)  // the table byte's shared address
-                        cq[k] = min(__float_as_uint(c[k]) + lut_lo, lut_hi);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        cq[k] = lutb + min((__float_as_uint(r[k]) >> S.shift) - S.u0, S.lut_last);
-                }
-                if (TRI) {  // pairs with j <= i: the out-of-range entry, never flagged
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        cq[k] = gv[k] > iv[q] ? cq[k] : lut_hi;
-                        g[k] = gv[k] > iv[q] ? g[k] : 1.0f;
-                    }
-                }
-                if (EVALS) {
-                    const int jv[4] = {jA, jA + 1, jA + JS, jA + JS + 1};
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        n_eval += (vv[q] && jv[k] >= jlo && jv[k] < jhi && (!TRI || gv[k] > iv[q]))
-                                      ? 1ull : 0ull;
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t e = lds_entry(cq[k]);  // flagged: -1, the row before bin 0
-                    const uint32_t m = min(__float_as_uint(qv[k]) - PI_MAGIC_BITS, npiu);
-                    red_shared(S.hbase + e * S.rowb + m * 4u, 1u);
-                    // pair (t, k) ends at bit 4 tend - 1 - (4 t + k): flagged rp cell or
-                    // near a pi edge (sign of g)
-                    fm[q] = push_sign(fm[q], e | __float_as_uint(g[k]));
-                }
-            }
-        }
-        uint32_t anyf = 0u;
-#pragma unroll
-        for (int q = 0; q < PP; ++q)
-            anyf |= fm[q];
-        if (__any_sync(FULL, anyf != 0u)) {
-#pragma unroll
-            for (int q = 0; q < PP; ++q) {
-                float xh, yh, zh, tmp;
-                unpack2(XH[q], xh, tmp);
-                unpack2(YH[q], yh, tmp);
-                unpack2(ZH[q], zh, tmp);
-                uint32_t m = fm[q];
-                while (m) {
-                    const int bit = __ffs(m) - 1;
-                    m &= m - 1u;
-                    const int tk = 4 * tend - 1 - bit, t = tk >> 2, k = tk & 3;
-                    const int jl = jAb + t * 2 * JS + ((k & 2) ? JS : 0) + (k & 1);
-                    n_rck += resolve_local_rppi<LIN>(smem, S, xh, yh, zh, sc, iv[q], jl);
-                }
-            }
-        }
-    }
-}
-
-// Float32 DD(rp, pi) without sums: I x PP primaries per chunk (lane ii holds
-// primaries ii, ii + I, ...), deferred flag resolution.  Tables, histograms and
-// the merge are those of Rppi32Path.
-template <int I, int PP, bool EVALS>
-struct Rppi32PathPP {
-    using Base = Rppi32Path<I, EVALS, false, false>;
-    static __device__ __forceinline__ void init(const PairParams &P, unsigned char *smem)
-    {
-        Base::init(P, smem);
-    }
-    static __device__ __forceinline__ void fini(const PairParams &P, unsigned char *smem, PathState &st)
-    {
-        Base::fini(P, smem, st);
-    }
-
-    static __device__ __forceinline__ bool item(const PairParams &P, const Item &it,
-                                                unsigned char *smem, PathState &st)
-    {
-        constexpr int CH = I * PP;
-        const int nb = P.nbins, npi = P.npibins;
-        uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
-        const float *tz = reinterpret_cast<const float *>(smem + TX_OFF + 2 * TSTRIDE);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + P.hist_off);
-        const int copy = rppi32_rows(nb) * (npi + 1);
-
-        const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-        unsigned &pending = st.pending;
-
-        uint32_t *hc = hist + (warp % P.hcopies) * copy + (npi + 1);  // row 0 of the warp's copy
-        const int ii = lane % I, jj = lane / I;
-        SweepRP S;
-        S.nb = nb;
-        S.npi = npi;
-        S.u0 = P.u0;
-        S.lut_last = (uint32_t)(P.lut_n - 1);
-        S.shift = P.lut_shift;
-        S.nthr = P.nthr;
-        S.lin = P.lut_lin;
-        S.lscale = P.lut_scale;
-        S.hbase = smem_u32(hc);
-        S.rowb = (uint32_t)(npi + 1) * 4u;
-        S.pband = P.pband;
-        S.pa = P.A.pos64;
-        S.pb = P.B.pos64;
-        S.acc = nullptr;
-        S.weighted = false;
-        S.want_r = false;
-        S.xlj = S.ylj = nullptr;
-        const u64 SC = pack2(P.pscale, P.pscale);
-        const unsigned flush_at = (1u << 30) / (unsigned)(WARPS / P.hcopies);
-        const float qnan = __int_as_float(0x7fc00000);
-
-        const float dzw = __fadd_ru(__double2float_ru(it.dzmax), P.zslack);
-        const float Sxf = __double2float_rn(it.Sx), Syf = __double2float_rn(it.Sy);
-        S.Sx = it.Sx;
-        S.Sy = it.Sy;
-        const int nchunks = (it.a1 - it.a0 + CH - 1) / CH;
-
-        for (int t0 = it.b0; t0 < it.b1; t0 += TILE32) {
-            const int nt = min(TILE32, it.b1 - t0);
-            if (!stage_tiles32(smem, P.B, t0, nt, bar, st.phase, P.err, P.wait_ns))
-                return false;
-            S.t0 = t0;
-            const float zt_lo = tz[0];
-            float zt_hi = tz[nt - 1];
-            if (isnan(zt_hi))
-                zt_hi = INFINITY;
-            auto zkey = [&](int q) { return tz[q]; };
-            int lo_prev[3] = {0, 0, 0}, hi_prev[3] = {0, 0, 0};
-            auto next_chunk = [&]() {  // chunks in increasing order, claimed by the warps
-                int v = 0;
-                if (lane == 0)
-                    v = atomicAdd(reinterpret_cast<int *>(smem + CLAIM_OFF), 1);
-                return __shfl_sync(FULL, v, 0);
-            };
-            for (int c = next_chunk(); c < nchunks; c = next_chunk()) {
-                const int ib = it.a0 + c * CH;
-                u64 XH[PP], YH[PP], ZH[PP];
-                int iv[PP];
-                bool vv[PP];
-                float zq[PP];
-                float zmax = qnan;
-#pragma unroll
-                for (int q = 0; q < PP; ++q) {
-                    const int i = ib + q * I + ii;
-                    float xi = qnan, yi = qnan, zi = qnan;
-                    if (i < it.a1) {
-                        xi = P.A.xs[i];
-                        yi = P.A.ys[i];
-                        zi = P.A.zs[i];
-                    }
-                    iv[q] = i;
-                    vv[q] = !isnan(xi);  // chunk tail and column padding are NaN
-                    const float xh = __fsub_rn(xi, Sxf), yh = __fsub_rn(yi, Syf);
-                    XH[q] = pack2(xh, xh);
-                    YH[q] = pack2(yh, yh);
-                    zq[q] = zi;
-                    zmax = (isnan(zmax) || zi > zmax) ? zi : zmax;
-                }
-                const float zlo = __shfl_sync(FULL, zq[0], 0);
-                float zhi = zmax;
-#pragma unroll
-                for (int o = 1; o < I; o <<= 1) {  // largest real z of the chunk
-                    const float t = __shfl_xor_sync(FULL, zhi, o);
-                    zhi = (isnan(zhi) || t > zhi) ? t : zhi;
-                }
-                if (isnan(zlo))
-                    continue;
-#pragma unroll
-                for (int kk = 0; kk < 3; ++kk) {
-                    const int k = kk - 1;
-                    if (k < it.kmin || k > it.kmax)
-                        continue;
-                    const float kz = (float)k * P.boxf[2];
-                    const float wlo = zlo - kz - dzw, whi = zhi - kz + dzw;
-                    if (whi < zt_lo || wlo > zt_hi)
-                        continue;
-                    int jlo = warp_bound_from(zkey, lo_prev[kk], nt, wlo, false, lane);
-                    const int jhi = warp_bound_from(zkey, max(hi_prev[kk], jlo), nt, whi, true, lane);
-                    lo_prev[kk] = jlo;
-                    hi_prev[kk] = jhi;
-                    const bool tri = it.self && k == 0;
-                    if (tri)
-                        jlo = max(jlo, ib + 1 - t0);
-                    if (jlo >= jhi)
-                        continue;
-                    pending += (unsigned)((jhi - jlo) / (64 / I) + 4) * 2u * PP;
-#pragma unroll
-                    for (int q = 0; q < PP; ++q) {
-                        const float zh = __fsub_rn(zq[q], kz);
-                        ZH[q] = pack2(zh, zh);
-                    }
-                    S.Sz = k == 0 ? 0.0 : (k > 0 ? P.g.box[2] : -P.g.box[2]);
-                    if (tri) {
-                        if (S.lin)
-                            sweep_rppi32_pp<I, PP, true, EVALS, true>(smem, S, jlo, jhi, jj, XH, YH, ZH, SC,
-                                                                      P.pscale, iv, vv, st.n_eval, st.n_rck);
-                        else
-                            sweep_rppi32_pp<I, PP, true, EVALS, false>(smem, S, jlo, jhi, jj, XH, YH, ZH, SC,
-                                                                       P.pscale, iv, vv, st.n_eval, st.n_rck);
-                    } else {
-                        if (S.lin)
-                            sweep_rppi32_pp<I, PP, false, EVALS, true>(smem, S, jlo, jhi, jj, XH, YH, ZH, SC,
-                                                                       P.pscale, iv, vv, st.n_eval, st.n_rck);
-                        else
-                            sweep_rppi32_pp<I, PP, false, EVALS, false>(smem, S, jlo, jhi, jj, XH, YH, ZH, SC,
-                                                                        P.pscale, iv, vv, st.n_eval, st.n_rck);
-                    }
-                }
-                if (pending > flush_at) {  // keep every shared u32 count far from overflow
-                    __syncwarp();
-                    flush_rppi(hc, nb, npi, P.hist, lane);
-                    pending = 0;
-                }
-            }
-        }
-        return true;
-    }
-};
-
-// Binary64 DD(rp, pi): canonical rp^2 and |dz|, exact edge compares.
-template <int I, bool EVALS, bool WACC>
-struct Rppi64Path {
-    static __device__ __forceinline__ void init(const PairParams &P, unsigned char *smem)
-    {
-        const int nb = P.nbins, npi = P.npibins, row = npi + 1, copy = (nb + 1) * row;
-        const Smem64 L = smem64_layout(P.tile_max, nb, npi, 0);
-        double *E2 = reinterpret_cast<double *>(smem + L.e2);
-        double *Pe = reinterpret_cast<double *>(smem + L.p);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + P.hist_off);
-        double *acc = WACC ? reinterpret_cast<double *>(smem + P.acc_off) : nullptr;
-
-        const int tid = threadIdx.x;
-        for (int q = tid; q <= nb; q += THREADS)
-            E2[q] = P.E2[q];
-        for (int q = tid; q <= npi; q += THREADS)
-            Pe[q] = P.P[q];
-        for (int q = tid; q < P.hcopies * copy; q += THREADS)
-            hist[q] = 0u;
-        if (WACC)
-            for (int q = tid; q < 2 * P.hcopies * copy; q += THREADS)
-                acc[q] = 0.0;
-    }
-
-    static __device__ __forceinline__ bool item(const PairParams &P, const Item &it,
-                                                unsigned char *smem, PathState &st)
-    {
-        constexpr int J = 32 / I;
-        const int nb = P.nbins, npi = P.npibins, row = npi + 1, copy = (nb + 1) * row;
-        const Smem64 L = smem64_layout(P.tile_max, nb, npi, 0);
-        uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
-        double4_32a *tile = reinterpret_cast<double4_32a *>(smem + L.tile);
-        double *E2 = reinterpret_cast<double *>(smem + L.e2);
-        double *Pe = reinterpret_cast<double *>(smem + L.p);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + P.hist_off);
-        double *acc = WACC ? reinterpret_cast<double *>(smem + P.acc_off) : nullptr;
-
-        const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-        unsigned &phase = st.phase;
-        u64 &n_eval = st.n_eval;
-        unsigned &pending = st.pending;
-
-        uint32_t *hc = hist + (warp % P.hcopies) * copy;
-        double *ac = WACC ? acc + 2 * (warp % P.hcopies) * copy : nullptr;
-        const unsigned flush_at = (1u << 30) / (unsigned)(WARPS / P.hcopies);
-        const int ii = lane % I, jj = lane / I;
-        const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-
-        const double dzw = __dadd_rn(it.dzmax, 1e-9 * (P.rz + P.g.box[2] + 1.0));
-        const int nchunks = (it.a1 - it.a0 + I - 1) / I;
-
-        for (int t0 = it.b0; t0 < it.b1; t0 += P.tile_max) {
-            const int nt = min(P.tile_max, it.b1 - t0);
-            if (!stage_tile(tile, P.B.pos64 + t0, nt, 32, bar, phase, P.err, P.wait_ns)) {
-                return false;
-            }
-            double zt_hi = tile[nt - 1].z;
-            if (isnan(zt_hi))
-                zt_hi = INFINITY;
-            const double zt_lo = tile[0].z;
-            auto zkey = [&](int p) { return tile[p].z; };
-            auto next_chunk = [&]() {  // chunks in increasing order, claimed by the warps
-                int v = 0;
-                if (lane == 0)
-                    v = atomicAdd(reinterpret_cast<int *>(smem + CLAIM_OFF), 1);
-                return __shfl_sync(FULL, v, 0);
-            };
-            for (int c = next_chunk(); c < nchunks; c = next_chunk()) {
-                const int ib = it.a0 + c * I;
-                const int nvi = min(I, it.a1 - ib);
-                const int i = ib + ii;
-                const bool vi = ii < nvi;
-                double4_32a pi = make_double4_32a(qnan, qnan, qnan, qnan);
-                if (vi)
-                    pi = P.A.pos64[i];
-                const double zlo = __shfl_sync(FULL, pi.z, 0);
-                double zhi = pi.z;
-    #pragma unroll
-                for (int o = 1; o < I; o <<= 1) {
-                    const double t = __shfl_xor_sync(FULL, zhi, o);
-                    zhi = (isnan(zhi) || t > zhi) ? t : zhi;
-                }
-                if (isnan(zlo))
-                    continue;
-                for (int k = it.kmin; k <= it.kmax; ++k) {
-                    const double kz = k * P.g.box[2];
-                    const double wlo = zlo - kz - dzw, whi = zhi - kz + dzw;
-                    if (whi < zt_lo || wlo > zt_hi)
-                        continue;
-                    int jlo = warp_bound(zkey, nt, wlo, false, lane);
-                    const int jhi = warp_bound(zkey, nt, whi, true, lane);
-                    const bool tri = it.self && k == 0;
-                    if (tri)
-                        jlo = max(jlo, ib + 1 - t0);
-                    if (jlo >= jhi)
-                        continue;
-                    pending += (unsigned)((jhi - jlo + J - 1) / J) * 32u;
-                    const bool noshift = it.Sx == 0.0 && it.Sy == 0.0 && kz == 0.0;  // as in Xi64Path
-                    for (int jb = jlo; jb < jhi; jb += J) {
-                        const int j = jb + jj;
-                        const double4_32a pj = tile[j];
-                        const bool live = !tri || (t0 + j > i);
-                        if (EVALS)
-                            n_eval += (vi && j < jhi && live) ? 1ull : 0ull;
-                        double dx, dy, dz;
-                        if (noshift) {
-                            dx = __dsub_rn(pj.x, pi.x);
-                            dy = __dsub_rn(pj.y, pi.y);
-                            dz = __dsub_rn(pj.z, pi.z);
-                        } else {
-                            dx = canon_comp(pi.x, pj.x, it.Sx);
-                            dy = canon_comp(pi.y, pj.y, it.Sy);
-                            dz = canon_comp(pi.z, pj.z, kz);
-                        }
-                        double rp2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
-                        if (!live)
-                            rp2 = qnan;
-                        const int kb = bin_f64(rp2, E2, nb);
-                        if (kb >= 0) {
-                            const int m = bin_f64(fabs(dz), Pe, npi);
-                            if (m >= 0) {
-                                atomicAdd(&hc[kb * row + m], 1u);
-                                if (WACC) {  // Code 1's weight; the oracle's product and sqrt
-                                    const double pw = P.weighted ? __dmul_rn(pi.w, pj.w) : 1.0;
-                                    atomicAdd(ac + 2 * (kb * row + m), pw);
-                                    if (P.want_r)
-                                        atomicAdd(ac + 2 * (kb * row + m) + 1,
-                                                  __dmul_rn(__dsqrt_rn(rp2), pw));
-                                }
-                            }
-                        }
-                    }
-                }
-                if (pending > flush_at) {
-                    __syncwarp();
-                    flush_rppi(hc, nb, npi, P.hist, lane);
-                    pending = 0;
-                }
-            }
-        }
-        return true;
-    }
-
-    static __device__ __forceinline__ void fini(const PairParams &P, unsigned char *smem, PathState &st)
-    {
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + P.hist_off);
-        double *acc = WACC ? reinterpret_cast<double *>(smem + P.acc_off) : nullptr;
-
-        const int tid = threadIdx.x, lane = tid & 31;
-        u64 &n_eval = st.n_eval;
-
-        __syncthreads();
-        merge_rppi(P, hist, acc, P.nbins + 1);
-        n_eval = warp_sum_u64(n_eval);
-        if (lane == 0 && n_eval)
-            atomicAdd(&P.diag[1], n_eval);
-    }
-};
-
 // One persistent kernel per path: init the CTA's tables and histograms, pull
 // kept column pairs from the global counter, merge at the end.
 template <class Path, int MINB>
@@ -2315,162 +1663,6 @@ __global__ void __launch_bounds__(THREADS, MINB) k_path(const __grid_constant__ 
     }
     __syncthreads();
     Path::fini(P, smem, st);
-}
-
-// ============================================================ batched kernel
-// Many independent jobs (catalogues, bins, modes) in one persistent launch: the
-// CTAs pull items from one global counter over the concatenation of the jobs'
-// kept column pairs; a CTA that moves on to another job merges its histograms
-// into the previous job's output and loads the next job's tables.
-using XiF32 = Xi32Path<16, 2, false, false>;
-using XiF32_8x2 = Xi32Path<8, 2, false, false>;
-using XiF32_16x1 = Xi32Path<16, 1, false, false>;
-using XiF32_32x1 = Xi32Path<32, 1, false, false>;
-using XiF64 = Xi64Path<8, false, false>;
-using RpF32 = Rppi32PathPP<16, 2, false>;
-using RpF64 = Rppi64Path<8, false, false>;
-
-__device__ __forceinline__ void batch_init(int path, const PairParams &P, unsigned char *smem)
-{
-    switch (path) {
-    case BATCH_XI32:
-    case BATCH_XI32_8x2:
-    case BATCH_XI32_16x1:
-    case BATCH_XI32_32x1: XiF32::init(P, smem); break;  // shape-independent
-    case BATCH_XI64: XiF64::init(P, smem); break;
-    case BATCH_RPPI32: RpF32::init(P, smem); break;
-    default: RpF64::init(P, smem); break;
-    }
-}
-
-__device__ __forceinline__ bool batch_item(int path, const PairParams &P, const Item &it,
-                                           unsigned char *smem, PathState &st)
-{
-    switch (path) {
-    case BATCH_XI32: return XiF32::item(P, it, smem, st);
-    case BATCH_XI32_8x2: return XiF32_8x2::item(P, it, smem, st);
-    case BATCH_XI32_16x1: return XiF32_16x1::item(P, it, smem, st);
-    case BATCH_XI32_32x1: return XiF32_32x1::item(P, it, smem, st);
-    case BATCH_XI64: return XiF64::item(P, it, smem, st);
-    case BATCH_RPPI32: return RpF32::item(P, it, smem, st);
-    default: return RpF64::item(P, it, smem, st);
-    }
-}
-
-__device__ __forceinline__ void batch_fini(int path, const PairParams &P, unsigned char *smem,
-                                           PathState &st)
-{
-    switch (path) {
-    case BATCH_XI32:
-    case BATCH_XI32_8x2:
-    case BATCH_XI32_16x1:
-    case BATCH_XI32_32x1: XiF32::fini(P, smem, st); break;  // shape-independent
-    case BATCH_XI64: XiF64::fini(P, smem, st); break;
-    case BATCH_RPPI32: RpF32::fini(P, smem, st); break;
-    default: RpF64::fini(P, smem, st); break;
-    }
-}
-
-// offsets[j] = kept column pairs of jobs 0..j-1 (one thread; a few thousand jobs at most).
-// Exclusive scan of the jobs' kept-item counts (one warp: each lane loads its
-// jobs' counts in parallel, 32 jobs per round).
-__global__ void k_batch_offsets(const __grid_constant__ BatchParams B)
-{
-    if (blockIdx.x != 0)
-        return;
-    const int lane = threadIdx.x & 31;
-    unsigned carry = 0;
-    for (int j0 = 0; j0 < B.njobs; j0 += 32) {
-        const int j = j0 + lane;
-        const unsigned v = j < B.njobs ? *B.jobs[j].work_count : 0u;
-        unsigned incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned t = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o)
-                incl += t;
-        }
-        if (j < B.njobs)
-            B.offsets[j] = carry + incl - v;
-        carry += __shfl_sync(FULL, incl, 31);
-    }
-    if (lane == 0)
-        B.offsets[B.njobs] = carry;
-}
-
-// Candidate pairs of a work item below which the batch kernel claims items in
-// groups (see k_batch).
-constexpr long long GROUP_PAIRS = 1ll << 16;
-
-__global__ void __launch_bounds__(THREADS, 2) k_batch(const __grid_constant__ BatchParams B)
-{
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ unsigned s_off[BATCH_MAX + 1];
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
-    volatile int *s_item = reinterpret_cast<volatile int *>(smem + 8);
-    for (int j = threadIdx.x; j <= B.njobs; j += THREADS)
-        s_off[j] = B.offsets[j];
-    if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    const unsigned total = s_off[B.njobs];
-    // Small items (column pairs of fewer than GROUP_PAIRS candidate pairs) are
-    // claimed in groups of consecutive items (up to 16, together about
-    // GROUP_PAIRS), so that a CTA stays on a small job for a while instead of
-    // every CTA switching to it for one item (each switch loads the job's table
-    // and merges its histogram); larger items are claimed one by one, which keeps
-    // the load balanced.  The size of the next group comes from the last item
-    // decoded (the next one is most often of the same job), so a claim stays one
-    // atomic.
-    PathState st = {0ull, 0ull, 0ull, 0u, 0u, 0u};
-    int cur = -1;
-    unsigned group = 1;
-    bool ok = true;
-    while (ok) {
-        if (threadIdx.x == 0)
-            *s_item = (int)atomicAdd(B.item_counter, group);
-        __syncthreads();
-        const unsigned base = (unsigned)*s_item;
-        __syncthreads();
-        if (base >= total)
-            break;
-        const unsigned stop = min(base + group, total);
-#pragma unroll 1
-        for (unsigned item = base; item < stop; ++item) {
-            int lo = 0, hi = B.njobs;  // largest job with s_off[job] <= item
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (s_off[mid] <= item)
-                    lo = mid;
-                else
-                    hi = mid;
-            }
-            const int job = lo;
-            if (job != cur) {  // CTA-uniform: every thread holds the same item
-                if (cur >= 0)
-                    batch_fini(B.path[cur], B.jobs[cur], smem, st);
-                __syncthreads();
-                batch_init(B.path[job], B.jobs[job], smem);
-                st.n_eval = st.n_rck = st.n_viol = 0ull;
-                st.pending = 0u;
-                __syncthreads();
-                cur = job;
-            }
-            const PairParams &P = B.jobs[job];
-            Item it;
-            decode_item(P, (int)(item - s_off[job]), it);
-            const long long pairs = (long long)max(it.a1 - it.a0, 1) * max(it.b1 - it.b0, 1);
-            group = pairs < GROUP_PAIRS ? (unsigned)min(16ll, GROUP_PAIRS / pairs) : 1u;
-            if (!batch_item(B.path[job], P, it, smem, st)) {
-                ok = false;
-                break;
-            }
-        }
-    }
-    if (cur >= 0)
-        batch_fini(B.path[cur], B.jobs[cur], smem, st);
 }
 
 template <class K>
@@ -2543,57 +1735,6 @@ cudaError_t occupancy_of(const void *kern, int smem, int &occ)
     if (g_nocc < 128)
         g_occ[g_nocc++] = OccCache{kern, dev, smem, occ};
     return cudaSuccess;
-}
-
-int batch_path(const PairParams &P, int f64, int chunk, int pp)
-{
-    if (P.kind == 0) {
-        if (f64)
-            return BATCH_XI64;
-        if (pp == 2 && chunk == 8)
-            return BATCH_XI32_8x2;
-        if (pp == 1 && chunk == 16)
-            return BATCH_XI32_16x1;
-        if (pp == 1 && chunk == 32)
-            return BATCH_XI32_32x1;
-        return BATCH_XI32;
-    }
-    return f64 ? BATCH_RPPI64 : BATCH_RPPI32;
-}
-
-cudaError_t launch_worklist(const PairParams &P, cudaStream_t st)
-{
-    if (P.n_items <= 0)
-        return cudaSuccess;
-    k_worklist<<<(P.n_items + 255) / 256, 256, 0, st>>>(P);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_worklist_batch(const PairParams *jobs, const unsigned *pre, int njobs,
-                                  unsigned blocks, cudaStream_t st)
-{
-    if (blocks == 0 || njobs < 1)
-        return cudaSuccess;
-    k_worklist_batch<<<blocks, 256, 0, st>>>(jobs, pre, njobs);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_batch(const BatchParams &B, int smem, int sms, int &blocks, cudaStream_t st)
-{
-    if (B.njobs < 1 || B.njobs > BATCH_MAX)
-        return cudaErrorInvalidValue;
-    k_batch_offsets<<<1, 32, 0, st>>>(B);
-    cudaError_t e = cudaGetLastError();
-    if (e)
-        return e;
-    int occ = 0;
-    if ((e = occupancy(k_batch, smem, occ)))
-        return e;
-    if (occ < 1)
-        return cudaErrorInvalidConfiguration;
-    blocks = sms * occ;
-    k_batch<<<blocks, THREADS, smem, st>>>(B);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_pairs(const PairParams &P0, PairLaunch &L, int sms, cudaStream_t st)

@@ -1,6 +1,8 @@
 // Host interface of the pair kernels (pairs.cu).
 #pragma once
 
+#include <vector>
+
 #include "cf_internal.cuh"
 
 namespace cf {
@@ -90,7 +92,7 @@ cudaError_t launch_count64(const PairParams &P, PairLaunch &L, int sms, cudaStre
 // (the work-list kernel, then the pair kernel).
 cudaError_t launch_pairs(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
 
-// ---- batched launch: jobs of these paths share one persistent kernel
+// ---- batched launch: one persistent kernel per kind of count
 enum : int {
     BATCH_XI32 = 0,       // float32 DD(r), chunks of 16 lanes x 2 primaries
     BATCH_XI64 = 1,
@@ -99,34 +101,41 @@ enum : int {
     BATCH_XI32_8x2 = 4,   // float32 DD(r) with the other tuned shapes
     BATCH_XI32_16x1 = 5,
     BATCH_XI32_32x1 = 6,
+    BATCH_LIN = 8,        // added: table cells linear in the squared distance
 };
 constexpr int BATCH_MAX = 1024;  // jobs per batched launch
 
-struct BatchParams {
-    const PairParams *jobs;  // device array, one per job (work lists already built)
-    const int *path;         // device array: BATCH_* per job
-    int njobs;
-    unsigned *offsets;       // device, njobs + 1 (written by the launch)
-    unsigned *item_counter;  // device, zeroed before the launch
+// The jobs of one kind of count: list[first .. first + n), CTA b's first job (index
+// into that range) at start[start0 + b].
+struct BatchGroup {
+    int path, first, n, blocks, start0, smem;
+};
+struct BatchPlan {
+    std::vector<BatchGroup> groups;
+    std::vector<int> list, start;
 };
 
 // Path of a job: float32 (float32 DD(r) in the kernel shape chunk x pp: 16 x 2,
 // 8 x 2, 16 x 1 or 32 x 1, else 16 x 2) or binary64, DD(r) or DD(rp, pi);
-// unweighted only.
+// unweighted only.  Needs P's table (lut_lin).
 int batch_path(const PairParams &P, int f64, int chunk = 16, int pp = 2);
 
-// The work-list kernel of one job (kept column pairs into P.work, count into
-// *P.work_count, which must be zero).
-cudaError_t launch_worklist(const PairParams &P, cudaStream_t st);
+// Shared memory of a job on that path; its offsets into P.
+int batch_smem(PairParams &P, int path);
 
-// The work lists of njobs jobs (device parameter array) in one launch; job j
-// owns blocks [pre[j], pre[j + 1]) of 256 candidates, blocks = pre[njobs].
-cudaError_t launch_worklist_batch(const PairParams *jobs, const unsigned *pre, int njobs,
-                                  unsigned blocks, cudaStream_t st);
+// Groups, lists and first jobs from every job's path, shared memory and estimated
+// work; the jobs' task splits into their parameters.
+cudaError_t plan_batch(const std::vector<int> &path, const std::vector<int> &smem,
+                       const std::vector<double> &work, int sms, std::vector<PairParams> &jobs,
+                       BatchPlan &plan);
 
-// Offsets over the jobs' kept pairs, then the batched persistent kernel with
-// smem bytes of dynamic shared memory (the largest job's plan); blocks returns
-// the grid size.
-cudaError_t launch_batch(const BatchParams &B, int smem, int sms, int &blocks, cudaStream_t st);
+// The neighbour lists of njobs jobs (device parameter array) in one launch; job j
+// owns blocks [pre[j], pre[j + 1]) of 8 columns, blocks = pre[njobs].
+cudaError_t launch_neighbours_batch(const PairParams *jobs, const unsigned *pre, int njobs, unsigned blocks,
+                                    cudaStream_t st);
+
+// The kernels of a plan; list and start are device copies of the plan's.
+cudaError_t launch_batch(const BatchPlan &plan, const PairParams *jobs, const int *list, const int *start,
+                         cudaStream_t st);
 
 }  // namespace cf

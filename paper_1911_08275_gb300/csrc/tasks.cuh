@@ -35,8 +35,8 @@ struct FlagQueue {
 
 // Tasks of nchunk chunks: one task per chunk, but the last eighth of the chunks
 // (TASK_TAIL) is split into parts, so that the last tasks to finish are short while
-// most chunks pay the set-up of a task once.  All chunks are split when there
-// are at most two per warp of the grid.  Measured on 1.2M points (kernel, ms at
+// most chunks pay the set-up of a task once.  All chunks are split where there
+// are few (at most two per warp of the grid).  Measured on 1.2M points (kernel, ms at
 // Rmax 5 / 10 / 25 / 50): every chunk in one part 0.218 / 0.288 / 1.248 / 5.600,
 // every chunk in two 0.246 / 0.305 / 1.231 / 5.462; then, with the queue of flagged
 // pairs, a tail of a quarter in 4 parts 0.232 / 0.280 / 1.135 / 5.166, of an eighth
@@ -44,8 +44,8 @@ struct FlagQueue {
 constexpr unsigned TASK_TAIL = 8;
 struct TaskSplit {
     unsigned whole, parts, ntask;
-    __device__ TaskSplit(unsigned nchunk, unsigned parts_)
-        : whole(parts_ == 1u ? nchunk : nchunk > 2u * gridDim.x * WARPS ? nchunk - nchunk / TASK_TAIL : 0u), parts(parts_),
+    __device__ TaskSplit(unsigned nchunk, unsigned parts_, bool all)
+        : whole(parts_ == 1u ? nchunk : all ? 0u : nchunk - nchunk / TASK_TAIL), parts(parts_),
           ntask(whole + (nchunk - whole) * parts_)
     {
     }
@@ -264,6 +264,34 @@ __device__ __forceinline__ void for_windows(const PairParams &P, int col, int ib
     }
 }
 
+// Neighbour lists (Sec. 2.1, 2.2): one warp per primary column, one stencil
+// offset per lane; the kept column pairs are listed in stencil order with
+// their z reach (float32, rounded up, with the window slack).
+__device__ __forceinline__ void neighbours_body(const PairParams &P, int col, int lane)
+{
+    if (col >= P.g.ncols)
+        return;
+    int n = 0;
+    for (int s0 = 0; s0 < P.nstencil; s0 += 32) {
+        const int s = s0 + lane;
+        WorkItem w;
+        const bool keep = s < P.nstencil && plan_item(P, col * P.nstencil + s, w);
+        const unsigned m = __ballot_sync(FULL, keep);
+        if (keep) {
+            Nbr r;
+            r.dz = __fadd_ru(__double2float_ru(w.dzmax), P.zslack);
+            r.code = w.code;
+            P.nbr[(long long)col * P.nstencil + n + __popc(m & ((1u << lane) - 1u))] = r;
+        }
+        n += __popc(m);
+    }
+    if (lane == 0) {
+        P.nbr_count[col] = (unsigned)n;
+        if (n)
+            atomicAdd(P.work_count, (unsigned)n);
+    }
+}
+
 // Persistent kernel over the chunk tasks of one count.  Path: CH (primaries per
 // chunk), State, init (false in every thread if the CTA has to give up), task,
 // fini.
@@ -275,7 +303,8 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tasks(const __grid_constant__
     if (!Path::init(P, smem, st))
         return;
     const int lane = threadIdx.x & 31;
-    const TaskSplit split(__ldg(P.A.cell_start + P.g.ncells) / Path::CH, (unsigned)P.parts);
+    const unsigned nchunk = __ldg(P.A.cell_start + P.g.ncells) / Path::CH;
+    const TaskSplit split(nchunk, (unsigned)P.parts, nchunk <= 2u * gridDim.x * WARPS);
     unsigned nxt = 0;
     if (lane == 0)
         nxt = atomicAdd(P.item_counter, 1u);
@@ -301,7 +330,7 @@ cudaError_t launch_tasks(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
     if (occ < 1)
         return cudaErrorInvalidConfiguration;
     const long long chunks = (P.A.n + (long long)P.g.ncols * (COL_PAD / 2)) / Path::CH + 1;
-    P.parts = std::min(P.nstencil, TASK_PARTS);
+    P.parts = task_parts((double)chunks, (double)sms * occ * WARPS, P.nstencil);
     L.blocks = (int)std::max(1ll, std::min<long long>((long long)sms * occ, (chunks * P.parts + WARPS - 1) / WARPS));
     k_tasks<Path, MINB><<<L.blocks, THREADS, L.smem, st>>>(P);
     return cudaGetLastError();
