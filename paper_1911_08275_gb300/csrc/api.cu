@@ -676,7 +676,6 @@ void base_params(const Request &q, const cf::Geom &g, const cf::Gridded &A, cons
     P.n_items = g.ncols * P.nstencil;
     P.shard_n = c->shard_count > 1 ? c->shard_count : 1;
     P.shard_k = c->shard_count > 1 ? c->shard_index : 0;
-    P.tile_max = 1024;
     P.flags = c->flags;
     P.wait_ns = wait_limit_ns(c->flags);
     M = std::max(g.extent[0], std::max(g.extent[1], g.extent[2]));
@@ -689,6 +688,8 @@ void base_params(const Request &q, const cf::Geom &g, const cf::Gridded &A, cons
     P.zslack = (float)(8.0 * U32 * (M + Ls + Rz) + 1e-6 * Rz);
     for (int a = 0; a < 3; ++a)
         P.boxf[a] = (float)g.box[a];
+    for (int a = 0; a < 3; ++a)
+        P.boxr[a] = (float)(g.box[a] - (double)P.boxf[a]);
     set_cull(P, q.edges.back(), q.kind == 0 ? 3 : 2, M, Ls, R);
     P.nbins = (int)q.edges.size() - 1;
     if (q.kind == 1) {
@@ -760,12 +761,8 @@ int run(Request &q)
     double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
     unsigned long long *bbox_keys = nullptr;
     unsigned *d_err = nullptr, *d_ctr = nullptr, *d_wcount = nullptr;
-    cf::WorkItem *work = nullptr;
-    cf::Win *wins = nullptr;
     cf::Nbr *nbr = nullptr;
     unsigned *nbr_count = nullptr;
-    long long win_cap = 0;
-    long long *wscratch = nullptr;
     unsigned long long *d_hist = nullptr, *d_diag = nullptr;
     float *d_thr = nullptr;
     uint8_t *d_lut = nullptr;
@@ -885,16 +882,11 @@ int run(Request &q)
             bump.off = 0;
             for (int t = 0; t < ncat; ++t) {
                 const long long n = cf::padded_max(cats[t]->n, g.ncols);
-                G[t].xs = bump.take<float>(n);
-                G[t].ys = bump.take<float>(n);
-                G[t].zs = bump.take<float>(n);
                 G[t].xyz = bump.take<float>(3 * n);
                 G[t].chunk_col = bump.take<int>(n / cf::COL_PAD);
                 G[t].ws = c->weighted ? bump.take<float>(n + 64) : nullptr;  // + slack for tile reads
                 if (resid) {  // float32 mean separation from inputs float32 cannot hold exactly
-                    G[t].xl = bump.take<float>(n + 64);
-                    G[t].yl = bump.take<float>(n + 64);
-                    G[t].zl = bump.take<float>(n + 64);
+                    G[t].res = bump.take<float>(3 * n);
                 }
                 G[t].wmax = c->weighted ? reinterpret_cast<unsigned *>(d_hist + nslots + 6) + t : nullptr;
                 G[t].pos64 = bump.take<double4_32a>(n);
@@ -913,17 +905,6 @@ int run(Request &q)
             const int nst = q.autocorr ? (sx * sy + 1) / 2 : sx * sy;
             nbr = bump.take<cf::Nbr>((size_t)g.ncols * nst);
             nbr_count = bump.take<unsigned>(g.ncols);
-            work = bump.take<cf::WorkItem>((size_t)g.ncols * cf::MAX_STENCIL);
-            if (q.kind == 0 && !f64 && wacc) {  // window records of the weighted float32 DD(r) kernels
-                const int ch = cf::xi32_chunk(c->pair_chunk ? c->pair_chunk : 16,
-                                              c->pair_pp ? c->pair_pp : 2, wacc,
-                                              (c->flags & CF_FLAG_VERIFY_BAND) != 0);
-                win_cap = cf::win_bound(cats[0]->n, g.ncols, nst, ch);
-                wins = bump.take<cf::Win>((size_t)win_cap);
-            }
-            // float32 weighted DD(r): 64-bit sums per thread of at most 2 CTAs per SM
-            wscratch = (wacc && !f64 && q.kind == 0) ? bump.take<long long>((size_t)sms * 2 * cf::THREADS * 3 * nb)
-                                                     : nullptr;
             if (pass == 0) {
                 const cudaError_t e = cudaMallocAsync(&ws2, bump.off, st);
                 if (e) {
@@ -947,13 +928,8 @@ int run(Request &q)
         // ---- pair kernel parameters
         double M = 0.0, Ls = 0.0;
         base_params(q, g, G[0], G[1], P, M, Ls);
-        P.work = work;
         P.nbr = nbr;
         P.nbr_count = nbr_count;
-        P.win = wins;
-        P.win_cap = win_cap;
-        P.win_count = d_err + 3;  // zeroed with the result block
-        P.wscratch = wscratch;
         if (q.kind == 1) {
             std::memcpy(ho->pe, Pe.data(), 8 * Pe.size());
             CF_CUDA(cudaMemcpyAsync(d_P, ho->pe, 8 * Pe.size(), cudaMemcpyHostToDevice, st), "H2D pi edges");
@@ -995,14 +971,10 @@ int run(Request &q)
         PL.pp = c->pair_pp ? c->pair_pp : 2;
         PL.evals = (c->flags & (CF_FLAG_COUNT_EVALS | CF_FLAG_VERIFY_BAND)) ? 1 : 0;
         PL.verify = (!f64 && (c->flags & CF_FLAG_VERIFY_BAND)) ? 1 : 0;
-        PL.max_blocks = wscratch ? sms * 2 : 0;
-        cf::plan_pairs(P, PL);
-        if (!f64 && PL.smem > cf::SMEM_MAX) {
-            // float32 weighted rows for this many bins exceed shared memory: count
-            // with the binary64 kernel instead (same results, exact per-pair terms)
+        // the float32 DD(r) rows of weights and mean separations fit an SM's shared memory
+        // up to 59 bins: beyond that the binary64 kernel counts (same results, exact terms)
+        if (!f64 && q.kind == 0 && c->weighted && c->want_ravg && nb > 59)
             PL.f64 = 1;
-            cf::plan_pairs(P, PL);
-        }
         trace.point("tables");
         CF_CUDA(cudaEventRecord(g_events.ev[1], st), "cudaEventRecord");
         if (P.n_items > 0) {
@@ -1068,7 +1040,7 @@ int run(Request &q)
         res->n_rechecked = ho->diag[2];
         res->n_band_violations = ho->diag[3];
         for (int t = 0; t < ncat; ++t)
-            res->n_kernels += cf::grid_kernels(cats[t]->n, G[t].xl != nullptr) +
+            res->n_kernels += cf::grid_kernels(cats[t]->n, G[t].res != nullptr) +
                               (c->periodic ? 0 : cf::bbox_kernels(cats[t]->n));
         res->n_kernels += PL.kernels;  // work list, window pre-pass, pair kernel
     }
@@ -1755,7 +1727,6 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
                                       : (2 * g.reach_x + 1) * (2 * g.reach_y + 1);
     cf::Gridded G[2] = {};
     cf::GridTemps tmp = {};
-    cf::WorkItem *work = nullptr;
     cf::Nbr *nbr = nullptr;
     unsigned *nbr_count = nullptr;
     // Carve the grids, temporaries and the work list for the current geometry
@@ -1769,9 +1740,6 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
         for (int t = 0; t < ncat; ++t) {
             const long long n = cf::padded_max(cats[t]->n, g.ncols);
             G[t] = cf::Gridded{};
-            G[t].xs = b.take<float>(n);
-            G[t].ys = b.take<float>(n);
-            G[t].zs = b.take<float>(n);
             G[t].xyz = b.take<float>(3 * n);
             G[t].chunk_col = b.take<int>(n / cf::COL_PAD);
             G[t].pos64 = b.take<double4_32a>(n);
@@ -1786,7 +1754,6 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
         tmp.counts = b.take<uint32_t>(g.ncells + 1);
         tmp.pad = b.take<uint32_t>(g.ncols);
         tmp.bsum = b.take<uint32_t>(g.ncells / 4096 + 2);
-        work = b.take<cf::WorkItem>((size_t)g.ncols * nstencil_max);
         nbr = b.take<cf::Nbr>((size_t)g.ncols * nstencil_max);
         nbr_count = b.take<unsigned>(g.ncols);
         if (b.off <= NOALLOC_BYTES) {
@@ -1836,11 +1803,9 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
             P.stencil[P.nstencil++] = make_int2(ox, oy);
         }
     P.n_items = g.ncols * P.nstencil;
-    P.work = work;
     P.work_count = d_ctr + 1;
     P.nbr = nbr;
     P.nbr_count = nbr_count;
-    P.tile_max = 1024;
     P.flags = c->flags & (CF_FLAG_NO_PRUNE | CF_FLAG_COUNT_EVALS);
     P.wait_ns = wait_limit_ns(P.flags);
     const double M = std::max(g.extent[0], std::max(g.extent[1], g.extent[2]));
@@ -1884,7 +1849,6 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     PL.chunk = 16;
     PL.pp = 2;
     PL.evals = (P.flags & CF_FLAG_COUNT_EVALS) ? 1 : 0;
-    cf::plan_pairs(P, PL);
     if (P.n_items > 0 && (e = cf::launch_pairs(P, PL, sms, st)))
         return cuda_fail(e, "pair kernel launch");
     if ((e = cudaMemcpyAsync(h.hist, d_hist, sizeof(unsigned long long) * nb, cudaMemcpyDeviceToHost, st)) ||
@@ -2236,9 +2200,6 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
                 const long long n = cf::padded_max(j.cat[t].n, j.g.ncols);
                 cf::Gridded &G = j.G[t];
                 G.n = j.cat[t].n;
-                G.xs = bump.take<float>(n);
-                G.ys = bump.take<float>(n);
-                G.zs = bump.take<float>(n);
                 G.xyz = bump.take<float>(3 * n);
                 G.chunk_col = bump.take<int>(n / cf::COL_PAD);
                 G.ws = nullptr;

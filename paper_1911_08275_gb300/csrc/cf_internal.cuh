@@ -13,7 +13,6 @@ constexpr int NB_MAX = 64;          // radial (xi) or rp bins
 constexpr int NBINS2D_MAX = 4096;   // rp bins * pi bins
 constexpr int NPI_MAX = 4096;
 constexpr int LUT_MAX = 16384;      // entries (bytes) of the float32 bin lookup table
-constexpr int TILE32 = 2048;        // secondary points per staged float32 tile
 constexpr int MAX_REACH = 4;        // column stencil half-width per axis
 constexpr int MAX_STENCIL = (2 * MAX_REACH + 1) * (2 * MAX_REACH + 1);
 constexpr int WARPS = 8;            // warps per pair-kernel CTA
@@ -35,29 +34,6 @@ enum : unsigned {
 // of the values -1 .. nbins (the row of -1 just before bin 0, never read) and
 // an entry is a row index without a clamp.
 constexpr unsigned char TAB_FLAGGED = 0xff;
-
-// Shared layout of the float32 DD(r) kernel (compile-time offsets):
-// [0,128) barrier + work item; LUT; x, y, z tiles of TILE32 + 64 floats each;
-// thresholds; squared edges; histogram copies ((nbins + 2) rows of 32 lanes each:
-// the flagged row, the bins, the not-counted row).
-constexpr int XI32_LUT_OFF = 128;
-constexpr int XI32_TX_OFF = XI32_LUT_OFF + LUT_MAX;
-constexpr int XI32_TSTRIDE = (TILE32 + 64) * 4;
-constexpr int XI32_THR_OFF = XI32_TX_OFF + 3 * XI32_TSTRIDE;
-constexpr int XI32_E2_OFF = XI32_THR_OFF + 2 * (NB_MAX + 1) * 4;
-constexpr int XI32_HIST_OFF = XI32_E2_OFF + (NB_MAX + 1) * 8;
-
-// The weighted float32 DD(rp, pi) kernel stages a weight tile after the squared
-// edges.
-constexpr int XIW_W_OFF = XI32_HIST_OFF;
-static_assert(XIW_W_OFF % 16 == 0, "bulk-copy destinations need 16 B");
-
-// The float32 DD(rp, pi) kernel uses the DD(r) layout up to the thresholds and
-// squared rp edges, then a weight tile (as above), the pi edges (binary64) and,
-// from a run-time offset, its histograms: hcopies copies of (nbins + 1) rows
-// of (npibins + 1) words (row nbins and column npibins collect pairs that are
-// not counted), then for weighted sums binary64 [copy][slot][w, r w].
-constexpr int RPPI_P_OFF = XIW_W_OFF + XI32_TSTRIDE;
 
 // Grid geometry: columns in (x, y), z-cells inside each column (sort keys).
 struct Geom {
@@ -97,12 +73,12 @@ __host__ __device__ __forceinline__ size_t quad_off(uint32_t d)
 // COL_PAD entries.
 struct Gridded {
     long long n;
-    float *xs, *ys, *zs;  // float32 coordinates in the grid frame (padded columns)
-    float *xyz;           // the same in quads (quad_off): one address serves three 16-byte loads
+    float *xyz;           // float32 coordinates in the grid frame, in quads (quad_off): one address
+                          // serves three 16-byte loads
     float *ws;            // float32 weights (padded columns, 64 floats of slack; NULL without weights)
     unsigned *wmax;       // bit pattern of max |w| as float (written by gridding; NULL without weights)
-    float *xl, *yl, *zl;  // rounding residuals fl32((X - O) - xs) of the float32 coordinates
-                          // (float32 mean separations from float64 inputs; else NULL)
+    float *res;           // rounding residuals fl32((X - O) - x~) of the float32 coordinates, in the
+                          // quad layout (float32 mean separations from float64 inputs; else NULL)
     double4_32a *pos64;       // (x, y, z, w) binary64, exact inputs
     int *perm;            // original index of each sorted point
     int *chunk_col;       // column of each run of COL_PAD entries
@@ -117,14 +93,6 @@ struct __align__(16) WorkItem {
     int code;            // bits 0-1: qx + 1, bits 2-3: qy + 1 (periodic image), bit 4: self pair,
                          // bits 5-31: column b
     int wbase;           // first window record of the pair's chunks (window pre-pass), else 0
-};
-
-// Window record of one chunk of column a against column b (window pre-pass):
-// for each periodic z image k = -1, 0, +1 the range [lo, hi) of column b (point
-// indices) whose float32 z can lie within the pair's z reach of the chunk; an
-// empty range (lo == hi) when the image does not apply.
-struct __align__(8) Win {
-    int lo[3], hi[3];
 };
 
 // A kept neighbour of a primary column: the column pair's z reach (float32,
@@ -152,17 +120,11 @@ struct PairParams {
     int2 stencil[MAX_STENCIL];
     int n_items;        // (column, stencil offset) candidates
     int shard_k, shard_n;  // keep columns whose first point lies in slice k of n (n > 1)
-    WorkItem *work;     // kept column pairs (work-list kernel output)
     unsigned *work_count;  // number of kept column pairs
-    Win *win;           // window records (window pre-pass), NULL = windows found in the sweep
-    unsigned *win_count;   // window records handed out by the work-list kernel
-    long long win_cap;  // capacity of win (records)
-    int win_chunk;      // primaries per chunk the windows are computed for (0 = no pre-pass)
     Nbr *nbr;           // chunk tasks: nstencil entries per primary column, kept ones first
     unsigned *nbr_count;   // kept entries per primary column
     int parts;          // chunk tasks: shares a chunk's neighbour list is split into
     int split_all;      // batches: every chunk is split (else the last eighth)
-    int tile_max;       // points per staged tile
     uint32_t flags;
     uint64_t wait_ns;   // limit of every tile-barrier wait (then the error word gets ERR_TIMEOUT)
     // radii (binary64 decisions on bounding boxes)
@@ -171,6 +133,7 @@ struct PairParams {
     double rxy2;        // squared xy reach for the z window: Rmax^2
     float zslack;       // float32 slack added to z windows
     float boxf[3];      // fl32(L)
+    float boxr[3];      // fl32(L - fl32(L))
     // binning
     int nbins;          // xi or rp bins
     int npibins;        // rp-pi only
@@ -191,7 +154,6 @@ struct PairParams {
     int wacc;           // weighted || want_r
     int rlo;            // float32 mean separation corrected with the coordinates' residuals
     int acc_off;        // byte offset of the binary64 accumulators in shared memory
-    long long *wscratch;  // float32 weighted DD(r): per-thread [bin][count, w, r w] int64 sums
     const float *thr;        // nthr
     const uint8_t *lut;      // lut_n
     const double *E2;        // nbins + 1

@@ -44,7 +44,7 @@ constexpr int C32_LUT = 128;
 constexpr int C32_THR = C32_LUT + LUT_MAX;
 constexpr int C32_E2 = C32_THR + 2 * (NB_MAX + 1) * 4;
 constexpr int C32_RING = (C32_E2 + (NB_MAX + 1) * 8 + 127) / 128 * 128;
-constexpr int C32_QUEUE = C32_RING + WARPS * RING_BYTES;
+constexpr int C32_QUEUE = C32_RING + WARPS * RingXYZ::BYTES;
 constexpr int C32_HIST = C32_QUEUE + WARPS * (int)sizeof(FlagQueue);
 
 // What a sweep needs beside the primaries.
@@ -274,14 +274,14 @@ struct Count32 {
                                                 unsigned c, unsigned part, unsigned parts)
     {
         const int lane = threadIdx.x & 31, ii = lane % I, jj = lane / I;
-        const uint32_t ring = smem_u32(smem + C32_RING) + (threadIdx.x >> 5) * (uint32_t)RING_BYTES;
+        const uint32_t ring = smem_u32(smem + C32_RING) + (threadIdx.x >> 5) * (uint32_t)RingXYZ::BYTES;
         const int ib = (int)(c * CH);
         Chunk<I, PP> C;
         if (!C.load(P, ib, ii))
             return;
         u64 XH[PP], YH[PP], ZH[PP];
         int image = 0;
-        for_windows<128 / I>(
+        for_windows<128 / I, RingXYZ>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) { image = C.shift(P, k, code, XH, YH, ZH); },
             [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {

@@ -16,7 +16,7 @@ int plan_count64(PairParams &P)
     P.guess_off = 128;
     P.e2_off = P.guess_off + GUESS;
     P.ring_off = align_up(P.e2_off + (P.nbins + 1 + (P.kind == 1 ? P.npibins + 1 : 0)) * 8, 128);
-    P.queue_off = P.ring_off + WARPS * RING_BYTES;
+    P.queue_off = P.ring_off + WARPS * RingXYZ::BYTES;
     P.hist_off = align_up(P.queue_off + WARPS * (int)sizeof(FlagQueue), 128);
     const int sums = P.wacc ? slots * 16 : 0;
     if (P.kind == 0) {

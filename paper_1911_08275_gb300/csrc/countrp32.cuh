@@ -39,7 +39,7 @@ constexpr int CRP_LUT = 128;
 constexpr int CRP_THR = CRP_LUT + LUT_MAX;
 constexpr int CRP_E2 = CRP_THR + 2 * (NB_MAX + 1) * 4;
 constexpr int CRP_RING = (CRP_E2 + (NB_MAX + 1) * 8 + 127) / 128 * 128;
-constexpr int CRP_QUEUE = CRP_RING + WARPS * RING_BYTES;
+constexpr int CRP_QUEUE = CRP_RING + WARPS * RingXYZ::BYTES;
 constexpr int CRP_HIST = CRP_QUEUE + WARPS * (int)sizeof(FlagQueue);
 
 __device__ __forceinline__ void red_shared_add(uint32_t addr, uint32_t v)
@@ -308,14 +308,14 @@ struct CountRp32 {
                                                 unsigned c, unsigned part, unsigned parts)
     {
         const int lane = threadIdx.x & 31, ii = lane % I, jj = lane / I;
-        const uint32_t ring = smem_u32(smem + CRP_RING) + (threadIdx.x >> 5) * (uint32_t)RING_BYTES;
+        const uint32_t ring = smem_u32(smem + CRP_RING) + (threadIdx.x >> 5) * (uint32_t)RingXYZ::BYTES;
         const int ib = (int)(c * CH);
         Chunk<I, PP> C;
         if (!C.load(P, ib, ii))
             return;
         u64 XH[PP], YH[PP], ZH[PP];
         int image = 0;
-        for_windows<JS>(
+        for_windows<JS, RingXYZ>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) { image = C.shift(P, k, code, XH, YH, ZH); },
             [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {

@@ -192,88 +192,19 @@ struct Cull64 {
     {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ii = lane % I, jj = lane / I;
         FlagQueue *fq = reinterpret_cast<FlagQueue *>(smem + P.queue_off) + warp;
-        const uint32_t ring = smem_u32(smem + P.ring_off) + (uint32_t)warp * RING_BYTES;
-        const u64 CULL = pack2(-P.cull, -P.cull), ZCULL = pack2(-P.zcull, -P.zcull);
+        const uint32_t ring = smem_u32(smem + P.ring_off) + (uint32_t)warp * RingXYZ::BYTES;
         const int ib = (int)(c * CH);
         Chunk<I, PP> C;
         if (!C.load(P, ib, ii))
             return;
         u64 XH[PP], YH[PP], ZH[PP];
         int image = 0;
-        for_windows<JS>(
+        for_windows<JS, RingXYZ>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) { image = C.shift(P, k, code, XH, YH, ZH); },
             [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {
-                const uint32_t p0 = addr + 48u * jj;
-                uint32_t p = p0;
-                for (int nit = (j1 - j0 + JS - 1) / JS; nit > 0; nit -= 8) {
-                    const int tend = min(8, nit);
-                    const uint32_t pb = p, pend = p + (uint32_t)tend * (12u * JS);
-                    uint32_t fm[PP];
-#pragma unroll
-                    for (int q = 0; q < PP; ++q)
-                        fm[q] = 0u;
-#pragma unroll 1
-                    for (; p != pend; p += 12 * JS) {
-                        ulonglong2 vx, vy, vz;
-                        lds128<0>(p, vx);
-                        lds128<16>(p, vy);
-                        lds128<32>(p, vz);
-#pragma unroll
-                        for (int q = 0; q < PP; ++q) {
-                            u64 s[2], dx, dy, dz;
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                dx = fsub2(h ? vx.y : vx.x, XH[q]);
-                                dy = fsub2(h ? vy.y : vy.x, YH[q]);
-                                dz = fsub2(h ? vz.y : vz.x, ZH[q]);
-                                // negative: within reach (a NaN of the padding is positive)
-                                s[h] = ffma2(dy, dy, ffma2(dx, dx, CULL));
-                                if (KIND == 0)
-                                    s[h] = ffma2(dz, dz, s[h]);
-                                else  // both signs set
-                                    s[h] &= ffma2(dz, dz, ZCULL);
-                            }
-                            float f[4];
-                            unpack2(s[0], f[0], f[1]);
-                            unpack2(s[1], f[2], f[3]);
-#pragma unroll
-                            for (int r = 0; r < 4; ++r)  // pair (t, r) ends at bit 4 tend - 1 - (4 t + r)
-                                fm[q] = push_sign(fm[q], __float_as_uint(f[r]));
-                        }
-                        if (EVALS) {
-                            const int jt = j0 + 4 * jj + (int)((p - p0) / 12u);
-#pragma unroll
-                            for (int q = 0; q < PP; ++q)
-#pragma unroll
-                                for (int r = 0; r < 4; ++r)
-                                    st.n_eval += (((C.vmask >> q) & 1u) && jt + r >= jlo && jt + r < jhi &&
-                                                  (!tri || jt + r > ib + q * I + ii)) ? 1ull : 0ull;
-                        }
-                    }
-                    const int jb = j0 + 4 * jj + (int)((pb - p0) / 12u);
-#pragma unroll
-                    for (int q = 0; q < PP; ++q) {
-                        const int i = ib + q * I + ii;
-                        uint32_t m = fm[q];
-                        for (unsigned bm; (bm = __ballot_sync(FULL, m != 0u)) != 0u;) {
-                            const int b = 4 * tend - __ffs(m);  // = 4 t + r
-                            const int j = jb + (b >> 2) * JS + (b & 3);
-                            const bool put = m != 0u && (!tri || j > i);
-                            m &= m - 1u;
-                            if (tri)
-                                bm = __ballot_sync(FULL, put);
-                            if (put) {
-                                const int at = st.qn + __popc(bm & ((1u << lane) - 1u));
-                                fq->i[at] = i;
-                                fq->j[at] = j;
-                                fq->image[at] = image;
-                            }
-                            st.qn += __popc(bm);
-                            drain(P, smem, st, fq, 31);
-                        }
-                    }
-                }
+                cull_piece<KIND, I, PP, EVALS>(P, fq, st.qn, st.n_eval, addr, j0, j1, jlo, jhi, tri, jj, ii, XH,
+                                               YH, ZH, ib, image, C.vmask, [&]() { drain(P, smem, st, fq, 31); });
                 flush(P, smem, st);
             });
         // entries name their points, so a partly filled queue waits for the next task

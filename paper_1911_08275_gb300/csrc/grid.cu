@@ -11,8 +11,8 @@
 //                           entries, so chunks of 8, 16 or 32 primaries and
 //                           aligned groups of secondaries never straddle two
 //                           columns; padding entries are NaN and never counted.
-//   xs, ys, zs[n']  float32 x - ox, y - oy, z - oz (grid frame), structure of arrays
-//   xyz[3 n']       the same in quads (x0..x3, y0..y3, z0..z3 per four points)
+//   xyz[3 n']       float32 x - ox, y - oy, z - oz (grid frame) in quads (x0..x3, y0..y3,
+//                   z0..z3 per four points)
 //   chunk_col[n'/32] column of each run of 32 entries
 //   pos64[n']       double4 (x, y, z, w) exact binary64 copies (re-checks, FP64 path)
 //   perm[n']        original index of each sorted point (-1 for padding)
@@ -255,9 +255,8 @@ __global__ void k_scatter(const T *__restrict__ z, long long n, const uint32_t *
 template <class T>
 __device__ __forceinline__ void put_entry(const T *__restrict__ x, const T *__restrict__ y,
                                           const double *__restrict__ w, const Geom &g, uint32_t d,
-                                          int iq, unsigned long long kq, float *__restrict__ xs,
-                                          float *__restrict__ ys, float *__restrict__ zs,
-                                          float *__restrict__ xyz, float *__restrict__ ws,
+                                          int iq, unsigned long long kq, float *__restrict__ xyz,
+                                          float *__restrict__ ws,
                                           double4_32a *__restrict__ pos64, int *__restrict__ perm,
                                           unsigned &wm)
 {
@@ -268,9 +267,6 @@ __device__ __forceinline__ void put_entry(const T *__restrict__ x, const T *__re
     coord(X, 0, g, fx);
     coord(Y, 1, g, fy);
     coord(Z, 2, g, fz);
-    xs[d] = fx;
-    ys[d] = fy;
-    zs[d] = fz;
     float *qd = xyz + quad_off(d);
     qd[0] = fx;
     qd[4] = fy;
@@ -310,8 +306,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
     k_sort_cells(const T *__restrict__ x, const T *__restrict__ y, const double *__restrict__ w,
                  long long ncells, Geom g, const uint32_t *__restrict__ count,
                  const uint32_t *__restrict__ start, const int *__restrict__ tmp_idx,
-                 const unsigned long long *__restrict__ tmp_key, float *__restrict__ xs,
-                 float *__restrict__ ys, float *__restrict__ zs, float *__restrict__ xyz,
+                 const unsigned long long *__restrict__ tmp_key, float *__restrict__ xyz,
                  float *__restrict__ ws, unsigned *__restrict__ wmax, double4_32a *__restrict__ pos64,
                  int *__restrict__ perm, unsigned *__restrict__ claim)
 {
@@ -339,7 +334,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
             __syncwarp();
             const uint32_t rank = rank_in(be + half * 16, max(cnt0, cnt1), kq, iq);
             if (mine)
-                put_entry(x, y, w, g, s + rank, iq, kq, xs, ys, zs, xyz, ws, pos64, perm, wm);
+                put_entry(x, y, w, g, s + rank, iq, kq, xyz, ws, pos64, perm, wm);
             continue;
         }
         for (int h = 0; h < 2; ++h) {  // whole warp, one cell after the other
@@ -379,7 +374,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
                     }
                 }
                 if (mine)
-                    put_entry(x, y, w, g, sc + rank, iq, kq, xs, ys, zs, xyz, ws, pos64, perm, wm);
+                    put_entry(x, y, w, g, sc + rank, iq, kq, xyz, ws, pos64, perm, wm);
             }
         }
     }
@@ -407,7 +402,6 @@ __device__ __forceinline__ void pad_column(const Gridded &G, int col, uint32_t s
     const double dn = __longlong_as_double(0x7ff8000000000000ll);
     if ((uint32_t)lane < pad) {
         const uint32_t q = e - 1u - lane;
-        G.xs[q] = G.ys[q] = G.zs[q] = fn;
         float *qd = G.xyz + quad_off(q);
         qd[0] = qd[4] = qd[8] = fn;
         if (G.ws)
@@ -540,25 +534,24 @@ inline int grid_blocks(long long n, int threads, int sms)
 // does (binary64; X itself in a periodic box, whose origin is 0).  The float32
 // mean separation uses them to restore the coordinates' lost bits.  Padding
 // entries get 0.
-__global__ void k_residual(const double4_32a *__restrict__ pos64, const float *__restrict__ xs,
-                           const float *__restrict__ ys, const float *__restrict__ zs,
-                           const uint32_t *__restrict__ cell_start, Geom g, float *__restrict__ xl,
-                           float *__restrict__ yl, float *__restrict__ zl)
+__global__ void k_residual(const __grid_constant__ Gridded G, const __grid_constant__ Geom g)
 {
-    const long long n = cell_start[g.ncells];  // padded length of the gridded catalogue
+    const long long n = G.cell_start[g.ncells];  // padded length of the gridded catalogue
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long d = (long long)blockIdx.x * blockDim.x + threadIdx.x; d < n; d += stride) {
-        const double4_32a p = pos64[d];
+        const double4_32a p = G.pos64[d];
+        const float *q = G.xyz + quad_off((uint32_t)d);
+        float *r = G.res + quad_off((uint32_t)d);
         if (isnan(p.x)) {
-            xl[d] = yl[d] = zl[d] = 0.0f;
+            r[0] = r[4] = r[8] = 0.0f;
             continue;
         }
         const double X = g.periodic ? p.x : __dsub_rn(p.x, g.origin[0]);
         const double Y = g.periodic ? p.y : __dsub_rn(p.y, g.origin[1]);
         const double Z = g.periodic ? p.z : __dsub_rn(p.z, g.origin[2]);
-        xl[d] = __double2float_rn(__dsub_rn(X, (double)xs[d]));
-        yl[d] = __double2float_rn(__dsub_rn(Y, (double)ys[d]));
-        zl[d] = __double2float_rn(__dsub_rn(Z, (double)zs[d]));
+        r[0] = __double2float_rn(__dsub_rn(X, (double)q[0]));
+        r[4] = __double2float_rn(__dsub_rn(Y, (double)q[4]));
+        r[8] = __double2float_rn(__dsub_rn(Z, (double)q[8]));
     }
 }
 
@@ -711,10 +704,10 @@ __device__ __forceinline__ void put_seg(const GridBatch &B, const GridSeg &S, ui
     const Geom &g = B.geom[S.job];
     if (S.f32)
         put_entry(static_cast<const float *>(S.x), static_cast<const float *>(S.y), nullptr, g, d, iq,
-                  kq, S.out.xs, S.out.ys, S.out.zs, S.out.xyz, nullptr, S.out.pos64, S.out.perm, wm);
+                  kq, S.out.xyz, nullptr, S.out.pos64, S.out.perm, wm);
     else
         put_entry(static_cast<const double *>(S.x), static_cast<const double *>(S.y), nullptr, g, d,
-                  iq, kq, S.out.xs, S.out.ys, S.out.zs, S.out.xyz, nullptr, S.out.pos64, S.out.perm, wm);
+                  iq, kq, S.out.xyz, nullptr, S.out.pos64, S.out.perm, wm);
 }
 
 // k_sort_cells over the concatenated cells of every segment (the two cells of
@@ -888,18 +881,14 @@ cudaError_t build_grid_t(const void *x, const void *y, const void *z, const doub
         const long long cwarps = std::min<long long>((nc + 1) / 2, (long long)sms * 64);
         k_sort_cells<T><<<(int)((cwarps * 32 + SORT_THREADS - 1) / SORT_THREADS), SORT_THREADS, 0, st>>>(
             (const T *)x, (const T *)y, w, nc, g, t.counts, out.cell_start, t.tmp_idx, t.tmp_key,
-            out.xs, out.ys, out.zs, out.xyz, out.ws, out.ws ? out.wmax : nullptr, out.pos64, out.perm,
+            out.xyz, out.ws, out.ws ? out.wmax : nullptr, out.pos64, out.perm,
             t.counts + nc);
     }
     k_padfill<<<cb, 256, 0, st>>>(t.pad, g.ncols, g.nz, out);
     k_colbox<<<std::min(g.ncols, sms * 8), 256, 0, st>>>(out.pos64, out.cell_start, g.ncols, g.nz,
                                                           out.colbox);
-    if (out.xl) {
-        const long long np = padded_max(n, g.ncols);
-        k_residual<<<grid_blocks(np, TB, sms), TB, 0, st>>>(out.pos64, out.xs, out.ys, out.zs,
-                                                            out.cell_start, g, out.xl, out.yl,
-                                                            out.zl);
-    }
+    if (out.res)
+        k_residual<<<grid_blocks(padded_max(n, g.ncols), TB, sms), TB, 0, st>>>(out, g);
     return cudaGetLastError();
 }
 

@@ -9,72 +9,16 @@ namespace cf {
 
 __host__ __device__ inline int align_up(int v, int a) { return (v + a - 1) / a * a; }
 
-// Shared-memory layout of the binary64 kernels (identical on host and device):
-// [0, 128) barrier + work item; tile of tile_max + 32 points (x, y, z, w);
-// squared edges; pi edges (rp-pi); histograms.
-struct Smem64 {
-    int tile, e2, p, hist, total;
-};
-
-__host__ __device__ inline Smem64 smem64_layout(int tile_max, int nbins, int npibins, int hist_words)
-{
-    Smem64 L;
-    int off = 128;
-    L.tile = off;
-    off += (tile_max + 32) * 32;
-    L.e2 = off = align_up(off, 16);
-    off += (nbins + 1) * 8;
-    L.p = off = align_up(off, 16);
-    off += (npibins > 0 ? npibins + 1 : 0) * 8;
-    L.hist = off = align_up(off, 128);
-    off += hist_words * 4;
-    L.total = align_up(off, 128);
-    return L;
-}
-
-constexpr int SMEM_MAX = 232448;  // dynamic shared memory a CTA may opt in to (227 KB)
-
 struct PairLaunch {
-    int f64;         // 1: binary64 path
-    int chunk;       // primary lanes per warp chunk (8, 16 or 32)
-    int pp;          // primaries per lane (1 or 2; float32 DD(r))
-    int evals;       // count evaluations
-    int verify;      // verify float32 decisions against binary64
-    int blocks;      // persistent CTAs
-    int smem;        // dynamic shared memory bytes
-    int hist_words;  // shared histogram words
-    int max_blocks;  // upper bound on the persistent grid (0 = none)
-    int kernels;     // kernels the launch issued (work list, window pre-pass, pair kernel)
+    int f64;      // 1: binary64 counts
+    int chunk;    // primary lanes per warp chunk (8, 16 or 32)
+    int pp;       // primaries per lane (1, 2 or 4; float32 counts)
+    int evals;    // count evaluations
+    int verify;   // verify float32 decisions against binary64
+    int blocks;   // persistent CTAs
+    int smem;     // dynamic shared memory bytes
+    int kernels;  // kernels the launch issued (neighbour lists, pair kernel)
 };
-
-// Primaries per chunk of the float32 DD(r) kernel for a requested shape (chunk
-// lanes x primaries per lane; the weighted sweep runs 16 x 1, the verifying
-// one 8 x 1); the window pre-pass writes one record per chunk of this size.
-inline int xi32_chunk(int chunk, int pp, bool weighted, bool verify)
-{
-    if (verify)
-        return 8;
-    if (weighted)
-        return 16;
-    if (pp == 4)
-        return 32;
-    if (pp == 2)
-        return chunk == 8 ? 16 : 32;
-    return chunk == 16 || chunk == 32 ? chunk : 8;
-}
-
-// Upper bound on the window records of one launch: every kept column pair
-// (at most nstencil per column of d1) has one record per chunk of its column a,
-// and the columns of d1 hold padded_max(n1, ncols) entries.
-inline long long win_bound(long long n1, int ncols, int nstencil, int chunk)
-{
-    return (long long)nstencil * (padded_max(n1, ncols) / chunk + ncols + 1);
-}
-
-// Fill the shared-memory plan of a launch: L.smem, L.hist_words and, for
-// rp-pi, P.hcopies and P.hist_off.  Needs P.kind, P.nbins, P.npibins,
-// P.tile_max and L.f64.
-void plan_pairs(PairParams &P, PairLaunch &L);
 
 // Chunk tasks (tasks.cuh): the neighbour lists of d1's columns (P.nbr,
 // P.nbr_count; kept pairs added to *P.work_count), and the float32 DD(r) counts.
@@ -88,8 +32,11 @@ int countrp32_smem(int nbins, int npibins);
 int plan_count64(PairParams &P);
 cudaError_t launch_count64(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
 
-// Configure (max dynamic smem), pick the occupancy-based grid and launch
-// (the work-list kernel, then the pair kernel).
+// Float32 sums: DD(r), DD(rp, pi).
+cudaError_t launch_sums32(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
+cudaError_t launch_sumsrp32(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
+
+// The kernels of one count: neighbour lists, then the pair kernel of its kind.
 cudaError_t launch_pairs(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
 
 // ---- batched launch: one persistent kernel per kind of count

@@ -95,14 +95,6 @@ __device__ __forceinline__ void zwindow(const float *__restrict__ q, const uint3
     hi = b0;
 }
 
-// Two pieces of secondaries per warp in shared memory: while the warp sweeps
-// one, the next (of this window or the one after) is on its way.  A 16-byte
-// global load of a value that 16 lanes share occupies the L1's data path four
-// times (once per quarter warp), a shared load twice.
-constexpr int PIECE = 192;                   // secondaries per piece
-constexpr int PIECE_BYTES = PIECE * 12;      // in the quad layout
-constexpr int RING_BYTES = 2 * PIECE_BYTES;  // per warp
-
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -113,6 +105,43 @@ __device__ __forceinline__ void cp_wait()
 {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+
+// Copy bytes (a multiple of 16, both sides aligned to 16) to shared memory, one
+// 16-byte unit per lane and round.
+__device__ __forceinline__ void warp_copy(uint32_t dst, const void *src, int bytes, int lane)
+{
+    for (int u = lane * 16; u < bytes; u += 512)
+        cp_async16(dst + u, static_cast<const char *>(src) + u);
+}
+
+// Two pieces of secondaries per warp in shared memory: while the warp sweeps
+// one, the next (of this window or the one after) is on its way.  A 16-byte
+// global load of a value that 16 lanes share occupies the L1's data path four
+// times (once per quarter warp), a shared load twice.  A Ring says what a piece
+// holds: N secondaries, SLOT bytes, copied by copy(P, dst, j, n, lane).
+struct RingXYZ {  // coordinates, in the quad layout
+    static constexpr int N = 192, SLOT = N * 12, BYTES = 2 * SLOT;
+    static __device__ __forceinline__ void copy(const PairParams &P, uint32_t dst, int j, int n, int lane)
+    {
+        warp_copy(dst, P.B.xyz + 3ll * j, n * 12, lane);
+    }
+};
+
+// Coordinates, then their residuals (RL) in the quad layout, then weights (W).
+// Short pieces: two CTAs with their rows of sums fill an SM's shared memory.
+template <bool W, bool RL>
+struct RingSums {
+    static constexpr int N = RL ? 32 : 64, RES_OFF = N * 12, W_OFF = N * (RL ? 24 : 12),
+                         SLOT = W_OFF + (W ? N * 4 : 0), BYTES = 2 * SLOT;
+    static __device__ __forceinline__ void copy(const PairParams &P, uint32_t dst, int j, int n, int lane)
+    {
+        warp_copy(dst, P.B.xyz + 3ll * j, n * 12, lane);
+        if (RL)
+            warp_copy(dst + RES_OFF, P.B.res + 3ll * j, n * 12, lane);
+        if (W)
+            warp_copy(dst + W_OFF, P.B.ws + j, n * 4, lane);
+    }
+};
 
 // The job's byte table by one bulk copy into smem + lut_off, while fill() writes
 // what else the CTA needs (the barrier at smem is initialised; its phase parity is
@@ -126,7 +155,7 @@ __device__ __forceinline__ bool load_table(const PairParams &P, unsigned char *s
         const unsigned bytes = ((unsigned)P.lut_n + 15u) & ~15u;
         fence_proxy_async_smem();
         mbar_arrive_expect_tx(bar, bytes);
-        if (!(P.flags & CF_FLAG_DEBUG_STALL) || P.kind != 0)  // diagnostic stall: never issued
+        if (!(P.flags & CF_FLAG_DEBUG_STALL) || P.kind != 0 || P.wacc)  // diagnostic stall: never issued
             bulk_g2s(smem + lut_off, P.lut, bytes, bar);
     }
     fill();
@@ -194,7 +223,7 @@ struct Chunk {
 // [j0, j1) of it (j0 a multiple of JS; secondaries outside the window are
 // farther than the reach in z) sweep(addr, j0, j1, jlo, jhi, tri) is called with
 // the shared address of secondary j0.
-template <int JS, class Open, class Sw>
+template <int JS, class Ring, class Open, class Sw>
 __device__ __forceinline__ void for_windows(const PairParams &P, int col, int ib, float zlo, float zhi,
                                             int part, int parts, int lane, uint32_t ring, Open open, Sw sw)
 {
@@ -235,10 +264,8 @@ __device__ __forceinline__ void for_windows(const PairParams &P, int col, int ib
                     pe = __shfl_sync(FULL, jhi, l);
                 }
                 if (pj < pe) {
-                    const int n = min(PIECE, (pe - pj + JS - 1) & ~(JS - 1));
-                    const char *src = reinterpret_cast<const char *>(P.B.xyz) + 12ll * pj;
-                    for (int u = lane * 16; u < n * 12; u += 512)
-                        cp_async16(dst + u, src + u);
+                    const int n = min(Ring::N, (pe - pj + JS - 1) & ~(JS - 1));
+                    Ring::copy(P, dst, pj, n, lane);
                     pj += n;
                 }
                 cp_commit();
@@ -251,14 +278,96 @@ __device__ __forceinline__ void for_windows(const PairParams &P, int col, int ib
                 const int cd = __shfl_sync(FULL, code, l);
                 const bool tri = (cd & 16) && k == 0;
                 open(k, cd);
-                for (int j0 = lo & ~(JS - 1); j0 < hi; j0 += PIECE) {
-                    request(2 * ring + PIECE_BYTES - cur);
+                for (int j0 = lo & ~(JS - 1); j0 < hi; j0 += Ring::N) {
+                    request(2 * ring + Ring::SLOT - cur);
                     cp_wait<1>();
                     __syncwarp();
-                    sw(cur, j0, min(j0 + PIECE, hi), lo, hi, tri);
+                    sw(cur, j0, min(j0 + Ring::N, hi), lo, hi, tri);
                     __syncwarp();
-                    cur = 2 * ring + PIECE_BYTES - cur;
+                    cur = 2 * ring + Ring::SLOT - cur;
                 }
+            }
+        }
+    }
+}
+
+// Queue the pairs of a piece [j0, j1) of a window [jlo, jhi) that the float32 bounds
+// do not prove out of reach (set_cull): KIND 0 by r^2, KIND 1 by rp^2 and |dz|.
+// drain() is called whenever pairs were added (at most 31 may be left waiting).
+template <int KIND, int I, int PP, bool EVALS, class Drain>
+__device__ __forceinline__ void cull_piece(const PairParams &P, FlagQueue *fq, int &qn, u64 &n_eval,
+                                           uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri, int jj,
+                                           int ii, const u64 (&XH)[PP], const u64 (&YH)[PP],
+                                           const u64 (&ZH)[PP], int ib, int image, unsigned vmask, Drain drain)
+{
+    constexpr int JS = 128 / I;
+    const u64 CULL = pack2(-P.cull, -P.cull), ZCULL = pack2(-P.zcull, -P.zcull);
+    const uint32_t p0 = addr + 48u * jj;
+    uint32_t p = p0;
+    for (int nit = (j1 - j0 + JS - 1) / JS; nit > 0; nit -= 8) {
+        const int tend = min(8, nit);
+        const uint32_t pb = p, pend = p + (uint32_t)tend * (12u * JS);
+        uint32_t fm[PP];
+#pragma unroll
+        for (int q = 0; q < PP; ++q)
+            fm[q] = 0u;
+#pragma unroll 1
+        for (; p != pend; p += 12 * JS) {
+            ulonglong2 vx, vy, vz;
+            lds128<0>(p, vx);
+            lds128<16>(p, vy);
+            lds128<32>(p, vz);
+#pragma unroll
+            for (int q = 0; q < PP; ++q) {
+                u64 s[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const u64 dx = fsub2(h ? vx.y : vx.x, XH[q]), dy = fsub2(h ? vy.y : vy.x, YH[q]),
+                              dz = fsub2(h ? vz.y : vz.x, ZH[q]);
+                    // negative: within reach (a NaN of the padding is positive)
+                    s[h] = ffma2(dy, dy, ffma2(dx, dx, CULL));
+                    if (KIND == 0)
+                        s[h] = ffma2(dz, dz, s[h]);
+                    else  // both signs set
+                        s[h] &= ffma2(dz, dz, ZCULL);
+                }
+                float f[4];
+                unpack2(s[0], f[0], f[1]);
+                unpack2(s[1], f[2], f[3]);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)  // pair (t, r) ends at bit 4 tend - 1 - (4 t + r)
+                    fm[q] = push_sign(fm[q], __float_as_uint(f[r]));
+            }
+            if (EVALS) {
+                const int jt = j0 + 4 * jj + (int)((p - p0) / 12u);
+#pragma unroll
+                for (int q = 0; q < PP; ++q)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        n_eval += (((vmask >> q) & 1u) && jt + r >= jlo && jt + r < jhi &&
+                                   (!tri || jt + r > ib + q * I + ii)) ? 1ull : 0ull;
+            }
+        }
+        const int lane = threadIdx.x & 31, jb = j0 + 4 * jj + (int)((pb - p0) / 12u);
+#pragma unroll
+        for (int q = 0; q < PP; ++q) {
+            const int i = ib + q * I + ii;
+            uint32_t m = fm[q];
+            for (unsigned bm; (bm = __ballot_sync(FULL, m != 0u)) != 0u;) {
+                const int b = 4 * tend - __ffs(m);  // = 4 t + r
+                const int j = jb + (b >> 2) * JS + (b & 3);
+                const bool put = m != 0u && (!tri || j > i);
+                m &= m - 1u;
+                if (tri)
+                    bm = __ballot_sync(FULL, put);
+                if (put) {
+                    const int at = qn + __popc(bm & ((1u << lane) - 1u));
+                    fq->i[at] = i;
+                    fq->j[at] = j;
+                    fq->image[at] = image;
+                }
+                qn += __popc(bm);
+                drain();
             }
         }
     }
