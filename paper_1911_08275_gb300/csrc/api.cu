@@ -760,7 +760,7 @@ int run(Request &q)
     long long nmax = 0, ntot = 0;
     double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
     unsigned long long *bbox_keys = nullptr;
-    unsigned *d_err = nullptr, *d_ctr = nullptr, *d_wcount = nullptr;
+    unsigned *d_err = nullptr, *d_ctr = nullptr, *d_wcount = nullptr, *d_bar = nullptr;
     cf::Nbr *nbr = nullptr;
     unsigned *nbr_count = nullptr;
     unsigned long long *d_hist = nullptr, *d_diag = nullptr;
@@ -769,7 +769,7 @@ int run(Request &q)
     double *d_E2 = nullptr, *d_P = nullptr;
     size_t total = 0;
     struct HostOut {
-        unsigned long long hist[3 * cf::NBINS2D_MAX + 7];  // hist | diag(4) | err, counter | kept | max |w| (2) | wsum | rsum
+        unsigned long long hist[3 * cf::NBINS2D_MAX + 8];  // hist | diag(4) | err, counter | kept | max |w| (2) | barriers (2) | wsum | rsum
         unsigned long long *diag;
         unsigned err;
         float thr[2 * (cf::NB_MAX + 1)];  // page-locked staging of the tables
@@ -814,11 +814,12 @@ int run(Request &q)
         }
         bbox_keys = bump.take<unsigned long long>(6);
         // one block, one memset, one copy back: [hist | diag(4) | err, counter | wsum | rsum]
-        d_hist = bump.take<unsigned long long>(nslots + 7 + nacc);
+        d_hist = bump.take<unsigned long long>(nslots + 8 + nacc);
         d_diag = d_hist + nslots;
         d_err = reinterpret_cast<unsigned *>(d_hist + nslots + 4);
         d_ctr = d_err + 1;
         d_wcount = d_err + 2;
+        d_bar = d_err + 6;
         d_thr = bump.take<float>(2 * (nb + 1));
         d_lut = bump.take<uint8_t>(cf::LUT_MAX);
         d_E2 = bump.take<double>(nb + 1);
@@ -838,7 +839,7 @@ int run(Request &q)
         if (dw[t])
             CF_CUDA(cudaMemcpyAsync((void *)dw[t], cats[t]->w, n * 8, cudaMemcpyHostToDevice, st), "H2D w");
     }
-    CF_CUDA(cudaMemsetAsync(d_hist, 0, sizeof(unsigned long long) * (nslots + 7 + nacc), st), "memset");
+    CF_CUDA(cudaMemsetAsync(d_hist, 0, sizeof(unsigned long long) * (nslots + 8 + nacc), st), "memset");
 
     ho = (HostOut *)g_pinned.get(sizeof(HostOut));
     if (!ho) {
@@ -892,15 +893,15 @@ int run(Request &q)
                 G[t].pos64 = bump.take<double4_32a>(n);
                 G[t].perm = bump.take<int>(n);
                 G[t].cell_start = bump.take<uint32_t>(g.ncells + 1);
-                G[t].colbox = bump.take<double4_32a>(g.ncols);
+                G[t].colbox = bump.take<cf::ColBox>(g.ncols);
             }
             tmp.cell_of = bump.take<uint32_t>(nmax);
             tmp.slot = bump.take<uint32_t>(nmax);
             tmp.tmp_idx = bump.take<int>(cf::padded_max(nmax, g.ncols));
             tmp.tmp_key = bump.take<unsigned long long>(cf::padded_max(nmax, g.ncols));
             tmp.counts = bump.take<uint32_t>(g.ncells + 1);
-            tmp.pad = bump.take<uint32_t>(g.ncols);
-            tmp.bsum = bump.take<uint32_t>(g.ncells / 4096 + 2);
+            tmp.coltot = bump.take<uint32_t>(g.ncols);
+            tmp.bsum = bump.take<uint32_t>(cf::grid_max_blocks(sms));
             const int sx = 2 * g.reach_x + 1, sy = 2 * g.reach_y + 1;
             const int nst = q.autocorr ? (sx * sy + 1) / 2 : sx * sy;
             nbr = bump.take<cf::Nbr>((size_t)g.ncols * nst);
@@ -915,7 +916,7 @@ int run(Request &q)
         }
         for (int t = 0; t < ncat; ++t) {
             const cudaError_t e = cf::build_grid(c->dtype, dx[t][0], dx[t][1], dx[t][2], dw[t],
-                                                 cats[t]->n, g, tmp, G[t], sms, d_err, st);
+                                                 cats[t]->n, g, tmp, G[t], sms, d_err, d_bar + t, st);
             if (e) {
                 rc = cuda_fail(e, "grid kernels");
                 goto cleanup;
@@ -959,7 +960,7 @@ int run(Request &q)
         P.want_r = c->want_ravg ? 1 : 0;
         P.wacc = wacc ? 1 : 0;
         P.rlo = resid ? 1 : 0;
-        P.wsum = wacc ? reinterpret_cast<double *>(d_hist + nslots + 7) : nullptr;
+        P.wsum = wacc ? reinterpret_cast<double *>(d_hist + nslots + 8) : nullptr;
         P.rsum = wacc ? P.wsum + nslots : nullptr;
         P.diag = d_diag;
         P.err = d_err;
@@ -986,7 +987,7 @@ int run(Request &q)
         }
         CF_CUDA(cudaEventRecord(g_events.ev[2], st), "cudaEventRecord");
         trace.point("pair kernel");
-        CF_CUDA(cudaMemcpyAsync(ho->hist, d_hist, sizeof(unsigned long long) * (nslots + 7 + nacc),
+        CF_CUDA(cudaMemcpyAsync(ho->hist, d_hist, sizeof(unsigned long long) * (nslots + 8 + nacc),
                                 cudaMemcpyDeviceToHost, st),
                 "D2H results");
     }
@@ -1021,7 +1022,7 @@ int run(Request &q)
         for (int k = 0; k < nslots; ++k)
             res->npairs[k] = ho->hist[k] * mult;
         if (wacc) {
-            const double *ws = reinterpret_cast<const double *>(ho->hist + nslots + 7);
+            const double *ws = reinterpret_cast<const double *>(ho->hist + nslots + 8);
             const double *rs = ws + nslots;
             for (int k = 0; k < nslots; ++k) {
                 const double wk = ws[k] * (double)mult, rk = rs[k] * (double)mult;
@@ -1040,7 +1041,7 @@ int run(Request &q)
         res->n_rechecked = ho->diag[2];
         res->n_band_violations = ho->diag[3];
         for (int t = 0; t < ncat; ++t)
-            res->n_kernels += cf::grid_kernels(cats[t]->n, G[t].res != nullptr) +
+            res->n_kernels += cf::grid_kernels() +
                               (c->periodic ? 0 : cf::bbox_kernels(cats[t]->n));
         res->n_kernels += PL.kernels;  // work list, window pre-pass, pair kernel
     }
@@ -1651,7 +1652,8 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     bump.base = (char *)scratch;
     unsigned long long *bbox_keys = bump.take<unsigned long long>(6);
     unsigned *d_err = bump.take<unsigned>(1);
-    unsigned *d_ctr = bump.take<unsigned>(3);  // [0] item counter, [1] kept column pairs, [2] window records
+    unsigned *d_ctr = bump.take<unsigned>(4);  // [0] item counter, [1] kept column pairs, [2, 3] gridding barriers
+    unsigned *d_bar = d_ctr + 2;
     unsigned long long *d_hist = bump.take<unsigned long long>(cf::NB_MAX);
     unsigned long long *d_diag = bump.take<unsigned long long>(4);
     float *d_thr = bump.take<float>(2 * (cf::NB_MAX + 1));
@@ -1745,15 +1747,15 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
             G[t].pos64 = b.take<double4_32a>(n);
             G[t].perm = b.take<int>(n);
             G[t].cell_start = b.take<uint32_t>(g.ncells + 1);
-            G[t].colbox = b.take<double4_32a>(g.ncols);
+            G[t].colbox = b.take<cf::ColBox>(g.ncols);
         }
         tmp.cell_of = b.take<uint32_t>(nmax);
         tmp.slot = b.take<uint32_t>(nmax);
         tmp.tmp_idx = b.take<int>(cf::padded_max(nmax, g.ncols));
         tmp.tmp_key = b.take<unsigned long long>(cf::padded_max(nmax, g.ncols));
         tmp.counts = b.take<uint32_t>(g.ncells + 1);
-        tmp.pad = b.take<uint32_t>(g.ncols);
-        tmp.bsum = b.take<uint32_t>(g.ncells / 4096 + 2);
+        tmp.coltot = b.take<uint32_t>(g.ncols);
+        tmp.bsum = b.take<uint32_t>(cf::grid_max_blocks(sms));
         nbr = b.take<cf::Nbr>((size_t)g.ncols * nstencil_max);
         nbr_count = b.take<unsigned>(g.ncols);
         if (b.off <= NOALLOC_BYTES) {
@@ -1775,13 +1777,13 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     g.inv_w[2] = g.nz / std::max(g.extent[2], 1e-300);
     finish_geom(g);
 
-    if ((e = cudaMemsetAsync(d_ctr, 0, 3 * sizeof(unsigned), st)) ||
+    if ((e = cudaMemsetAsync(d_ctr, 0, 4 * sizeof(unsigned), st)) ||
         (e = cudaMemsetAsync(d_hist, 0, sizeof(unsigned long long) * nb, st)) ||
         (e = cudaMemsetAsync(d_diag, 0, sizeof(unsigned long long) * 4, st)))
         return cuda_fail(e, "memset");
     for (int t = 0; t < ncat; ++t)
         if ((e = cf::build_grid(c->dtype, cats[t]->x, cats[t]->y, cats[t]->z, nullptr, cats[t]->n,
-                                g, tmp, G[t], sms, d_err, st)))
+                                g, tmp, G[t], sms, d_err, d_bar + t, st)))
             return cuda_fail(e, "grid kernels");
     if (autocorr)
         G[1] = G[0];
@@ -1870,7 +1872,7 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     res->n_evaluated = h.diag[1];
     res->n_rechecked = h.diag[2];
     for (int t = 0; t < ncat; ++t)
-        res->n_kernels += cf::grid_kernels(cats[t]->n) + (c->periodic ? 0 : cf::bbox_kernels(cats[t]->n));
+        res->n_kernels += cf::grid_kernels() + (c->periodic ? 0 : cf::bbox_kernels(cats[t]->n));
     res->n_kernels += PL.kernels;  // work list, window pre-pass, pair kernel
     return CF_OK;
 }
@@ -2148,6 +2150,7 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
     // concatenated per-cell arrays start at c0 (ncells + 1 each)
     std::vector<cf::GridSeg> seg;
     long long ctot = 0;
+    int cols = 0;
     for (int k = 0; k < nj; ++k) {
         const BatchJob &j = b->jobs[k];
         for (int t = 0; t < j.ncat; ++t) {
@@ -2160,6 +2163,8 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
             sg.job = k;
             sg.n = j.cat[t].n;
             sg.c0 = ctot;
+            sg.col0 = cols;
+            cols += j.g.ncols;
             ctot += j.g.ncells + 1;
             seg.push_back(sg);
         }
@@ -2206,7 +2211,7 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
                 G.pos64 = bump.take<double4_32a>(n);
                 G.perm = bump.take<int>(n);
                 G.cell_start = bump.take<uint32_t>(j.g.ncells + 1);
-                G.colbox = bump.take<double4_32a>(j.g.ncols);
+                G.colbox = bump.take<cf::ColBox>(j.g.ncols);
                 cf::GridSeg &sg = seg[q];
                 sg.out = G;
                 sg.cell_of = bump.take<uint32_t>(j.cat[t].n);

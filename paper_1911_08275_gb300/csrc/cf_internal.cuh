@@ -69,6 +69,12 @@ __host__ __device__ __forceinline__ size_t quad_off(uint32_t d)
     return (size_t)(d >> 2) * 12u + (d & 3u);
 }
 
+// Extent of a column's points in x and y, as order-preserving keys (order_key) of the
+// binary64 coordinates, so that it can be gathered with integer atomics; x1 = 0: empty.
+struct __align__(32) ColBox {
+    unsigned long long x0, x1, y0, y1;
+};
+
 // A gridded catalogue, in (column, z, original index) order, columns padded to
 // COL_PAD entries.
 struct Gridded {
@@ -83,20 +89,12 @@ struct Gridded {
     int *perm;            // original index of each sorted point
     int *chunk_col;       // column of each run of COL_PAD entries
     uint32_t *cell_start; // ncells + 1
-    double4_32a *colbox;      // per column (xmin, xmax, ymin, ymax)
-};
-
-// One kept column pair (Sec. 2.2 pruning done), written by the work-list kernel.
-struct __align__(16) WorkItem {
-    int a0, a1, b0, b1;  // point ranges of columns a and b
-    double dzmax;        // z reach of the pair (binary64, already widened)
-    int code;            // bits 0-1: qx + 1, bits 2-3: qy + 1 (periodic image), bit 4: self pair,
-                         // bits 5-31: column b
-    int wbase;           // first window record of the pair's chunks (window pre-pass), else 0
+    ColBox *colbox;       // per column
 };
 
 // A kept neighbour of a primary column: the column pair's z reach (float32,
-// rounded up, with the window slack) and its code (as WorkItem::code).
+// rounded up, with the window slack) and its code (bits 0-1: qx + 1, bits 2-3: qy + 1 of
+// the periodic image, bit 4: self pair, bits 5-31: the neighbour column).
 struct __align__(8) Nbr {
     float dz;
     int code;
@@ -167,6 +165,18 @@ struct PairParams {
 };
 
 // ----------------------------------------------------------------- device helpers
+// Order-preserving map of a binary64 bit pattern onto uint64 (and back).
+__device__ __forceinline__ unsigned long long order_key(long long b)
+{
+    const unsigned long long u = (unsigned long long)b;
+    return (b < 0) ? ~u : (u | 0x8000000000000000ull);
+}
+__device__ __forceinline__ double key_value(unsigned long long k)
+{
+    const unsigned long long b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
+    return __longlong_as_double((long long)b);
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));

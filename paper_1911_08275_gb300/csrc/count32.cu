@@ -10,6 +10,11 @@ namespace {
 
 __global__ void __launch_bounds__(128) k_neighbours(const __grid_constant__ PairParams P)
 {
+    if (*P.err & ERR_TIMEOUT) {  // the gridding gave up: leave the pair kernel no task
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            P.A.cell_start[P.g.ncells] = 0u;
+        return;
+    }
     neighbours_body(P, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), threadIdx.x & 31);
 }
 

@@ -28,35 +28,53 @@
 
 #include "cf_internal.cuh"
 #include "grid.cuh"
+#include "launch.cuh"
 
 namespace cf {
 
 namespace {
 
-// Order-preserving map of a binary64 bit pattern onto uint64 (and back).
-__device__ __forceinline__ unsigned long long order_key(long long b)
+// Binary64 -> float32, round to nearest even, and back, in integer arithmetic: the
+// conversion instructions run in the binary64 pipe, two lanes per SM (gridding
+// 1.2M points held it busy for half of the time).  Zeros are taken as they are;
+// values whose float32 is not a normal number take the instruction.
+__device__ __forceinline__ float d2f(double v)
 {
-    const unsigned long long u = (unsigned long long)b;
-    return (b < 0) ? ~u : (u | 0x8000000000000000ull);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+    if (e - 897u < 253u) {  // 2^-126 <= |v| < 2^127
+        const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
+        return __uint_as_float((((unsigned)(r >> 29) - (896u << 23)) & 0x7fffffffu) |
+                               ((unsigned)(b >> 32) & 0x80000000u));
+    }
+    if ((b << 1) == 0ull)
+        return __uint_as_float((unsigned)(b >> 32));
+    return __double2float_rn(v);
 }
-__device__ __forceinline__ double key_value(unsigned long long k)
+__device__ __forceinline__ double f2d(float v)
 {
-    const unsigned long long b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
-    return __longlong_as_double((long long)b);
+    const unsigned u = __float_as_uint(v);
+    if (((u >> 23) & 0xffu) - 1u < 254u)
+        return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))),
+                                (int)(u << 29));
+    if ((u << 1) == 0u)
+        return __hiloint2double((int)u, 0);
+    return (double)v;
 }
-
+__device__ __forceinline__ double to_f64(double v) { return v; }
+__device__ __forceinline__ double to_f64(float v) { return f2d(v); }
 
 // Validity and float32 frame coordinate of one input coordinate, without
-// binary64 arithmetic (the binary64 pipe of this GPU is narrow): range tests on
-// bit patterns, one conversion.
+// binary64 arithmetic in a periodic box (the binary64 pipe of this GPU is narrow):
+// range tests on bit patterns.
 __device__ __forceinline__ bool coord(double v, int a, const Geom &g, float &f)
 {
     const long long b = __double_as_longlong(v);
     if (g.periodic) {
-        f = __double2float_rn(v);  // frame origin is 0
+        f = d2f(v);  // frame origin is 0
         return (b >= 0 && b < g.box_bits[a]) || b == (long long)0x8000000000000000ull;
     }
-    f = __double2float_rn(__dsub_rn(v, g.origin[a]));
+    f = d2f(__dsub_rn(v, g.origin[a]));
     return (b & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
 }
 __device__ __forceinline__ bool coord(float v, int a, const Geom &g, float &f)
@@ -66,15 +84,29 @@ __device__ __forceinline__ bool coord(float v, int a, const Geom &g, float &f)
         f = v;
         return (b >= 0 && b < g.box_bits32[a]) || b == (int)0x80000000u;
     }
-    f = __double2float_rn(__dsub_rn((double)v, g.origin[a]));
+    f = d2f(__dsub_rn(f2d(v), g.origin[a]));
     return (b & 0x7f800000) != 0x7f800000;
 }
 
+// Sum over the block (every thread gets it; red: one word per warp).
+__device__ __forceinline__ uint32_t block_sum(uint32_t v, uint32_t *red)
+{
+    v = __reduce_add_sync(FULL, v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0)
+        red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    uint32_t s = 0;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q)
+        s += red[q];
+    return s;
+}
+
+// Cell and slot in the cell of every point (counts of the cells in count, zeroed).
 template <class T>
-__global__ void k_assign(const T *__restrict__ x, const T *__restrict__ y, const T *__restrict__ z,
-                         long long n, Geom g, uint32_t *__restrict__ cell_of,
-                         uint32_t *__restrict__ slot, uint32_t *__restrict__ count,
-                         unsigned *__restrict__ err)
+__device__ __forceinline__ void assign_points(const T *__restrict__ x, const T *__restrict__ y,
+                                              const T *__restrict__ z, long long n, const Geom &g,
+                                              uint32_t *cell_of, uint32_t *slot, uint32_t *count, unsigned *err)
 {
     const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -210,72 +242,42 @@ __global__ void k_scan_add(uint32_t *__restrict__ out, long long n, const uint32
         out[i] += bsum[i / SCAN_ITEMS];
 }
 
-// One warp per column: padding that rounds the column up to a multiple of COL_PAD,
-// written into the padded count of the column's last cell.
-__global__ void k_colpad(const uint32_t *__restrict__ count, int ncols, int nz,
-                         uint32_t *__restrict__ pad, uint32_t *__restrict__ padded)
-{
-    const int lane = threadIdx.x & 31;
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= ncols)
-        return;
-    const long long c0 = (long long)col * nz;
-    uint32_t tot = 0;
-    for (int z = lane; z < nz; z += 32) {
-        const uint32_t v = count[c0 + z];
-        padded[c0 + z] = v;
-        tot += v;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        tot += __shfl_xor_sync(FULL, tot, o);
-    const uint32_t pd = (COL_PAD - (tot & (COL_PAD - 1u))) & (COL_PAD - 1u);
-    __syncwarp();
-    if (lane == 0) {
-        pad[col] = pd;
-        padded[c0 + nz - 1] += pd;
-    }
-}
-
-template <class T>
-__global__ void k_scatter(const T *__restrict__ z, long long n, const uint32_t *__restrict__ cell_of,
-                          const uint32_t *__restrict__ slot, const uint32_t *__restrict__ start,
-                          int *__restrict__ tmp_idx, unsigned long long *__restrict__ tmp_key)
-{
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
-         p += (long long)gridDim.x * blockDim.x) {
-        const uint32_t q = start[cell_of[p]] + slot[p];
-        tmp_idx[q] = (int)p;
-        tmp_key[q] = order_key(__double_as_longlong((double)z[p]));
-    }
-}
-
-// Write one ranked entry: binary64 copy, float32 frame coordinates, weight,
-// original index.
+// Write one ranked entry: binary64 copy, float32 frame coordinates, their rounding
+// residuals fl32((X - O) - x~) if wanted, weight, original index.
 template <class T>
 __device__ __forceinline__ void put_entry(const T *__restrict__ x, const T *__restrict__ y,
                                           const double *__restrict__ w, const Geom &g, uint32_t d,
-                                          int iq, unsigned long long kq, float *__restrict__ xyz,
-                                          float *__restrict__ ws,
-                                          double4_32a *__restrict__ pos64, int *__restrict__ perm,
-                                          unsigned &wm)
+                                          int iq, unsigned long long kq, const Gridded &G, unsigned &wm,
+                                          ColBox &box)
 {
-    const double X = (double)x[iq], Y = (double)y[iq], Z = key_value(kq);
+    const double X = to_f64(x[iq]), Y = to_f64(y[iq]), Z = key_value(kq);
+    const unsigned long long kx = order_key(__double_as_longlong(X)), ky = order_key(__double_as_longlong(Y));
+    box.x0 = min(box.x0, kx);
+    box.x1 = max(box.x1, kx);
+    box.y0 = min(box.y0, ky);
+    box.y1 = max(box.y1, ky);
     const double W = w ? w[iq] : 0.0;
-    pos64[d] = make_double4_32a(X, Y, Z, W);
-    float fx, fy, fz;
-    coord(X, 0, g, fx);
-    coord(Y, 1, g, fy);
-    coord(Z, 2, g, fz);
-    float *qd = xyz + quad_off(d);
-    qd[0] = fx;
-    qd[4] = fy;
-    qd[8] = fz;
-    if (ws) {
-        ws[d] = (float)W;
-        wm = max(wm, __float_as_uint(fabsf((float)W)));
+    G.pos64[d] = make_double4_32a(X, Y, Z, W);
+    const double fx = g.periodic ? X : __dsub_rn(X, g.origin[0]);
+    const double fy = g.periodic ? Y : __dsub_rn(Y, g.origin[1]);
+    const double fz = g.periodic ? Z : __dsub_rn(Z, g.origin[2]);
+    const float sx = d2f(fx), sy = d2f(fy), sz = d2f(fz);
+    float *qd = G.xyz + quad_off(d);
+    qd[0] = sx;
+    qd[4] = sy;
+    qd[8] = sz;
+    if (G.res) {  // float32 mean separations restore the coordinates' lost bits
+        float *rd = G.res + quad_off(d);
+        rd[0] = d2f(__dsub_rn(fx, f2d(sx)));
+        rd[4] = d2f(__dsub_rn(fy, f2d(sy)));
+        rd[8] = d2f(__dsub_rn(fz, f2d(sz)));
     }
-    perm[d] = iq;
+    if (G.ws) {
+        const float wf = d2f(W);
+        G.ws[d] = wf;
+        wm = max(wm, __float_as_uint(fabsf(wf)));
+    }
+    G.perm[d] = iq;
 }
 
 constexpr int SORT_THREADS = 256;
@@ -293,92 +295,134 @@ __device__ __forceinline__ uint32_t rank_in(const ulonglong2 *e, uint32_t n, uns
     return rank;
 }
 
-// Rank the cells' real entries by (z, original index) and write the sorted
-// float32 / binary64 copies.  Each warp claims two cells at a time from a
-// counter (cell sizes vary, and a fixed split leaves a partial second wave of
-// blocks): cells of up to 16 entries are ranked by a half warp each; otherwise
-// the whole warp ranks the two cells one after the other, up to SORT_BUF
-// entries, beyond that against the cell in global memory.  The entries being ranked are copied to a
-// per-warp shared buffer as 16-byte (key, index) records: one broadcast load
-// per comparison.
-template <class T>
-__global__ void __launch_bounds__(SORT_THREADS)
-    k_sort_cells(const T *__restrict__ x, const T *__restrict__ y, const double *__restrict__ w,
-                 long long ncells, Geom g, const uint32_t *__restrict__ count,
-                 const uint32_t *__restrict__ start, const int *__restrict__ tmp_idx,
-                 const unsigned long long *__restrict__ tmp_key, float *__restrict__ xyz,
-                 float *__restrict__ ws, unsigned *__restrict__ wmax, double4_32a *__restrict__ pos64,
-                 int *__restrict__ perm, unsigned *__restrict__ claim)
+__device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
 {
-    __shared__ ulonglong2 s_ent[SORT_THREADS / 32][SORT_BUF];
-    const int lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15, wid = threadIdx.x >> 5;
-    ulonglong2 *be = s_ent[wid];
+    const unsigned hi = __reduce_min_sync(FULL, (unsigned)(v >> 32));
+    const unsigned lo = __reduce_min_sync(FULL, (unsigned)(v >> 32) == hi ? (unsigned)v : ~0u);
+    return ((unsigned long long)hi << 32) | lo;
+}
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) { return ~warp_min_u64(~v); }
+
+__device__ __forceinline__ ColBox empty_box() { return ColBox{~0ull, 0ull, ~0ull, 0ull}; }
+
+// Rank the real entries of a warp's cells by (z, original index) and write the
+// sorted outputs; lane l holds cell l of a run of consecutive cells (count n,
+// offset s, column col; n = 0 past the run's end).  Cells are ordered by z within a
+// column, so neighbouring cells of one column that hold at most 32 entries
+// together are ranked as one group, one entry per lane; a larger cell by itself,
+// from the warp's buffer up to SORT_BUF entries, beyond that in global memory.  The
+// entries being ranked are 16-byte (key, index) records: one broadcast load per
+// comparison.  at(l, col): the arrays of lane l's cell and the box of its column (all
+// lanes call it); put(src, d, iq, kq, box): write entry d.
+template <class At, class Put>
+__device__ __forceinline__ void sort_run(uint32_t n, uint32_t s, int col, int lane, ulonglong2 *be, At at,
+                                         Put put)
+{
+    uint32_t incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o)
+            incl += t;
+    }
+    for (unsigned todo = __ballot_sync(FULL, n > 0u); todo;) {
+        const int k = __ffs(todo) - 1;
+        const uint32_t before = __shfl_sync(FULL, incl - n, k), nk = __shfl_sync(FULL, n, k);
+        const uint32_t sk = __shfl_sync(FULL, s, k);
+        const int ck = __shfl_sync(FULL, col, k);
+        unsigned grp = __ballot_sync(FULL, n > 0u && lane >= k && col == ck && incl - before <= 32u);
+        if (nk > 32u)
+            grp = 1u << k;
+        const uint32_t cn = __shfl_sync(FULL, incl, 31 - __clz(grp)) - before;  // entries of the group
+        todo &= ~grp;
+        const auto src = at(k, ck);
+        ColBox box = empty_box();
+        const bool buffered = cn <= (uint32_t)SORT_BUF;
+        if (buffered) {
+            __syncwarp();
+            for (uint32_t e = lane; e < cn; e += 32)
+                be[e] = make_ulonglong2(src.key[sk + e], (unsigned long long)(unsigned)src.idx[sk + e]);
+            __syncwarp();
+        }
+        for (uint32_t e0 = 0; e0 < cn; e0 += 32) {
+            const uint32_t e = e0 + lane;
+            if (e < cn) {
+                unsigned long long kq;
+                int iq;
+                uint32_t rank = 0;
+                if (buffered) {
+                    kq = be[e].x;
+                    iq = (int)be[e].y;
+                    rank = rank_in(be, cn, kq, iq);
+                } else {
+                    kq = src.key[sk + e];
+                    iq = src.idx[sk + e];
+                    for (uint32_t m = 0; m < cn; ++m) {
+                        const unsigned long long km = src.key[sk + m];
+                        const int im = src.idx[sk + m];
+                        rank += (km < kq) || (km == kq && im < iq);
+                    }
+                }
+                put(src, sk + rank, iq, kq, box);
+            }
+        }
+        __syncwarp();
+        box.x0 = warp_min_u64(box.x0);
+        box.x1 = warp_max_u64(box.x1);
+        box.y0 = warp_min_u64(box.y0);
+        box.y1 = warp_max_u64(box.y1);
+        if (lane == 0) {
+            atomicMin(&src.box->x0, box.x0);
+            atomicMax(&src.box->x1, box.x1);
+            atomicMin(&src.box->y0, box.y0);
+            atomicMax(&src.box->y1, box.y1);
+        }
+    }
+}
+
+struct SortSrc {
+    const unsigned long long *key;
+    const int *idx;
+    ColBox *box;
+};
+struct SegSrc : SortSrc {
+    const GridSeg *seg;
+};
+
+// Cells of one claim: enough claims for four per warp, up to 32 cells.
+__device__ __forceinline__ unsigned claim_cells(long long ncells)
+{
+    const long long per = ncells / (4ll * gridDim.x * (SORT_THREADS / 32));
+    return per >= 32 ? 32u : per < 2 ? 2u : (unsigned)per;
+}
+
+template <class T>
+__device__ __forceinline__ void sort_cells(const T *__restrict__ x, const T *__restrict__ y,
+                                           const double *__restrict__ w, long long ncells, const Geom &g,
+                                           const uint32_t *count, const int *tmp_idx,
+                                           const unsigned long long *tmp_key, const Gridded &G, unsigned *claim,
+                                           ulonglong2 (*s_ent)[SORT_BUF])
+{
+    const uint32_t *start = G.cell_start;  // written earlier in the same launch: plain loads
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned per = claim_cells(ncells);
     unsigned wm = 0;  // bit pattern of the largest |w| (float) this thread stored
     for (;;) {
         unsigned v = 0u;
         if (lane == 0)
-            v = atomicAdd(claim, 1u);  // the next pair of cells (zeroed with the counts)
-        const long long c0 = 2ll * __shfl_sync(FULL, v, 0);
-        if (c0 >= ncells)
+            v = atomicAdd(claim, per);  // the next run of cells (zeroed with the counts)
+        const long long c = (long long)__shfl_sync(FULL, v, 0) + lane;
+        if (c - lane >= ncells)
             break;
-        const long long cm = c0 + half;  // this half warp's cell
-        const uint32_t cnt = cm < ncells ? count[cm] : 0u;
-        const uint32_t s = cm < ncells ? start[cm] : 0u;
-        const uint32_t cnt0 = __shfl_sync(FULL, cnt, 0), cnt1 = __shfl_sync(FULL, cnt, 16);
-        if (max(cnt0, cnt1) <= 16u) {
-            const bool mine = (uint32_t)hl < cnt;
-            const unsigned long long kq = mine ? tmp_key[s + hl] : ~0ull;  // absent: ranks last
-            const int iq = mine ? tmp_idx[s + hl] : 0x7fffffff;
-            __syncwarp();
-            be[lane] = make_ulonglong2(kq, (unsigned long long)(unsigned)iq);
-            __syncwarp();
-            const uint32_t rank = rank_in(be + half * 16, max(cnt0, cnt1), kq, iq);
-            if (mine)
-                put_entry(x, y, w, g, s + rank, iq, kq, xyz, ws, pos64, perm, wm);
-            continue;
-        }
-        for (int h = 0; h < 2; ++h) {  // whole warp, one cell after the other
-            const uint32_t cn = h ? cnt1 : cnt0;
-            const uint32_t sc = __shfl_sync(FULL, s, h * 16);
-            if (cn == 0)
-                continue;
-            const bool buffered = cn <= (uint32_t)SORT_BUF;
-            if (buffered) {
-                __syncwarp();
-                for (uint32_t e = lane; e < cn; e += 32)
-                    be[e] = make_ulonglong2(tmp_key[sc + e], (unsigned long long)(unsigned)tmp_idx[sc + e]);
-                __syncwarp();
-            }
-            for (uint32_t e0 = 0; e0 < cn; e0 += 32) {
-                const uint32_t e = e0 + lane;
-                const bool mine = e < cn;
-                unsigned long long kq = ~0ull;
-                int iq = 0x7fffffff;
-                if (mine) {
-                    if (buffered) {
-                        kq = be[e].x;
-                        iq = (int)be[e].y;
-                    } else {
-                        kq = tmp_key[sc + e];
-                        iq = tmp_idx[sc + e];
-                    }
-                }
-                uint32_t rank = 0;
-                if (buffered) {
-                    rank = rank_in(be, cn, kq, iq);
-                } else {
-                    for (uint32_t m = 0; m < cn; ++m) {
-                        const unsigned long long km = tmp_key[sc + m];
-                        const int im = tmp_idx[sc + m];
-                        rank += (km < kq) || (km == kq && im < iq);
-                    }
-                }
-                if (mine)
-                    put_entry(x, y, w, g, sc + rank, iq, kq, xyz, ws, pos64, perm, wm);
-            }
-        }
+        const bool mine = (unsigned)lane < per && c < ncells;
+        const uint32_t n = mine ? count[c] : 0u, s = mine ? start[c] : 0u;
+        sort_run(n, s, mine ? (int)c / g.nz : -1, lane, s_ent[wid],
+                 [&](int, int k) { return SortSrc{tmp_key, tmp_idx, G.colbox + k}; },
+                 [&](const SortSrc &, uint32_t d, int iq, unsigned long long kq, ColBox &box) {
+                     put_entry(x, y, w, g, d, iq, kq, G, wm, box);
+                 });
     }
-    if (wmax) {  // one atomic per block
+    if (G.ws) {  // one atomic per block
         __shared__ unsigned red[SORT_THREADS / 32];
         wm = __reduce_max_sync(FULL, wm);
         if (lane == 0)
@@ -388,7 +432,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
             unsigned m = 0;
             for (int q = 0; q < SORT_THREADS / 32; ++q)
                 m = max(m, red[q]);
-            atomicMax(wmax, m);
+            atomicMax(G.wmax, m);
         }
     }
 }
@@ -404,6 +448,10 @@ __device__ __forceinline__ void pad_column(const Gridded &G, int col, uint32_t s
         const uint32_t q = e - 1u - lane;
         float *qd = G.xyz + quad_off(q);
         qd[0] = qd[4] = qd[8] = fn;
+        if (G.res) {
+            float *rd = G.res + quad_off(q);
+            rd[0] = rd[4] = rd[8] = 0.0f;
+        }
         if (G.ws)
             G.ws[q] = 0.0f;
         G.pos64[q] = make_double4_32a(dn, dn, dn, dn);
@@ -413,72 +461,165 @@ __device__ __forceinline__ void pad_column(const Gridded &G, int col, uint32_t s
         G.chunk_col[k] = col;
 }
 
-__global__ void __launch_bounds__(256) k_padfill(const uint32_t *__restrict__ pad, int ncols, int nz,
-                                                 const __grid_constant__ Gridded G)
+// Everything one catalogue's gridding needs (kernel parameter).
+struct GridArgs {
+    const void *x, *y, *z;
+    const double *w;
+    long long n;
+    Geom g;
+    GridTemps t;
+    Gridded out;
+    unsigned *err, *bar;  // error word; arrivals at the grid barriers (zero before the launch)
+};
+
+// Barrier of the whole (cooperatively launched) grid: arrive, then wait until the
+// count reaches goal, at most 2 s.  False in every thread of the block if the wait
+// gave up (the error word says so; no later kernel touches the results).
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned goal, unsigned *err)
 {
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col < ncols)
-        pad_column(G, col, G.cell_start[(long long)col * nz], G.cell_start[(long long)(col + 1) * nz],
-                   pad[col], threadIdx.x & 31);
+    __syncthreads();
+    bool ok = true;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        const uint64_t t0 = global_ns();
+        for (unsigned it = 0;; ++it) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if (v >= goal)
+                break;
+            if ((it & 63u) == 63u && global_ns() - t0 > 2000000000ull) {
+                atomicOr(err, ERR_TIMEOUT);
+                ok = false;
+                break;
+            }
+        }
+        __threadfence();
+    }
+    return !__syncthreads_or(!ok);
 }
 
-// One block per column: (xmin, xmax, ymin, ymax) of its points, with min / max
-// taken on order-preserving integer keys (padding entries, NaN, are skipped).
-__global__ void __launch_bounds__(256) k_colbox(const double4_32a *__restrict__ pos64,
-                                                const uint32_t *__restrict__ start, int ncols,
-                                                int nz, double4_32a *__restrict__ colbox)
+// One catalogue's gridding in one cooperative launch; the stages are separated by
+// grid barriers:
+//   clear the cell counts | cell and slot of every point | padded size of every
+//   column, each block over a range of columns | offsets, padding, chunk_col |
+//   scatter into cells | rank the cells' entries, write the outputs and column boxes
+// Bound: latency (barriers of 1.5 us, dependent loads) for small catalogues, the
+// scattered reads of x and y by the ranked order for large ones.  Measured, with ten
+// kernels before, one per stage and with conversions in the binary64 pipe: 20,000
+// points 36 us of kernels and as much in gaps -> 18 us; 1.2M 113 -> 73 us; 12M
+// weighted with residuals 2.2 -> 1.5 ms (k_sort 1,137 -> 850 us by ranking small cells
+// together and claiming up to 32 at a time).
+template <class T>
+__global__ void __launch_bounds__(SORT_THREADS) k_grid(const __grid_constant__ GridArgs A)
 {
-    __shared__ unsigned long long red[4][8];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int col = blockIdx.x; col < ncols; col += gridDim.x) {
-        const uint32_t s = start[(long long)col * nz], e = start[(long long)(col + 1) * nz];
-        unsigned long long x0 = ~0ull, x1 = 0ull, y0 = ~0ull, y1 = 0ull;
-        for (uint32_t r = s + threadIdx.x; r < e; r += blockDim.x) {
-            const long long bx = __double_as_longlong(pos64[r].x);
-            const long long by = __double_as_longlong(pos64[r].y);
-            if ((bx & 0x7ff0000000000000ll) == 0x7ff0000000000000ll)
-                continue;  // padding
-            const unsigned long long kx = order_key(bx), ky = order_key(by);
-            x0 = min(x0, kx);
-            x1 = max(x1, kx);
-            y0 = min(y0, ky);
-            y1 = max(y1, ky);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            x0 = min(x0, __shfl_xor_sync(FULL, x0, o));
-            x1 = max(x1, __shfl_xor_sync(FULL, x1, o));
-            y0 = min(y0, __shfl_xor_sync(FULL, y0, o));
-            y1 = max(y1, __shfl_xor_sync(FULL, y1, o));
-        }
+    __shared__ ulonglong2 s_ent[SORT_THREADS / 32][SORT_BUF];
+    __shared__ uint32_t s_red[32], s_scan[32], s_tot;
+    __shared__ uint32_t s_off[SORT_THREADS];
+    const Geom &g = A.g;
+    const T *x = (const T *)A.x, *y = (const T *)A.y, *z = (const T *)A.z;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = SORT_THREADS / 32;
+    const unsigned nblk = gridDim.x, blk = blockIdx.x;
+    const long long nc = g.ncells, stride = (long long)nblk * SORT_THREADS, first = (long long)blk * SORT_THREADS + tid;
+    uint32_t *counts = A.t.counts, *start = A.out.cell_start;
+
+    for (long long q = first; q <= nc; q += stride)  // + the sort's claim counter
+        counts[q] = 0u;
+    for (long long q = first; q < g.ncols; q += stride)
+        A.out.colbox[q] = empty_box();
+    if (!grid_barrier(A.bar, nblk, A.err))
+        return;
+    assign_points<T>(x, y, z, A.n, g, A.t.cell_of, A.t.slot, counts, A.err);
+    if (!grid_barrier(A.bar, 2u * nblk, A.err))
+        return;
+
+    // this block's columns: a warp per column adds up its cells
+    const int c0 = (int)((long long)g.ncols * blk / nblk), c1 = (int)((long long)g.ncols * (blk + 1) / nblk);
+    uint32_t mine = 0;
+    for (int col = c0 + wid; col < c1; col += nwarp) {
+        uint32_t tot = 0;
+        for (int q = lane; q < g.nz; q += 32)
+            tot += counts[(long long)col * g.nz + q];
+        tot = __reduce_add_sync(FULL, tot);
         if (lane == 0) {
-            red[0][wid] = x0;
-            red[1][wid] = x1;
-            red[2][wid] = y0;
-            red[3][wid] = y1;
+            A.t.coltot[col] = tot;
+            mine += (tot + COL_PAD - 1u) & ~(COL_PAD - 1u);
         }
+    }
+    mine = block_sum(lane == 0 ? mine : 0u, s_red);
+    if (tid == 0)
+        A.t.bsum[blk] = mine;
+    if (!grid_barrier(A.bar, 3u * nblk, A.err))
+        return;
+
+    uint32_t base = 0;
+    for (unsigned q = tid; q < blk; q += SORT_THREADS)
+        base += __ldcg(A.t.bsum + q);
+    base = block_sum(base, s_red);
+    for (int r0 = c0; r0 < c1; r0 += SORT_THREADS) {
+        const int col = r0 + tid;
+        const uint32_t tot = col < c1 ? A.t.coltot[col] : 0u;
+        s_off[tid] = base + block_exclusive_scan((tot + COL_PAD - 1u) & ~(COL_PAD - 1u), s_scan, &s_tot);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int q = 1; q < (int)(blockDim.x >> 5); ++q) {
-                x0 = min(x0, red[0][q]);
-                x1 = max(x1, red[1][q]);
-                y0 = min(y0, red[2][q]);
-                y1 = max(y1, red[3][q]);
+        for (int k = wid; k < min(SORT_THREADS, c1 - r0); k += nwarp) {
+            uint32_t off = s_off[k];
+            const uint32_t s = off;
+            const long long cell = (long long)(r0 + k) * g.nz;
+            for (int q0 = 0; q0 < g.nz; q0 += 32) {
+                const uint32_t v = q0 + lane < g.nz ? counts[cell + q0 + lane] : 0u;
+                uint32_t incl = v;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o)
+                        incl += t;
+                }
+                if (q0 + lane < g.nz)
+                    start[cell + q0 + lane] = off + incl - v;
+                off += __shfl_sync(FULL, incl, 31);
             }
-            // empty column: keys keep their start values; mark the box empty
-            colbox[col] = x1 == 0ull ? make_double4_32a(DBL_MAX, -DBL_MAX, DBL_MAX, -DBL_MAX)
-                                     : make_double4_32a(key_value(x0), key_value(x1),
-                                                        key_value(y0), key_value(y1));
+            const uint32_t e = s + ((off - s + COL_PAD - 1u) & ~(COL_PAD - 1u));
+            pad_column(A.out, r0 + k, s, e, e - off, lane);
+            if (r0 + k == g.ncols - 1 && lane == 0)
+                start[nc] = e;
         }
+        base += s_tot;
         __syncthreads();
     }
+    if (!grid_barrier(A.bar, 4u * nblk, A.err))
+        return;
+
+    for (long long p = first; p < A.n; p += stride) {
+        const uint32_t q = start[A.t.cell_of[p]] + A.t.slot[p];
+        A.t.tmp_idx[q] = (int)p;
+        A.t.tmp_key[q] = order_key(__double_as_longlong(to_f64(z[p])));
+    }
+    if (!grid_barrier(A.bar, 5u * nblk, A.err))
+        return;
+    sort_cells<T>(x, y, A.w, nc, g, counts, A.t.tmp_idx, A.t.tmp_key, A.out, counts + nc, s_ent);
 }
 
-// Order-preserving map of a double onto uint64 (for atomic min / max).
-__device__ __forceinline__ unsigned long long dkey(double v)
+// Bounding box, on order-preserving integer keys (binary64 compares would hold the
+// narrow binary64 pipe).
+__device__ __forceinline__ uint32_t order_key32(int b)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+    return b < 0 ? ~(uint32_t)b : ((uint32_t)b | 0x80000000u);
+}
+__device__ __forceinline__ unsigned long long key_of(double v) { return order_key(__double_as_longlong(v)); }
+__device__ __forceinline__ uint32_t key_of(float v) { return order_key32(__float_as_int(v)); }
+__device__ __forceinline__ bool finite_bits(double v)
+{
+    return (__double_as_longlong(v) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool finite_bits(float v)
+{
+    return (__float_as_int(v) & 0x7f800000) != 0x7f800000;
+}
+__device__ __forceinline__ unsigned long long wide_key(unsigned long long k) { return k; }
+__device__ __forceinline__ unsigned long long wide_key(uint32_t k)
+{
+    const uint32_t b = (k >> 31) ? (k & 0x7fffffffu) : ~k;
+    return key_of(f2d(__uint_as_float(b)));
 }
 
 template <class T>
@@ -486,19 +627,21 @@ __global__ void k_bbox(const T *__restrict__ x, const T *__restrict__ y, const T
                        long long n, unsigned long long *__restrict__ out /* 6: min xyz, max xyz */,
                        unsigned *__restrict__ err)
 {
-    double lo[3] = {DBL_MAX, DBL_MAX, DBL_MAX}, hi[3] = {-DBL_MAX, -DBL_MAX, -DBL_MAX};
+    using K = decltype(key_of(T(0)));
+    K lo[3] = {~K(0), ~K(0), ~K(0)}, hi[3] = {K(0), K(0), K(0)};
     bool bad = false;
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
          p += (long long)gridDim.x * blockDim.x) {
-        const double v[3] = {(double)x[p], (double)y[p], (double)z[p]};
+        const T v[3] = {x[p], y[p], z[p]};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            if (!isfinite(v[a])) {
+            if (!finite_bits(v[a])) {
                 bad = true;
                 continue;
             }
-            lo[a] = fmin(lo[a], v[a]);
-            hi[a] = fmax(hi[a], v[a]);
+            const K k = key_of(v[a]);
+            lo[a] = min(lo[a], k);
+            hi[a] = max(hi[a], k);
         }
     }
     if (bad)
@@ -507,16 +650,17 @@ __global__ void k_bbox(const T *__restrict__ x, const T *__restrict__ y, const T
     for (int a = 0; a < 3; ++a) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            lo[a] = fmin(lo[a], __shfl_xor_sync(FULL, lo[a], o));
-            hi[a] = fmax(hi[a], __shfl_xor_sync(FULL, hi[a], o));
+            lo[a] = min(lo[a], (K)__shfl_xor_sync(FULL, lo[a], o));
+            hi[a] = max(hi[a], (K)__shfl_xor_sync(FULL, hi[a], o));
         }
     }
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            atomicMin(&out[a], dkey(lo[a]));
-            atomicMax(&out[3 + a], dkey(hi[a]));
-        }
+        for (int a = 0; a < 3; ++a)
+            if (lo[a] <= hi[a]) {
+                atomicMin(&out[a], wide_key(lo[a]));
+                atomicMax(&out[3 + a], wide_key(hi[a]));
+            }
     }
 }
 
@@ -527,32 +671,6 @@ inline int grid_blocks(long long n, int threads, int sms)
     if (b > cap)
         b = cap;
     return (int)(b < 1 ? 1 : b);
-}
-
-// Rounding residuals of the float32 frame coordinates, from the sorted binary64
-// copies: r = fl32((X - O) - x~) with (X - O) evaluated as the frame conversion
-// does (binary64; X itself in a periodic box, whose origin is 0).  The float32
-// mean separation uses them to restore the coordinates' lost bits.  Padding
-// entries get 0.
-__global__ void k_residual(const __grid_constant__ Gridded G, const __grid_constant__ Geom g)
-{
-    const long long n = G.cell_start[g.ncells];  // padded length of the gridded catalogue
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long d = (long long)blockIdx.x * blockDim.x + threadIdx.x; d < n; d += stride) {
-        const double4_32a p = G.pos64[d];
-        const float *q = G.xyz + quad_off((uint32_t)d);
-        float *r = G.res + quad_off((uint32_t)d);
-        if (isnan(p.x)) {
-            r[0] = r[4] = r[8] = 0.0f;
-            continue;
-        }
-        const double X = g.periodic ? p.x : __dsub_rn(p.x, g.origin[0]);
-        const double Y = g.periodic ? p.y : __dsub_rn(p.y, g.origin[1]);
-        const double Z = g.periodic ? p.z : __dsub_rn(p.z, g.origin[2]);
-        r[0] = __double2float_rn(__dsub_rn(X, (double)q[0]));
-        r[4] = __double2float_rn(__dsub_rn(Y, (double)q[4]));
-        r[8] = __double2float_rn(__dsub_rn(Z, (double)q[8]));
-    }
 }
 
 // ============================================================ batched gridding
@@ -642,7 +760,8 @@ __global__ void __launch_bounds__(256) kb_assign(const GridBatch B)
     }
 }
 
-// One warp per column (as k_colpad), into the concatenated padded counts; the
+// One warp per column: its cells' counts into the concatenated padded counts, the
+// padding that rounds the column up to a multiple of COL_PAD in its last cell; the
 // last column also zeroes the segment's extra entry.
 __global__ void __launch_bounds__(256) kb_colpad(const GridBatch B)
 {
@@ -669,6 +788,7 @@ __global__ void __launch_bounds__(256) kb_colpad(const GridBatch B)
     __syncwarp();
     if (lane == 0) {
         S.pad[col] = pd;
+        S.out.colbox[col] = empty_box();
         padded[c0 + nz - 1] += pd;
         if (col == ncols - 1)
             padded[g.ncells] = 0u;
@@ -693,104 +813,54 @@ __global__ void __launch_bounds__(256) kb_scatter(const GridBatch B)
     if (p >= S.n)
         return;
     const uint32_t q = S.out.cell_start[S.cell_of[p]] + S.slot[p];
-    const double zv = S.f32 ? (double)static_cast<const float *>(S.z)[p] : static_cast<const double *>(S.z)[p];
+    const double zv = S.f32 ? f2d(static_cast<const float *>(S.z)[p]) : static_cast<const double *>(S.z)[p];
     S.tmp_idx[q] = (int)p;
     S.tmp_key[q] = order_key(__double_as_longlong(zv));
 }
 
 __device__ __forceinline__ void put_seg(const GridBatch &B, const GridSeg &S, uint32_t d, int iq,
-                                        unsigned long long kq, unsigned &wm)
+                                        unsigned long long kq, unsigned &wm, ColBox &box)
 {
     const Geom &g = B.geom[S.job];
     if (S.f32)
-        put_entry(static_cast<const float *>(S.x), static_cast<const float *>(S.y), nullptr, g, d, iq,
-                  kq, S.out.xyz, nullptr, S.out.pos64, S.out.perm, wm);
+        put_entry(static_cast<const float *>(S.x), static_cast<const float *>(S.y), nullptr, g, d, iq, kq, S.out,
+                  wm, box);
     else
-        put_entry(static_cast<const double *>(S.x), static_cast<const double *>(S.y), nullptr, g, d,
-                  iq, kq, S.out.xyz, nullptr, S.out.pos64, S.out.perm, wm);
+        put_entry(static_cast<const double *>(S.x), static_cast<const double *>(S.y), nullptr, g, d, iq, kq,
+                  S.out, wm, box);
 }
 
-// k_sort_cells over the concatenated cells of every segment (the two cells of
-// a claim may belong to different segments; a segment's extra entry has no
-// points).
+// sort_cells over the concatenated cells of every segment (the cells of a claim may
+// belong to different segments; a segment's extra entry has no points).
 __global__ void __launch_bounds__(SORT_THREADS) kb_sort_cells(const GridBatch B)
 {
     __shared__ ulonglong2 s_ent[SORT_THREADS / 32][SORT_BUF];
-    const int lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15, wid = threadIdx.x >> 5;
-    ulonglong2 *be = s_ent[wid];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned per = claim_cells(B.ctot);
     unsigned wm = 0;
     for (;;) {
         unsigned v = 0u;
         if (lane == 0)
-            v = atomicAdd(B.counts + B.ctot, 1u);  // the next pair of entries (zeroed with the counts)
-        const long long c0 = 2ll * __shfl_sync(FULL, v, 0);
-        if (c0 >= B.ctot)
+            v = atomicAdd(B.counts + B.ctot, per);  // the next run of entries (zeroed with the counts)
+        const long long c = (long long)__shfl_sync(FULL, v, 0) + lane;
+        if (c - lane >= B.ctot)
             break;
-        const long long cm = c0 + half;  // this half warp's entry
-        int sg = 0;
-        uint32_t cnt = 0u, s0 = 0u;
-        if (cm < B.ctot) {
-            sg = seg_of_entry(B, cm);
-            cnt = B.counts[cm];
-            if (cnt)
-                s0 = B.seg[sg].out.cell_start[cm - B.seg[sg].c0];
+        int sg = 0, col = -1;
+        uint32_t n = 0u, s = 0u;
+        if ((unsigned)lane < per && c < B.ctot && (n = B.counts[c]) != 0u) {
+            sg = seg_of_entry(B, c);
+            const long long cell = c - B.seg[sg].c0;
+            s = B.seg[sg].out.cell_start[cell];
+            col = B.seg[sg].col0 + (int)cell / B.geom[B.seg[sg].job].nz;
         }
-        const uint32_t cnt0 = __shfl_sync(FULL, cnt, 0), cnt1 = __shfl_sync(FULL, cnt, 16);
-        if (max(cnt0, cnt1) <= 16u) {
-            const GridSeg &S = B.seg[sg];
-            const bool mine = (uint32_t)hl < cnt;
-            const unsigned long long kq = mine ? S.tmp_key[s0 + hl] : ~0ull;
-            const int iq = mine ? S.tmp_idx[s0 + hl] : 0x7fffffff;
-            __syncwarp();
-            be[lane] = make_ulonglong2(kq, (unsigned long long)(unsigned)iq);
-            __syncwarp();
-            const uint32_t rank = rank_in(be + half * 16, max(cnt0, cnt1), kq, iq);
-            if (mine)
-                put_seg(B, S, s0 + rank, iq, kq, wm);
-            continue;
-        }
-        for (int h = 0; h < 2; ++h) {  // whole warp, one cell after the other
-            const uint32_t cn = h ? cnt1 : cnt0;
-            const uint32_t sc = __shfl_sync(FULL, s0, h * 16);
-            const int sh = __shfl_sync(FULL, sg, h * 16);
-            if (cn == 0)
-                continue;
-            const GridSeg &S = B.seg[sh];
-            const bool buffered = cn <= (uint32_t)SORT_BUF;
-            if (buffered) {
-                __syncwarp();
-                for (uint32_t e = lane; e < cn; e += 32)
-                    be[e] = make_ulonglong2(S.tmp_key[sc + e], (unsigned long long)(unsigned)S.tmp_idx[sc + e]);
-                __syncwarp();
-            }
-            for (uint32_t e0 = 0; e0 < cn; e0 += 32) {
-                const uint32_t e = e0 + lane;
-                const bool mine = e < cn;
-                unsigned long long kq = ~0ull;
-                int iq = 0x7fffffff;
-                if (mine) {
-                    if (buffered) {
-                        kq = be[e].x;
-                        iq = (int)be[e].y;
-                    } else {
-                        kq = S.tmp_key[sc + e];
-                        iq = S.tmp_idx[sc + e];
-                    }
-                }
-                uint32_t rank = 0;
-                if (buffered) {
-                    rank = rank_in(be, cn, kq, iq);
-                } else {
-                    for (uint32_t m = 0; m < cn; ++m) {
-                        const unsigned long long km = S.tmp_key[sc + m];
-                        const int im = S.tmp_idx[sc + m];
-                        rank += (km < kq) || (km == kq && im < iq);
-                    }
-                }
-                if (mine)
-                    put_seg(B, S, sc + rank, iq, kq, wm);
-            }
-        }
+        sort_run(n, s, col, lane, s_ent[wid],
+                 [&](int k, int ck) {
+                     const GridSeg *S = B.seg + __shfl_sync(FULL, sg, k);
+                     return SegSrc{{S->tmp_key, S->tmp_idx, S->out.colbox + (ck - S->col0)}, S};
+                 },
+                 [&](const SegSrc &src, uint32_t d, int iq, unsigned long long kq, ColBox &box) {
+                     put_seg(B, *src.seg, d, iq, kq, wm, box);
+                 });
     }
 }
 
@@ -805,91 +875,24 @@ __global__ void __launch_bounds__(256) kb_padfill(const GridBatch B)
                    S.out.cell_start[(long long)(col + 1) * g.nz], S.pad[col], threadIdx.x & 31);
 }
 
-// One block per column (as k_colbox).
-__global__ void __launch_bounds__(256) kb_colbox(const GridBatch B)
-{
-    __shared__ unsigned long long red[4][8];
-    const int s = block_seg(B.pre[GB_COLBLK], B.nseg);
-    const GridSeg &S = B.seg[s];
-    const int nz = B.geom[S.job].nz;
-    const int col = (int)(blockIdx.x - B.pre[GB_COLBLK][s]);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t st = S.out.cell_start[(long long)col * nz], en = S.out.cell_start[(long long)(col + 1) * nz];
-    unsigned long long x0 = ~0ull, x1 = 0ull, y0 = ~0ull, y1 = 0ull;
-    for (uint32_t r = st + threadIdx.x; r < en; r += blockDim.x) {
-        const long long bx = __double_as_longlong(S.out.pos64[r].x);
-        const long long by = __double_as_longlong(S.out.pos64[r].y);
-        if ((bx & 0x7ff0000000000000ll) == 0x7ff0000000000000ll)
-            continue;  // padding
-        const unsigned long long kx = order_key(bx), ky = order_key(by);
-        x0 = min(x0, kx);
-        x1 = max(x1, kx);
-        y0 = min(y0, ky);
-        y1 = max(y1, ky);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        x0 = min(x0, __shfl_xor_sync(FULL, x0, o));
-        x1 = max(x1, __shfl_xor_sync(FULL, x1, o));
-        y0 = min(y0, __shfl_xor_sync(FULL, y0, o));
-        y1 = max(y1, __shfl_xor_sync(FULL, y1, o));
-    }
-    if (lane == 0) {
-        red[0][wid] = x0;
-        red[1][wid] = x1;
-        red[2][wid] = y0;
-        red[3][wid] = y1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int q = 1; q < (int)(blockDim.x >> 5); ++q) {
-            x0 = min(x0, red[0][q]);
-            x1 = max(x1, red[1][q]);
-            y0 = min(y0, red[2][q]);
-            y1 = max(y1, red[3][q]);
-        }
-        S.out.colbox[col] = x1 == 0ull ? make_double4_32a(DBL_MAX, -DBL_MAX, DBL_MAX, -DBL_MAX)
-                                       : make_double4_32a(key_value(x0), key_value(x1),
-                                                          key_value(y0), key_value(y1));
-    }
-}
-
 template <class T>
-cudaError_t build_grid_t(const void *x, const void *y, const void *z, const double *w, long long n,
-                         const Geom &g, const GridTemps &t, Gridded &out, int sms, unsigned *err,
-                         cudaStream_t st)
+cudaError_t build_grid_t(GridArgs &A, int sms, cudaStream_t st)
 {
-    cudaError_t e;
-    const long long nc = g.ncells;
-    if ((e = cudaMemsetAsync(t.counts, 0, sizeof(uint32_t) * (nc + 1), st)))  // + the sort's claim counter
+    int occ = 0;
+    const cudaError_t e = occupancy(k_grid<T>, 0, occ);
+    if (e)
         return e;
-    const int TB = 256;
-    if (n > 0) {
-        k_assign<T><<<grid_blocks(n, TB, sms), TB, 0, st>>>((const T *)x, (const T *)y,
-                                                            (const T *)z, n, g, t.cell_of, t.slot,
-                                                            t.counts, err);
-    }
-    const int cb = (g.ncols * 32 + 255) / 256;
-    k_colpad<<<cb, 256, 0, st>>>(t.counts, g.ncols, g.nz, t.pad, out.cell_start);
-    const int nb = (int)((nc + SCAN_ITEMS - 1) / SCAN_ITEMS);
-    k_scan_blocks<<<nb, SCAN_THREADS, 0, st>>>(out.cell_start, out.cell_start, nc, t.bsum);
-    k_scan_sums<<<1, SCAN_THREADS, 0, st>>>(t.bsum, (long long)nb, out.cell_start + nc);
-    k_scan_add<<<(int)((nc + 255) / 256), 256, 0, st>>>(out.cell_start, nc, t.bsum);
-    if (n > 0) {
-        k_scatter<T><<<grid_blocks(n, TB, sms), TB, 0, st>>>((const T *)z, n, t.cell_of, t.slot,
-                                                             out.cell_start, t.tmp_idx, t.tmp_key);
-        const long long cwarps = std::min<long long>((nc + 1) / 2, (long long)sms * 64);
-        k_sort_cells<T><<<(int)((cwarps * 32 + SORT_THREADS - 1) / SORT_THREADS), SORT_THREADS, 0, st>>>(
-            (const T *)x, (const T *)y, w, nc, g, t.counts, out.cell_start, t.tmp_idx, t.tmp_key,
-            out.xyz, out.ws, out.ws ? out.wmax : nullptr, out.pos64, out.perm,
-            t.counts + nc);
-    }
-    k_padfill<<<cb, 256, 0, st>>>(t.pad, g.ncols, g.nz, out);
-    k_colbox<<<std::min(g.ncols, sms * 8), 256, 0, st>>>(out.pos64, out.cell_start, g.ncols, g.nz,
-                                                          out.colbox);
-    if (out.res)
-        k_residual<<<grid_blocks(padded_max(n, g.ncols), TB, sms), TB, 0, st>>>(out, g);
-    return cudaGetLastError();
+    if (occ < 1)
+        return cudaErrorInvalidConfiguration;
+    // a thread per point or cell, a warp per column; all blocks resident, as the barriers
+    // need
+    const long long work = std::max(A.n, std::max(A.g.ncells, 32ll * A.g.ncols));
+    long long blocks = std::min<long long>((long long)sms * occ, (work + SORT_THREADS - 1) / SORT_THREADS);
+    if (blocks < 1)
+        blocks = 1;
+    void *args[] = {&A};
+    return cudaLaunchCooperativeKernel((const void *)k_grid<T>, dim3((unsigned)blocks), dim3(SORT_THREADS), args, 0,
+                                       st);
 }
 
 template <class T>
@@ -907,12 +910,14 @@ cudaError_t bbox_t(const void *x, const void *y, const void *z, long long n,
 
 cudaError_t build_grid(cf_dtype dt, const void *x, const void *y, const void *z, const double *w,
                        long long n, const Geom &g, const GridTemps &t, Gridded &out, int sms,
-                       unsigned *err, cudaStream_t st)
+                       unsigned *err, unsigned *bar, cudaStream_t st)
 {
     out.n = n;
-    return dt == CF_FLOAT32 ? build_grid_t<float>(x, y, z, w, n, g, t, out, sms, err, st)
-                            : build_grid_t<double>(x, y, z, w, n, g, t, out, sms, err, st);
+    GridArgs A{x, y, z, w, n, g, t, out, err, bar};
+    return dt == CF_FLOAT32 ? build_grid_t<float>(A, sms, st) : build_grid_t<double>(A, sms, st);
 }
+
+int grid_max_blocks(int sms) { return sms * 8; }  // 2,048 threads per SM
 
 cudaError_t launch_bbox(cf_dtype dt, const void *x, const void *y, const void *z, long long n,
                         unsigned long long *out6, int sms, unsigned *err, cudaStream_t st)
@@ -933,8 +938,6 @@ unsigned grid_batch_blocks(int k, long long n, const Geom &g)
         return (unsigned)((n + 255) / 256);
     case GB_COLWARPS:
         return (unsigned)((g.ncols + 7) / 8);
-    case GB_COLBLK:
-        return (unsigned)g.ncols;
     default:
         return (unsigned)((g.ncells + 1 + 255) / 256);
     }
@@ -961,7 +964,6 @@ cudaError_t build_grid_batch(const GridBatch &B, int sms, cudaStream_t st)
         kb_sort_cells<<<(unsigned)((cwarps * 32 + SORT_THREADS - 1) / SORT_THREADS), SORT_THREADS, 0, st>>>(B);
     }
     kb_padfill<<<B.blocks[GB_COLWARPS], 256, 0, st>>>(B);
-    kb_colbox<<<B.blocks[GB_COLBLK], 256, 0, st>>>(B);
     return cudaGetLastError();
 }
 

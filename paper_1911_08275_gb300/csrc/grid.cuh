@@ -14,14 +14,18 @@ struct GridTemps {
     int *tmp_idx;        // padded_max(n, ncols)
     unsigned long long *tmp_key;  // padded_max(n, ncols): order-preserving keys of z
     uint32_t *counts;    // ncells + 1 (the last: the in-cell sort's claim counter)
-    uint32_t *pad;       // ncols
-    uint32_t *bsum;      // ceil(ncells / 4096)
+    uint32_t *coltot;    // ncols: points per column
+    uint32_t *bsum;      // grid_max_blocks: padded entries of each block's columns
 };
 
-// Grid one catalogue into `out` (whose arrays are preallocated).
+// Blocks of one gridding launch, at most.
+int grid_max_blocks(int sms);
+
+// Grid one catalogue into `out` (whose arrays are preallocated): one cooperative
+// launch.  *bar must be zero (arrivals at the launch's grid barriers).
 cudaError_t build_grid(cf_dtype dt, const void *x, const void *y, const void *z, const double *w,
                        long long n, const Geom &g, const GridTemps &t, Gridded &out, int sms,
-                       unsigned *err, cudaStream_t st);
+                       unsigned *err, unsigned *bar, cudaStream_t st);
 
 // Bounding box of a catalogue: out6 = order-preserving keys of (min x,y,z, max x,y,z);
 // initialise out6[0..2] to ~0 and out6[3..5] to 0 first.
@@ -44,6 +48,7 @@ struct GridSeg {
     int *tmp_idx;                  // padded_max(n, ncols)
     unsigned long long *tmp_key;   // padded_max(n, ncols)
     uint32_t *pad;                 // ncols
+    int col0;                      // columns of the segments before this one
     unsigned *err;                 // the job's error word
 };
 
@@ -52,7 +57,6 @@ struct GridSeg {
 enum GridBatchShape {
     GB_POINTS,    // 256 points per block
     GB_COLWARPS,  // 8 columns per block (one warp each)
-    GB_COLBLK,    // one column per block
     GB_CELLS,     // 256 entries of cell_start per block
     GB_SHAPES
 };
@@ -79,13 +83,10 @@ unsigned grid_batch_blocks(int k, long long n, const Geom &g);
 cudaError_t build_grid_batch(const GridBatch &B, int sms, cudaStream_t st);
 
 // Kernel launches (and memsets) of one build_grid_batch.
-inline int grid_batch_kernels() { return 11; }
+inline int grid_batch_kernels() { return 10; }
 
 // Kernels launched by build_grid / launch_bbox for a catalogue of n points.
-inline int grid_kernels(long long n, bool residuals = false)
-{
-    return (n > 0 ? 9 : 6) + (residuals ? 1 : 0);
-}
+inline int grid_kernels() { return 1; }
 inline int bbox_kernels(long long n) { return n > 0 ? 1 : 0; }
 
 }  // namespace cf

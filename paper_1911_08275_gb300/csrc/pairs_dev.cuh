@@ -232,8 +232,8 @@ __device__ __forceinline__ uint32_t push_sign(uint32_t m, uint32_t v)
 }
 
 // Candidate (column a, stencil offset) -> column pair, image, pruning
-// (Sec. 2.2) and z reach, in binary64.  Returns false if the pair has no work.
-__device__ __forceinline__ bool plan_item(const PairParams &P, int item, WorkItem &w)
+// (Sec. 2.2) in binary64 and z reach.  Returns false if the pair has no work.
+__device__ __forceinline__ bool plan_item(const PairParams &P, int item, Nbr &w)
 {
     const int a = item / P.nstencil, s = item - a * P.nstencil;
     const int2 o = P.stencil[s];
@@ -252,7 +252,6 @@ __device__ __forceinline__ bool plan_item(const PairParams &P, int item, WorkIte
     } else if (bx < 0 || bx >= P.g.ncx || by < 0 || by >= P.g.ncy) {
         return false;
     }
-    const double Sx = qx * P.g.box[0], Sy = qy * P.g.box[1];
     const int b = bx * P.g.ncy + by;
     const long long nz = P.g.nz;
     if (P.shard_n > 1) {  // deterministic split of the primary columns over shards
@@ -263,29 +262,35 @@ __device__ __forceinline__ bool plan_item(const PairParams &P, int item, WorkIte
         if (first < lo || first >= hi)
             return false;
     }
-    w.a0 = (int)P.A.cell_start[a * nz];
-    w.a1 = (int)P.A.cell_start[(a + 1) * nz];
-    w.b0 = (int)P.B.cell_start[b * nz];
-    w.b1 = (int)P.B.cell_start[(b + 1) * nz];
-    if (w.a0 >= w.a1 || w.b0 >= w.b1)
+    if (P.A.cell_start[a * nz] >= P.A.cell_start[(a + 1) * nz] || P.B.cell_start[b * nz] >= P.B.cell_start[(b + 1) * nz])
         return false;
-    // minimum possible (x, y) separation of the two columns' bounding boxes
-    const double4_32a ba = P.A.colbox[a], bb = P.B.colbox[b];
-    const double gx = fmax(0.0, fmax(__dsub_rn(__dadd_rn(bb.x, Sx), ba.y),
-                                     __dsub_rn(ba.x, __dadd_rn(bb.y, Sx))));
-    const double gy = fmax(0.0, fmax(__dsub_rn(__dadd_rn(bb.z, Sy), ba.w),
-                                     __dsub_rn(ba.z, __dadd_rn(bb.w, Sy))));
+    // minimum possible (x, y) separation of the two columns' bounding boxes; signs and
+    // compares on the bits (the binary64 pipe is narrow)
+    const ColBox ba = P.A.colbox[a], bb = P.B.colbox[b];
+    auto gap = [](double a0, double a1, double b0, double b1, int q, double box) {
+        if (q) {
+            const double S = q > 0 ? box : -box;
+            b0 = __dadd_rn(b0, S);
+            b1 = __dadd_rn(b1, S);
+        }
+        const double up = __dsub_rn(b0, a1), dn = __dsub_rn(a0, b1);
+        return __double_as_longlong(up) > 0 ? up : __double_as_longlong(dn) > 0 ? dn : 0.0;
+    };
+    const double gx = gap(key_value(ba.x0), key_value(ba.x1), key_value(bb.x0), key_value(bb.x1), qx, P.g.box[0]);
+    const double gy = gap(key_value(ba.y0), key_value(ba.y1), key_value(bb.y0), key_value(bb.y1), qy, P.g.box[1]);
     const double g2 = __dadd_rn(__dmul_rn(gx, gx), __dmul_rn(gy, gy));
-    if (!(P.flags & CF_FLAG_NO_PRUNE) && g2 >= P.prune_r2)
+    if (!(P.flags & CF_FLAG_NO_PRUNE) && __double_as_longlong(g2) >= __double_as_longlong(P.prune_r2))
         return false;
-    // z reach: dz_max,all of Sec. 2.2 (xi); pimax (rp-pi)
-    double dzmax = P.rz;
-    if (P.kind == 0)
-        dzmax = sqrt(fmax(0.0, __dsub_rn(P.rxy2, __dmul_rn(g2, 1.0 - 1e-12))));
-    w.dzmax = __dmul_rn(dzmax, 1.0 + 1e-9);
+    // z reach, rounded up: dz_max,all of Sec. 2.2 (xi); pimax (rp-pi)
+    if (P.kind == 0) {
+        const double t = __dsub_rn(P.rxy2, __dmul_rn(g2, 1.0 - 1e-12));
+        w.dz = __double_as_longlong(t) > 0 ? __fmul_ru(__fsqrt_ru(__double2float_ru(t)), 1.0f + 0x1p-22f) : 0.0f;
+    } else {
+        w.dz = __double2float_ru(P.rz);
+    }
+    w.dz = __fadd_ru(w.dz, P.zslack);
     const bool self = P.autocorr && o.x == 0 && o.y == 0;
     w.code = (qx + 1) | ((qy + 1) << 2) | (self ? 16 : 0) | (b << 5);
-    w.wbase = 0;
     return true;
 }
 

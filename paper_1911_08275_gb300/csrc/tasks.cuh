@@ -383,15 +383,11 @@ __device__ __forceinline__ void neighbours_body(const PairParams &P, int col, in
     int n = 0;
     for (int s0 = 0; s0 < P.nstencil; s0 += 32) {
         const int s = s0 + lane;
-        WorkItem w;
-        const bool keep = s < P.nstencil && plan_item(P, col * P.nstencil + s, w);
+        Nbr r;
+        const bool keep = s < P.nstencil && plan_item(P, col * P.nstencil + s, r);
         const unsigned m = __ballot_sync(FULL, keep);
-        if (keep) {
-            Nbr r;
-            r.dz = __fadd_ru(__double2float_ru(w.dzmax), P.zslack);
-            r.code = w.code;
+        if (keep)
             P.nbr[(long long)col * P.nstencil + n + __popc(m & ((1u << lane) - 1u))] = r;
-        }
         n += __popc(m);
     }
     if (lane == 0) {
