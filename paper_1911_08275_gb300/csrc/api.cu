@@ -749,8 +749,6 @@ int run(Request &q)
     cf::PairLaunch PL = {};
     std::vector<double> E2(nb + 1);
     std::vector<double> Pe(q.kind == 1 ? q.npibins + 1 : 0);
-    float T[2 * (cf::NB_MAX + 1)];
-    uint8_t tab[cf::LUT_MAX];
     cf::Gridded G[2] = {};
     cf::GridTemps tmp = {};
     Bump bump;
@@ -759,7 +757,10 @@ int run(Request &q)
     bool host_in[2] = {false, false};
     long long nmax = 0, ntot = 0;
     double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
-    unsigned long long *bbox_keys = nullptr;
+    struct {
+        unsigned long long *keys;
+    } stage = {nullptr};
+    bool resid = false;
     unsigned *d_err = nullptr, *d_ctr = nullptr, *d_wcount = nullptr, *d_bar = nullptr;
     cf::Nbr *nbr = nullptr;
     unsigned *nbr_count = nullptr;
@@ -767,15 +768,13 @@ int run(Request &q)
     float *d_thr = nullptr;
     uint8_t *d_lut = nullptr;
     double *d_E2 = nullptr, *d_P = nullptr;
-    size_t total = 0;
-    struct HostOut {
-        unsigned long long hist[3 * cf::NBINS2D_MAX + 8];  // hist | diag(4) | err, counter | kept | max |w| (2) | barriers (2) | wsum | rsum
+    struct HostOut {  // page-locked
+        unsigned long long hist[3 * cf::NBINS2D_MAX + 16];  // results read back
         unsigned long long *diag;
         unsigned err;
-        float thr[2 * (cf::NB_MAX + 1)];  // page-locked staging of the tables
-        double e2[cf::NB_MAX + 1];
-        double pe[cf::NPI_MAX + 1];
-        uint8_t lut[cf::LUT_MAX];
+        // image of the staged block (at most: keys, results, both edge arrays, thresholds, table)
+        alignas(16) unsigned long long stage[6 + 3 * cf::NBINS2D_MAX + 8 + 2 * (cf::NB_MAX + 1) + cf::NPI_MAX + 1 +
+                                             cf::LUT_MAX / 8 + 2];
     } *ho = nullptr;
 
     CF_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
@@ -795,101 +794,45 @@ int run(Request &q)
         E2[k] = q.edges[k] * q.edges[k];
     pi_edges(q, Pe);
 
-    // Pass 1: sizes of everything except the grid (known only after the bbox).
-    for (int pass = 0; pass < 2; ++pass) {
-        bump.base = pass ? (char *)ws : nullptr;
-        bump.off = 0;
-        for (int t = 0; t < ncat; ++t) {
-            const long long n = cats[t]->n;
-            if (host_in[t]) {
-                for (int a = 0; a < 3; ++a)
-                    dx[t][a] = bump.take<char>(n * esz);
-                dw[t] = cats[t]->w ? bump.take<double>(n) : nullptr;
-            } else {
-                dx[t][0] = cats[t]->x;
-                dx[t][1] = cats[t]->y;
-                dx[t][2] = cats[t]->z;
-                dw[t] = cats[t]->w;
-            }
-        }
-        bbox_keys = bump.take<unsigned long long>(6);
-        // one block, one memset, one copy back: [hist | diag(4) | err, counter | wsum | rsum]
-        d_hist = bump.take<unsigned long long>(nslots + 8 + nacc);
-        d_diag = d_hist + nslots;
-        d_err = reinterpret_cast<unsigned *>(d_hist + nslots + 4);
-        d_ctr = d_err + 1;
-        d_wcount = d_err + 2;
-        d_bar = d_err + 6;
-        d_thr = bump.take<float>(2 * (nb + 1));
-        d_lut = bump.take<uint8_t>(cf::LUT_MAX);
-        d_E2 = bump.take<double>(nb + 1);
-        d_P = bump.take<double>(Pe.size());
-        if (pass == 0) {
-            total = bump.off;
-            CF_CUDA(cudaMallocAsync(&ws, total, st), "cudaMallocAsync (inputs)");
-        }
-    }
-    for (int t = 0; t < ncat; ++t) {
-        if (!host_in[t])
-            continue;
-        const long long n = cats[t]->n;
-        CF_CUDA(cudaMemcpyAsync((void *)dx[t][0], cats[t]->x, n * esz, cudaMemcpyHostToDevice, st), "H2D x");
-        CF_CUDA(cudaMemcpyAsync((void *)dx[t][1], cats[t]->y, n * esz, cudaMemcpyHostToDevice, st), "H2D y");
-        CF_CUDA(cudaMemcpyAsync((void *)dx[t][2], cats[t]->z, n * esz, cudaMemcpyHostToDevice, st), "H2D z");
-        if (dw[t])
-            CF_CUDA(cudaMemcpyAsync((void *)dw[t], cats[t]->w, n * 8, cudaMemcpyHostToDevice, st), "H2D w");
-    }
-    CF_CUDA(cudaMemsetAsync(d_hist, 0, sizeof(unsigned long long) * (nslots + 8 + nacc), st), "memset");
-
     ho = (HostOut *)g_pinned.get(sizeof(HostOut));
     if (!ho) {
         rc = fail(CF_ENOMEM, "cudaHostAlloc failed");
         goto cleanup;
     }
 
-    if (!c->periodic) {  // open box: grid over the union bounding box
-        unsigned long long init[6] = {~0ull, ~0ull, ~0ull, 0ull, 0ull, 0ull};
-        std::memcpy(ho->hist, init, sizeof(init));
-        CF_CUDA(cudaMemcpyAsync(bbox_keys, ho->hist, sizeof(init), cudaMemcpyHostToDevice, st), "H2D bbox");
-        for (int t = 0; t < ncat; ++t)
-            CF_CUDA(cf::launch_bbox(c->dtype, dx[t][0], dx[t][1], dx[t][2], cats[t]->n, bbox_keys, sms,
-                                    d_err, st),
-                    "bbox kernel");
-        CF_CUDA(cudaMemcpyAsync(ho->hist, bbox_keys, sizeof(init), cudaMemcpyDeviceToHost, st), "D2H bbox");
-        CF_CUDA(cudaMemcpyAsync(&ho->err, d_err, 4, cudaMemcpyDeviceToHost, st), "D2H err");
-        CF_CUDA(cudaStreamSynchronize(st), "sync (bbox)");
-        if (ho->err & cf::ERR_COORD) {
-            rc = fail(CF_EINVAL, "non-finite coordinate");
-            goto cleanup;
-        }
-        if (ntot > 0)
-            for (int a = 0; a < 3; ++a) {
-                lo[a] = cf::decode_dkey(ho->hist[a]);
-                hi[a] = cf::decode_dkey(ho->hist[3 + a]);
+    {
+        // Inputs and the staged block.  The block is one host image and one copy: the
+        // bounding-box keys, the zeroed results [hist | diag(4) | err, counter | kept, - |
+        // max |w| (2) | barriers (2) | wsum | rsum], squared edges, pi edges, thresholds, table.
+        const size_t nres = nslots + 8 + nacc;
+        auto carve_inputs = [&]() {
+            for (int t = 0; t < ncat; ++t) {
+                const long long n = cats[t]->n;
+                if (host_in[t]) {
+                    for (int a = 0; a < 3; ++a)
+                        dx[t][a] = bump.take<char>(n * esz);
+                    dw[t] = cats[t]->w ? bump.take<double>(n) : nullptr;
+                } else {
+                    dx[t][0] = cats[t]->x;
+                    dx[t][1] = cats[t]->y;
+                    dx[t][2] = cats[t]->z;
+                    dw[t] = cats[t]->w;
+                }
             }
-    }
-    trace.point("setup");
-    plan_geom(q, lo, hi, ntot, g);
-    res->refine_used[0] = g.reach_x;
-    res->refine_used[1] = g.reach_y;
-    res->refine_used[2] = g.reach_z;
-
-    {  // grid workspace
+            stage.keys = bump.take<unsigned long long>(6 + nres + (nb + 1) + Pe.size() + (nb + 1) +
+                                                       cf::LUT_MAX / 8 + 2);  // + the table's alignment
+        };
         // float32 mean separations: the coordinates' float32 rounding residuals,
         // unless the inputs are float32 in a periodic box (exact)
-        const bool resid = !f64 && c->want_ravg && !(c->dtype == CF_FLOAT32 && c->periodic);
-        for (int pass = 0; pass < 2; ++pass) {
-            bump.base = pass ? (char *)ws2 : nullptr;
-            bump.off = 0;
+        resid = !f64 && c->want_ravg && !(c->dtype == CF_FLOAT32 && c->periodic);
+        auto carve_grid = [&]() {
             for (int t = 0; t < ncat; ++t) {
                 const long long n = cf::padded_max(cats[t]->n, g.ncols);
                 G[t].xyz = bump.take<float>(3 * n);
                 G[t].chunk_col = bump.take<int>(n / cf::COL_PAD);
-                G[t].ws = c->weighted ? bump.take<float>(n + 64) : nullptr;  // + slack for tile reads
-                if (resid) {  // float32 mean separation from inputs float32 cannot hold exactly
-                    G[t].res = bump.take<float>(3 * n);
-                }
-                G[t].wmax = c->weighted ? reinterpret_cast<unsigned *>(d_hist + nslots + 6) + t : nullptr;
+                G[t].ws = c->weighted ? bump.take<float>(n) : nullptr;
+                G[t].res = resid ? bump.take<float>(3 * n) : nullptr;
+                G[t].wmax = c->weighted ? d_err + 4 + t : nullptr;
                 G[t].pos64 = bump.take<double4_32a>(n);
                 G[t].perm = bump.take<int>(n);
                 G[t].cell_start = bump.take<uint32_t>(g.ncells + 1);
@@ -903,40 +846,98 @@ int run(Request &q)
             tmp.coltot = bump.take<uint32_t>(g.ncols);
             tmp.bsum = bump.take<uint32_t>(cf::grid_max_blocks(sms));
             const int sx = 2 * g.reach_x + 1, sy = 2 * g.reach_y + 1;
-            const int nst = q.autocorr ? (sx * sy + 1) / 2 : sx * sy;
-            nbr = bump.take<cf::Nbr>((size_t)g.ncols * nst);
+            nbr = bump.take<cf::Nbr>((size_t)g.ncols * (q.autocorr ? (sx * sy + 1) / 2 : sx * sy));
             nbr_count = bump.take<unsigned>(g.ncols);
-            if (pass == 0) {
-                const cudaError_t e = cudaMallocAsync(&ws2, bump.off, st);
-                if (e) {
-                    rc = cuda_fail(e, "cudaMallocAsync (grid)");
-                    goto cleanup;
-                }
-            }
-        }
+        };
+        // In a periodic box the grid is known at once and one allocation serves all; an
+        // open box's grid follows from the points' extent, read back first.
+        if (c->periodic)
+            plan_geom(q, lo, hi, ntot, g);
+        carve_inputs();
+        if (c->periodic)
+            carve_grid();
+        CF_CUDA(cudaMallocAsync(&ws, bump.off, st), "cudaMallocAsync");
+        bump.base = (char *)ws;
+        bump.off = 0;
+        carve_inputs();
+        d_hist = stage.keys + 6;
+        d_diag = d_hist + nslots;
+        d_err = reinterpret_cast<unsigned *>(d_hist + nslots + 4);
+        d_ctr = d_err + 1;
+        d_wcount = d_err + 2;
+        d_bar = d_err + 6;
+        d_E2 = reinterpret_cast<double *>(d_hist + nres);
+        d_P = d_E2 + nb + 1;
+        d_thr = reinterpret_cast<float *>(d_P + Pe.size());
+        d_lut = reinterpret_cast<uint8_t *>(d_thr + 2 * (nb + 1));
+        d_lut += (16 - (d_lut - reinterpret_cast<uint8_t *>(stage.keys)) % 16) % 16;  // bulk copies start on 16 bytes
+        if (c->periodic)
+            carve_grid();
         for (int t = 0; t < ncat; ++t) {
-            const cudaError_t e = cf::build_grid(c->dtype, dx[t][0], dx[t][1], dx[t][2], dw[t],
-                                                 cats[t]->n, g, tmp, G[t], sms, d_err, d_bar + t, st);
-            if (e) {
-                rc = cuda_fail(e, "grid kernels");
+            if (!host_in[t])
+                continue;
+            const long long n = cats[t]->n;
+            CF_CUDA(cudaMemcpyAsync((void *)dx[t][0], cats[t]->x, n * esz, cudaMemcpyHostToDevice, st), "H2D x");
+            CF_CUDA(cudaMemcpyAsync((void *)dx[t][1], cats[t]->y, n * esz, cudaMemcpyHostToDevice, st), "H2D y");
+            CF_CUDA(cudaMemcpyAsync((void *)dx[t][2], cats[t]->z, n * esz, cudaMemcpyHostToDevice, st), "H2D z");
+            if (dw[t])
+                CF_CUDA(cudaMemcpyAsync((void *)dw[t], cats[t]->w, n * 8, cudaMemcpyHostToDevice, st), "H2D w");
+        }
+        if (!c->periodic) {  // grid over the union bounding box
+            for (int a = 0; a < 6; ++a)
+                ho->stage[a] = a < 3 ? ~0ull : 0ull;
+            std::memset(ho->stage + 6, 0, 8 * nres);
+            CF_CUDA(cudaMemcpyAsync(stage.keys, ho->stage, 8 * (6 + nres), cudaMemcpyHostToDevice, st), "H2D bbox");
+            for (int t = 0; t < ncat; ++t)
+                CF_CUDA(cf::launch_bbox(c->dtype, dx[t][0], dx[t][1], dx[t][2], cats[t]->n, stage.keys, sms,
+                                        d_err, st),
+                        "bbox kernel");
+            CF_CUDA(cudaMemcpyAsync(ho->hist, stage.keys, 8 * (6 + nslots + 5), cudaMemcpyDeviceToHost, st),
+                    "D2H bbox");
+            CF_CUDA(cudaStreamSynchronize(st), "sync (bbox)");
+            unsigned err = 0;
+            std::memcpy(&err, ho->hist + 6 + nslots + 4, 4);
+            if (err & cf::ERR_COORD) {
+                rc = fail(CF_EINVAL, "non-finite coordinate");
                 goto cleanup;
             }
+            if (ntot > 0)
+                for (int a = 0; a < 3; ++a) {
+                    lo[a] = cf::decode_dkey(ho->hist[a]);
+                    hi[a] = cf::decode_dkey(ho->hist[3 + a]);
+                }
+            plan_geom(q, lo, hi, ntot, g);
+            bump.base = nullptr;
+            bump.off = 0;
+            carve_grid();
+            CF_CUDA(cudaMallocAsync(&ws2, bump.off, st), "cudaMallocAsync (grid)");
+            bump.base = (char *)ws2;
+            bump.off = 0;
+            carve_grid();
         }
+    }
+    trace.point("setup");
+    res->refine_used[0] = g.reach_x;
+    res->refine_used[1] = g.reach_y;
+    res->refine_used[2] = g.reach_z;
+
+    {
         if (q.autocorr)
             G[1] = G[0];
-        trace.point("gridding");
 
-        // ---- pair kernel parameters
+        // ---- pair kernel parameters and tables, then the staged block
         double M = 0.0, Ls = 0.0;
         base_params(q, g, G[0], G[1], P, M, Ls);
-        P.nbr = nbr;
-        P.nbr_count = nbr_count;
-        if (q.kind == 1) {
-            std::memcpy(ho->pe, Pe.data(), 8 * Pe.size());
-            CF_CUDA(cudaMemcpyAsync(d_P, ho->pe, 8 * Pe.size(), cudaMemcpyHostToDevice, st), "H2D pi edges");
-        }
+        unsigned long long *h0 = ho->stage;  // host image, at the same offsets
+        std::memcpy(h0 + (reinterpret_cast<unsigned long long *>(d_E2) - stage.keys), E2.data(), 8 * E2.size());
+        if (q.kind == 1)
+            std::memcpy(h0 + (reinterpret_cast<unsigned long long *>(d_P) - stage.keys), Pe.data(), 8 * Pe.size());
+        size_t staged = reinterpret_cast<uint8_t *>(d_thr) - reinterpret_cast<uint8_t *>(stage.keys);
         if (!f64) {
-            const Tables tb = cached_tables(E2.data(), nb + 1, q.kind == 0 ? 3 : 2, M, Ls, R, T, tab);
+            uint8_t *hb = reinterpret_cast<uint8_t *>(h0);
+            const size_t at_lut = d_lut - reinterpret_cast<uint8_t *>(stage.keys);
+            const Tables tb = cached_tables(E2.data(), nb + 1, q.kind == 0 ? 3 : 2, M, Ls, R,
+                                            reinterpret_cast<float *>(hb + staged), hb + at_lut);
             P.nthr = tb.nthr;
             P.lut_n = tb.lut_n;
             P.lut_shift = tb.shift;
@@ -944,13 +945,31 @@ int run(Request &q)
             P.lut_lin = tb.lin;
             P.lut_scale = tb.lscale;
             res->table_linear = tb.lin;
-            std::memcpy(ho->thr, T, 4 * P.nthr);
-            std::memcpy(ho->lut, tab, P.lut_n);
-            CF_CUDA(cudaMemcpyAsync(d_thr, ho->thr, 4 * P.nthr, cudaMemcpyHostToDevice, st), "H2D thresholds");
-            CF_CUDA(cudaMemcpyAsync(d_lut, ho->lut, P.lut_n, cudaMemcpyHostToDevice, st), "H2D lut");
+            staged = at_lut + tb.lut_n;
         }
-        std::memcpy(ho->e2, E2.data(), 8 * E2.size());
-        CF_CUDA(cudaMemcpyAsync(d_E2, ho->e2, 8 * E2.size(), cudaMemcpyHostToDevice, st), "H2D E2");
+        if (c->periodic) {  // results and tables in one copy
+            std::memset(h0, 0, 8 * (6 + nslots + 8 + nacc));
+            CF_CUDA(cudaMemcpyAsync(stage.keys, h0, staged, cudaMemcpyHostToDevice, st), "H2D tables");
+        } else {  // the results were cleared with the bounding box
+            const size_t from = reinterpret_cast<uint8_t *>(d_E2) - reinterpret_cast<uint8_t *>(stage.keys);
+            CF_CUDA(cudaMemcpyAsync(d_E2, reinterpret_cast<uint8_t *>(h0) + from, staged - from,
+                                    cudaMemcpyHostToDevice, st),
+                    "H2D tables");
+        }
+        trace.point("tables");
+        for (int t = 0; t < ncat; ++t) {
+            const cudaError_t e = cf::build_grid(c->dtype, dx[t][0], dx[t][1], dx[t][2], dw[t],
+                                                 cats[t]->n, g, tmp, G[t], sms, d_err, d_bar + t, st);
+            if (e) {
+                rc = cuda_fail(e, "grid kernel");
+                goto cleanup;
+            }
+        }
+        trace.point("gridding");
+        P.A.n = cats[0]->n;
+        P.B.n = cats[ncat - 1]->n;
+        P.nbr = nbr;
+        P.nbr_count = nbr_count;
         P.thr = d_thr;
         P.lut = d_lut;
         P.E2 = d_E2;
@@ -976,7 +995,6 @@ int run(Request &q)
         // up to 59 bins: beyond that the binary64 kernel counts (same results, exact terms)
         if (!f64 && q.kind == 0 && c->weighted && c->want_ravg && nb > 59)
             PL.f64 = 1;
-        trace.point("tables");
         CF_CUDA(cudaEventRecord(g_events.ev[1], st), "cudaEventRecord");
         if (P.n_items > 0) {
             const cudaError_t e = cf::launch_pairs(P, PL, sms, st);
@@ -992,7 +1010,11 @@ int run(Request &q)
                 "D2H results");
     }
     CF_CUDA(cudaEventRecord(g_events.ev[3], st), "cudaEventRecord");
-    CF_CUDA(cudaEventSynchronize(g_events.ev[3]), "synchronize");
+    if (ws2)  // released in stream order, before the call's one wait
+        cudaFreeAsync(ws2, st);
+    cudaFreeAsync(ws, st);
+    ws = ws2 = nullptr;
+    CF_CUDA(cudaStreamSynchronize(st), "synchronize");
     trace.point("readback");
     {
         float ms = 0.f;
@@ -1049,14 +1071,10 @@ int run(Request &q)
 cleanup:
     if (ws2)
         cudaFreeAsync(ws2, st);
-    if (ws) {
+    if (ws)
         cudaFreeAsync(ws, st);
-        if (rc == CF_OK) {
-            cudaError_t e = cudaStreamSynchronize(st);
-            if (e)
-                rc = cuda_fail(e, "final synchronize");
-        }
-    }
+    if (rc != CF_OK && ws)
+        cudaStreamSynchronize(st);  // the staged block's copy may still be on its way
     return rc;
 }
 
