@@ -27,7 +27,7 @@ cudaError_t launch_shape(const PairParams &P, PairLaunch &L, int sms, cudaStream
 
 }  // namespace
 
-int count32_smem(int nbins) { return align_up(C32_HIST + (nbins + 2) * 128, 128); }
+int count32_smem(int nbins) { return Lay32<false>::total(nbins); }
 
 cudaError_t launch_neighbours(const PairParams &P, cudaStream_t st)
 {

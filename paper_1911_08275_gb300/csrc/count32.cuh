@@ -25,7 +25,13 @@
 // blocks of 8 steps, a whole warp waiting for one lane); without the queue the
 // chunk tasks took 1.218 ms, and reading the secondaries through the L1 instead
 // of the ring 1.245 ms (four wavefronts per 16-byte load).  Rmax 5 / 10 / 50: 0.282 /
-// 0.280 / 5.285 ms before, 0.219 / 0.270 / 5.12 ms now.
+// 0.280 / 5.285 ms before, 0.219 / 0.270 / 5.12 ms so.
+//
+// Where (nbins + 2)^2 rows fit beside the rings of 24 warps, an atomic takes two pairs
+// (D2): the row is that of the pair of entries, and a bin's count is the sum of the
+// rows with the bin as either entry.  Four fewer atomics (8 -> 4) and the four
+// multiply-adds that join two entries in the place of eight addresses: 24 wavefronts
+// a step.  Kernel at Rmax 25 1.052 ms, at Rmax 5 / 10 / 50 0.212 / 0.255 / 4.73 ms.
 #pragma once
 
 #include <type_traits>
@@ -44,25 +50,55 @@ constexpr int C32_LUT = 128;
 constexpr int C32_THR = C32_LUT + LUT_MAX;
 constexpr int C32_E2 = C32_THR + 2 * (NB_MAX + 1) * 4;
 constexpr int C32_RING = (C32_E2 + (NB_MAX + 1) * 8 + 127) / 128 * 128;
-constexpr int C32_QUEUE = C32_RING + WARPS * RingXYZ::BYTES;
-constexpr int C32_HIST = C32_QUEUE + WARPS * (int)sizeof(FlagQueue);
+
+// D2: one histogram word for two pairs (a row per pair of entries, (nbins + 2)^2 rows),
+// which halves the atomics; a CTA of 24 warps shares it.
+template <bool D2>
+struct Lay32 {
+    static constexpr int NW = D2 ? 24 : WARPS;
+    using Ring = RingXYZ;
+    static constexpr int QUEUE = C32_RING + NW * Ring::BYTES;
+    static constexpr int HIST = QUEUE + NW * (int)sizeof(FlagQueue);
+    static __host__ __device__ int words(int nb) { return (D2 ? (nb + 2) * (nb + 2) : nb + 2) * 32; }
+    static __host__ __device__ int total(int nb) { return align_up(HIST + words(nb) * 4, 128); }
+};
+
+// Secondaries a D2 count may have, so that no word overflows: a warp flushes between
+// tasks once it has evaluated 2^30 / 24 pairs per lane, and one task evaluates at most
+// 3 (images in z) x 2 (padding) x n pairs per lane, each up to 1.5 additions:
+// 24 * 1.5 * 6 * 2^23 + 1.5 * 2^30 < 2^32.  Where the stencil is wider than the grid, a
+// column comes up under up to 9 images in x and y.
+constexpr long long D2_MAX_POINTS = 1ll << 23;
 
 // What a sweep needs beside the primaries.
 struct Sweep {
     uint32_t lutb, hl;  // shared addresses: table, this lane's histogram column (row 0)
     uint32_t u0, lut_last;
     int shift, nthr, nb;
+    uint32_t nrow;      // D2: nbins + 2
+    // where settled pairs go: row 0 of this lane's column (D2: with a pair that does not
+    // count), bytes per row
+    template <bool D2>
+    __device__ __forceinline__ uint32_t settle_at() const
+    {
+        return D2 ? hl + (nrow - 2u) * 128u : hl;
+    }
+    template <bool D2>
+    __device__ __forceinline__ uint32_t settle_row() const
+    {
+        return D2 ? nrow * 128u : 128u;
+    }
     float lscale;
     FlagQueue *fq;
     int qn;  // flagged pairs waiting in the warp's queue
 };
 
-// Settle the last min(32, qn) flagged pairs of the warp's queue, one per lane: the
-// float32 d2 with the sweep's operations, counted against the thresholds; inside
-// a band re-evaluated in binary64.  Each pair goes to its true bin (the sweep has
+// Settle the last min(32, qn) flagged pairs of the warp's queue, one per lane (their
+// rows are rowb bytes apart from hl): the float32 d2 with the sweep's operations,
+// counted against the thresholds; inside a band re-evaluated in binary64.  Each pair goes to its true bin (the sweep has
 // put it in row -1, which is never read).  Returns 1 in lanes that re-evaluated.
 __device__ __noinline__ int settle(const PairParams &P, const unsigned char *smem, uint32_t hl,
-                                   const FlagQueue *fq, int qn)
+                                   uint32_t rowb, const FlagQueue *fq, int qn)
 {
     const int lane = threadIdx.x & 31, first = max(0, qn - 32);
     int row = -1, re = 0;
@@ -86,7 +122,7 @@ __device__ __noinline__ int settle(const PairParams &P, const unsigned char *sme
         }
     }
     if (row >= 0)
-        red_shared1(hl + (uint32_t)row * 128u);
+        red_shared1(hl + (uint32_t)row * rowb);
     __syncwarp();
     return re;
 }
@@ -97,7 +133,7 @@ __device__ __noinline__ int settle(const PairParams &P, const unsigned char *sme
 // secondaries and starts at a multiple of JS, so it never leaves the column
 // (columns are padded to 32).  Secondaries outside the window are farther than
 // Rmax in z and never counted.  TRI: pairs with j <= i do not count.
-template <int I, int PP, bool TRI, bool EVALS, bool VERIFY, bool LIN>
+template <int I, int PP, bool TRI, bool EVALS, bool VERIFY, bool LIN, bool D2>
 __device__ __forceinline__ void sweep(const PairParams &P, const unsigned char *smem, Sweep &S,
                                       uint32_t addr, int j0, int j1, int jlo, int jhi, int jj,
                                       const u64 (&XH)[PP], const u64 (&YH)[PP], const u64 (&ZH)[PP], int ib,
@@ -169,13 +205,18 @@ __device__ __forceinline__ void sweep(const PairParams &P, const unsigned char *
                                    (!TRI || jt + r > ib + q * I + ii)) ? 1ull : 0ull;
             }
 #pragma unroll
-            for (int q = 0; q < PP; ++q)
+            for (int q = 0; q < PP; ++q) {
+                uint32_t e[4];
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    const uint32_t e = lds_entry(cq[q][r]);  // the row: bin, dummy or flagged (-1)
-                    red_shared1(S.hl + e * 128u);
-                    fm[q] = push_sign(fm[q], e);  // pair (t, r) ends at bit 4 tend - 1 - (4 t + r)
+                    e[r] = lds_entry(cq[q][r]);  // the row: bin, dummy or flagged (-1)
+                    if (!D2)
+                        red_shared1(S.hl + e[r] * 128u);
+                    fm[q] = push_sign(fm[q], e[r]);  // pair (t, r) ends at bit 4 tend - 1 - (4 t + r)
+                    if (D2 && (r & 1))
+                        red_shared1(S.hl + (e[r - 1] * S.nrow + e[r]) * 128u);
                 }
+            }
             if (VERIFY) {
                 const float *T = reinterpret_cast<const float *>(smem + C32_THR);
                 const double *E2 = reinterpret_cast<const double *>(smem + C32_E2);
@@ -210,7 +251,7 @@ __device__ __forceinline__ void sweep(const PairParams &P, const unsigned char *
                     }
                     S.qn += __popc(bm);
                     if (S.qn >= 32) {
-                        n_rck += settle(P, smem, S.hl, S.fq, S.qn);
+                        n_rck += settle(P, smem, S.template settle_at<D2>(), S.template settle_row<D2>(), S.fq, S.qn);
                         S.qn -= 32;
                     }
                 }
@@ -221,9 +262,10 @@ __device__ __forceinline__ void sweep(const PairParams &P, const unsigned char *
 
 // LT: table cells linear in d2 (1) or on float bits (0), or as the launch's tables
 // say (-1).
-template <int I, int PP, bool EVALS, bool VERIFY, int LT>
+template <int I, int PP, bool EVALS, bool VERIFY, int LT, bool D2 = false>
 struct Count32 {
-    static constexpr int CH = I * PP;
+    using Lay = Lay32<D2>;
+    static constexpr int CH = I * PP, NW = Lay::NW, NT = NW * 32;
     struct State {
         Sweep S;
         u64 n_eval, n_rck, n_viol;
@@ -244,28 +286,29 @@ struct Count32 {
     static __device__ __forceinline__ bool load(const PairParams &P, unsigned char *smem, State &st,
                                                 unsigned phase)
     {
-        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + C32_HIST);
+        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + Lay::HIST);
         const int tid = threadIdx.x, nb = P.nbins;
         const bool ok = load_table(P, smem, C32_LUT, phase, [&]() {
-            for (int q = tid; q < P.nthr; q += THREADS)
+            for (int q = tid; q < P.nthr; q += NT)
                 reinterpret_cast<float *>(smem + C32_THR)[q] = P.thr[q];
-            for (int q = tid; q <= nb; q += THREADS)
+            for (int q = tid; q <= nb; q += NT)
                 reinterpret_cast<double *>(smem + C32_E2)[q] = P.E2[q];
-            for (int q = tid; q < (nb + 2) * 32; q += THREADS)
+            for (int q = tid; q < Lay::words(nb); q += NT)
                 hist[q] = 0u;
         });
         st.n_eval = st.n_rck = st.n_viol = 0ull;
         st.pending = 0u;
         Sweep &S = st.S;
         S.lutb = smem_u32(smem + C32_LUT);
-        S.hl = smem_u32(hist + 32 + (tid & 31));  // row 0 (row -1 before it)
+        S.nrow = (uint32_t)nb + 2u;
+        S.hl = smem_u32(hist + (D2 ? nb + 3 : 1) * 32 + (tid & 31));  // row 0 (row -1 before it)
         S.u0 = P.u0;
         S.lut_last = (uint32_t)(P.lut_n - 1);
         S.shift = P.lut_shift;
         S.nthr = P.nthr;
         S.nb = nb;
         S.lscale = P.lut_scale;
-        S.fq = reinterpret_cast<FlagQueue *>(smem + C32_QUEUE) + (tid >> 5);
+        S.fq = reinterpret_cast<FlagQueue *>(smem + Lay::QUEUE) + (tid >> 5);
         S.qn = 0;
         return ok;
     }
@@ -274,19 +317,19 @@ struct Count32 {
                                                 unsigned c, unsigned part, unsigned parts)
     {
         const int lane = threadIdx.x & 31, ii = lane % I, jj = lane / I;
-        const uint32_t ring = smem_u32(smem + C32_RING) + (threadIdx.x >> 5) * (uint32_t)RingXYZ::BYTES;
+        const uint32_t ring = smem_u32(smem + C32_RING) + (threadIdx.x >> 5) * (uint32_t)Lay::Ring::BYTES;
         const int ib = (int)(c * CH);
         Chunk<I, PP> C;
         if (!C.load(P, ib, ii))
             return;
         u64 XH[PP], YH[PP], ZH[PP];
         int image = 0;
-        for_windows<128 / I, RingXYZ>(
+        for_windows<128 / I, typename Lay::Ring>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) { image = C.shift(P, k, code, XH, YH, ZH); },
             [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {
                 auto go = [&](auto tr, auto li) {
-                    sweep<I, PP, decltype(tr)::value, EVALS, VERIFY, decltype(li)::value>(
+                    sweep<I, PP, decltype(tr)::value, EVALS, VERIFY, decltype(li)::value, D2>(
                         P, smem, st.S, addr, j0, j1, jlo, jhi, jj, XH, YH, ZH, ib, image, C.vmask, st.n_eval,
                         st.n_rck, st.n_viol);
                 };
@@ -302,28 +345,62 @@ struct Count32 {
                     else
                         go(std::false_type{}, std::false_type{});
                 }
-                if (st.pending > (1u << 30) / WARPS) {  // keep every shared u32 count far from overflow
+                if (!D2 && st.pending > (1u << 30) / NW) {  // keep every shared u32 count far from overflow
                     __syncwarp();
-                    warp_flush_shared(reinterpret_cast<uint32_t *>(smem + C32_HIST) + 32, P.nbins, P.hist,
+                    warp_flush_shared(reinterpret_cast<uint32_t *>(smem + Lay::HIST) + 32, P.nbins, P.hist,
                                       lane);
                     st.pending = 0;
                 }
             });
+        if (D2 && st.pending > (1u << 30) / NW) {
+            __syncwarp();
+            flush(P, smem, lane, 1, 0);
+            st.pending = 0;
+        }
+    }
+
+    // Rows w0, w0 + step, ... to the global counts, each word taken by one exchange (other
+    // warps may be adding).  D2: a row's pairs belong to two bins.
+    static __device__ __noinline__ void flush(const PairParams &P, unsigned char *smem, int lane, int step, int w0)
+    {
+        uint32_t *hist = reinterpret_cast<uint32_t *>(smem + Lay::HIST);
+        const int nb = P.nbins, nr = nb + 2;
+        for (int r = w0; r < (D2 ? nr * nr : nr); r += step) {
+            const int b1 = (D2 ? r % nr : r) - 1, b0 = D2 ? r / nr - 1 : -1;
+            const bool in1 = b1 >= 0 && b1 < nb, in0 = b0 >= 0 && b0 < nb;
+            if (!in0 && !in1)
+                continue;
+            const u64 v = warp_sum_u64(atomicExch(&hist[r * 32 + lane], 0u));
+            if (lane == 0 && v) {
+                if (in1)
+                    atomicAdd(&P.hist[b1], v);
+                if (in0)
+                    atomicAdd(&P.hist[b0], v);
+            }
+        }
     }
 
     static __device__ __forceinline__ void fini(const PairParams &P, unsigned char *smem, State &st)
     {
         const int lane = threadIdx.x & 31;
-        const uint32_t *hist = reinterpret_cast<const uint32_t *>(smem + C32_HIST);
         if (st.S.qn) {
-            st.n_rck += settle(P, smem, st.S.hl, st.S.fq, st.S.qn);
+            st.n_rck += settle(P, smem, st.S.template settle_at<D2>(), st.S.template settle_row<D2>(), st.S.fq, st.S.qn);
             st.S.qn = 0;
         }
         __syncthreads();
-        for (int b = threadIdx.x >> 5; b < P.nbins; b += WARPS) {
-            const u64 v = warp_sum_u64(hist[(b + 1) * 32 + lane]);
-            if (lane == 0 && v)
-                atomicAdd(&P.hist[b], v);
+        if (D2) {  // a warp per bin: the rows with the bin as either entry
+            const uint32_t *hist = reinterpret_cast<const uint32_t *>(smem + Lay::HIST);
+            const int nr = P.nbins + 2;
+            for (int b = threadIdx.x >> 5; b < P.nbins; b += NW) {
+                u64 v = 0;
+                for (int c = 0; c < nr; ++c)
+                    v += (u64)hist[((b + 1) * nr + c) * 32 + lane] + hist[(c * nr + b + 1) * 32 + lane];
+                v = warp_sum_u64(v);
+                if (lane == 0 && v)
+                    atomicAdd(&P.hist[b], v);
+            }
+        } else {
+            flush(P, smem, lane, NW, threadIdx.x >> 5);
         }
         const u64 n_rck = warp_sum_u64(st.n_rck);
         if (lane == 0 && n_rck)

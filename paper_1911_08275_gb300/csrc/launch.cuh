@@ -5,14 +5,14 @@
 
 namespace cf {
 
-// CTAs of THREADS threads per SM for a kernel with smem bytes of dynamic shared
+// CTAs of `threads` threads per SM for a kernel with smem bytes of dynamic shared
 // memory; raises the kernel's shared-memory limit when needed (cached).
-cudaError_t occupancy_of(const void *kern, int smem, int &occ);
+cudaError_t occupancy_of(const void *kern, int smem, int &occ, int threads = 256);
 
 template <class K>
-cudaError_t occupancy(K kern, int smem, int &occ)
+cudaError_t occupancy(K kern, int smem, int &occ, int threads = 256)
 {
-    return occupancy_of((const void *)kern, smem, occ);
+    return occupancy_of((const void *)kern, smem, occ, threads);
 }
 
 // Parts a split chunk task has (TaskSplit; a part takes every parts-th

@@ -25,7 +25,7 @@ int g_nocc = 0, g_nattr = 0;
 std::mutex g_occ_mu;
 }  // namespace
 
-cudaError_t occupancy_of(const void *kern, int smem, int &occ)
+cudaError_t occupancy_of(const void *kern, int smem, int &occ, int threads)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -50,7 +50,7 @@ cudaError_t occupancy_of(const void *kern, int smem, int &occ)
             occ = g_occ[q].occ;
             return cudaSuccess;
         }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, THREADS, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
     if (e)
         return e;
     if (g_nocc < 128)
@@ -71,7 +71,9 @@ cudaError_t launch_pairs(const PairParams &P, PairLaunch &L, int sms, cudaStream
         return launch_count64(P, L, sms, st);
     if (P.wacc)
         return P.kind == 0 ? launch_sums32(P, L, sms, st) : launch_sumsrp32(P, L, sms, st);
-    return P.kind == 0 ? launch_count32(P, L, sms, st) : launch_countrp32(P, L, sms, st);
+    if (P.kind == 1)
+        return launch_countrp32(P, L, sms, st);
+    return count32_paired(P, L) ? launch_count32_paired(P, L, sms, st) : launch_count32(P, L, sms, st);
 }
 
 }  // namespace cf

@@ -9,6 +9,8 @@ namespace cf {
 
 __host__ __device__ inline int align_up(int v, int a) { return (v + a - 1) / a * a; }
 
+constexpr int SMEM_MAX = 232448;  // dynamic shared memory a CTA may opt in to (227 KB)
+
 struct PairLaunch {
     int f64;      // 1: binary64 counts
     int chunk;    // primary lanes per warp chunk (8, 16 or 32)
@@ -25,6 +27,9 @@ struct PairLaunch {
 cudaError_t launch_neighbours(const PairParams &P, cudaStream_t st);
 cudaError_t launch_count32(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
 int count32_smem(int nbins);
+// The same with one histogram word for two pairs, where that is faster.
+bool count32_paired(const PairParams &P, const PairLaunch &L);
+cudaError_t launch_count32_paired(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
 // Float32 DD(rp, pi) counts.
 cudaError_t launch_countrp32(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st);
 int countrp32_smem(int nbins, int npibins);

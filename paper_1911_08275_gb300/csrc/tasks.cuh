@@ -119,13 +119,16 @@ __device__ __forceinline__ void warp_copy(uint32_t dst, const void *src, int byt
 // global load of a value that 16 lanes share occupies the L1's data path four
 // times (once per quarter warp), a shared load twice.  A Ring says what a piece
 // holds: N secondaries, SLOT bytes, copied by copy(P, dst, j, n, lane).
-struct RingXYZ {  // coordinates, in the quad layout
-    static constexpr int N = 192, SLOT = N * 12, BYTES = 2 * SLOT;
+template <int LEN>
+struct RingCoords {  // coordinates, in the quad layout
+    static constexpr int N = LEN, SLOT = N * 12, BYTES = 2 * SLOT;
     static __device__ __forceinline__ void copy(const PairParams &P, uint32_t dst, int j, int n, int lane)
     {
         warp_copy(dst, P.B.xyz + 3ll * j, n * 12, lane);
     }
 };
+
+using RingXYZ = RingCoords<192>;
 
 // Coordinates, then their residuals (RL) in the quad layout, then weights (W).
 // Short pieces: two CTAs with their rows of sums fill an SM's shared memory.
@@ -397,11 +400,28 @@ __device__ __forceinline__ void neighbours_body(const PairParams &P, int col, in
     }
 }
 
+// Warps per CTA of a path: Path::NW, or WARPS.
+template <class Path>
+constexpr auto path_warps_of(int) -> decltype(Path::NW)
+{
+    return Path::NW;
+}
+template <class Path>
+constexpr int path_warps_of(long)
+{
+    return WARPS;
+}
+template <class Path>
+constexpr int path_warps()
+{
+    return path_warps_of<Path>(0);
+}
+
 // Persistent kernel over the chunk tasks of one count.  Path: CH (primaries per
 // chunk), State, init (false in every thread if the CTA has to give up), task,
 // fini.
 template <class Path, int MINB>
-__global__ void __launch_bounds__(THREADS, MINB) k_tasks(const __grid_constant__ PairParams P)
+__global__ void __launch_bounds__(32 * path_warps<Path>(), MINB) k_tasks(const __grid_constant__ PairParams P)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     typename Path::State st;
@@ -409,7 +429,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tasks(const __grid_constant__
         return;
     const int lane = threadIdx.x & 31;
     const unsigned nchunk = __ldg(P.A.cell_start + P.g.ncells) / Path::CH;
-    const TaskSplit split(nchunk, (unsigned)P.parts, nchunk <= 2u * gridDim.x * WARPS);
+    const TaskSplit split(nchunk, (unsigned)P.parts, nchunk <= 2u * gridDim.x * path_warps<Path>());
     unsigned nxt = 0;
     if (lane == 0)
         nxt = atomicAdd(P.item_counter, 1u);
@@ -429,15 +449,16 @@ cudaError_t launch_tasks(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
 {
     PairParams P = P0;
     int occ = 0;
-    const cudaError_t e = occupancy(k_tasks<Path, MINB>, L.smem, occ);
+    constexpr int NW = path_warps<Path>();
+    const cudaError_t e = occupancy(k_tasks<Path, MINB>, L.smem, occ, 32 * NW);
     if (e)
         return e;
     if (occ < 1)
         return cudaErrorInvalidConfiguration;
     const long long chunks = (P.A.n + (long long)P.g.ncols * (COL_PAD / 2)) / Path::CH + 1;
-    P.parts = task_parts((double)chunks, (double)sms * occ * WARPS, P.nstencil);
-    L.blocks = (int)std::max(1ll, std::min<long long>((long long)sms * occ, (chunks * P.parts + WARPS - 1) / WARPS));
-    k_tasks<Path, MINB><<<L.blocks, THREADS, L.smem, st>>>(P);
+    P.parts = task_parts((double)chunks, (double)sms * occ * NW, P.nstencil);
+    L.blocks = (int)std::max(1ll, std::min<long long>((long long)sms * occ, (chunks * P.parts + NW - 1) / NW));
+    k_tasks<Path, MINB><<<L.blocks, 32 * NW, L.smem, st>>>(P);
     return cudaGetLastError();
 }
 
