@@ -74,9 +74,9 @@ typedef enum {
                                          binary64 and count float32 decisions that
                                          disagree into n_band_violations (debug)  */
 #define CF_FLAG_DEBUG_STALL (1u << 3) /* diagnostic (float32 DD(r) without sums):
-                                         each CTA's first tile barrier is armed for
-                                         a copy that is never issued, and the waits
-                                         give up after 1 ms, so the call returns
+                                         each CTA's table barrier is armed for a
+                                         copy that is never issued, and the wait
+                                         gives up after 1 ms, so the call returns
                                          CF_ETIMEOUT; tests the bounded waits.
                                          Ignored by the other kernels.          */
 

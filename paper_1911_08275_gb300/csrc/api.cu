@@ -503,7 +503,7 @@ void finish_geom(cf::Geom &g)
 }
 
 // Points per column the default refinement aims at: fewer make the per-work-item
-// and per-chunk costs (window records, claims, tile copies) dominate, more make
+// and per-chunk costs (window searches, claims, ring fills) dominate, more make
 // the columns' square cross-section a poorer fit to the sphere (more pairs
 // evaluated beyond Rmax).
 constexpr double DEFAULT_COL_POINTS = 1024.0;
@@ -629,7 +629,7 @@ int plan_geom(const Request &q, const double lo[3], const double hi[3], long lon
     return CF_OK;
 }
 
-// Limit of a kernel's tile-barrier waits: 2 s (a tile copy of a few tens of KB
+// Limit of a kernel's table-barrier waits: 2 s (a copy of a few tens of KB
 // that has not landed by then never will), 1 ms under CF_FLAG_DEBUG_STALL.
 uint64_t wait_limit_ns(uint32_t flags)
 {
@@ -1032,7 +1032,7 @@ int run(Request &q)
         goto cleanup;
     }
     if (ho->err & cf::ERR_TIMEOUT) {
-        rc = fail(CF_ETIMEOUT, "a bounded device wait (TMA tile barrier) gave up");
+        rc = fail(CF_ETIMEOUT, "a bounded device wait (table copy or gridding barrier) gave up");
         goto cleanup;
     }
     if (ho->err) {
@@ -1065,7 +1065,7 @@ int run(Request &q)
         for (int t = 0; t < ncat; ++t)
             res->n_kernels += cf::grid_kernels() +
                               (c->periodic ? 0 : cf::bbox_kernels(cats[t]->n));
-        res->n_kernels += PL.kernels;  // work list, window pre-pass, pair kernel
+        res->n_kernels += PL.kernels;  // neighbour lists, pair kernel
     }
     rc = CF_OK;
 cleanup:
@@ -1513,43 +1513,6 @@ namespace {
 
 std::mutex g_noalloc_mu;
 
-// Unique id of the calling thread's current CUDA context (cuCtxGetId, reached
-// through the runtime's driver entry points so the library does not link the
-// driver library).  A device reset or a new context gets a new id.
-typedef int (*PfnCtxGetCurrent)(void **);
-typedef int (*PfnCtxGetId)(void *, unsigned long long *);
-
-bool current_context_id(int dev, unsigned long long &id)
-{
-    static PfnCtxGetCurrent get_current = nullptr;
-    static PfnCtxGetId get_id = nullptr;
-    static bool looked_up = false;
-    if (!looked_up) {  // under g_noalloc_mu
-        looked_up = true;
-        cudaDriverEntryPointQueryResult q1, q2;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", (void **)&get_current, 12000,
-                                             cudaEnableDefault, &q1) != cudaSuccess ||
-            q1 != cudaDriverEntryPointSuccess)
-            get_current = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", (void **)&get_id, 12000,
-                                             cudaEnableDefault, &q2) != cudaSuccess ||
-            q2 != cudaDriverEntryPointSuccess)
-            get_id = nullptr;
-        cudaGetLastError();
-    }
-    if (!get_current || !get_id)
-        return false;
-    void *ctx = nullptr;
-    if (get_current(&ctx) != 0 || !ctx) {
-        // no current context yet: make the device's primary context current
-        if (cudaSetDevice(dev) != cudaSuccess || get_current(&ctx) != 0 || !ctx) {
-            cudaGetLastError();
-            return false;
-        }
-    }
-    return get_id(ctx, &id) == 0;
-}
-
 // Device address of the static scratch in the current context.  The lookup
 // (cudaGetSymbolAddress, with the device current) runs once per CUDA context:
 // the first call on a device, and again after a device reset or on another
@@ -1565,7 +1528,7 @@ int noalloc_scratch(int dev, void **out)
 {
     std::lock_guard<std::mutex> lock(g_noalloc_mu);
     unsigned long long id = 0;
-    const bool have_id = current_context_id(dev, id);
+    const bool have_id = cf::current_context_id(dev, id);
     if (have_id)
         for (const NoallocAddr &a : g_noalloc_addr)
             if (a.ptr && a.ctx_id == id) {
@@ -1749,7 +1712,7 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     cf::GridTemps tmp = {};
     cf::Nbr *nbr = nullptr;
     unsigned *nbr_count = nullptr;
-    // Carve the grids, temporaries and the work list for the current geometry
+    // Carve the grids, temporaries and the neighbour lists for the current geometry
     // out of the array; if they do not fit, plan coarser (columns at least
     // Rmax / refine wide stay correct at any width, and fewer z-cells only make
     // the in-column sort work harder) and try again.
@@ -1880,7 +1843,7 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     if (h.err & cf::ERR_COORD)
         return fail(CF_EINVAL, "coordinate outside [0, boxsize) or non-finite");
     if (h.err & cf::ERR_TIMEOUT)
-        return fail(CF_ETIMEOUT, "a bounded device wait (TMA tile barrier) gave up");
+        return fail(CF_ETIMEOUT, "a bounded device wait (table copy or gridding barrier) gave up");
     if (h.err)
         return fail(CF_EDEVICE, "kernel reported an internal inconsistency");
     const uint64_t mult = autocorr ? 2u : 1u;
@@ -1891,7 +1854,7 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     res->n_rechecked = h.diag[2];
     for (int t = 0; t < ncat; ++t)
         res->n_kernels += cf::grid_kernels() + (c->periodic ? 0 : cf::bbox_kernels(cats[t]->n));
-    res->n_kernels += PL.kernels;  // work list, window pre-pass, pair kernel
+    res->n_kernels += PL.kernels;  // neighbour lists, pair kernel
     return CF_OK;
 }
 

@@ -124,7 +124,7 @@ struct PairParams {
     int parts;          // chunk tasks: shares a chunk's neighbour list is split into
     int split_all;      // batches: every chunk is split (else the last eighth)
     uint32_t flags;
-    uint64_t wait_ns;   // limit of every tile-barrier wait (then the error word gets ERR_TIMEOUT)
+    uint64_t wait_ns;   // limit of every table-barrier wait (then the error word gets ERR_TIMEOUT)
     // radii (binary64 decisions on bounding boxes)
     double prune_r2;    // prune a column pair if its xy gap^2 >= prune_r2
     double rz;          // z reach: Rmax (xi) or pimax (rp-pi)

@@ -25,12 +25,53 @@
 #include <float.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "cf_internal.cuh"
 #include "grid.cuh"
 #include "launch.cuh"
 
 namespace cf {
+
+namespace {
+
+// Unique id of the calling thread's current CUDA context (cuCtxGetId, reached
+// through the runtime's driver entry points so the library does not link the
+// driver library).  A device reset or a new context gets a new id.
+typedef int (*PfnCtxGetCurrent)(void **);
+typedef int (*PfnCtxGetId)(void *, unsigned long long *);
+
+}  // namespace
+
+bool current_context_id(int dev, unsigned long long &id)
+{
+    static PfnCtxGetCurrent get_current = nullptr;
+    static PfnCtxGetId get_id = nullptr;
+    static std::once_flag once;
+    std::call_once(once, []() {
+        cudaDriverEntryPointQueryResult q1, q2;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", (void **)&get_current, 12000,
+                                             cudaEnableDefault, &q1) != cudaSuccess ||
+            q1 != cudaDriverEntryPointSuccess)
+            get_current = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", (void **)&get_id, 12000,
+                                             cudaEnableDefault, &q2) != cudaSuccess ||
+            q2 != cudaDriverEntryPointSuccess)
+            get_id = nullptr;
+        cudaGetLastError();
+    });
+    if (!get_current || !get_id)
+        return false;
+    void *ctx = nullptr;
+    if (get_current(&ctx) != 0 || !ctx) {
+        // no current context yet: make the device's primary context current
+        if (cudaSetDevice(dev) != cudaSuccess || get_current(&ctx) != 0 || !ctx) {
+            cudaGetLastError();
+            return false;
+        }
+    }
+    return get_id(ctx, &id) == 0;
+}
 
 namespace {
 
@@ -473,9 +514,11 @@ struct GridArgs {
 };
 
 // Barrier of the whole (cooperatively launched) grid: arrive, then wait until the
-// count reaches goal, at most 2 s.  False in every thread of the block if the wait
+// count reaches goal, at most limit_s seconds: 2, but 300 at the first barrier, where
+// blocks may still wait for another call's kernels to leave the SMs.  False in every thread of the block if the wait
 // gave up (the error word says so; no later kernel touches the results).
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned goal, unsigned *err)
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned goal, unsigned *err,
+                                             unsigned limit_s = 2u)
 {
     __syncthreads();
     bool ok = true;
@@ -488,7 +531,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned goal, unsig
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if (v >= goal)
                 break;
-            if ((it & 63u) == 63u && global_ns() - t0 > 2000000000ull) {
+            if ((it & 63u) == 63u && global_ns() - t0 > limit_s * 1000000000ull) {
                 atomicOr(err, ERR_TIMEOUT);
                 ok = false;
                 break;
@@ -527,7 +570,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_grid(const __grid_constant__ G
         counts[q] = 0u;
     for (long long q = first; q < g.ncols; q += stride)
         A.out.colbox[q] = empty_box();
-    if (!grid_barrier(A.bar, nblk, A.err))
+    if (!grid_barrier(A.bar, nblk, A.err, 300u))
         return;
     assign_points<T>(x, y, z, A.n, g, A.t.cell_of, A.t.slot, counts, A.err);
     if (!grid_barrier(A.bar, 2u * nblk, A.err))
@@ -875,6 +918,49 @@ __global__ void __launch_bounds__(256) kb_padfill(const GridBatch B)
                    S.out.cell_start[(long long)(col + 1) * g.nz], S.pad[col], threadIdx.x & 31);
 }
 
+// Gridding launches of one device run one after another, whatever their streams: two
+// grids half resident each would wait for one another.  One event per context (it dies
+// with its context: after a device reset the context has a new id), kept for the life
+// of the process.
+struct GridOrder {
+    std::mutex mu;
+    unsigned long long ctx[64] = {};
+    cudaEvent_t done[64] = {};
+    int next = 0;
+};
+GridOrder g_order;
+
+template <class F>
+cudaError_t in_order(cudaStream_t st, F &&launch)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    int dev = 0;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e || (e = cudaGetDevice(&dev)))
+        return e;
+    unsigned long long id = 0;
+    if (cap != cudaStreamCaptureStatusNone)  // an event recorded here would belong to the capture
+        return launch();
+    if (!current_context_id(dev, id))
+        id = ~(unsigned long long)dev;
+    std::lock_guard<std::mutex> lock(g_order.mu);
+    int k = 0;
+    while (k < 64 && !(g_order.done[k] && g_order.ctx[k] == id))
+        ++k;
+    if (k < 64) {
+        e = cudaStreamWaitEvent(st, g_order.done[k], 0);
+    } else {
+        k = g_order.next;
+        g_order.next = (k + 1) % 64;
+        g_order.ctx[k] = id;
+        g_order.done[k] = nullptr;
+        e = cudaEventCreateWithFlags(&g_order.done[k], cudaEventDisableTiming);
+    }
+    if (!e)
+        e = launch();
+    return e ? e : cudaEventRecord(g_order.done[k], st);
+}
+
 template <class T>
 cudaError_t build_grid_t(GridArgs &A, int sms, cudaStream_t st)
 {
@@ -891,8 +977,10 @@ cudaError_t build_grid_t(GridArgs &A, int sms, cudaStream_t st)
     if (blocks < 1)
         blocks = 1;
     void *args[] = {&A};
-    return cudaLaunchCooperativeKernel((const void *)k_grid<T>, dim3((unsigned)blocks), dim3(SORT_THREADS), args, 0,
-                                       st);
+    return in_order(st, [&]() {
+        return cudaLaunchCooperativeKernel((const void *)k_grid<T>, dim3((unsigned)blocks), dim3(SORT_THREADS), args,
+                                           0, st);
+    });
 }
 
 template <class T>

@@ -18,6 +18,10 @@ struct GridTemps {
     uint32_t *bsum;      // grid_max_blocks: padded entries of each block's columns
 };
 
+// Unique id of the calling thread's current CUDA context (device dev's primary context
+// if there is none yet); false if the driver does not say.
+bool current_context_id(int dev, unsigned long long &id);
+
 // Blocks of one gridding launch, at most.
 int grid_max_blocks(int sms);
 
