@@ -224,7 +224,8 @@ int cf_countpairs_xi_noalloc(int autocorr, const cf_catalog *d1, const cf_catalo
  * one persistent kernel per kind of count (DD(r) or DD(rp, pi), float32 or
  * binary64, kernel shape) whose CTAs attach to one job after another (the GPU
  * analogue of the paper's OpenMP loop over cell pairs, Sec. 2.1): a run is 13
- * launches plus one per kind, whatever the number of jobs.  With
+ * launches plus one per kind (two per kind where a batch has float32 and binary64
+ * jobs: those run beside each other on a second stream), whatever the number of jobs.  With
  * use_graph the whole sequence is captured once into a CUDA graph and replayed
  * by later runs.  A job's res->n_kernels is 0 (the launches are shared; the
  * batch's count is in cf_batch_stats).

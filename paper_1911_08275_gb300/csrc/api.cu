@@ -1909,6 +1909,7 @@ struct cf_batch {
     unsigned *d_wpre = nullptr;          // neighbour-list blocks: prefix over the jobs
     unsigned wblocks = 0;
     cudaStream_t own = nullptr;
+    cf::BatchSide side = {};             // second stream of runs with both kinds of precision
     cudaEvent_t ev[4] = {};
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -2290,7 +2291,7 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
     if (b->plan.start.size() > (size_t)BATCH_STARTS * b->sms)
         return fail(CF_EDEVICE, "batch plan: more CTAs than expected");
     b->blocks = 0;
-    for (const auto &gr : b->plan.groups)
+    for (const auto &gr : b->plan.launches)
         b->blocks = std::max(b->blocks, gr.blocks);
     if ((e = cudaMemcpy(b->d_jobs, hp.data(), sizeof(cf::PairParams) * nj, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(b->d_list, b->plan.list.data(), sizeof(int) * nj, cudaMemcpyHostToDevice)) ||
@@ -2305,7 +2306,7 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
                             cudaMemcpyHostToDevice)))
             return cuda_fail(e, "H2D batch gridding plan");
     // a memset, the batched gridding, the neighbour lists, a pair kernel per kind of count
-    b->n_kernels = 1 + cf::grid_batch_kernels() + 1 + b->plan.groups.size();
+    b->n_kernels = 1 + cf::grid_batch_kernels() + 1 + b->plan.launches.size();
     b->planned = true;
     (void)st;
     return CF_OK;
@@ -2326,7 +2327,7 @@ int batch_issue(cf_batch *b, cudaStream_t st, bool capturing)
     if ((e = cf::launch_neighbours_batch(b->d_jobs, b->d_wpre, nj, b->wblocks, st)))
         return cuda_fail(e, "batched neighbour lists");
     if ((!capturing && (e = cudaEventRecord(b->ev[1], st))) ||
-        (e = cf::launch_batch(b->plan, b->d_jobs, b->d_list, b->d_start, st)) ||
+        (e = cf::launch_batch(b->plan, b->d_jobs, b->d_list, b->d_start, b->side, st)) ||
         (!capturing && (e = cudaEventRecord(b->ev[2], st))) ||
         (e = cudaMemcpyAsync(b->h_out, b->d_out, b->out_words * 8, cudaMemcpyDeviceToHost, st)) ||
         (!capturing && (e = cudaEventRecord(b->ev[3], st))))
@@ -2351,6 +2352,10 @@ int batch_run(cf_batch *b, cudaStream_t user, int use_graph, cf_batch_stats *sta
         if ((e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev)))
             return cuda_fail(e, "device attribute");
         if ((e = cudaStreamCreateWithFlags(&b->own, cudaStreamNonBlocking)))
+            return cuda_fail(e, "batch stream");
+        if ((e = cudaStreamCreateWithFlags(&b->side.stream, cudaStreamNonBlocking)) ||
+            (e = cudaEventCreateWithFlags(&b->side.fork, cudaEventDisableTiming)) ||
+            (e = cudaEventCreateWithFlags(&b->side.join, cudaEventDisableTiming)))
             return cuda_fail(e, "batch stream");
         for (auto &ev : b->ev)
             if ((e = cudaEventCreate(&ev)))
@@ -2515,8 +2520,12 @@ int cf_batch_destroy(cf_batch *b)
     if (!b)
         return CF_OK;
     batch_free_plan(b);
-    if (b->own)
-        cudaStreamDestroy(b->own);
+    for (cudaStream_t s : {b->own, b->side.stream})
+        if (s)
+            cudaStreamDestroy(s);
+    for (cudaEvent_t s : {b->side.fork, b->side.join})
+        if (s)
+            cudaEventDestroy(s);
     for (auto &ev : b->ev)
         if (ev)
             cudaEventDestroy(ev);

@@ -13,9 +13,9 @@
 // Measured (a run's device time, graph replay, GB300), before -- one kernel for all
 // kinds, CTAs claiming column pairs from one queue over all jobs, so that nearly
 // every CTA loaded nearly every job's tables -- and now: 480 jobs of 200 to 8,000
-// points 6.5 -> 1.06 ms; 48 jobs of 12,500 to 500,000 points 283 -> 49 ms (with
+// points 6.5 -> 0.97 ms; 48 jobs of 12,500 to 500,000 points 283 -> 44.7 ms (with
 // every chunk of a dense job one task the last tasks ran alone for a third of the
-// time: 75 ms); 100 jobs 140 -> 2.1 ms.
+// time: 75 ms; all kinds on one stream 49 ms); 100 jobs 140 -> 2.1 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -29,6 +29,9 @@
 namespace cf {
 
 namespace {
+
+// CTAs per SM of the binary64 counts beside float32 counts (of three in all).
+constexpr int F64_BESIDE = 2;
 
 // Fewest unclaimed tasks for which a CTA joins a job that others work on.
 constexpr unsigned JOIN_TASKS = 4 * WARPS;
@@ -198,39 +201,80 @@ cudaError_t plan_batch(const std::vector<int> &path, const std::vector<int> &sme
     std::sort(order.begin(), order.end(), [&](int a, int b) {
         return path[a] != path[b] ? path[a] < path[b] : work[a] != work[b] ? work[a] > work[b] : a < b;
     });
+    struct Kind {
+        BatchLaunch g;
+        int per_sm, f64;
+        double total;
+    };
+    std::vector<Kind> kinds;
+    int has[2] = {0, 0};
     for (size_t k = 0; k < order.size();) {
-        BatchGroup g{};
+        Kind q{};
+        BatchLaunch &g = q.g;
         g.path = path[order[k]];
         g.first = (int)k;
-        double total = 0.0;
         for (; k < order.size() && path[order[k]] == g.path; ++k) {
             g.smem = std::max(g.smem, smem[order[k]]);
-            total += work[order[k]];
+            q.total += work[order[k]];
             ++g.n;
         }
-        int occ = 0;
-        const cudaError_t e = occupancy_of(group_of(g.path).kern, g.smem, occ);
+        cudaError_t e = occupancy_of(group_of(g.path).kern, g.smem, q.per_sm);
         if (e)
             return e;
-        if (occ < 1)
+        if (q.per_sm < 1)
             return cudaErrorInvalidConfiguration;
-        g.blocks = sms * occ;
-        for (int q = g.first; q < g.first + g.n; ++q) {
-            PairParams &P = jobs[order[q]];
-            const double warps = std::max(1.0, work[order[q]] / total * g.blocks) * WARPS;
+        // both streams' CTAs share SMs: one split of the L1 for all, the largest
+        if ((e = cudaFuncSetAttribute(group_of(g.path).kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      cudaSharedmemCarveoutMaxShared)))
+            return e;
+        q.f64 = g.path == BATCH_XI64 || g.path == BATCH_RPPI64;
+        has[q.f64] = 1;
+        for (int j = g.first; j < g.first + g.n; ++j) {
+            PairParams &P = jobs[order[j]];
+            const double warps = std::max(1.0, work[order[j]] / q.total * sms * q.per_sm) * WARPS;
             const double chunks = (double)(P.A.n + (long long)P.g.ncols * (COL_PAD / 2)) / group_of(g.path).ch + 1.0;
             P.parts = task_parts(chunks, warps, P.nstencil);
             P.split_all = chunks < 8.0 * warps ? 1 : 0;
         }
+        kinds.push_back(q);
+    }
+    const auto add = [&](const Kind &q, int per_sm, int side) {
+        if (per_sm < 1)
+            return;
+        BatchLaunch g = q.g;
+        g.blocks = sms * per_sm;
+        g.side = side;
         g.start0 = (int)plan.start.size();
         double sum = 0.0;
         int j = -1;
         for (int b = 0; b < g.blocks; ++b) {
-            while (j + 1 < g.n && (j < 0 || sum < total * (b + 0.5) / g.blocks))
+            while (j + 1 < g.n && (j < 0 || sum < q.total * (b + 0.5) / g.blocks))
                 sum += work[order[g.first + ++j]];
             plan.start.push_back(j);
         }
-        plan.groups.push_back(g);
+        plan.launches.push_back(g);
+    };
+    // Binary64 jobs beside float32 jobs: the binary64 counts wait for their pipe and
+    // leave four fifths of the issue slots, the float32 counts issue and leave that pipe
+    // idle.  So the binary64 kinds run on a second stream with F64_BESIDE CTAs per SM, the
+    // float32 kinds with the rest of theirs; each stream ends with the other's
+    // kinds in what room it had, which join the jobs that are not done.  Measured (graph
+    // replay, one stream / two with 1 / 2 CTAs per SM): 48 jobs of 12,500 to 500,000 points
+    // 49.3 / 47.8 / 44.7 ms; 480 small jobs 1.042 / 0.979 / 0.967; 900 tiny jobs 0.613 / 0.496 /
+    // 0.527; 100 jobs 2.18 / 2.04 / 2.09.
+    plan.forked = has[0] && has[1];
+    if (!plan.forked) {
+        for (const Kind &q : kinds)
+            add(q, q.per_sm, 0);
+    } else {
+        for (int pass = 0; pass < 2; ++pass)  // its own kinds first, then the other's
+            for (int side = 1; side >= 0; --side)
+                for (const Kind &q : kinds) {
+                    if (q.f64 != (pass ? !side : side))
+                        continue;
+                    const int beside = std::min(F64_BESIDE, std::max(1, q.per_sm - 1));
+                    add(q, side ? beside : std::max(pass ? 0 : 1, q.per_sm - beside), side);
+                }
     }
     plan.list = order;
     return cudaSuccess;
@@ -246,18 +290,24 @@ cudaError_t launch_neighbours_batch(const PairParams *jobs, const unsigned *pre,
 }
 
 cudaError_t launch_batch(const BatchPlan &plan, const PairParams *jobs, const int *list, const int *start,
-                         cudaStream_t st)
+                         const BatchSide &side, cudaStream_t st)
 {
-    for (const BatchGroup &g : plan.groups) {
+    cudaError_t e = cudaSuccess;
+    if (plan.forked && ((e = cudaEventRecord(side.fork, st)) || (e = cudaStreamWaitEvent(side.stream, side.fork, 0))))
+        return e;
+    for (size_t k = 0; k < plan.launches.size() && !e; ++k) {
+        const BatchLaunch &g = plan.launches[k];
         const int *l = list + g.first, *s = start + g.start0;
         int n = g.n;
         void *args[] = {(void *)&jobs, (void *)&l, (void *)&s, (void *)&n};
-        const cudaError_t e = cudaLaunchKernel(group_of(g.path).kern, dim3(g.blocks), dim3(THREADS), args,
-                                               (size_t)g.smem, st);
-        if (e)
-            return e;
+        e = cudaLaunchKernel(group_of(g.path).kern, dim3(g.blocks), dim3(THREADS), args, (size_t)g.smem,
+                             g.side ? side.stream : st);
     }
-    return cudaSuccess;
+    if (plan.forked) {  // the streams join also after a failed launch
+        const cudaError_t r = cudaEventRecord(side.join, side.stream), w = cudaStreamWaitEvent(st, side.join, 0);
+        e = e ? e : r ? r : w;
+    }
+    return e;
 }
 
 }  // namespace cf

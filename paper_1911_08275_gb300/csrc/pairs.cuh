@@ -57,14 +57,21 @@ enum : int {
 };
 constexpr int BATCH_MAX = 1024;  // jobs per batched launch
 
-// The jobs of one kind of count: list[first .. first + n), CTA b's first job (index
-// into that range) at start[start0 + b].
-struct BatchGroup {
-    int path, first, n, blocks, start0, smem;
+// A launch over the jobs of one kind of count: list[first .. first + n), CTA b's first
+// job (index into that range) at start[start0 + b]; side: on the second stream.
+struct BatchLaunch {
+    int path, first, n, blocks, start0, smem, side;
 };
 struct BatchPlan {
-    std::vector<BatchGroup> groups;
+    std::vector<BatchLaunch> launches;  // in the order they are issued
+    bool forked;                        // some are on the second stream
     std::vector<int> list, start;
+};
+
+// The second stream of a plan that forks and the events that bracket it.
+struct BatchSide {
+    cudaStream_t stream;
+    cudaEvent_t fork, join;
 };
 
 // Path of a job: float32 (float32 DD(r) in the kernel shape chunk x pp: 16 x 2,
@@ -88,6 +95,6 @@ cudaError_t launch_neighbours_batch(const PairParams *jobs, const unsigned *pre,
 
 // The kernels of a plan; list and start are device copies of the plan's.
 cudaError_t launch_batch(const BatchPlan &plan, const PairParams *jobs, const int *list, const int *start,
-                         cudaStream_t st);
+                         const BatchSide &side, cudaStream_t st);
 
 }  // namespace cf
