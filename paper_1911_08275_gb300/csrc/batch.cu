@@ -13,7 +13,7 @@
 // Measured (a run's device time, graph replay, GB300), before -- one kernel for all
 // kinds, CTAs claiming column pairs from one queue over all jobs, so that nearly
 // every CTA loaded nearly every job's tables -- and now: 480 jobs of 200 to 8,000
-// points 6.5 -> 0.97 ms; 48 jobs of 12,500 to 500,000 points 283 -> 44.7 ms (with
+// points 6.5 -> 0.97 ms; 48 jobs of 12,500 to 500,000 points 283 -> 43.6 ms (with
 // every chunk of a dense job one task the last tasks ran alone for a third of the
 // time: 75 ms; all kinds on one stream 49 ms); 100 jobs 140 -> 2.1 ms.
 #include <cuda_runtime.h>
@@ -157,8 +157,8 @@ Group group_of(int path)
     case BATCH_XI32_32x1 + BATCH_LIN: return group<Count32<32, 1, false, false, 1>, 3>();
     case BATCH_RPPI32: return group<CountRp32<16, 2, false, false, 0>, 3>();
     case BATCH_RPPI32 + BATCH_LIN: return group<CountRp32<16, 2, false, false, 1>, 3>();
-    case BATCH_XI64: return group<Cull64<0, false, false>, 3>();
-    default: return group<Cull64<1, false, false>, 3>();
+    case BATCH_XI64: return group<Cull64<0, false, false, 2>, 3>();
+    default: return group<Cull64<1, false, false, 2>, 3>();
     }
 }
 

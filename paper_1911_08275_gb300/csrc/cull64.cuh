@@ -7,15 +7,15 @@
 // pair is dropped when its float32 distance proves it out of reach (the bound
 // that brackets the last edge in the float32 tables, build_thresholds; pimax plus
 // the window slack for |dz|), as the bounding boxes and z windows drop it.  The
-// others are queued per warp, and 32 at a time are evaluated, one per lane, so
-// the binary64 pipe works on full warps of pairs that count (all but those in
+// others are queued per warp, and 32 or 64 at a time are evaluated, one or two per lane,
+// so the binary64 pipe works on full warps of pairs that count (all but those in
 // the thin shell of the bound and below the first edge).
 //
 // Bound: the binary64 pipe, 8 instructions per counted pair (DD(rp, pi): 6).  1.2M
 // clustered points, kernel ms at Rmax 10 / 25 / 50 (GB300): 5.78 / 40.8 / 198 when every
-// pair of the windows was evaluated in binary64, 0.93 / 10.3 / 80.5 now (0.65e9 pairs
+// pair of the windows was evaluated in binary64, 0.91 / 10.2 / 80.4 now (0.65e9 pairs
 // within reach at Rmax 25, 5.1e9 at 50: the pipe alone takes 8.9 and 69.5 ms);
-// DD(rp, pi) 14 x 40, pimax 40: 56.8 -> 22.0 (15.8).  Tests of the periodic shift as
+// DD(rp, pi) 14 x 40, pimax 40: 56.8 -> 21.6 (15.8).  Tests of the periodic shift as
 // doubles had cost 11.5 instead of 10.3 ms at Rmax 25, a binary search of the
 // edges instead of the start table 24.3 instead of 22.0 ms for DD(rp, pi).
 #pragma once
@@ -68,21 +68,37 @@ __device__ __forceinline__ int bin_pi(double v, const double *Pe, int n, float s
     return p;
 }
 
-// Evaluate the n <= 32 pairs from entry `first` of the warp's queue, one per lane.
-template <int KIND, bool WACC>
-__device__ __noinline__ void eval64(const PairParams &P, unsigned char *smem, const FlagQueue *fq,
+// Pairs waiting to be evaluated (one queue per warp; at most 32 EV - 1 <= 63 wait when up
+// to 32 more are pushed).
+struct CullQueue {
+    int i[96], j[96], image[96];
+};
+
+// Evaluate the n <= 32 EV pairs from entry `first` of the warp's queue, EV per lane,
+// their points requested together.
+template <int KIND, bool WACC, int EV>
+__device__ __noinline__ void eval64(const PairParams &P, unsigned char *smem, const CullQueue *fq,
                                     int first, int n, uint32_t hist, double *acc)
 {
     const int lane = threadIdx.x & 31, nb = P.nbins, npi = P.npibins;
     const double *E2 = reinterpret_cast<const double *>(smem + P.e2_off), *Pe = E2 + nb + 1;
     const unsigned char *guess = smem + P.guess_off;
     __syncwarp();
-    if (lane < n) {
-        const int i = fq->i[first + lane], j = fq->j[first + lane], m = fq->image[first + lane];
-        const double4_32a a = P.A.pos64[i], b = P.B.pos64[j];
+    double4_32a a[EV], b[EV];
+#pragma unroll
+    for (int u = 0; u < EV; ++u) {  // (entry `first` in the place of those beyond n)
+        const int e = first + (lane + 32 * u < n ? lane + 32 * u : 0);
+        a[u] = P.A.pos64[fq->i[e]];
+        b[u] = P.B.pos64[fq->j[e]];
+    }
+#pragma unroll
+    for (int u = 0; u < EV; ++u) {
+        if (lane + 32 * u >= n)
+            continue;
+        const int m = fq->image[first + lane + 32 * u];
         // canonical differences: fl(x_j - x_i), then fl(+ S) where the image is shifted
         // (integer tests: a compare of doubles would hold the binary64 pipe too)
-        double dx = __dsub_rn(b.x, a.x), dy = __dsub_rn(b.y, a.y), dz = __dsub_rn(b.z, a.z);
+        double dx = __dsub_rn(b[u].x, a[u].x), dy = __dsub_rn(b[u].y, a[u].y), dz = __dsub_rn(b[u].z, a[u].z);
         if (m != IMAGE_NONE) {
             const int qx = (m & 3) - 1, qy = ((m >> 2) & 3) - 1, qz = ((m >> 4) & 3) - 1;
             if (qx)
@@ -103,7 +119,7 @@ __device__ __noinline__ void eval64(const PairParams &P, unsigned char *smem, co
         if (k >= 0) {
             red_shared1(hist + (uint32_t)k * (KIND == 0 ? 128u : 4u));
             if (WACC) {  // Code 1's weight: the exact product and square root
-                const double pw = P.weighted ? __dmul_rn(a.w, b.w) : 1.0;
+                const double pw = P.weighted ? __dmul_rn(a[u].w, b[u].w) : 1.0;
                 atomicAdd(acc + 2 * k, pw);
                 if (P.want_r)
                     atomicAdd(acc + 2 * k + 1, __dmul_rn(__dsqrt_rn(s2), pw));
@@ -115,8 +131,9 @@ __device__ __noinline__ void eval64(const PairParams &P, unsigned char *smem, co
 
 // KIND 0: DD(r), a histogram of nbins rows of 32 words (a word per lane) shared by
 // the CTA's warps.  KIND 1: DD(rp, pi), P.hcopies copies of nbins * npibins words.
-// WACC: binary64 sums [copy][slot][w, r w] (DD(r): one copy per warp).
-template <int KIND, bool EVALS, bool WACC>
+// WACC: binary64 sums [copy][slot][w, r w] (DD(r): one copy per warp).  EV: pairs per
+// lane of one evaluation.
+template <int KIND, bool EVALS, bool WACC, int EV>
 struct Cull64 {
     static constexpr int I = 16, PP = 2, CH = I * PP, JS = 128 / I;
     struct State {
@@ -171,19 +188,19 @@ struct Cull64 {
         return true;
     }
 
-    // Evaluate what the warp's queue holds beyond `keep` pairs (keep = 31: full
-    // warps only; 0: everything).
+    // Evaluate what the warp's queue holds beyond `keep` pairs (keep = 32 EV - 1:
+    // full warps only; 0: everything).
     static __device__ __forceinline__ void drain(const PairParams &P, unsigned char *smem, State &st,
-                                                 const FlagQueue *fq, int keep)
+                                                 const CullQueue *fq, int keep)
     {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, copy = warp % P.hcopies;
         uint32_t *hw = reinterpret_cast<uint32_t *>(smem + P.hist_off) + (KIND == 0 ? lane : copy * slots(P));
         double *acc = reinterpret_cast<double *>(smem + P.acc_off) + (long long)copy * slots(P) * 2;
         while (st.qn > keep) {
-            const int n = min(32, st.qn);
+            const int n = min(32 * EV, st.qn);
             st.qn -= n;
-            eval64<KIND, WACC>(P, smem, fq, st.qn, n, smem_u32(hw), acc);
-            ++st.pending;
+            eval64<KIND, WACC, EV>(P, smem, fq, st.qn, n, smem_u32(hw), acc);
+            st.pending += EV;
         }
     }
 
@@ -191,7 +208,7 @@ struct Cull64 {
                                                 unsigned c, unsigned part, unsigned parts)
     {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ii = lane % I, jj = lane / I;
-        FlagQueue *fq = reinterpret_cast<FlagQueue *>(smem + P.queue_off) + warp;
+        CullQueue *fq = reinterpret_cast<CullQueue *>(smem + P.queue_off) + warp;
         const uint32_t ring = smem_u32(smem + P.ring_off) + (uint32_t)warp * RingXYZ::BYTES;
         const int ib = (int)(c * CH);
         Chunk<I, PP> C;
@@ -204,7 +221,7 @@ struct Cull64 {
             [&](int k, int code) { image = C.shift(P, k, code, XH, YH, ZH); },
             [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {
                 cull_piece<KIND, I, PP, EVALS>(P, fq, st.qn, st.n_eval, addr, j0, j1, jlo, jhi, tri, jj, ii, XH,
-                                               YH, ZH, ib, image, C.vmask, [&]() { drain(P, smem, st, fq, 31); });
+                                               YH, ZH, ib, image, C.vmask, [&]() { drain(P, smem, st, fq, 32 * EV - 1); });
                 flush(P, smem, st);
             });
         // entries name their points, so a partly filled queue waits for the next task
@@ -234,7 +251,7 @@ struct Cull64 {
     static __device__ __forceinline__ void fini(const PairParams &P, unsigned char *smem, State &st)
     {
         const int tid = threadIdx.x, lane = tid & 31, n = slots(P);
-        drain(P, smem, st, reinterpret_cast<FlagQueue *>(smem + P.queue_off) + (tid >> 5), 0);
+        drain(P, smem, st, reinterpret_cast<CullQueue *>(smem + P.queue_off) + (tid >> 5), 0);
         __syncthreads();
         const uint32_t *hist = reinterpret_cast<const uint32_t *>(smem + P.hist_off);
         const double *acc = reinterpret_cast<const double *>(smem + P.acc_off);

@@ -296,9 +296,9 @@ __device__ __forceinline__ void for_windows(const PairParams &P, int col, int ib
 
 // Queue the pairs of a piece [j0, j1) of a window [jlo, jhi) that the float32 bounds
 // do not prove out of reach (set_cull): KIND 0 by r^2, KIND 1 by rp^2 and |dz|.
-// drain() is called whenever pairs were added (at most 31 may be left waiting).
-template <int KIND, int I, int PP, bool EVALS, class Drain>
-__device__ __forceinline__ void cull_piece(const PairParams &P, FlagQueue *fq, int &qn, u64 &n_eval,
+// drain() is called whenever pairs were added and leaves room for 32 more.
+template <int KIND, int I, int PP, bool EVALS, class Queue, class Drain>
+__device__ __forceinline__ void cull_piece(const PairParams &P, Queue *fq, int &qn, u64 &n_eval,
                                            uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri, int jj,
                                            int ii, const u64 (&XH)[PP], const u64 (&YH)[PP],
                                            const u64 (&ZH)[PP], int ib, int image, unsigned vmask, Drain drain)

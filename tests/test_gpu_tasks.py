@@ -189,3 +189,22 @@ def test_calls_from_threads_on_their_own_streams(cuda_device):
     for t in threads:
         t.join()
     assert not bad
+
+
+@pytest.mark.parametrize("n2", [599_999, 600_000])
+def test_binary64_evaluation_widths(cuda_device, n2):
+    # a few primaries against more secondaries than the size where DD(r) goes from two
+    # pairs per lane and evaluation to one, with sums (tolerance: order of summation)
+    a = synth.uniform_box(301, 200.0, seed=270)
+    b = synth.uniform_box(n2, 200.0, seed=271)
+    rng = np.random.default_rng(272)
+    w, w2 = rng.uniform(0.5, 1.5, a.n), rng.uniform(0.5, 1.5, b.n)
+    e = synth.log_edges(0.5, 12.0, 9)
+    x, y, z, wd = dev(a.x, a.y, a.z, w)
+    x2, y2, z2, wd2 = dev(b.x, b.y, b.z, w2)
+    r = cf.countpairs_xi(x, y, z, e, x2=x2, y2=y2, z2=z2, boxsize=200.0, mode="fp64")
+    s = cf.countpairs_xi(x, y, z, e, w=wd, x2=x2, y2=y2, z2=z2, w2=wd2, boxsize=200.0, mode="fp64")
+    cnt, ref, _ = oracle.xi(a.x, a.y, a.z, w1=w, x2=b.x, y2=b.y, z2=b.z, w2=w2, edges=e, autocorr=False,
+                            periodic=True, box=200.0)
+    assert np.array_equal(r.npairs, cnt) and np.array_equal(s.npairs, cnt)
+    assert np.allclose(s.wsum, ref, rtol=1e-12, atol=0.0)
