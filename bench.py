@@ -122,7 +122,7 @@ def load_peaks():
 
 PROFILE = os.path.join(ROOT, "profiles", "k_xi32_xi_auto_1.2M_rmax25.md")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1911_08275_gb300", "csrc", f)
-                  for f in ("pairs.cu", "cf_internal.cuh")]
+                  for f in ("count32.cuh", "tasks.cuh", "pairs_dev.cuh", "cf_internal.cuh")]
 
 
 def profile_traffic():
@@ -326,7 +326,7 @@ def batch_workload(cf, synth, torch, dev, flush):
     first run plans the batch), against the same jobs as 48 single calls
     (per-job counts must be identical); the float32 and the binary64 jobs as
     batches of their own; and 480 small jobs (launch-bound: every gridding
-    stage and the work lists of all jobs run as one launch each) with and
+    stage and the neighbour lists of all jobs run as one launch each) with and
     without the graph, and as 480 single calls."""
     jobs = [synth.batch_job(j) for j in range(48)]
     xyz = [[torch.from_numpy(v).to(dev) for v in (jb["cat"].x, jb["cat"].y, jb["cat"].z)]

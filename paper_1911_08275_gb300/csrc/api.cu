@@ -528,9 +528,8 @@ void cap_columns(long long ntot, int &ncx, int &ncy)
 // (2, 2, 1) as a good start): the column side s over which the smaller
 // catalogue holds DEFAULT_COL_POINTS points on average (an ex x ey
 // cross-section), and r = round(Rxy / s) in [1, MAX_REACH].  The smaller one
-// decides because a work item's tile copies of the secondaries are spread over
-// its primaries and its per-chunk costs over the secondaries in the windows;
-// both want enough points per column.  Degenerate extents give 2.
+// decides because a chunk's costs are spread over the secondaries in its windows and
+// a window's over its primaries; both want enough points per column.  Degenerate extents give 2.
 int default_reach(double R, double ex, double ey, double na, double nb)
 {
     const double area = ex * ey, n = std::max(std::min(na, nb), 1.0);
