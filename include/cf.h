@@ -132,7 +132,7 @@ typedef struct {
                             w_i*w_j when weighted; 0 for empty bins.  Binary64
                             mode: exact per-pair terms, sums within 1e-12
                             relative (summation order).  Float32 mode: r from
-                            the float32 squared distance corrected with the
+                            float32 differences corrected with the
                             coordinates' float32 rounding residuals (~3e-7
                             relative per pair); DD(r) terms rounded to a fixed-
                             point grid scaled by the largest weights (2^-22
