@@ -6,7 +6,7 @@
 namespace cf {
 
 // CTAs of `threads` threads per SM for a kernel with smem bytes of dynamic shared
-// memory; raises the kernel's shared-memory limit when needed (cached).
+// memory; raises the kernel's shared-memory limit when needed, never lowers it (cached).
 cudaError_t occupancy_of(const void *kern, int smem, int &occ, int threads = 256);
 
 template <class K>

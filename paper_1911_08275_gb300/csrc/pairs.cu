@@ -3,26 +3,57 @@
 
 #include <mutex>
 
+#include "grid.cuh"
 #include "launch.cuh"
 #include "pairs.cuh"
 
 namespace cf {
 
-// Per (kernel, device): the dynamic shared-memory limit set so far (only ever
-// raised) and the occupancy per shared-memory size, queried once.
+// Per kernel and context: the dynamic shared-memory limit known to be set, and the
+// occupancy per shared-memory size.  The limit is only ever raised, also when the table
+// is full and it has to be asked for: a planned batch launches with the size it was
+// planned for, whatever other calls have needed since.  (Fixed tables: the calls that
+// allocate nothing come through here too.)
 namespace {
-struct OccCache {
+struct KernelKey {
     const void *kern;
-    int dev, smem, occ;
+    unsigned long long ctx;  // a device reset drops the limits with the context
+    bool operator==(const KernelKey &o) const { return kern == o.kern && ctx == o.ctx; }
 };
-struct AttrCache {
-    const void *kern;
-    int dev, limit;
+struct LimitEntry {
+    KernelKey key;
+    int limit;
 };
-OccCache g_occ[128];
-AttrCache g_attr[64];
-int g_nocc = 0, g_nattr = 0;
+struct OccEntry {
+    KernelKey key;
+    int smem, occ;
+};
+LimitEntry g_limit[256];
+OccEntry g_occ[256];
+int g_nlimit = 0, g_nocc = 0;
 std::mutex g_occ_mu;
+
+cudaError_t raise_limit(const KernelKey &key, int smem)
+{
+    for (int q = 0; q < g_nlimit; ++q)
+        if (g_limit[q].key == key && g_limit[q].limit >= smem)
+            return cudaSuccess;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, key.kern);
+    if (!e && a.maxDynamicSharedSizeBytes < smem)
+        e = cudaFuncSetAttribute(key.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e)
+        return e;
+    const int limit = smem > a.maxDynamicSharedSizeBytes ? smem : a.maxDynamicSharedSizeBytes;
+    for (int q = 0; q < g_nlimit; ++q)
+        if (g_limit[q].key == key) {
+            g_limit[q].limit = limit;
+            return cudaSuccess;
+        }
+    if (g_nlimit < 256)
+        g_limit[g_nlimit++] = LimitEntry{key, limit};
+    return cudaSuccess;
+}
 }  // namespace
 
 cudaError_t occupancy_of(const void *kern, int smem, int &occ, int threads)
@@ -31,31 +62,21 @@ cudaError_t occupancy_of(const void *kern, int smem, int &occ, int threads)
     cudaError_t e = cudaGetDevice(&dev);
     if (e)
         return e;
+    KernelKey key{kern, 0};
+    if (!current_context_id(dev, key.ctx))
+        key.ctx = ~(unsigned long long)dev;
     std::lock_guard<std::mutex> lock(g_occ_mu);
-    AttrCache *a = nullptr;
-    for (int q = 0; q < g_nattr; ++q)
-        if (g_attr[q].kern == kern && g_attr[q].dev == dev)
-            a = &g_attr[q];
-    if (!a || a->limit < smem) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e)
-            return e;
-        if (!a && g_nattr < 64)
-            a = &g_attr[g_nattr++];
-        if (a)
-            *a = AttrCache{kern, dev, smem};
-    }
+    if ((e = raise_limit(key, smem)))
+        return e;
     for (int q = 0; q < g_nocc; ++q)
-        if (g_occ[q].kern == kern && g_occ[q].dev == dev && g_occ[q].smem == smem) {
+        if (g_occ[q].key == key && g_occ[q].smem == smem) {
             occ = g_occ[q].occ;
             return cudaSuccess;
         }
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
-    if (e)
-        return e;
-    if (g_nocc < 128)
-        g_occ[g_nocc++] = OccCache{kern, dev, smem, occ};
-    return cudaSuccess;
+    if (!e && g_nocc < 256)
+        g_occ[g_nocc++] = OccEntry{key, smem, occ};
+    return e;
 }
 
 cudaError_t launch_pairs(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st)
