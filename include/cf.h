@@ -345,6 +345,16 @@ int cf_debug_bin_tables(const double *edges, int nedges, int ncomp, double coord
 int cf_debug_pi_band(double pimax, int npibins, double coord_max, double shift_max,
                      float *pscale, float *pband);
 
+/*
+ * The grid a DD(r) call of these sizes plans, for diagnostics and tests (host
+ * only): cells gets the columns along x and y and the z-cells of a column.
+ * extent: the points' extent per axis (open box; a periodic one takes
+ * cfg->boxsize); cfg: periodic, boxsize and refine are read.  Errors: CF_EINVAL
+ * for NULL pointers, negative sizes, rmax not positive and finite.
+ */
+int cf_debug_grid(int autocorr, int64_t n1, int64_t n2, const double *extent, double rmax,
+                  const cf_config *cfg, int *cells);
+
 /* Text of the last non-zero status returned on the calling thread. */
 const char *cf_last_error(void);
 

@@ -39,7 +39,8 @@ _STATUS = {CF_EINVAL: "CF_EINVAL", CF_ENOMEM: "CF_ENOMEM", CF_ECUDA: "CF_ECUDA",
 EXPORTS = ("cf_countpairs_xi", "cf_countpairs_rp_pi", "cf_last_error", "cf_version",
            "cf_countpairs_xi_noalloc", "cf_tune_save", "cf_tune_load", "cf_tune_clear",
            "cf_tune_count", "cf_batch_create", "cf_batch_add_xi", "cf_batch_add_rp_pi",
-           "cf_batch_run", "cf_batch_destroy", "cf_debug_bin_tables", "cf_debug_pi_band")
+           "cf_batch_run", "cf_batch_destroy", "cf_debug_bin_tables", "cf_debug_pi_band",
+           "cf_debug_grid")
 
 
 class cf_catalog(ctypes.Structure):
@@ -352,6 +353,23 @@ def debug_pi_band(pimax, npibins, *, coord_max, shift_max=0.0):
     if st < 0:
         raise CfError(st, L.cf_last_error().decode())
     return np.float32(ps.value), np.float32(pb.value)
+
+
+def debug_grid(n1, n2=None, *, extent=(0.0, 0.0, 0.0), rmax, periodic=True, boxsize=420.0, refine=(0, 0, 0)):
+    """(columns in x, columns in y, z-cells) that a DD(r) call plans (``cf_debug_grid``, host only)."""
+    L = lib()
+    f = L.cf_debug_grid
+    P = ctypes.POINTER
+    f.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_int64, P(ctypes.c_double), ctypes.c_double, P(cf_config),
+                  P(ctypes.c_int)]
+    f.restype = ctypes.c_int
+    cfg = _config(CF_FLOAT64, periodic, boxsize, "fp64", False, False, refine, 0, None, False)
+    cells = (ctypes.c_int * 3)()
+    st = f(int(n2 is None), int(n1), int(n2 or 0), (ctypes.c_double * 3)(*extent), float(rmax), ctypes.byref(cfg),
+           cells)
+    if st < 0:
+        raise CfError(st, L.cf_last_error().decode())
+    return tuple(cells)
 
 
 def countpairs_xi_noalloc(x, y, z, edges, *, x2=None, y2=None, z2=None, autocorr=None,

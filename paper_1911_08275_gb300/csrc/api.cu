@@ -604,8 +604,9 @@ int plan_geom(const Request &q, const double lo[3], const double hi[3], long lon
         g.ncy = std::max(1, g.ncy / 2);
     }
     cap_columns(ntot, g.ncx, g.ncy);
-    // padded entries are indexed with 32-bit integers
-    while ((long long)g.ncx * g.ncy > 1 && ntot + 31ll * g.ncx * g.ncy > (1ll << 31) - 64) {
+    // the padded entries of a catalogue are indexed with 32-bit integers
+    const long long nmax = std::max(q.d1->n, q.autocorr ? q.d1->n : q.d2->n);
+    while ((long long)g.ncx * g.ncy > 1 && cf::padded_max(nmax, g.ncx * g.ncy) > (1ll << 31) - 64) {
         g.ncx = std::max(1, g.ncx / 2);
         g.ncy = std::max(1, g.ncy / 2);
     }
@@ -1434,6 +1435,31 @@ int cf_debug_pi_band(double pimax, int npibins, double coord_max, double shift_m
         return fail(CF_EINVAL, "bounds must be finite and >= 0");
     pi_band(pimax, npibins, coord_max, shift_max, *pscale, *pband);
     return CF_OK;
+}
+
+int cf_debug_grid(int autocorr, int64_t n1, int64_t n2, const double *extent, double rmax, const cf_config *cfg,
+                  int *cells)
+{
+    if (!extent || !cfg || !cells)
+        return fail(CF_EINVAL, "NULL argument");
+    if (n1 < 0 || n2 < 0 || !(rmax > 0.0 && std::isfinite(rmax)))
+        return fail(CF_EINVAL, "sizes must be >= 0, rmax positive and finite");
+    const double lo[3] = {0.0, 0.0, 0.0};
+    cf_catalog d1 = {}, d2 = {};
+    d1.n = n1;
+    d2.n = autocorr ? n1 : n2;
+    Request q = {};
+    q.autocorr = autocorr ? 1 : 0;
+    q.d1 = &d1;
+    q.d2 = &d2;
+    q.edges = {0.0, rmax};
+    q.cfg = cfg;
+    cf::Geom g;
+    const int rc = plan_geom(q, lo, extent, n1 + (autocorr ? 0 : n2), g);
+    cells[0] = g.ncx;
+    cells[1] = g.ncy;
+    cells[2] = g.nz;
+    return rc;
 }
 
 static_assert(CF_BIN_TABLE_MAX == cf::LUT_MAX, "the header states the table size");
