@@ -56,8 +56,9 @@ extern "C" {
 #define CF_EINVAL (-1)    /* invalid argument (see cf_last_error)               */
 #define CF_ENOMEM (-2)    /* device or host allocation failed                   */
 #define CF_ECUDA (-3)     /* a CUDA runtime call failed                         */
-#define CF_ETIMEOUT (-4)  /* a bounded device-side wait gave up (after ~2 s;
-                             the kernel returns, the context stays usable)      */
+#define CF_ETIMEOUT (-4)  /* a bounded device-side wait gave up (after ~2 s, in
+                             the gridding ~20 s; the kernel returns, the context
+                             stays usable)                                      */
 #define CF_EDEVICE (-5)   /* a kernel reported an inconsistency (error word)    */
 
 typedef enum { CF_FLOAT32 = 0, CF_FLOAT64 = 1 } cf_dtype;
@@ -79,6 +80,10 @@ typedef enum {
                                          gives up after 1 ms, so the call returns
                                          CF_ETIMEOUT; tests the bounded waits.
                                          Ignored by the other kernels.          */
+#define CF_FLAG_DEBUG_STALL_GRID (1u << 4) /* diagnostic: the gridding's stages wait
+                                         for one more block than there is and give
+                                         up after 1 ms (CF_ETIMEOUT).  Ignored by
+                                         the no-alloc entry point and by batches. */
 
 /* One catalogue: n points with coordinates x[i], y[i], z[i] of type
  * cf_config.dtype, contiguous, in device or host memory, and optional float64

@@ -413,6 +413,10 @@ struct Trace {
     }
 };
 
+// Words of 8 bytes behind a call's histogram on the device: diag(4) | err, counter | kept, - |
+// max |w| (2) | gridding tickets (one word per catalogue).
+constexpr int NTAIL = 9;
+
 struct Request {
     int kind;  // 0 xi, 1 rp-pi
     int autocorr;
@@ -761,10 +765,10 @@ int run(Request &q)
         unsigned long long *keys;
     } stage = {nullptr};
     bool resid = false;
-    unsigned *d_err = nullptr, *d_ctr = nullptr, *d_wcount = nullptr, *d_bar = nullptr;
+    unsigned *d_err = nullptr, *d_ctr = nullptr, *d_wcount = nullptr;
     cf::Nbr *nbr = nullptr;
     unsigned *nbr_count = nullptr;
-    unsigned long long *d_hist = nullptr, *d_diag = nullptr;
+    unsigned long long *d_hist = nullptr, *d_diag = nullptr, *d_ticket = nullptr;
     float *d_thr = nullptr;
     uint8_t *d_lut = nullptr;
     double *d_E2 = nullptr, *d_P = nullptr;
@@ -773,7 +777,7 @@ int run(Request &q)
         unsigned long long *diag;
         unsigned err;
         // image of the staged block (at most: keys, results, both edge arrays, thresholds, table)
-        alignas(16) unsigned long long stage[6 + 3 * cf::NBINS2D_MAX + 8 + 2 * (cf::NB_MAX + 1) + cf::NPI_MAX + 1 +
+        alignas(16) unsigned long long stage[6 + 3 * cf::NBINS2D_MAX + NTAIL + 2 * (cf::NB_MAX + 1) + cf::NPI_MAX + 1 +
                                              cf::LUT_MAX / 8 + 2];
     } *ho = nullptr;
 
@@ -802,9 +806,9 @@ int run(Request &q)
 
     {
         // Inputs and the staged block.  The block is one host image and one copy: the
-        // bounding-box keys, the zeroed results [hist | diag(4) | err, counter | kept, - |
-        // max |w| (2) | barriers (2) | wsum | rsum], squared edges, pi edges, thresholds, table.
-        const size_t nres = nslots + 8 + nacc;
+        // bounding-box keys, the zeroed results [hist | NTAIL words | wsum | rsum], squared
+        // edges, pi edges, thresholds, table.
+        const size_t nres = nslots + NTAIL + nacc;
         auto carve_inputs = [&]() {
             for (int t = 0; t < ncat; ++t) {
                 const long long n = cats[t]->n;
@@ -865,7 +869,7 @@ int run(Request &q)
         d_err = reinterpret_cast<unsigned *>(d_hist + nslots + 4);
         d_ctr = d_err + 1;
         d_wcount = d_err + 2;
-        d_bar = d_err + 6;
+        d_ticket = d_diag + 7;
         d_E2 = reinterpret_cast<double *>(d_hist + nres);
         d_P = d_E2 + nb + 1;
         d_thr = reinterpret_cast<float *>(d_P + Pe.size());
@@ -948,7 +952,7 @@ int run(Request &q)
             staged = at_lut + tb.lut_n;
         }
         if (c->periodic) {  // results and tables in one copy
-            std::memset(h0, 0, 8 * (6 + nslots + 8 + nacc));
+            std::memset(h0, 0, 8 * (6 + nslots + NTAIL + nacc));
             CF_CUDA(cudaMemcpyAsync(stage.keys, h0, staged, cudaMemcpyHostToDevice, st), "H2D tables");
         } else {  // the results were cleared with the bounding box
             const size_t from = reinterpret_cast<uint8_t *>(d_E2) - reinterpret_cast<uint8_t *>(stage.keys);
@@ -959,7 +963,7 @@ int run(Request &q)
         trace.point("tables");
         for (int t = 0; t < ncat; ++t) {
             const cudaError_t e = cf::build_grid(c->dtype, dx[t][0], dx[t][1], dx[t][2], dw[t],
-                                                 cats[t]->n, g, tmp, G[t], sms, d_err, d_bar + t, st);
+                                                 cats[t]->n, g, tmp, G[t], sms, d_err, d_ticket + t, c->flags, st);
             if (e) {
                 rc = cuda_fail(e, "grid kernel");
                 goto cleanup;
@@ -979,7 +983,7 @@ int run(Request &q)
         P.want_r = c->want_ravg ? 1 : 0;
         P.wacc = wacc ? 1 : 0;
         P.rlo = resid ? 1 : 0;
-        P.wsum = wacc ? reinterpret_cast<double *>(d_hist + nslots + 8) : nullptr;
+        P.wsum = wacc ? reinterpret_cast<double *>(d_hist + nslots + NTAIL) : nullptr;
         P.rsum = wacc ? P.wsum + nslots : nullptr;
         P.diag = d_diag;
         P.err = d_err;
@@ -1005,7 +1009,7 @@ int run(Request &q)
         }
         CF_CUDA(cudaEventRecord(g_events.ev[2], st), "cudaEventRecord");
         trace.point("pair kernel");
-        CF_CUDA(cudaMemcpyAsync(ho->hist, d_hist, sizeof(unsigned long long) * (nslots + 8 + nacc),
+        CF_CUDA(cudaMemcpyAsync(ho->hist, d_hist, sizeof(unsigned long long) * (nslots + NTAIL + nacc),
                                 cudaMemcpyDeviceToHost, st),
                 "D2H results");
     }
@@ -1032,7 +1036,7 @@ int run(Request &q)
         goto cleanup;
     }
     if (ho->err & cf::ERR_TIMEOUT) {
-        rc = fail(CF_ETIMEOUT, "a bounded device wait (table copy or gridding barrier) gave up");
+        rc = fail(CF_ETIMEOUT, "a bounded device wait (table copy or gridding stage) gave up");
         goto cleanup;
     }
     if (ho->err) {
@@ -1044,7 +1048,7 @@ int run(Request &q)
         for (int k = 0; k < nslots; ++k)
             res->npairs[k] = ho->hist[k] * mult;
         if (wacc) {
-            const double *ws = reinterpret_cast<const double *>(ho->hist + nslots + 8);
+            const double *ws = reinterpret_cast<const double *>(ho->hist + nslots + NTAIL);
             const double *rs = ws + nslots;
             for (int k = 0; k < nslots; ++k) {
                 const double wk = ws[k] * (double)mult, rk = rs[k] * (double)mult;
@@ -1658,8 +1662,8 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     bump.base = (char *)scratch;
     unsigned long long *bbox_keys = bump.take<unsigned long long>(6);
     unsigned *d_err = bump.take<unsigned>(1);
-    unsigned *d_ctr = bump.take<unsigned>(4);  // [0] item counter, [1] kept column pairs, [2, 3] gridding barriers
-    unsigned *d_bar = d_ctr + 2;
+    unsigned *d_ctr = bump.take<unsigned>(6);  // [0] item counter, [1] kept column pairs, [2 .. 5] gridding tickets
+    unsigned long long *d_ticket = reinterpret_cast<unsigned long long *>(d_ctr + 2);
     unsigned long long *d_hist = bump.take<unsigned long long>(cf::NB_MAX);
     unsigned long long *d_diag = bump.take<unsigned long long>(4);
     float *d_thr = bump.take<float>(2 * (cf::NB_MAX + 1));
@@ -1783,13 +1787,13 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     g.inv_w[2] = g.nz / std::max(g.extent[2], 1e-300);
     finish_geom(g);
 
-    if ((e = cudaMemsetAsync(d_ctr, 0, 4 * sizeof(unsigned), st)) ||
+    if ((e = cudaMemsetAsync(d_ctr, 0, 6 * sizeof(unsigned), st)) ||
         (e = cudaMemsetAsync(d_hist, 0, sizeof(unsigned long long) * nb, st)) ||
         (e = cudaMemsetAsync(d_diag, 0, sizeof(unsigned long long) * 4, st)))
         return cuda_fail(e, "memset");
     for (int t = 0; t < ncat; ++t)
         if ((e = cf::build_grid(c->dtype, cats[t]->x, cats[t]->y, cats[t]->z, nullptr, cats[t]->n,
-                                g, tmp, G[t], sms, d_err, d_bar + t, st)))
+                                g, tmp, G[t], sms, d_err, d_ticket + t, 0u, st)))
             return cuda_fail(e, "grid kernels");
     if (autocorr)
         G[1] = G[0];
@@ -1868,7 +1872,7 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     if (h.err & cf::ERR_COORD)
         return fail(CF_EINVAL, "coordinate outside [0, boxsize) or non-finite");
     if (h.err & cf::ERR_TIMEOUT)
-        return fail(CF_ETIMEOUT, "a bounded device wait (table copy or gridding barrier) gave up");
+        return fail(CF_ETIMEOUT, "a bounded device wait (table copy or gridding stage) gave up");
     if (h.err)
         return fail(CF_EDEVICE, "kernel reported an internal inconsistency");
     const uint64_t mult = autocorr ? 2u : 1u;

@@ -147,12 +147,13 @@ __device__ __forceinline__ uint32_t block_sum(uint32_t v, uint32_t *red)
 template <class T>
 __device__ __forceinline__ void assign_points(const T *__restrict__ x, const T *__restrict__ y,
                                               const T *__restrict__ z, long long n, const Geom &g,
-                                              uint32_t *cell_of, uint32_t *slot, uint32_t *count, unsigned *err)
+                                              uint32_t *cell_of, uint32_t *slot, uint32_t *count, unsigned *err,
+                                              unsigned blk, unsigned nblk)
 {
     const int lane = threadIdx.x & 31;
-    const long long stride = (long long)gridDim.x * blockDim.x;
+    const long long stride = (long long)nblk * blockDim.x;
     // every lane of a warp runs the same number of iterations (warp-wide match)
-    const long long first = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+    const long long first = (long long)blk * blockDim.x + (threadIdx.x & ~31);
     for (long long base = first; base < n; base += stride) {
         const long long p = base + lane;
         const bool live = p < n;
@@ -510,49 +511,75 @@ struct GridArgs {
     Geom g;
     GridTemps t;
     Gridded out;
-    unsigned *err, *bar;  // error word; arrivals at the grid barriers (zero before the launch)
+    unsigned *err;
+    unsigned long long *tickets;  // low half: handed out, high half: finished (zero before the launch)
+    int stall;                    // diagnostic: wait for a ticket that does not exist, 1 ms at most
 };
 
-// Barrier of the whole (cooperatively launched) grid: arrive, then wait until the
-// count reaches goal, at most limit_s seconds: 2, but 300 at the first barrier, where
-// blocks may still wait for another call's kernels to leave the SMs.  False in every thread of the block if the wait
-// gave up (the error word says so; no later kernel touches the results).
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned goal, unsigned *err,
-                                             unsigned limit_s = 2u)
+// The stages of a launch are split into one ticket per block.  Blocks take the tickets in
+// order, a stage's after all of the stage before, and begin one when every ticket of the
+// earlier stages is finished: those were taken before it, by blocks that are running, so
+// nobody waits for a block that has not started (its place may be held by another
+// kernel for any time; the running blocks then take its tickets).
+
+// A block's ticket: share blk of the stage.
+struct Ticket {
+    unsigned stage, blk;
+};
+
+// Finishes the block's ticket (but for the first call) and takes the next, t; false in
+// every thread if the wait for the earlier stages gave up (the error word says so; no
+// later kernel touches the results).  The limit is 20 s of the GPU's timer and a million
+// tries: the timer runs on while another process has the GPU.  One atomic finishes and
+// takes: two words cost 1 us more per stage.
+__device__ __forceinline__ bool next_ticket(const GridArgs &A, bool first, Ticket &t)
 {
-    __syncthreads();
+    __shared__ Ticket s_t;
     bool ok = true;
+    __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(bar, 1u);
-        const uint64_t t0 = global_ns();
-        for (unsigned it = 0;; ++it) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= goal)
-                break;
-            if ((it & 63u) == 63u && global_ns() - t0 > limit_s * 1000000000ull) {
-                atomicOr(err, ERR_TIMEOUT);
-                ok = false;
-                break;
+        unsigned long long v = atomicAdd(A.tickets, first ? 1ull : (1ull << 32) + 1ull);
+        unsigned stage = first ? 0u : t.stage, blk = (unsigned)v - stage * gridDim.x;
+        for (; blk >= gridDim.x; blk -= gridDim.x)
+            ++stage;
+        if (!first)
+            v += 1ull << 32;
+        const unsigned goal = stage * gridDim.x;  // the tickets of the earlier stages
+        uint64_t t0 = 0;
+        for (unsigned it = 0; (unsigned)(v >> 32) < goal || (A.stall && goal); ++it) {
+            if ((it & 63u) == 63u) {
+                const uint64_t now = global_ns();
+                t0 = t0 ? t0 : now;
+                if (A.stall ? now - t0 > 1000000ull : it >= 1u << 20 && now - t0 > 20000000000ull) {
+                    atomicOr(A.err, ERR_TIMEOUT);
+                    ok = false;
+                    break;
+                }
             }
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(A.tickets) : "memory");
         }
         __threadfence();
+        s_t = Ticket{stage, blk};
     }
-    return !__syncthreads_or(!ok);
+    ok = !__syncthreads_or(!ok);
+    t = s_t;
+    return ok;
 }
 
-// One catalogue's gridding in one cooperative launch; the stages are separated by
-// grid barriers:
+// One catalogue's gridding in one launch; its stages:
 //   clear the cell counts | cell and slot of every point | padded size of every
 //   column, each block over a range of columns | offsets, padding, chunk_col |
 //   scatter into cells | rank the cells' entries, write the outputs and column boxes
-// Bound: latency (barriers of 1.5 us, dependent loads) for small catalogues, the
-// scattered reads of x and y by the ranked order for large ones.  Measured, with ten
-// kernels before, one per stage and with conversions in the binary64 pipe: 20,000
+// Bound: latency (waits of 1.5 us between the stages, dependent loads) for small
+// catalogues, the scattered reads of x and y by the ranked order for large ones.  Measured,
+// with ten kernels before, one per stage and with conversions in the binary64 pipe: 20,000
 // points 36 us of kernels and as much in gaps -> 18 us; 1.2M 113 -> 73 us; 12M
 // weighted with residuals 2.2 -> 1.5 ms (k_sort 1,137 -> 850 us by ranking small cells
-// together and claiming up to 32 at a time).
+// together and claiming up to 32 at a time).  A cooperative launch with barriers of the whole
+// grid in the place of the tickets took as long (100,000 to 12M points: within 3 us), but two
+// of them must not run at once: 40 calls with 300,000 points on each of four streams
+// 31.6 ms so, 29.2 ms with tickets.
 template <class T>
 __global__ void __launch_bounds__(SORT_THREADS) k_grid(const __grid_constant__ GridArgs A)
 {
@@ -562,84 +589,94 @@ __global__ void __launch_bounds__(SORT_THREADS) k_grid(const __grid_constant__ G
     const Geom &g = A.g;
     const T *x = (const T *)A.x, *y = (const T *)A.y, *z = (const T *)A.z;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = SORT_THREADS / 32;
-    const unsigned nblk = gridDim.x, blk = blockIdx.x;
-    const long long nc = g.ncells, stride = (long long)nblk * SORT_THREADS, first = (long long)blk * SORT_THREADS + tid;
+    const unsigned nblk = gridDim.x;
+    const long long nc = g.ncells, stride = (long long)nblk * SORT_THREADS;
     uint32_t *counts = A.t.counts, *start = A.out.cell_start;
 
-    for (long long q = first; q <= nc; q += stride)  // + the sort's claim counter
-        counts[q] = 0u;
-    for (long long q = first; q < g.ncols; q += stride)
-        A.out.colbox[q] = empty_box();
-    if (!grid_barrier(A.bar, nblk, A.err, 300u))
-        return;
-    assign_points<T>(x, y, z, A.n, g, A.t.cell_of, A.t.slot, counts, A.err);
-    if (!grid_barrier(A.bar, 2u * nblk, A.err))
-        return;
-
-    // this block's columns: a warp per column adds up its cells
-    const int c0 = (int)((long long)g.ncols * blk / nblk), c1 = (int)((long long)g.ncols * (blk + 1) / nblk);
-    uint32_t mine = 0;
-    for (int col = c0 + wid; col < c1; col += nwarp) {
-        uint32_t tot = 0;
-        for (int q = lane; q < g.nz; q += 32)
-            tot += counts[(long long)col * g.nz + q];
-        tot = __reduce_add_sync(FULL, tot);
-        if (lane == 0) {
-            A.t.coltot[col] = tot;
-            mine += (tot + COL_PAD - 1u) & ~(COL_PAD - 1u);
-        }
-    }
-    mine = block_sum(lane == 0 ? mine : 0u, s_red);
-    if (tid == 0)
-        A.t.bsum[blk] = mine;
-    if (!grid_barrier(A.bar, 3u * nblk, A.err))
-        return;
-
-    uint32_t base = 0;
-    for (unsigned q = tid; q < blk; q += SORT_THREADS)
-        base += __ldcg(A.t.bsum + q);
-    base = block_sum(base, s_red);
-    for (int r0 = c0; r0 < c1; r0 += SORT_THREADS) {
-        const int col = r0 + tid;
-        const uint32_t tot = col < c1 ? A.t.coltot[col] : 0u;
-        s_off[tid] = base + block_exclusive_scan((tot + COL_PAD - 1u) & ~(COL_PAD - 1u), s_scan, &s_tot);
-        __syncthreads();
-        for (int k = wid; k < min(SORT_THREADS, c1 - r0); k += nwarp) {
-            uint32_t off = s_off[k];
-            const uint32_t s = off;
-            const long long cell = (long long)(r0 + k) * g.nz;
-            for (int q0 = 0; q0 < g.nz; q0 += 32) {
-                const uint32_t v = q0 + lane < g.nz ? counts[cell + q0 + lane] : 0u;
-                uint32_t incl = v;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t t = __shfl_up_sync(FULL, incl, o);
-                    if (lane >= o)
-                        incl += t;
+    Ticket t;
+    for (bool begin = true; next_ticket(A, begin, t); begin = false) {
+        const unsigned blk = t.blk;
+        const long long first = (long long)blk * SORT_THREADS + tid;
+        // this ticket's columns (stages 2 and 3)
+        const int c0 = (int)((long long)g.ncols * blk / nblk), c1 = (int)((long long)g.ncols * (blk + 1) / nblk);
+        switch (t.stage) {
+        case 0:
+            for (long long q = first; q <= nc; q += stride)  // + the sort's claim counter
+                counts[q] = 0u;
+            for (long long q = first; q < g.ncols; q += stride)
+                A.out.colbox[q] = empty_box();
+            break;
+        case 1:
+            assign_points<T>(x, y, z, A.n, g, A.t.cell_of, A.t.slot, counts, A.err, blk, nblk);
+            break;
+        case 2: {  // a warp per column adds up its cells
+            uint32_t mine = 0;
+            for (int col = c0 + wid; col < c1; col += nwarp) {
+                uint32_t tot = 0;
+                for (int q = lane; q < g.nz; q += 32)
+                    tot += counts[(long long)col * g.nz + q];
+                tot = __reduce_add_sync(FULL, tot);
+                if (lane == 0) {
+                    A.t.coltot[col] = tot;
+                    mine += (tot + COL_PAD - 1u) & ~(COL_PAD - 1u);
                 }
-                if (q0 + lane < g.nz)
-                    start[cell + q0 + lane] = off + incl - v;
-                off += __shfl_sync(FULL, incl, 31);
             }
-            const uint32_t e = s + ((off - s + COL_PAD - 1u) & ~(COL_PAD - 1u));
-            pad_column(A.out, r0 + k, s, e, e - off, lane);
-            if (r0 + k == g.ncols - 1 && lane == 0)
-                start[nc] = e;
+            mine = block_sum(lane == 0 ? mine : 0u, s_red);
+            if (tid == 0)
+                A.t.bsum[blk] = mine;
+            break;
         }
-        base += s_tot;
-        __syncthreads();
+        case 3: {
+            uint32_t base = 0;
+            for (unsigned q = tid; q < blk; q += SORT_THREADS)
+                base += __ldcg(A.t.bsum + q);
+            base = block_sum(base, s_red);
+            for (int r0 = c0; r0 < c1; r0 += SORT_THREADS) {
+                const int col = r0 + tid;
+                const uint32_t tot = col < c1 ? A.t.coltot[col] : 0u;
+                s_off[tid] = base + block_exclusive_scan((tot + COL_PAD - 1u) & ~(COL_PAD - 1u), s_scan, &s_tot);
+                __syncthreads();
+                for (int k = wid; k < min(SORT_THREADS, c1 - r0); k += nwarp) {
+                    uint32_t off = s_off[k];
+                    const uint32_t s = off;
+                    const long long cell = (long long)(r0 + k) * g.nz;
+                    for (int q0 = 0; q0 < g.nz; q0 += 32) {
+                        const uint32_t v = q0 + lane < g.nz ? counts[cell + q0 + lane] : 0u;
+                        uint32_t incl = v;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const uint32_t u = __shfl_up_sync(FULL, incl, o);
+                            if (lane >= o)
+                                incl += u;
+                        }
+                        if (q0 + lane < g.nz)
+                            start[cell + q0 + lane] = off + incl - v;
+                        off += __shfl_sync(FULL, incl, 31);
+                    }
+                    const uint32_t e = s + ((off - s + COL_PAD - 1u) & ~(COL_PAD - 1u));
+                    pad_column(A.out, r0 + k, s, e, e - off, lane);
+                    if (r0 + k == g.ncols - 1 && lane == 0)
+                        start[nc] = e;
+                }
+                base += s_tot;
+                __syncthreads();
+            }
+            break;
+        }
+        case 4:
+            for (long long p = first; p < A.n; p += stride) {
+                const uint32_t q = start[A.t.cell_of[p]] + A.t.slot[p];
+                A.t.tmp_idx[q] = (int)p;
+                A.t.tmp_key[q] = order_key(__double_as_longlong(to_f64(z[p])));
+            }
+            break;
+        case 5:  // the cells are claimed one run at a time: after this ticket none is left
+            sort_cells<T>(x, y, A.w, nc, g, counts, A.t.tmp_idx, A.t.tmp_key, A.out, counts + nc, s_ent);
+            return;
+        default:  // a block that began when all was handed out
+            return;
+        }
     }
-    if (!grid_barrier(A.bar, 4u * nblk, A.err))
-        return;
-
-    for (long long p = first; p < A.n; p += stride) {
-        const uint32_t q = start[A.t.cell_of[p]] + A.t.slot[p];
-        A.t.tmp_idx[q] = (int)p;
-        A.t.tmp_key[q] = order_key(__double_as_longlong(to_f64(z[p])));
-    }
-    if (!grid_barrier(A.bar, 5u * nblk, A.err))
-        return;
-    sort_cells<T>(x, y, A.w, nc, g, counts, A.t.tmp_idx, A.t.tmp_key, A.out, counts + nc, s_ent);
 }
 
 // Bounding box, on order-preserving integer keys (binary64 compares would hold the
@@ -918,51 +955,8 @@ __global__ void __launch_bounds__(256) kb_padfill(const GridBatch B)
                    S.out.cell_start[(long long)(col + 1) * g.nz], S.pad[col], threadIdx.x & 31);
 }
 
-// Gridding launches of one device run one after another, whatever their streams: two
-// grids half resident each would wait for one another.  One event per context (it dies
-// with its context: after a device reset the context has a new id), kept for the life
-// of the process.
-struct GridOrder {
-    std::mutex mu;
-    unsigned long long ctx[64] = {};
-    cudaEvent_t done[64] = {};
-    int next = 0;
-};
-GridOrder g_order;
-
-template <class F>
-cudaError_t in_order(cudaStream_t st, F &&launch)
-{
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    int dev = 0;
-    cudaError_t e = cudaStreamIsCapturing(st, &cap);
-    if (e || (e = cudaGetDevice(&dev)))
-        return e;
-    unsigned long long id = 0;
-    if (cap != cudaStreamCaptureStatusNone)  // an event recorded here would belong to the capture
-        return launch();
-    if (!current_context_id(dev, id))
-        id = ~(unsigned long long)dev;
-    std::lock_guard<std::mutex> lock(g_order.mu);
-    int k = 0;
-    while (k < 64 && !(g_order.done[k] && g_order.ctx[k] == id))
-        ++k;
-    if (k < 64) {
-        e = cudaStreamWaitEvent(st, g_order.done[k], 0);
-    } else {
-        k = g_order.next;
-        g_order.next = (k + 1) % 64;
-        g_order.ctx[k] = id;
-        g_order.done[k] = nullptr;
-        e = cudaEventCreateWithFlags(&g_order.done[k], cudaEventDisableTiming);
-    }
-    if (!e)
-        e = launch();
-    return e ? e : cudaEventRecord(g_order.done[k], st);
-}
-
 template <class T>
-cudaError_t build_grid_t(GridArgs &A, int sms, cudaStream_t st)
+cudaError_t build_grid_t(const GridArgs &A, int sms, cudaStream_t st)
 {
     int occ = 0;
     const cudaError_t e = occupancy(k_grid<T>, 0, occ);
@@ -970,17 +964,11 @@ cudaError_t build_grid_t(GridArgs &A, int sms, cudaStream_t st)
         return e;
     if (occ < 1)
         return cudaErrorInvalidConfiguration;
-    // a thread per point or cell, a warp per column; all blocks resident, as the barriers
-    // need
+    // a thread per point or cell, a warp per column; no more blocks than fit at once
     const long long work = std::max(A.n, std::max(A.g.ncells, 32ll * A.g.ncols));
-    long long blocks = std::min<long long>((long long)sms * occ, (work + SORT_THREADS - 1) / SORT_THREADS);
-    if (blocks < 1)
-        blocks = 1;
-    void *args[] = {&A};
-    return in_order(st, [&]() {
-        return cudaLaunchCooperativeKernel((const void *)k_grid<T>, dim3((unsigned)blocks), dim3(SORT_THREADS), args,
-                                           0, st);
-    });
+    const long long blocks = std::min<long long>((long long)sms * occ, (work + SORT_THREADS - 1) / SORT_THREADS);
+    k_grid<T><<<(unsigned)std::max(blocks, 1ll), SORT_THREADS, 0, st>>>(A);
+    return cudaGetLastError();
 }
 
 template <class T>
@@ -998,10 +986,10 @@ cudaError_t bbox_t(const void *x, const void *y, const void *z, long long n,
 
 cudaError_t build_grid(cf_dtype dt, const void *x, const void *y, const void *z, const double *w,
                        long long n, const Geom &g, const GridTemps &t, Gridded &out, int sms,
-                       unsigned *err, unsigned *bar, cudaStream_t st)
+                       unsigned *err, unsigned long long *tickets, uint32_t flags, cudaStream_t st)
 {
     out.n = n;
-    GridArgs A{x, y, z, w, n, g, t, out, err, bar};
+    const GridArgs A{x, y, z, w, n, g, t, out, err, tickets, (flags & CF_FLAG_DEBUG_STALL_GRID) != 0};
     return dt == CF_FLOAT32 ? build_grid_t<float>(A, sms, st) : build_grid_t<double>(A, sms, st);
 }
 

@@ -25,11 +25,11 @@ bool current_context_id(int dev, unsigned long long &id);
 // Blocks of one gridding launch, at most.
 int grid_max_blocks(int sms);
 
-// Grid one catalogue into `out` (whose arrays are preallocated): one cooperative
-// launch.  *bar must be zero (arrivals at the launch's grid barriers).
+// Grid one catalogue into `out` (whose arrays are preallocated): one launch.  *tickets must
+// be zero.
 cudaError_t build_grid(cf_dtype dt, const void *x, const void *y, const void *z, const double *w,
                        long long n, const Geom &g, const GridTemps &t, Gridded &out, int sms,
-                       unsigned *err, unsigned *bar, cudaStream_t st);
+                       unsigned *err, unsigned long long *tickets, uint32_t flags, cudaStream_t st);
 
 // Bounding box of a catalogue: out6 = order-preserving keys of (min x,y,z, max x,y,z);
 // initialise out6[0..2] to ~0 and out6[3..5] to 0 first.
