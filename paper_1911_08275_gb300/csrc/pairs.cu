@@ -3,13 +3,12 @@
 
 #include <mutex>
 
-#include "grid.cuh"
 #include "launch.cuh"
 #include "pairs.cuh"
 
 namespace cf {
 
-// Per kernel and context: the dynamic shared-memory limit known to be set, and the
+// Per kernel and device: the dynamic shared-memory limit known to be set, and the
 // occupancy per shared-memory size.  The limit is only ever raised, also when the table
 // is full and it has to be asked for: a planned batch launches with the size it was
 // planned for, whatever other calls have needed since.  (Fixed tables: the calls that
@@ -17,8 +16,8 @@ namespace cf {
 namespace {
 struct KernelKey {
     const void *kern;
-    unsigned long long ctx;  // a device reset drops the limits with the context
-    bool operator==(const KernelKey &o) const { return kern == o.kern && ctx == o.ctx; }
+    int dev;
+    bool operator==(const KernelKey &o) const { return kern == o.kern && dev == o.dev; }
 };
 struct LimitEntry {
     KernelKey key;
@@ -62,9 +61,7 @@ cudaError_t occupancy_of(const void *kern, int smem, int &occ, int threads)
     cudaError_t e = cudaGetDevice(&dev);
     if (e)
         return e;
-    KernelKey key{kern, 0};
-    if (!current_context_id(dev, key.ctx))
-        key.ctx = ~(unsigned long long)dev;
+    const KernelKey key{kern, dev};
     std::lock_guard<std::mutex> lock(g_occ_mu);
     if ((e = raise_limit(key, smem)))
         return e;
