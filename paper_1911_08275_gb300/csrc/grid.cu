@@ -640,18 +640,28 @@ __global__ void __launch_bounds__(SORT_THREADS) k_grid(const __grid_constant__ G
                     uint32_t off = s_off[k];
                     const uint32_t s = off;
                     const long long cell = (long long)(r0 + k) * g.nz;
-                    for (int q0 = 0; q0 < g.nz; q0 += 32) {
-                        const uint32_t v = q0 + lane < g.nz ? counts[cell + q0 + lane] : 0u;
-                        uint32_t incl = v;
+                    // four loads in flight: few columns have many cells each (2M points, 49 columns:
+                    // the whole gridding 380 -> 339 us)
+                    for (int q0 = 0; q0 < g.nz; q0 += 128) {
+                        uint32_t v[4];
 #pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const uint32_t u = __shfl_up_sync(FULL, incl, o);
-                            if (lane >= o)
-                                incl += u;
+                        for (int h = 0; h < 4; ++h)
+                            v[h] = q0 + 32 * h + lane < g.nz ? counts[cell + q0 + 32 * h + lane] : 0u;
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            if (q0 + 32 * h >= g.nz)
+                                break;
+                            uint32_t incl = v[h];
+#pragma unroll
+                            for (int o = 1; o < 32; o <<= 1) {
+                                const uint32_t u = __shfl_up_sync(FULL, incl, o);
+                                if (lane >= o)
+                                    incl += u;
+                            }
+                            if (q0 + 32 * h + lane < g.nz)
+                                start[cell + q0 + 32 * h + lane] = off + incl - v[h];
+                            off += __shfl_sync(FULL, incl, 31);
                         }
-                        if (q0 + lane < g.nz)
-                            start[cell + q0 + lane] = off + incl - v;
-                        off += __shfl_sync(FULL, incl, 31);
                     }
                     const uint32_t e = s + ((off - s + COL_PAD - 1u) & ~(COL_PAD - 1u));
                     pad_column(A.out, r0 + k, s, e, e - off, lane);
