@@ -137,9 +137,10 @@ typedef struct {
                             w_i*w_j when weighted; 0 for empty bins.  Binary64
                             mode: exact per-pair terms, sums within 1e-12
                             relative (summation order).  Float32 mode: r from
-                            float32 differences corrected with the
+                            the float32 squared distance corrected with the
                             coordinates' float32 rounding residuals (~3e-7
-                            relative per pair); DD(r) terms rounded to a fixed-
+                            relative per pair, down to Rmax / 32; closer pairs
+                            from corrected differences where that is less); DD(r) terms rounded to a fixed-
                             point grid scaled by the largest weights (2^-22
                             max|w w| / |w w| relative per term), so wsum and
                             ravg agree to 1e-5 relative for weights within a

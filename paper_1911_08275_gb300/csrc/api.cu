@@ -106,6 +106,18 @@ double eps_axis(double r, double M, double Ls)
     return E * (1.0 + u) + u * (r + E);
 }
 
+// Squared separation (ncomp components) below which the float32 mean separations correct the
+// differences with the coordinates' residuals, not the squared sum (sums32.cuh): there
+// the square of the residuals, at most e2, may be more than 6e-7 of it (3e-7 of r).  It
+// stays below Rmax / 32 squared, where a thousandth of the pairs is, unless that is less
+// than four times the residuals.
+float near_sq(int ncomp, double M, double Ls, double R)
+{
+    const double E = 2.0 * U32 * M + (Ls > 0 ? 2.0 * U32 * Ls + U32 * M : 0.0);
+    const double e2 = 1.1 * ncomp * E * E;
+    return f32_up(std::min(e2 / 6e-7, std::max(R * R / 1024.0, 16.0 * e2)));
+}
+
 // Bound on |d2~(float32) - d2(canonical binary64)| for squared separations near S
 // (3 components for xi, 2 for rp).  Doubled for safety.
 double band_sq(double S, int ncomp, double M, double Ls, double R)
@@ -257,8 +269,9 @@ double lin_table(const float *T, int nthr, int nbins, int ncomp, uint8_t *tab, T
     return fm;
 }
 
-// Both cell shapes, keeping the one whose flagged cells hold less pair mass.
-Tables build_tables(const double *E2, int ne, int ncomp, double M, double Ls, double R, float *T,
+// Both cell shapes, keeping the one whose flagged cells hold less pair mass; then the cells
+// of values below near are flagged too.
+Tables build_tables(const double *E2, int ne, int ncomp, double M, double Ls, double R, float near, float *T,
                     uint8_t *tab)
 {
     Tables tl, tg;
@@ -269,17 +282,24 @@ Tables build_tables(const double *E2, int ne, int ncomp, double M, double Ls, do
     other.resize(cf::LUT_MAX);
     const double fl = lin_table(T, nthr, nbins, ncomp, tab, tl);
     const double fg = log_table(T, nthr, nbins, ncomp, other.data(), tg);
-    if (fl <= fg)
-        return tl;
-    std::memcpy(tab, other.data(), tg.lut_n);
-    return tg;
+    const Tables t = fl <= fg ? tl : tg;
+    if (!t.lin)
+        std::memcpy(tab, other.data(), tg.lut_n);
+    for (int q = 0; q < t.lut_n - 1; ++q) {  // cells that hold values below near
+        const double lo = !t.lin ? bitsf((t.u0s + (uint32_t)q) << t.shift)
+                          : q == 0 ? 0.0 : (q - 0.5) / t.lscale * (1.0 - 1e-12);
+        if (!(lo < near))
+            break;
+        tab[q] = cf::TAB_FLAGGED;
+    }
+    return t;
 }
 
 // The last tables built on this thread, reused when the inputs repeat (a
 // benchmark or an MCMC chain calls with the same bins and box every time).
 struct TableCache {
     bool valid = false;
-    double key[cf::NB_MAX + 1 + 5];
+    double key[cf::NB_MAX + 1 + 6];
     int nkey = 0;
     Tables t;
     float T[2 * (cf::NB_MAX + 1)];
@@ -287,22 +307,22 @@ struct TableCache {
 };
 thread_local TableCache g_tables;
 
-Tables cached_tables(const double *E2, int ne, int ncomp, double M, double Ls, double R, float *T,
+Tables cached_tables(const double *E2, int ne, int ncomp, double M, double Ls, double R, float near, float *T,
                      uint8_t *tab)
 {
     TableCache &c = g_tables;
-    const int nk = ne + 5;
+    const int nk = ne + 6;
     bool hit = c.valid && c.nkey == nk;
-    const double extra[5] = {(double)ne, (double)ncomp, M, Ls, R};
+    const double extra[6] = {(double)ne, (double)ncomp, M, Ls, R, near};
     for (int k = 0; hit && k < ne; ++k)
         hit = c.key[k] == E2[k];
-    for (int k = 0; hit && k < 5; ++k)
+    for (int k = 0; hit && k < 6; ++k)
         hit = c.key[ne + k] == extra[k];
     if (!hit) {
-        c.t = build_tables(E2, ne, ncomp, M, Ls, R, c.T, c.tab);
+        c.t = build_tables(E2, ne, ncomp, M, Ls, R, near, c.T, c.tab);
         for (int k = 0; k < ne; ++k)
             c.key[k] = E2[k];
-        for (int k = 0; k < 5; ++k)
+        for (int k = 0; k < 6; ++k)
             c.key[ne + k] = extra[k];
         c.nkey = nk;
         c.valid = true;
@@ -932,6 +952,7 @@ int run(Request &q)
         // ---- pair kernel parameters and tables, then the staged block
         double M = 0.0, Ls = 0.0;
         base_params(q, g, G[0], G[1], P, M, Ls);
+        P.near = resid ? near_sq(q.kind == 0 ? 3 : 2, M, Ls, R) : 0.0f;
         unsigned long long *h0 = ho->stage;  // host image, at the same offsets
         std::memcpy(h0 + (reinterpret_cast<unsigned long long *>(d_E2) - stage.keys), E2.data(), 8 * E2.size());
         if (q.kind == 1)
@@ -940,7 +961,7 @@ int run(Request &q)
         if (!f64) {
             uint8_t *hb = reinterpret_cast<uint8_t *>(h0);
             const size_t at_lut = d_lut - reinterpret_cast<uint8_t *>(stage.keys);
-            const Tables tb = cached_tables(E2.data(), nb + 1, q.kind == 0 ? 3 : 2, M, Ls, R,
+            const Tables tb = cached_tables(E2.data(), nb + 1, q.kind == 0 ? 3 : 2, M, Ls, R, P.near,
                                             reinterpret_cast<float *>(hb + staged), hb + at_lut);
             P.nthr = tb.nthr;
             P.lut_n = tb.lut_n;
@@ -1490,7 +1511,7 @@ int cf_debug_bin_tables(const double *edges, int nedges, int ncomp, double coord
     std::vector<double> E2(nedges);
     for (int k = 0; k < nedges; ++k)
         E2[k] = edges[k] * edges[k];
-    const Tables tb = build_tables(E2.data(), nedges, ncomp, coord_max, shift_max, rmax, thr, table);
+    const Tables tb = build_tables(E2.data(), nedges, ncomp, coord_max, shift_max, rmax, 0.0f, thr, table);
     info->nthr = tb.nthr;
     info->lut_n = tb.lut_n;
     info->lin = tb.lin;
@@ -1834,7 +1855,7 @@ int noalloc_xi(int autocorr, const cf_catalog *d1, const cf_catalog *d2, const d
     float T[2 * (cf::NB_MAX + 1)];
     uint8_t tab[cf::LUT_MAX];
     if (!f64) {
-        const Tables tb = cached_tables(E2, nb + 1, 3, M, Ls, R, T, tab);
+        const Tables tb = cached_tables(E2, nb + 1, 3, M, Ls, R, 0.0f, T, tab);
         P.nthr = tb.nthr;
         P.lut_n = tb.lut_n;
         P.lut_shift = tb.shift;
@@ -2279,7 +2300,7 @@ int batch_plan(cf_batch *b, cudaStream_t st, const std::vector<std::array<double
         if (!f64) {
             T[k].resize(2 * (nb + 1));
             tab[k].resize(cf::LUT_MAX);
-            tb[k] = build_tables(E2[k].data(), nb + 1, j.q.kind == 0 ? 3 : 2, M, Ls, j.edges.back(),
+            tb[k] = build_tables(E2[k].data(), nb + 1, j.q.kind == 0 ? 3 : 2, M, Ls, j.edges.back(), 0.0f,
                                  T[k].data(), tab[k].data());
             j.P.nthr = tb[k].nthr;
             j.P.lut_n = tb[k].lut_n;

@@ -162,6 +162,7 @@ struct PairParams {
     unsigned long long *diag;  // [0] kept items, [1] evaluations, [2] rechecks, [3] band violations
     unsigned *err;
     unsigned *item_counter;
+    float near;         // rlo: squared separations below it are corrected by their differences
 };
 
 // ----------------------------------------------------------------- device helpers

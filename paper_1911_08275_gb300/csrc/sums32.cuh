@@ -167,7 +167,7 @@ __device__ __noinline__ int settle_sums(const PairParams &P, const unsigned char
 {
     const int lane = threadIdx.x & 31, first = max(0, qn - 32);
     int row = -1, re = 0;
-    float pw = 1.0f, d2 = 0.0f;
+    float pw = 1.0f, dc = 0.0f;
     __syncwarp();
     if (first + lane < qn) {
         const int i = fq->i[first + lane], j = fq->j[first + lane], m = fq->image[first + lane];
@@ -175,17 +175,21 @@ __device__ __noinline__ int settle_sums(const PairParams &P, const unsigned char
         const float *a = P.A.xyz + quad_off((uint32_t)i), *b = P.B.xyz + quad_off((uint32_t)j);
         const float Sx = (float)qx * P.boxf[0], Sy = (float)qy * P.boxf[1], Sz = (float)qz * P.boxf[2];
         const float xh = __fsub_rn(a[0], Sx), yh = __fsub_rn(a[4], Sy), zh = __fsub_rn(a[8], Sz);
-        float dx = __fsub_rn(b[0], xh), dy = __fsub_rn(b[4], yh), dz = __fsub_rn(b[8], zh);
+        const float dx = __fsub_rn(b[0], xh), dy = __fsub_rn(b[4], yh), dz = __fsub_rn(b[8], zh);
+        const float d2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+        dc = d2;
         if (RL) {
             const float *ra = P.A.res + quad_off((uint32_t)i), *rb = P.B.res + quad_off((uint32_t)j);
             const float lx = shifted_residual(ra[0], a[0], Sx, xh, qx, P.boxr[0]);
             const float ly = shifted_residual(ra[4], a[4], Sy, yh, qy, P.boxr[1]);
             const float lz = shifted_residual(ra[8], a[8], Sz, zh, qz, P.boxr[2]);
-            dx = __fadd_rn(dx, __fsub_rn(rb[0], lx));
-            dy = __fadd_rn(dy, __fsub_rn(rb[4], ly));
-            dz = __fadd_rn(dz, __fsub_rn(rb[8], lz));
+            const float ex = __fsub_rn(rb[0], lx), ey = __fsub_rn(rb[4], ly), ez = __fsub_rn(rb[8], lz);
+            dc = __fmaf_rn(2.0f, __fmaf_rn(dz, ez, __fmaf_rn(dy, ey, __fmul_rn(dx, ex))), d2);
+            if (d2 < P.near) {
+                const float cx = __fadd_rn(dx, ex), cy = __fadd_rn(dy, ey), cz = __fadd_rn(dz, ez);
+                dc = __fmaf_rn(cz, cz, __fmaf_rn(cy, cy, __fmul_rn(cx, cx)));
+            }
         }
-        d2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
         if (W)
             pw = __fmul_rn(P.B.ws[j], P.A.ws[i]);
         const int c = thr_count(reinterpret_cast<const float *>(smem + S32_THR), P.nthr, d2);
@@ -199,19 +203,16 @@ __device__ __noinline__ int settle_sums(const PairParams &P, const unsigned char
         }
     }
     if (row >= 0)
-        sum_add<W, RV>(hl, srb, sw, (uint32_t)row, pw, d2);
+        sum_add<W, RV>(hl, srb, sw, (uint32_t)row, pw, dc);
     __syncwarp();
     return re;
 }
 
-// RL: the distance from differences corrected with the coordinates' float32 rounding
-// residuals, d2 = (dx~ + ex)^2 + (dy~ + ey)^2 + (dz~ + ez)^2 (primaries' residuals include
-// the roundings of the shift).  An axis is then off by at most the two roundings of its
-// difference and by a few 2^-48 of the coordinates, less than eps_axis allows, so the
-// same tables and thresholds decide the bin.  The first-order form
-// d2~ + 2 (dx~ ex + dy~ ey + dz~ ez) beside d2~ takes one packed instruction more, and is
-// negative for points closer than their residuals (3e-5 in a box of 420), where its root
-// is NaN; 1.2M x 12M points with weights took 46.9 ms a call so, 45.2 this way.
+// RL: r from the squared distance corrected with the coordinates' float32 rounding
+// residuals, d2 = d2~ + 2 (dx~ ex + dy~ ey + dz~ ez) up to the square of the residuals
+// (primaries' residuals include the roundings of the shift).  Of points no farther apart
+// than their residuals that square is all there is, and the sum negative: pairs with
+// d2~ < near are flagged in the table, and the settling adds up corrected differences.
 template <int PP, bool W, bool RV, bool RL, bool EVALS, int LT>
 struct Sums32 {
     static constexpr int I = 16, CH = I * PP, JS = 128 / I;
@@ -281,6 +282,7 @@ struct Sums32 {
                                                  const u64 (&WI)[PP], int ib, int image, unsigned vmask)
     {
         const u64 LS = pack2(P.lut_scale, P.lut_scale), LM = pack2(LIN_MAGIC, LIN_MAGIC);
+        const u64 TWO = pack2(2.0f, 2.0f);
         const uint32_t lutb = smem_u32(smem + S32_LUT), lut_lo = lutb - LIN_MAGIC_BITS,
                        lut_last = (uint32_t)(P.lut_n - 1), lut_hi = lutb + lut_last;
         const uint32_t p0 = addr + 48u * jj;  // this lane's first quad
@@ -314,19 +316,20 @@ struct Sums32 {
                     lds128<0>(pw4, wv);
 #pragma unroll
                 for (int q = 0; q < PP; ++q) {
-                    float d[4], pw[4];
+                    float d[4], dr[4], pw[4];
                     uint32_t cq[4];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        u64 dx = fsub2(h ? vx.y : vx.x, XH[q]), dy = fsub2(h ? vy.y : vy.x, YH[q]),
-                            dz = fsub2(h ? vz.y : vz.x, ZH[q]);
-                        if (RL) {
-                            dx = fadd2(dx, fsub2(h ? rx.y : rx.x, LX[q]));
-                            dy = fadd2(dy, fsub2(h ? ry.y : ry.x, LY[q]));
-                            dz = fadd2(dz, fsub2(h ? rz.y : rz.x, LZ[q]));
-                        }
+                        const u64 dx = fsub2(h ? vx.y : vx.x, XH[q]), dy = fsub2(h ? vy.y : vy.x, YH[q]),
+                                  dz = fsub2(h ? vz.y : vz.x, ZH[q]);
                         const u64 d2 = ffma2(dz, dz, ffma2(dy, dy, fmul2(dx, dx)));
                         unpack2(d2, d[2 * h], d[2 * h + 1]);
+                        if (RL) {
+                            const u64 c = ffma2(dz, fsub2(h ? rz.y : rz.x, LZ[q]),
+                                                ffma2(dy, fsub2(h ? ry.y : ry.x, LY[q]),
+                                                      fmul2(dx, fsub2(h ? rx.y : rx.x, LX[q]))));
+                            unpack2(ffma2(TWO, c, d2), dr[2 * h], dr[2 * h + 1]);
+                        }
                         if (W)
                             unpack2(fmul2(h ? wv.y : wv.x, WI[q]), pw[2 * h], pw[2 * h + 1]);
                         if (LIN) {
@@ -348,7 +351,7 @@ struct Sums32 {
                             st.n_eval += (((vmask >> q) & 1u) && jt + r >= jlo && jt + r < jhi &&
                                           (!TRI || jt + r > ib + q * I + ii)) ? 1ull : 0ull;
                         const uint32_t e = lds_entry(cq[r]);  // the row: bin, dummy or flagged (-1)
-                        sum_add<W, RV>(st.hl, st.srb, st.sw, e, W ? pw[r] : 1.0f, d[r]);
+                        sum_add<W, RV>(st.hl, st.srb, st.sw, e, W ? pw[r] : 1.0f, RL ? dr[r] : d[r]);
                         fm[q] = push_sign(fm[q], e);  // pair (t, r) ends at bit 4 tend - 1 - (4 t + r)
                     }
                 }

@@ -91,8 +91,13 @@ __device__ __noinline__ int settle_sums_rp(const PairParams &P, unsigned char *s
                 const float lx = shifted_residual(ra[0], a[0], Sx, xh, qx, P.boxr[0]);
                 const float ly = shifted_residual(ra[4], a[4], Sy, yh, qy, P.boxr[1]);
                 const float dx = __fsub_rn(b[0], xh), dy = __fsub_rn(b[4], yh);
-                const float cx = __fadd_rn(dx, __fsub_rn(rb[0], lx)), cy = __fadd_rn(dy, __fsub_rn(rb[4], ly));
-                rp2 = __fmaf_rn(cy, cy, __fmul_rn(cx, cx));
+                const float ex = __fsub_rn(rb[0], lx), ey = __fsub_rn(rb[4], ly);
+                if (rp2 < P.near) {
+                    const float cx = __fadd_rn(dx, ex), cy = __fadd_rn(dy, ey);
+                    rp2 = __fmaf_rn(cy, cy, __fmul_rn(cx, cx));
+                } else {
+                    rp2 = __fmaf_rn(2.0f, __fmaf_rn(dy, ey, __fmul_rn(dx, ex)), rp2);
+                }
             }
             const int k = s / (P.npibins + 1);
             add_slot<W, RV>(P, slots, reinterpret_cast<const float *>(smem + SRP_SR), k, s - k * (P.npibins + 1),
@@ -103,8 +108,9 @@ __device__ __noinline__ int settle_sums_rp(const PairParams &P, unsigned char *s
     return re;
 }
 
-// RL: rp^2 from the differences corrected with the coordinates' float32 rounding
-// residuals, (dx~ + ex)^2 + (dy~ + ey)^2; it also decides the bin (see sums32.cuh).
+// RL: rp^2 corrected to first order with the coordinates' float32 rounding residuals,
+// rp2 = rp2~ + 2 (dx~ ex + dy~ ey), but of pairs with rp2~ < near from corrected
+// differences (see sums32.cuh).
 template <int PP, bool W, bool RV, bool RL, bool EVALS, bool LIN>
 struct SumsRp32 {
     static constexpr int I = 16, CH = I * PP, JS = 128 / I;
@@ -170,7 +176,7 @@ struct SumsRp32 {
                                                  int ib, int image, unsigned vmask)
     {
         const u64 MG = pack2(PI_MAGIC, PI_MAGIC), LS = pack2(P.lut_scale, P.lut_scale),
-                  LM = pack2(LIN_MAGIC, LIN_MAGIC);
+                  LM = pack2(LIN_MAGIC, LIN_MAGIC), TWO = pack2(2.0f, 2.0f);
         const float sc = P.pscale, pband = P.pband;
         const uint32_t npi = (uint32_t)P.npibins, nbu = (uint32_t)P.nbins;
         const uint32_t lutb = smem_u32(smem + CRP_LUT), lut_lo = lutb - LIN_MAGIC_BITS,
@@ -202,15 +208,11 @@ struct SumsRp32 {
                     lds128<0>(pw4, wv);
 #pragma unroll
                 for (int q = 0; q < PP; ++q) {
-                    float r[4], t[4], s[4], w[4], pw[4];
+                    float r[4], rc[4], t[4], s[4], w[4], pw[4];
                     uint32_t cq[4];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        u64 dx = fsub2(h ? vx.y : vx.x, XH[q]), dy = fsub2(h ? vy.y : vy.x, YH[q]);
-                        if (RL) {
-                            dx = fadd2(dx, fsub2(h ? rx.y : rx.x, LX[q]));
-                            dy = fadd2(dy, fsub2(h ? ry.y : ry.x, LY[q]));
-                        }
+                        const u64 dx = fsub2(h ? vx.y : vx.x, XH[q]), dy = fsub2(h ? vy.y : vy.x, YH[q]);
                         const u64 r2 = ffma2(dy, dy, fmul2(dx, dx));
                         float za, zb;
                         unpack2(fsub2(h ? vz.y : vz.x, ZH[q]), za, zb);
@@ -221,6 +223,10 @@ struct SumsRp32 {
                         unpack2(r2, r[2 * h], r[2 * h + 1]);
                         unpack2(s2, s[2 * h], s[2 * h + 1]);
                         unpack2(fsub2(t2, fsub2(s2, MG)), w[2 * h], w[2 * h + 1]);
+                        if (RL)
+                            unpack2(ffma2(TWO, ffma2(dy, fsub2(h ? ry.y : ry.x, LY[q]),
+                                                     fmul2(dx, fsub2(h ? rx.y : rx.x, LX[q]))), r2),
+                                    rc[2 * h], rc[2 * h + 1]);
                         if (W)
                             unpack2(fmul2(h ? wv.y : wv.x, WI[q]), pw[2 * h], pw[2 * h + 1]);
                         if (LIN) {
@@ -252,7 +258,7 @@ struct SumsRp32 {
                         fm[q] = push_sign(fm[q], f);  // pair (t, k) ends at bit 4 tend - 1 - (4 t + k)
                         if ((int)f >= 0 && e < nbu && m < npi)
                             add_slot<W, RV>(P, smem + SLOTS, sr, (int)e, (int)m, W ? pw[k] : 1.0f, st.sw,
-                                            r[k]);
+                                            RL ? rc[k] : r[k]);
                     }
                 }
             }
