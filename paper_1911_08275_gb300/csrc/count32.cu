@@ -21,8 +21,11 @@ __global__ void __launch_bounds__(128) k_neighbours(const __grid_constant__ Pair
 template <int I, int PP, bool EVALS, bool VERIFY, int MINB>
 cudaError_t launch_shape(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st)
 {
-    return P.lut_lin ? launch_tasks<Count32<I, PP, EVALS, VERIFY, 1>, MINB>(P, L, sms, st)
-                     : launch_tasks<Count32<I, PP, EVALS, VERIFY, 0>, MINB>(P, L, sms, st);
+    constexpr bool SL = I == 16 && PP == 2 && !EVALS;  // the default shape
+    return P.lut_lin ? launch_tasks<Count32<I, PP, EVALS, VERIFY, 1>, MINB,
+                                    Count32<I, PP, EVALS, VERIFY, 1, false, SL>>(P, L, sms, st)
+                     : launch_tasks<Count32<I, PP, EVALS, VERIFY, 0>, MINB,
+                                    Count32<I, PP, EVALS, VERIFY, 0, false, SL>>(P, L, sms, st);
 }
 
 }  // namespace

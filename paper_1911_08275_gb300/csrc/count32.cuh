@@ -262,7 +262,7 @@ __device__ __forceinline__ void sweep(const PairParams &P, const unsigned char *
 
 // LT: table cells linear in d2 (1) or on float bits (0), or as the launch's tables
 // say (-1).
-template <int I, int PP, bool EVALS, bool VERIFY, int LT, bool D2 = false>
+template <int I, int PP, bool EVALS, bool VERIFY, int LT, bool D2 = false, bool SL = false>
 struct Count32 {
     using Lay = Lay32<D2>;
     static constexpr int CH = I * PP, NW = Lay::NW, NT = NW * 32;
@@ -324,7 +324,7 @@ struct Count32 {
             return;
         u64 XH[PP], YH[PP], ZH[PP];
         int image = 0;
-        for_windows<128 / I, typename Lay::Ring>(
+        for_windows<128 / I, typename Lay::Ring, SL>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) { image = C.shift(P, k, code, XH, YH, ZH); },
             [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {

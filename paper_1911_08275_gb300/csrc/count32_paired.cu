@@ -24,8 +24,10 @@ bool count32_paired(const PairParams &P, const PairLaunch &L)
 cudaError_t launch_count32_paired(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st)
 {
     L.smem = Lay32<true>::total(P.nbins);
-    return P.lut_lin ? launch_tasks<Count32<16, 2, false, false, 1, true>, 1>(P, L, sms, st)
-                     : launch_tasks<Count32<16, 2, false, false, 0, true>, 1>(P, L, sms, st);
+    return P.lut_lin ? launch_tasks<Count32<16, 2, false, false, 1, true>, 1,
+                                    Count32<16, 2, false, false, 1, true, true>>(P, L, sms, st)
+                     : launch_tasks<Count32<16, 2, false, false, 0, true>, 1,
+                                    Count32<16, 2, false, false, 0, true, true>>(P, L, sms, st);
 }
 
 }  // namespace cf

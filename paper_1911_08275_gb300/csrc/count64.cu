@@ -41,9 +41,9 @@ cudaError_t launch_kind(const PairParams &P, PairLaunch &L, int sms, cudaStream_
 {
     if (P.wacc)
         return L.evals ? launch_tasks<Cull64<KIND, true, true, EV>, 3>(P, L, sms, st)
-                       : launch_tasks<Cull64<KIND, false, true, EV>, 3>(P, L, sms, st);
+                       : launch_tasks<Cull64<KIND, false, true, EV>, 3, Cull64<KIND, false, true, EV, true>>(P, L, sms, st);
     return L.evals ? launch_tasks<Cull64<KIND, true, false, EV>, 3>(P, L, sms, st)
-                   : launch_tasks<Cull64<KIND, false, false, EV>, 3>(P, L, sms, st);
+                   : launch_tasks<Cull64<KIND, false, false, EV>, 3, Cull64<KIND, false, false, EV, true>>(P, L, sms, st);
 }
 
 }  // namespace

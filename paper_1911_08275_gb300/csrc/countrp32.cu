@@ -10,8 +10,10 @@ namespace {
 template <int I, int PP, bool EVALS, bool VERIFY, int MINB>
 cudaError_t launch_shape(const PairParams &P, PairLaunch &L, int sms, cudaStream_t st)
 {
-    return P.lut_lin ? launch_tasks<CountRp32<I, PP, EVALS, VERIFY, 1>, MINB>(P, L, sms, st)
-                     : launch_tasks<CountRp32<I, PP, EVALS, VERIFY, 0>, MINB>(P, L, sms, st);
+    constexpr bool SL = I == 16 && PP == 2 && !EVALS;  // the default shape
+    return P.lut_lin
+               ? launch_tasks<CountRp32<I, PP, EVALS, VERIFY, 1>, MINB, CountRp32<I, PP, EVALS, VERIFY, 1, SL>>(P, L, sms, st)
+               : launch_tasks<CountRp32<I, PP, EVALS, VERIFY, 0>, MINB, CountRp32<I, PP, EVALS, VERIFY, 0, SL>>(P, L, sms, st);
 }
 
 }  // namespace

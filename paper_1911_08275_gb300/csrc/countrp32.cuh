@@ -156,7 +156,7 @@ __device__ __noinline__ int verify_rp(const PairParams &P, const unsigned char *
 
 // LT: table cells linear in rp^2 (1) or on float bits (0), or as the launch's tables
 // say (-1).
-template <int I, int PP, bool EVALS, bool VERIFY, int LT>
+template <int I, int PP, bool EVALS, bool VERIFY, int LT, bool SL = false>
 struct CountRp32 {
     static constexpr int CH = I * PP, JS = 128 / I;
     struct State {
@@ -315,7 +315,7 @@ struct CountRp32 {
             return;
         u64 XH[PP], YH[PP], ZH[PP];
         int image = 0;
-        for_windows<JS, RingXYZ>(
+        for_windows<JS, RingXYZ, SL>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) { image = C.shift(P, k, code, XH, YH, ZH); },
             [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {

@@ -133,7 +133,7 @@ __device__ __noinline__ void eval64(const PairParams &P, unsigned char *smem, co
 // the CTA's warps.  KIND 1: DD(rp, pi), P.hcopies copies of nbins * npibins words.
 // WACC: binary64 sums [copy][slot][w, r w] (DD(r): one copy per warp).  EV: pairs per
 // lane of one evaluation.
-template <int KIND, bool EVALS, bool WACC, int EV>
+template <int KIND, bool EVALS, bool WACC, int EV, bool SL = false>
 struct Cull64 {
     static constexpr int I = 16, PP = 2, CH = I * PP, JS = 128 / I;
     struct State {
@@ -216,7 +216,7 @@ struct Cull64 {
             return;
         u64 XH[PP], YH[PP], ZH[PP];
         int image = 0;
-        for_windows<JS, RingXYZ>(
+        for_windows<JS, RingXYZ, SL>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) { image = C.shift(P, k, code, XH, YH, ZH); },
             [&](uint32_t addr, int j0, int j1, int jlo, int jhi, bool tri) {

@@ -14,8 +14,9 @@ cudaError_t launch_kind(const PairParams &P, PairLaunch &L, int sms, cudaStream_
     if (L.evals)
         return P.lut_lin ? launch_tasks<Sums32<PP, W, RV, RL, true, 1>, 2>(P, L, sms, st)
                          : launch_tasks<Sums32<PP, W, RV, RL, true, 0>, 2>(P, L, sms, st);
-    return P.lut_lin ? launch_tasks<Sums32<PP, W, RV, RL, false, 1>, 2>(P, L, sms, st)
-                     : launch_tasks<Sums32<PP, W, RV, RL, false, 0>, 2>(P, L, sms, st);
+    return P.lut_lin
+               ? launch_tasks<Sums32<PP, W, RV, RL, false, 1>, 2, Sums32<PP, W, RV, RL, false, 1, true>>(P, L, sms, st)
+               : launch_tasks<Sums32<PP, W, RV, RL, false, 0>, 2, Sums32<PP, W, RV, RL, false, 0, true>>(P, L, sms, st);
 }
 
 }  // namespace

@@ -213,7 +213,7 @@ __device__ __noinline__ int settle_sums(const PairParams &P, const unsigned char
 // (primaries' residuals include the roundings of the shift).  Of points no farther apart
 // than their residuals that square is all there is, and the sum negative: pairs with
 // d2~ < near are flagged in the table, and the settling adds up corrected differences.
-template <int PP, bool W, bool RV, bool RL, bool EVALS, int LT>
+template <int PP, bool W, bool RV, bool RL, bool EVALS, int LT, bool SL = false>
 struct Sums32 {
     static constexpr int I = 16, CH = I * PP, JS = 128 / I;
     using Lay = SumLayout<W, RV, RL>;
@@ -410,7 +410,7 @@ struct Sums32 {
             }
         }
         int image = 0;
-        for_windows<JS, Ring>(
+        for_windows<JS, Ring, SL>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) {
                 image = C.shift(P, k, code, XH, YH, ZH);

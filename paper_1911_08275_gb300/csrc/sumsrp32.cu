@@ -13,8 +13,9 @@ cudaError_t launch_kind(const PairParams &P, PairLaunch &L, int sms, cudaStream_
     if (L.evals)
         return P.lut_lin ? launch_tasks<SumsRp32<2, W, RV, RL, true, true>, 3>(P, L, sms, st)
                          : launch_tasks<SumsRp32<2, W, RV, RL, true, false>, 3>(P, L, sms, st);
-    return P.lut_lin ? launch_tasks<SumsRp32<2, W, RV, RL, false, true>, 3>(P, L, sms, st)
-                     : launch_tasks<SumsRp32<2, W, RV, RL, false, false>, 3>(P, L, sms, st);
+    return P.lut_lin
+               ? launch_tasks<SumsRp32<2, W, RV, RL, false, true>, 3, SumsRp32<2, W, RV, RL, false, true, true>>(P, L, sms, st)
+               : launch_tasks<SumsRp32<2, W, RV, RL, false, false>, 3, SumsRp32<2, W, RV, RL, false, false, true>>(P, L, sms, st);
 }
 
 }  // namespace

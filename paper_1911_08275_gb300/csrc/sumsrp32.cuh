@@ -111,7 +111,7 @@ __device__ __noinline__ int settle_sums_rp(const PairParams &P, unsigned char *s
 // RL: rp^2 corrected to first order with the coordinates' float32 rounding residuals,
 // rp2 = rp2~ + 2 (dx~ ex + dy~ ey), but of pairs with rp2~ < near from corrected
 // differences (see sums32.cuh).
-template <int PP, bool W, bool RV, bool RL, bool EVALS, bool LIN>
+template <int PP, bool W, bool RV, bool RL, bool EVALS, bool LIN, bool SL = false>
 struct SumsRp32 {
     static constexpr int I = 16, CH = I * PP, JS = 128 / I;
     using Ring = RingSums<W, RL>;
@@ -324,7 +324,7 @@ struct SumsRp32 {
             }
         }
         int image = 0;
-        for_windows<JS, Ring>(
+        for_windows<JS, Ring, SL>(
             P, C.col, ib, C.zlo, C.zhi, (int)part, (int)parts, lane, ring,
             [&](int k, int code) {
                 image = C.shift(P, k, code, XH, YH, ZH);

@@ -13,6 +13,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "launch.cuh"
 #include "pairs.cuh"
@@ -221,17 +222,24 @@ struct Chunk {
 };
 
 // The windows of the chunk [ib, ib + CH) of column col against its neighbours
-// part, part + parts, ...; all lanes call it together.  For every window,
+// part, part + parts, ...; all lanes call it together.  SL: parts is a multiple of
+// nstencil, a part one neighbour (or all, parts 1) and one of parts / nstencil slices
+// of its windows.  For every window,
 // open(k, code) sets the primaries up for the image, then for every piece
 // [j0, j1) of it (j0 a multiple of JS; secondaries outside the window are
 // farther than the reach in z) sweep(addr, j0, j1, jlo, jhi, tri) is called with
 // the shared address of secondary j0.
-template <int JS, class Ring, class Open, class Sw>
+template <int JS, class Ring, bool SL, class Open, class Sw>
 __device__ __forceinline__ void for_windows(const PairParams &P, int col, int ib, float zlo, float zhi,
                                             int part, int parts, int lane, uint32_t ring, Open open, Sw sw)
 {
     const int nn = (int)__ldg(P.nbr_count + col), nz = P.g.nz;
     const Nbr *nb = P.nbr + (long long)col * P.nstencil;
+    const int slices = SL && parts > 1 ? parts / P.nstencil : 1, slice = SL ? part % slices : 0;
+    if (SL) {
+        part /= slices;
+        parts /= slices;
+    }
     const int k0 = P.g.periodic ? -1 : 0, k1 = P.g.periodic ? 1 : 0;
     for (int base = part; base < nn; base += 32 * parts) {
         const int e = base + lane * parts;
@@ -254,6 +262,12 @@ __device__ __forceinline__ void for_windows(const PairParams &P, int col, int ib
                 zwindow(P.B.xyz, cs, nz, P.g.inv_wf[2], wlo, whi, jlo, jhi);
                 if ((code & 16) && k == 0)
                     jlo = max(jlo, ib + 1);
+                if (SL && jlo < jhi) {  // whole steps: a sweep takes all that its steps hold
+                    const int s0 = jlo / JS, n = (jhi - 1) / JS + 1 - s0, per = (n + slices - 1) / slices;
+                    const int a = min(n, per * slice), b = min(n, a + per);
+                    jlo = max(jlo, (s0 + a) * JS);
+                    jhi = min(jhi, (s0 + b) * JS);
+                }
             }
             unsigned m = __ballot_sync(FULL, jlo < jhi), pm = m;
             if (!m)
@@ -443,8 +457,9 @@ __global__ void __launch_bounds__(32 * path_warps<Path>(), MINB) k_tasks(const _
     Path::fini(P, smem, st);
 }
 
-// Launch k_tasks with L.smem bytes of shared memory per CTA.
-template <class Path, int MINB>
+// Launch k_tasks with L.smem bytes of shared memory per CTA; Sliced: the path's variant for
+// sliced windows (SL), if it has one.
+template <class Path, int MINB, class Sliced = Path>
 cudaError_t launch_tasks(const PairParams &P0, PairLaunch &L, int sms, cudaStream_t st)
 {
     PairParams P = P0;
@@ -457,6 +472,20 @@ cudaError_t launch_tasks(const PairParams &P0, PairLaunch &L, int sms, cudaStrea
         return cudaErrorInvalidConfiguration;
     const long long chunks = (P.A.n + (long long)P.g.ncols * (COL_PAD / 2)) / Path::CH + 1;
     P.parts = task_parts((double)chunks, (double)sms * occ * NW, P.nstencil);
+    if (!std::is_same<Path, Sliced>::value) {
+        const int slices = task_slices((double)chunks, (double)sms * occ * NW, P.nstencil, window_points(P, Path::CH));
+        if (slices > 1) {
+            P.parts = P.nstencil * slices;
+            const cudaError_t es = occupancy(k_tasks<Sliced, MINB>, L.smem, occ, 32 * NW);
+            if (es)
+                return es;
+            if (occ < 1)
+                return cudaErrorInvalidConfiguration;
+            L.blocks = (int)std::min<long long>((long long)sms * occ, (chunks * P.parts + NW - 1) / NW);
+            k_tasks<Sliced, MINB><<<L.blocks, 32 * NW, L.smem, st>>>(P);
+            return cudaGetLastError();
+        }
+    }
     L.blocks = (int)std::max(1ll, std::min<long long>((long long)sms * occ, (chunks * P.parts + NW - 1) / NW));
     k_tasks<Path, MINB><<<L.blocks, 32 * NW, L.smem, st>>>(P);
     return cudaGetLastError();
