@@ -18,6 +18,12 @@ constexpr int MAX_STENCIL = (2 * MAX_REACH + 1) * (2 * MAX_REACH + 1);
 constexpr int WARPS = 8;            // warps per pair-kernel CTA
 constexpr int THREADS = WARPS * 32;
 constexpr unsigned FULL = 0xffffffffu;
+// The shared 32-bit counts are moved on before they can overflow, after some 1e12 pairs of a
+// call: a test build moves them on 2^CF_FLUSH_SHIFT times as often.
+#ifndef CF_FLUSH_SHIFT
+#define CF_FLUSH_SHIFT 0
+#endif
+constexpr unsigned FLUSH_SHIFT = CF_FLUSH_SHIFT;
 
 // Error-word bits written by kernels (read back once per call).
 enum : unsigned {

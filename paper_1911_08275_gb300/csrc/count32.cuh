@@ -345,14 +345,14 @@ struct Count32 {
                     else
                         go(std::false_type{}, std::false_type{});
                 }
-                if (!D2 && st.pending > (1u << 30) / NW) {  // keep every shared u32 count far from overflow
+                if (!D2 && st.pending > (1u << 30) / NW >> FLUSH_SHIFT) {  // keep every shared u32 count far from overflow
                     __syncwarp();
                     warp_flush_shared(reinterpret_cast<uint32_t *>(smem + Lay::HIST) + 32, P.nbins, P.hist,
                                       lane);
                     st.pending = 0;
                 }
             });
-        if (D2 && st.pending > (1u << 30) / NW) {
+        if (D2 && st.pending > (1u << 30) / NW >> FLUSH_SHIFT) {
             __syncwarp();
             flush(P, smem, lane, 1, 0);
             st.pending = 0;

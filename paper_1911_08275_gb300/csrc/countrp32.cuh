@@ -336,7 +336,7 @@ struct CountRp32 {
                         go(std::false_type{}, std::false_type{});
                 }
                 // a warp adds at most 32 to one word per lane pair: keep it below 2^30
-                if (st.pending > (1u << 30) / (32u * WARPS)) {
+                if (st.pending > (1u << 30) / (32u * WARPS) >> FLUSH_SHIFT) {
                     __syncwarp();
                     const int row = P.npibins + 1;
                     uint32_t *hist = reinterpret_cast<uint32_t *>(smem + CRP_HIST) + row;

@@ -230,7 +230,7 @@ struct Cull64 {
     // Keep every shared u32 count far from overflow.
     static __device__ __forceinline__ void flush(const PairParams &P, unsigned char *smem, State &st)
     {
-        if (st.pending < (KIND == 0 ? 1u << 27 : 1u << 22))
+        if (st.pending < (KIND == 0 ? 1u << 27 : 1u << 22) >> FLUSH_SHIFT)
             return;
         const int lane = threadIdx.x & 31;
         uint32_t *hist = reinterpret_cast<uint32_t *>(smem + P.hist_off);
