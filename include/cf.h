@@ -152,8 +152,8 @@ typedef struct {
     double kernel_ms;           /* device time of the pair kernel                 */
     double total_ms;            /* device time of the whole call                  */
     uint64_t n_kernels;         /* kernels the call launched (gridding, bounding
-                                   box, work list, pair kernel; copies and memsets
-                                   excluded)                                      */
+                                   box, neighbour lists, pair kernel; copies and
+                                   memsets excluded)                              */
     int refine_used[3];         /* refinement the call used                        */
     int chunk_used, pp_used;    /* float32 DD(r) kernel shape the call used        */
     int tuned;                  /* 0 no autotuning, 1 this call tuned (timed the

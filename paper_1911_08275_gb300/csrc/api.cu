@@ -534,7 +534,7 @@ constexpr double DEFAULT_COL_POINTS = 1024.0;
 
 // Fewest points per column (both catalogues) the grid keeps: a sparse catalogue
 // in a large box would otherwise get more columns than points, and the
-// gridding and work-list costs grow with the columns.
+// gridding and neighbour-list costs grow with the columns.
 constexpr double MIN_COL_POINTS = 32.0;
 
 // Halve the columns on both axes until there are at most max(1, ntot /

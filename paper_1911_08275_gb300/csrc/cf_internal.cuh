@@ -28,8 +28,7 @@ constexpr unsigned FLUSH_SHIFT = CF_FLUSH_SHIFT;
 // Error-word bits written by kernels (read back once per call).
 enum : unsigned {
     ERR_COORD = 1u,     // non-finite coordinate or outside [0, L) in periodic mode
-    ERR_TIMEOUT = 2u,   // a bounded mbarrier wait gave up
-    ERR_INTERNAL = 4u,  // an index or table inconsistency that must never happen
+    ERR_TIMEOUT = 2u,   // a bounded wait (table copy, gridding stage) gave up
 };
 
 // Lookup-table entry (one byte): 0..nbins-1 -> the bin (the cell lies wholly
@@ -87,7 +86,7 @@ struct Gridded {
     long long n;
     float *xyz;           // float32 coordinates in the grid frame, in quads (quad_off): one address
                           // serves three 16-byte loads
-    float *ws;            // float32 weights (padded columns, 64 floats of slack; NULL without weights)
+    float *ws;            // float32 weights (NULL without weights)
     unsigned *wmax;       // bit pattern of max |w| as float (written by gridding; NULL without weights)
     float *res;           // rounding residuals fl32((X - O) - x~) of the float32 coordinates, in the
                           // quad layout (float32 mean separations from float64 inputs; else NULL)
@@ -200,12 +199,6 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, unsigned by
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
                  "r"(bytes)
                  : "memory");
-}
-
-// Plain arrive (no transaction bytes): completes a phase that carries no copy.
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // Nanoseconds of the GPU's global timer.

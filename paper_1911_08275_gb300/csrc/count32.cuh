@@ -260,8 +260,7 @@ __device__ __forceinline__ void sweep(const PairParams &P, const unsigned char *
     }
 }
 
-// LT: table cells linear in d2 (1) or on float bits (0), or as the launch's tables
-// say (-1).
+// LT: table cells linear in d2 (1) or on float bits (0).
 template <int I, int PP, bool EVALS, bool VERIFY, int LT, bool D2 = false, bool SL = false>
 struct Count32 {
     using Lay = Lay32<D2>;
@@ -334,12 +333,12 @@ struct Count32 {
                         st.n_rck, st.n_viol);
                 };
                 st.pending += (unsigned)((j1 - j0) / (128 / I) + 1) * 4u * PP;
-                if (LT == 1 || (LT < 0 && P.lut_lin)) {
+                if (LT == 1) {
                     if (tri)
                         go(std::true_type{}, std::true_type{});
                     else
                         go(std::false_type{}, std::true_type{});
-                } else if (LT <= 0) {
+                } else {
                     if (tri)
                         go(std::true_type{}, std::false_type{});
                     else

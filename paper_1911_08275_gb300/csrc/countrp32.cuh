@@ -154,8 +154,7 @@ __device__ __noinline__ int verify_rp(const PairParams &P, const unsigned char *
     return c32 != c64 || (c32 && (k32 != k64 || m32 != m64));
 }
 
-// LT: table cells linear in rp^2 (1) or on float bits (0), or as the launch's tables
-// say (-1).
+// LT: table cells linear in rp^2 (1) or on float bits (0).
 template <int I, int PP, bool EVALS, bool VERIFY, int LT, bool SL = false>
 struct CountRp32 {
     static constexpr int CH = I * PP, JS = 128 / I;
@@ -324,12 +323,12 @@ struct CountRp32 {
                                                                     XH, YH, ZH, ib, image, C.vmask);
                 };
                 st.pending += (unsigned)((j1 - j0) / JS + 1) * 4u * PP;
-                if (LT == 1 || (LT < 0 && P.lut_lin)) {
+                if (LT == 1) {
                     if (tri)
                         go(std::true_type{}, std::true_type{});
                     else
                         go(std::false_type{}, std::true_type{});
-                } else if (LT <= 0) {
+                } else {
                     if (tri)
                         go(std::true_type{}, std::false_type{});
                     else

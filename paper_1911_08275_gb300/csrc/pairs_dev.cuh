@@ -54,31 +54,6 @@ __device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c)
 }
 
 // ---------------------------------------------------------------- searches
-// First index p in [0, n) with key(p) >= v (upper = false) or key(p) > v
-// (upper = true); n if none.  Keys must be sorted.  All lanes call it with the
-// same arguments; each round probes 32 positions.
-template <class Key, class V>
-__device__ __forceinline__ int warp_bound(Key key, int n, V v, bool upper, int lane)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int s = (hi - lo + 31) >> 5;
-        const int p = lo + lane * s;
-        bool q = false;
-        if (p < hi) {
-            const V z = key(p);
-            q = upper ? (z <= v) : (z < v);
-        }
-        const int c = __popc(__ballot_sync(FULL, q));
-        if (c == 0)
-            break;
-        const int nlo = lo + (c - 1) * s + 1;
-        hi = min(hi, lo + c * s);
-        lo = nlo;
-    }
-    return lo;
-}
-
 // Bin of a binary64 squared separation: k with E2[k] <= r2 < E2[k+1], else -1.
 // Non-negative doubles order like their bit patterns, so integer compares suffice.
 __device__ __forceinline__ int bin_f64(double r2, const double *E2, int nb)
@@ -107,24 +82,6 @@ __device__ __forceinline__ double canon_r2(const double4_32a &p, const double4_3
     return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
-// The same for an image whose shifts are all zero (canon_comp's adds are then
-// skipped, so the value is bit-identical).  The binary64 sweeps choose between
-// the two once per window: a shift test inside the pair loop is compiled into
-// adds issued under a predicate, which still occupy the narrow binary64 pipe.
-__device__ __forceinline__ double plain_r2(const double4_32a &p, const double4_32a &q)
-{
-    const double dx = __dsub_rn(q.x, p.x), dy = __dsub_rn(q.y, p.y), dz = __dsub_rn(q.z, p.z);
-    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-}
-
-// Binary64 re-evaluation of one pair inside an error band: bin row or -1.
-__device__ __noinline__ int recheck64(const double *E2, int nb, const double4_32a *pa,
-                                      const double4_32a *pb, int i, int j, double Sx, double Sy,
-                                      double Sz)
-{
-    return bin_f64(canon_r2(pa[i], pb[j], Sx, Sy, Sz), E2, nb);
-}
-
 // Debug: does the float32 decision for d2 agree with binary64?  (1 = violation)
 __device__ __noinline__ int verify_pair(float d2, const float *thr, int nthr, int nb,
                                         const double *E2, const double4_32a *pa,
@@ -149,19 +106,8 @@ __device__ __forceinline__ u64 warp_sum_u64(u64 v)
     return v;
 }
 
-// Move one warp's per-lane counts to the global histogram (overflow guard).
-__device__ void warp_flush(uint32_t *hw, int nb, unsigned long long *ghist, int lane)
-{
-    for (int b = 0; b < nb; ++b) {
-        const u64 v = warp_sum_u64(hw[b * 32 + lane]);
-        hw[b * 32 + lane] = 0u;
-        if (lane == 0 && v)
-            atomicAdd(&ghist[b], v);
-    }
-}
-
-// The same for a copy that other warps add to concurrently: each count is read
-// and cleared in one atomic exchange, so no concurrent increment is lost.
+// Move a copy's counts (a word per lane and bin) to the global histogram while other warps
+// add to it: each count is read and cleared in one atomic exchange, so no increment is lost.
 __device__ void warp_flush_shared(uint32_t *hw, int nb, unsigned long long *ghist, int lane)
 {
     for (int b = 0; b < nb; ++b) {
@@ -176,17 +122,6 @@ __device__ void warp_flush_shared(uint32_t *hw, int nb, unsigned long long *ghis
 // larger bit patterns and clamp to the out-of-range entry).
 constexpr float LIN_MAGIC = 8388608.0f;  // 2^23: spacing 1 in [2^23, 2^24)
 constexpr uint32_t LIN_MAGIC_BITS = 0x4b000000u;
-
-// Number of thresholds T[c] <= d2 (T non-decreasing, d2 not NaN), scanning
-// down from the top: flagged cells are dominated by the largest edges (the
-// pair density grows with the separation), where this ends in a step or two.
-__device__ __forceinline__ int thr_count_top(const float *T, int nthr, float d2)
-{
-    int c = nthr;
-    while (c > 0 && T[c - 1] > d2)
-        --c;
-    return c;
-}
 
 // Number of thresholds T[c] <= d2 (T is non-decreasing; NaN counts none).
 __device__ __forceinline__ int thr_count(const float *T, int nthr, float d2)

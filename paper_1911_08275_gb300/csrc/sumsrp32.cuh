@@ -14,8 +14,8 @@
 // box, 14 x 40 bins, weights and mean rp (8.6e7 pairs counted): 5.13 -> 0.90 ms;
 // 1.2M points auto: 79 -> 10.1 ms.  Queueing every pair within reach and evaluating
 // full warps from global memory took 2.09 ms: fourteen gathers of 32 addresses.
-// Two primaries per lane at three CTAs per SM (the compiler spills little): 0.90
-// ms, at two CTAs 1.03, one primary per lane 1.03 and 1.16.
+// Two primaries per lane at three CTAs per SM (200 bytes of spill stores and 300 of loads per
+// thread): 0.90 ms, at two CTAs 1.03, one primary per lane 1.03 and 1.16.
 #pragma once
 
 #include "countrp32.cuh"
