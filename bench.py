@@ -122,7 +122,8 @@ def load_peaks():
 
 PROFILE = os.path.join(ROOT, "profiles", "k_xi32_xi_auto_1.2M_rmax25.md")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1911_08275_gb300", "csrc", f)
-                  for f in ("count32.cuh", "tasks.cuh", "pairs_dev.cuh", "cf_internal.cuh")]
+                  for f in ("count32.cuh", "tasks.cuh", "pairs_dev.cuh", "cf_internal.cuh", "count32.cu",
+                            "count32_paired.cu", "launch.cuh")]
 
 
 def profile_traffic():
