@@ -139,8 +139,8 @@ typedef struct {
                             relative (summation order).  Float32 mode: r from
                             the float32 squared distance corrected with the
                             coordinates' float32 rounding residuals (~3e-7
-                            relative per pair, down to Rmax / 32; closer pairs
-                            from corrected differences where that is less); DD(r) terms rounded to a fixed-
+                            relative per pair; pairs so close that it could be
+                            more than 3e-6 from corrected differences); DD(r) terms rounded to a fixed-
                             point grid scaled by the largest weights (2^-22
                             max|w w| / |w w| relative per term), so wsum and
                             ravg agree to 1e-5 relative for weights within a

@@ -108,14 +108,14 @@ double eps_axis(double r, double M, double Ls)
 
 // Squared separation (ncomp components) below which the float32 mean separations correct the
 // differences with the coordinates' residuals, not the squared sum (sums32.cuh): there
-// the square of the residuals, at most e2, may be more than 6e-7 of it (3e-7 of r).  It
-// stays below Rmax / 32 squared, where a thousandth of the pairs is, unless that is less
-// than four times the residuals.
+// the square of the residuals, at most e2, may be more than 6e-6 of it (3e-6 of r; a hundredth
+// of that for most pairs).  It stays below Rmax / 32 squared, where a thousandth of the
+// pairs is, unless that is less than four times the residuals.
 float near_sq(int ncomp, double M, double Ls, double R)
 {
     const double E = 2.0 * U32 * M + (Ls > 0 ? 2.0 * U32 * Ls + U32 * M : 0.0);
     const double e2 = 1.1 * ncomp * E * E;
-    return f32_up(std::min(e2 / 6e-7, std::max(R * R / 1024.0, 16.0 * e2)));
+    return f32_up(std::min(e2 / 6e-6, std::max(R * R / 1024.0, 16.0 * e2)));
 }
 
 // Bound on |d2~(float32) - d2(canonical binary64)| for squared separations near S

@@ -2,8 +2,9 @@
 
 Two float64 points 1e-8 apart may round to float32 neighbours 3e-5 apart (box of 420) or to
 the same value: the separation then comes from the rounding residuals alone.  Per pair
-r may be off by 1e-10 (a few residuals of at most 1e-4, each rounded to 2^-24 of itself)
-and by a few float32 roundings of r; DD(r) rounds r w to a grid of at most
+r may be off by 1e-10 (a few residuals of at most 1e-4, each rounded to 2^-24 of itself),
+by a few float32 roundings of r and, where only the squared distance is corrected, by
+3e-6 of r; DD(r) rounds r w to a grid of at most
 e_{k+1} max(w w) 2^-19, so by half of that (weights within [0.5, 1.5]: 9 times as much
 relative to the weight).  wsum has the documented 1e-5.
 """
